@@ -1,615 +1,80 @@
-// Chunk gradients (Sec. I): g_{D_i} = sum_{rows r of chunk i} grad l(x_r, y_r, w)
-//                                    = X_i^T (f(X_i w) - y01_i),
-// f = identity (least squares) or the logistic sigmoid, un-normalised as in
-// Sec. I; the loss L = (1/N~) sum_r l(x_r, y_r, w) is fused in.
-//
-// GB300 design: the path is HBM bound (2 flops per element read), so X is read
-// exactly once.  A cluster of CL CTAs owns a contiguous range of rows (a flat
-// partition of all N~ rows, so every SM gets the same amount of X); CTA rank q
-// of the cluster owns the column slice [q*Wc, (q+1)*Wc).  Rows arrive through
-// a ring of S shared-memory stages filled by TMA bulk copies
-// (cp.async.bulk, one per row slice, completion on an mbarrier).  For each
-// stage of RB rows:
-//   pass 1: every thread forms partial dot products of its columns with w;
-//           they are reduced across the CTA (warp shuffles + shared memory)
-//           and, when CL > 1, across the cluster through distributed shared
-//           memory (st.shared::cluster + barrier.cluster);
-//   then:   residual r = f(z) - y01 per row (and the loss term);
-//   pass 2: acc[col] += r * x[row, col] from the same shared-memory stage.
-// acc lives in registers; when the row range crosses into a new chunk the
-// cluster writes its partial chunk gradient to a scratch slot, and a small
-// second kernel adds the (at most a few) partials of every chunk in a fixed
-// order, so results are deterministic.
-//
-// Rows that are not 16-byte multiples, or unaligned X, take the same kernel
-// with plain cooperative loads instead of TMA (use_tma = 0).
-#include <math.h>
-#include <stdlib.h>
-
+// Chunk gradients: the host-side plan, the launches and the reduction of the
+// partial gradients (the gradient kernel and its design: k_chunkgrad.cuh).
 #include <algorithm>
-#include <mutex>
-#include <type_traits>
+#include <atomic>
 
-#include "gc_internal.cuh"
-#include "tc_ptx.cuh"
+#include "k_chunkgrad.cuh"
 
 namespace gc {
 
 namespace {
 
-// the CTA-local mbarrier wrappers are the shared ones (tc_ptx.cuh); the
-// cluster-scope ones below are this kernel's own
-using tcw::mbar_expect_tx;
-using tcw::mbar_init;
-using tcw::mbar_try_wait;
-using tcw::smem_u32;
-
-__device__ __forceinline__ void fence_mbar_init() {
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes,
-                                         uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-          "r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
-  uint32_t out;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(addr), "r"(rank));
-  return out;
-}
-__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
-                   : "memory");
-}
-
-// Load V elements (16 bytes) of a row slice from shared memory as floats.
-template <typename T>
-struct Vec;
-template <>
-struct Vec<float> {
-  static constexpr int V = 4;
-  __device__ static __forceinline__ void load(const float* p, float (&o)[4]) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
-  }
-  __device__ static __forceinline__ uint4 load_raw(const float* p) {
-    return *reinterpret_cast<const uint4*>(p);
-  }
-  __device__ static __forceinline__ void unpack(const uint4& u, float (&o)[4]) {
-    o[0] = __uint_as_float(u.x); o[1] = __uint_as_float(u.y);
-    o[2] = __uint_as_float(u.z); o[3] = __uint_as_float(u.w);
-  }
-  __device__ static __forceinline__ float scalar(const float* p) { return *p; }
-};
-template <>
-struct Vec<__nv_bfloat16> {
-  static constexpr int V = 8;
-  __device__ static __forceinline__ void load(const __nv_bfloat16* p, float (&o)[8]) {
-    unpack(load_raw(p), o);
-  }
-  __device__ static __forceinline__ uint4 load_raw(const __nv_bfloat16* p) {
-    return *reinterpret_cast<const uint4*>(p);
-  }
-  __device__ static __forceinline__ void unpack(const uint4& u, float (&o)[8]) {
-    const uint32_t w[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      o[2 * k] = __uint_as_float(w[k] << 16);
-      o[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
-    }
-  }
-  __device__ static __forceinline__ float scalar(const __nv_bfloat16* p) {
-    return __bfloat162float(*p);
-  }
-};
-
-constexpr int kMaxStages = 4;
-// DSMEM exchange slots: a peer can run at most ~1.5 batches ahead of this CTA
-// (it needs this CTA's sums of batch n + 1 before writing batch n + 4), so
-// four slots keep a slot from being rewritten before it is read.
-constexpr int kZSlots = 4;
-constexpr long long kSpinLimit = 1LL << 31;  // clock cycles (~1 s) per wait
-
-struct CGArgs {
-  const void* X;
-  const float* y;
-  const float* w;
-  int d;          // row length (elements)
-  int Wc;         // columns per CTA slice (multiple of V)
-  int ld_s;       // shared-memory row stride of a stage (elements, multiple of V)
-  int n_c;        // rows per chunk
-  long long Ntil; // rows
-  long long rpc;  // rows per cluster (multiple of RB)
-  int RB;         // rows per stage
-  int S;          // stages
-  int maxt;       // chunk slots per cluster in `parts`
-  int loss;
-  int want_loss;
-  int use_tma;
-  long long spin_limit;  // clock cycles a wait may take before the kernel gives up
-  int stall;             // failure-path test: the loader issues nothing
-  float* parts;        // [clusters][maxt][d]
-  double* loss_parts;  // [clusters]
-  uint32_t* status;
-};
-
-// Arrive on the mbarrier at the same offset in cluster peer `rank`, releasing
-// this thread's prior shared::cluster stores to it.
-__device__ __forceinline__ void mbar_arrive_remote(uint64_t* bar, uint32_t rank) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
-                   mapa(smem_u32(bar), rank))
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait; `cl` selects cluster-scope acquire (remote arrivals).
-__device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                             uint32_t* status, long long limit, bool cl = false) {
-  auto tw = [&]() { return cl ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
-  if (tw()) return true;
-  const long long t0 = clock64();
-  while (!tw()) {
-    if (*abort_flag) return false;
-    if (clock64() - t0 > limit) {
-      atomicOr(status, ST_TIMEOUT);
-      *abort_flag = 1;
-      return false;
-    }
-  }
-  return true;
-}
-__device__ __forceinline__ void consumer_sync(int nthreads) {
-  asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
-}
-
-// Warp sums of R row partials with a halving butterfly: log2(R) exchange
-// levels that each halve the vector, then plain xor levels -- 5 + R - 1
-// shuffles instead of 5 R.  Lane l ends with the warp sum of row l >> (5 - log2 R).
-template <int R>
-__device__ __forceinline__ float warp_sum_rows(const float (&p)[R], int lane) {
-  constexpr int LR = R >= 4 ? 2 : (R >= 2 ? 1 : 0);
-  static_assert((1 << LR) == R, "rows per batch must be 1, 2 or 4");
-  float v[R];
-#pragma unroll
-  for (int j = 0; j < R; ++j) v[j] = p[j];
-#pragma unroll
-  for (int lvl = 0; lvl < LR; ++lvl) {
-    const int off = 16 >> lvl;
-    const int half = R >> (lvl + 1);
-    const bool hi = (lane & off) != 0;
-#pragma unroll
-    for (int j = 0; j < half; ++j) {
-      const float keep = hi ? v[half + j] : v[j];
-      const float send = hi ? v[j] : v[half + j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-    }
-  }
-#pragma unroll
-  for (int lvl = LR; lvl < 5; ++lvl) v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16 >> lvl);
-  return v[0];
-}
-
-// Position in the ring of stages: the stage index and the parity of its phase.
-struct Ring {
-  int s;
-  uint32_t ph;
-  __device__ __forceinline__ void next(int S) {
-    if (++s == S) {
-      s = 0;
-      ph ^= 1u;
-    }
-  }
-};
-
-// NT consumer threads (warps 0 .. NW-1) plus one producer warp (warp NW).
-template <typename T, int CL, int NT, int NVT, int RBM>
-__device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
-  constexpr int V = Vec<T>::V;
-  constexpr int NW = NT / 32;
-  extern __shared__ __align__(128) unsigned char smem[];
-  T* stages = reinterpret_cast<T*>(smem);
-  const size_t stage_elems = (size_t)RBM * a.ld_s;
-  float* red = reinterpret_cast<float*>(smem + a.S * stage_elems * sizeof(T));  // [2][NW][RBM]
-  float* zcl = red + 2 * NW * RBM;                                               // [kZSlots][CL][RBM]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(zcl + kZSlots * CL * RBM + 2);    // 8-byte aligned
-  uint64_t* full = bars;                    // [kMaxStages] data landed
-  uint64_t* empty = bars + kMaxStages;      // [kMaxStages] consumers done with the stage
-  uint64_t* zfull = bars + 2 * kMaxStages;  // [kZSlots] every peer's partial dots arrived
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kMaxStages + kZSlots);
-
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rank = CL > 1 ? (int)cluster_rank() : 0;
-  const long long q = blockIdx.x / CL;
-  const long long r0 = q * a.rpc;
-  const long long r1 = min(r0 + a.rpc, a.Ntil);
-  const int nb = r0 < r1 ? (int)((r1 - r0) / a.RB) : 0;
-  const int c0 = rank * a.Wc;
-  const int nvs = a.Wc / V;  // vectors in this CTA's slice
-  const T* X = static_cast<const T*>(a.X);
-
-  if (tid == 0) {
-    *abort_flag = 0;
-    for (int s = 0; s < a.S; ++s) {
-      mbar_init(&full[s], a.use_tma ? 1 : 32);
-      mbar_init(&empty[s], NW);
-    }
-    for (int z = 0; z < kZSlots; ++z) mbar_init(&zfull[z], CL);
-    fence_mbar_init();
-  }
-  {
-    // Stage bytes the producer never writes -- rows RB..RBM-1, and with TMA
-    // the vectors past the slice -- are zeroed once, so that the consumers
-    // read whole stages without masks (zeros add nothing to either pass).
-    const int vpr = a.ld_s / V;  // 16-byte vectors per stage row
-    const int vfrom = a.use_tma ? nvs : vpr;
-    for (int s = 0; s < a.S; ++s) {
-      uint4* st = reinterpret_cast<uint4*>(stages + (size_t)s * stage_elems);
-      for (int r = 0; r < RBM; ++r)
-        for (int v = (r < a.RB ? vfrom : 0) + tid; v < vpr; v += blockDim.x)
-          st[(size_t)r * vpr + v] = make_uint4(0u, 0u, 0u, 0u);
-    }
-  }
-  __syncthreads();
-  if (CL > 1) cluster_sync_all();  // every peer has started and initialised its barriers
-
-  if (warp == NW) {
-    // ------------------------------------------------------------ producer warp
-    // A batch is issued only while no wait has failed: then every earlier
-    // batch of the stage has landed (its consumers' waits succeeded), so each
-    // stage holds at most one copy in flight and the phases stay in order.
-    // The decision is warp-uniform.
-    const uint32_t row_bytes = (uint32_t)(a.Wc * sizeof(T));
-    int issued = 0;
-    for (int n = 0; n < (a.stall ? 0 : nb); ++n) {
-      const int s = n % a.S;
-      const uint32_t ph = (uint32_t)((n / a.S) & 1);
-      const bool ok = bounded_wait(&empty[s], ph ^ 1, abort_flag, a.status, a.spin_limit);
-      if (!__all_sync(0xffffffffu, ok && !*abort_flag)) break;
-      T* st = stages + s * stage_elems;
-      const long long row = r0 + (long long)n * a.RB;
-      if (a.use_tma) {
-        if (lane == 0) {
-          mbar_expect_tx(&full[s], row_bytes * a.RB);
-          for (int r = 0; r < a.RB; ++r)
-            bulk_g2s(st + (size_t)r * a.ld_s, X + (row + r) * a.d + c0, row_bytes, &full[s]);
-        }
-      } else {
-        // plain loads with bounds (zero fill past d), then every lane arrives
-        for (int r = 0; r < a.RB; ++r) {
-          const T* src = X + (row + r) * a.d;
-          for (int c = lane; c < a.ld_s; c += 32) {
-            const int col = c0 + c;
-            st[(size_t)r * a.ld_s + c] = (c < a.Wc && col < a.d) ? src[col] : T(0.f);
-          }
-        }
-        tcw::mbar_arrive(&full[s]);
-      }
-      issued = n + 1;
-    }
-    // drain: the CTA must not exit with copies in flight
-    if (a.use_tma && lane == 0) {
-      volatile int no_abort = 0;
-      for (int n = max(0, issued - a.S); n < issued; ++n)
-        bounded_wait(&full[n % a.S], (uint32_t)((n / a.S) & 1), &no_abort, a.status, kSpinLimit);
-    }
-  } else {
-    // ------------------------------------------------------------ consumer warps
-    // w and the gradient accumulators as column pairs: the passes use packed
-    // two-wide FMAs (__ffma2_rn, the rounding of two fmaf)
-    constexpr int V2 = V / 2;
-    float2 wv[NVT][V2];
-#pragma unroll
-    for (int u = 0; u < NVT; ++u) {
-      const int v = tid + u * NT;
-#pragma unroll
-      for (int e = 0; e < V; ++e) {
-        const int col = c0 + v * V + e;
-        const float wc = (v < nvs && col < a.d) ? a.w[col] : 0.f;
-        if (e & 1)
-          wv[u][e >> 1].y = wc;
-        else
-          wv[u][e >> 1].x = wc;
-      }
-    }
-    float2 acc[NVT][V2];
-#pragma unroll
-    for (int u = 0; u < NVT; ++u)
-#pragma unroll
-      for (int e = 0; e < V2; ++e) acc[u][e] = make_float2(0.f, 0.f);
-    const long long first_chunk = r0 / a.n_c;
-    long long cur = -1;     // chunk whose gradient acc holds
-    long long next_row = r0;  // first row past chunk `cur` (a batch never straddles chunks: RB | n_c)
-    double loss_acc = 0.0;
-    auto flush = [&](long long chunk) {
-      float* dst = a.parts + ((size_t)q * a.maxt + (size_t)(chunk - first_chunk)) * a.d;
-#pragma unroll
-      for (int u = 0; u < NVT; ++u) {
-        const int v = tid + u * NT;
-        if (v < nvs) {
-#pragma unroll
-          for (int e = 0; e < V; ++e) {
-            const int col = c0 + v * V + e;
-            if (col < a.d) dst[col] = (e & 1) ? acc[u][e >> 1].y : acc[u][e >> 1].x;
-          }
-        }
-      }
-    };
-
-    // Stage access.  Every stage row is NVT * NT vectors long and the parts
-    // the producer never writes are zero, so the reads need no masks.
-    auto wait_stage = [&](const Ring& g) {
-      bounded_wait(&full[g.s], g.ph, abort_flag, a.status, a.spin_limit);
-    };
-    auto from_stage = [&](const Ring& g) {
-      const T* st = stages + (size_t)g.s * stage_elems + tid * V;
-      const int ld = a.ld_s;
-      return [=](int r, int u) { return Vec<T>::load_raw(st + r * ld + u * NT * V); };
-    };
-    // x of a batch copied to registers once (kept from the dot products to pass 2)
-    auto load_x = [&](const Ring& g, uint4 (&xr)[RBM][NVT]) {
-      auto src = from_stage(g);
-#pragma unroll
-      for (int r = 0; r < RBM; ++r)
-#pragma unroll
-        for (int u = 0; u < NVT; ++u) xr[r][u] = src(r, u);
-    };
-    // hand a stage back to the producer (every lane of the warp is done reading it)
-    auto release = [&](const Ring& g) {
-      __syncwarp();
-      if (lane == 0) tcw::mbar_arrive(&empty[g.s]);
-    };
-    // Dot products of batch n, reduced over the CTA (warp butterfly, then
-    // lane-parallel over (warp, row) pairs) and, with clusters, sent to every
-    // peer.  Returns the CTA sums in every lane.
-    auto dots = [&](int n, auto&& xget, float (&z)[RBM]) {
-      // two packed partial sums a row (vectors u even / odd), so that the
-      // FMA chain of a row is a quarter as long
-      float pd[RBM];
-#pragma unroll
-      for (int r = 0; r < RBM; ++r) {
-        float2 p2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
-#pragma unroll
-        for (int u = 0; u < NVT; ++u) {
-          float x[V];
-          Vec<T>::unpack(xget(r, u), x);
-#pragma unroll
-          for (int e = 0; e < V2; ++e)
-            p2[u & 1] = __ffma2_rn(make_float2(x[2 * e], x[2 * e + 1]), wv[u][e], p2[u & 1]);
-        }
-        pd[r] = (p2[0].x + p2[0].y) + (p2[1].x + p2[1].y);
-      }
-      constexpr int kRowShift = 5 - (RBM >= 4 ? 2 : (RBM >= 2 ? 1 : 0));
-      const float ws_ = warp_sum_rows<RBM>(pd, lane);
-      float* redn = red + (n & 1) * NW * RBM;
-      if ((lane & ((1 << kRowShift) - 1)) == 0) redn[warp * RBM + (lane >> kRowShift)] = ws_;
-      consumer_sync(NT);
-      // CTA sums: the NW x RBM partials are spread over the lanes (entry
-      // j*32 + lane is warp (idx % NW) of row idx / NW), summed over aligned
-      // groups of NW lanes, then row r is read from the first lane of its group.
-      constexpr int E = NW * RBM, NCH = (E + 31) / 32;
-      float cs[NCH];
-#pragma unroll
-      for (int j = 0; j < NCH; ++j) {
-        const int idx = j * 32 + lane;
-        float t = idx < E ? redn[(idx % NW) * RBM + idx / NW] : 0.f;
-#pragma unroll
-        for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        cs[j] = t;
-      }
-#pragma unroll
-      for (int r = 0; r < RBM; ++r) z[r] = __shfl_sync(0xffffffffu, cs[(r * NW) / 32], (r * NW) % 32);
-      if (CL > 1 && tid < CL && !*abort_flag) {
-        // thread p writes the CTA sums into peer p's slot and arrives there
-        // (release).  After a failed wait the CTA sends no more: a peer then
-        // never receives more arrivals in one phase than it expects.
-        float* zc = zcl + (n % kZSlots) * CL * RBM;
-        const uint32_t peer = (uint32_t)tid;
-#pragma unroll
-        for (int r = 0; r < RBM; ++r)
-          st_cluster_f32(mapa(smem_u32(zc + rank * RBM + r), peer), z[r]);
-        mbar_arrive_remote(&zfull[n % kZSlots], peer);
-      }
-    };
-    // Cluster sums of batch n once every peer's CTA sums have arrived: lane
-    // p * RBM + r reads peer p's sum of row r, a xor tree adds the peers.
-    auto cluster_sums = [&](int n, float (&z)[RBM]) {
-      bounded_wait(&zfull[n % kZSlots], (uint32_t)((n / kZSlots) & 1), abort_flag, a.status,
-                   a.spin_limit, true);
-      const float* zc = zcl + (n % kZSlots) * CL * RBM;
-      float t = lane < CL * RBM ? zc[lane] : 0.f;
-#pragma unroll
-      for (int o = RBM; o < CL * RBM; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-#pragma unroll
-      for (int r = 0; r < RBM; ++r) z[r] = __shfl_sync(0xffffffffu, t, r);
-    };
-
-    // y of batch n for lane r < RB, loaded two batches ahead (off the
-    // critical path between the dot products and the residuals)
-    auto load_y = [&](int n) {
-      return (lane < a.RB && n < nb) ? __ldg(a.y + r0 + (long long)n * a.RB + lane) : 0.f;
-    };
-    float y0 = load_y(0), y1 = load_y(1);
-    // Residuals, loss and pass 2 (acc += r * x) of batch n from its row sums z.
-    auto finish = [&](int n, const float (&z)[RBM], auto&& xget) {
-      const long long row = r0 + (long long)n * a.RB;
-      if (row >= next_row) {
-        if (cur >= 0) flush(cur);
-#pragma unroll
-        for (int u = 0; u < NVT; ++u)
-#pragma unroll
-          for (int e = 0; e < V2; ++e) acc[u][e] = make_float2(0.f, 0.f);
-        cur = cur < 0 ? first_chunk : cur + 1;
-        next_row = (cur + 1) * a.n_c;
-      }
-      const float yv = y0;
-      y0 = y1;
-      y1 = load_y(n + 2);
-      // ---- residuals: lane r < RBM takes row r (rows past RB are zero
-      // padding whose residual multiplies zeros), then a broadcast
-      float zr = z[0];
-#pragma unroll
-      for (int r = 1; r < RBM; ++r) zr = lane == r ? z[r] : zr;
-      const float mine =
-          a.loss == GC_LSQ ? zr - yv : 1.f / (1.f + __expf(-zr)) - 0.5f * (yv + 1.f);
-      float res[RBM];
-#pragma unroll
-      for (int r = 0; r < RBM; ++r) res[r] = __shfl_sync(0xffffffffu, mine, r);
-      // ---- the loss: lane r < RB of warp 0 takes row r (fp32), one fp64 add per batch
-      if (a.want_loss && rank == 0 && warp == 0) {
-        float lr = 0.f;
-        if (lane < a.RB) {
-          if (a.loss == GC_LSQ) {
-            const float e = zr - yv;
-            lr = 0.5f * e * e;
-          } else {
-            // log(1 + e^t) = max(t, 0) + log(1 + e^-|t|); the fast intrinsics
-            // are accurate to ~1e-6 absolute per row here (1 + e^-|t| lies in
-            // [1, 2]), far below the loss's 1e-5 relative tolerance, and keep
-            // warp 0 from lagging behind the others at every batch
-            const float t = -yv * zr;
-            lr = fmaxf(t, 0.f) + __logf(1.f + __expf(-fabsf(t)));
-          }
-        }
-#pragma unroll
-        for (int o = 2; o > 0; o >>= 1) lr += __shfl_xor_sync(0xffffffffu, lr, o);
-        if (lane == 0) loss_acc += (double)lr;
-      }
-      // ---- pass 2
-#pragma unroll
-      for (int r = 0; r < RBM; ++r) {
-        const float2 rr = make_float2(res[r], res[r]);
-#pragma unroll
-        for (int u = 0; u < NVT; ++u) {
-          float x[V];
-          Vec<T>::unpack(xget(r, u), x);
-#pragma unroll
-          for (int e = 0; e < V2; ++e)
-            acc[u][e] = __ffma2_rn(rr, make_float2(x[2 * e], x[2 * e + 1]), acc[u][e]);
-        }
-      }
-    };
-
-    // x in registers when they fit beside acc and w (fp32 rows; not bf16,
-    // whose unpacked vectors would spill)
-    constexpr bool kXRegs = NVT * RBM * V <= 32;
-    Ring g{0, 0u};
-    if (CL == 1 && kXRegs) {
-      // One pass over the stage: x stays in registers from the dot products to
-      // pass 2, so the stage goes back to the producer as soon as it is read.
-      for (int n = 0; n < nb; ++n, g.next(a.S)) {
-        uint4 xr[RBM][NVT];
-        float z[RBM];
-        wait_stage(g);
-        load_x(g, xr);
-        release(g);
-        auto xget = [&](int r, int u) { return xr[r][u]; };
-        dots(n, xget, z);
-        finish(n, z, xget);
-      }
-    } else if (CL == 1) {
-      for (int n = 0; n < nb; ++n, g.next(a.S)) {
-        float z[RBM];
-        wait_stage(g);
-        dots(n, from_stage(g), z);
-        finish(n, z, from_stage(g));
-        release(g);
-      }
-    } else {
-      // Clusters: batch n + 1's dot products and send run before the wait for
-      // batch n's cluster sums (software pipelining); pass 2 re-reads the
-      // stage, which is handed back afterwards.
-      float znext[RBM];
-      Ring g1 = g;
-      if (nb > 0) {
-        wait_stage(g1);
-        dots(0, from_stage(g1), znext);
-        g1.next(a.S);
-      }
-      for (int n = 0; n < nb; ++n, g.next(a.S), g1.next(a.S)) {
-        if (n + 1 < nb) {
-          wait_stage(g1);
-          dots(n + 1, from_stage(g1), znext);
-        }
-        float z[RBM];
-        cluster_sums(n, z);
-        finish(n, z, from_stage(g));
-        release(g);
-      }
-    }
-    // the reduction kernel may be scheduled now (it waits for this grid to
-    // finish); not earlier, so that work on other streams keeps the SMs' room
-    if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (cur >= 0) flush(cur);
-    if (tid == 0 && rank == 0) a.loss_parts[q] = loss_acc;
-  }
-  if (CL > 1) cluster_sync_all();  // no CTA leaves while a peer may still address it
-}
-
-template <typename T, int CL, int NT, int NVT, int RBM>
-__global__ void __launch_bounds__(NT + 32, 1) k_chunkgrad(CGArgs a) {
-  chunkgrad_body<T, CL, NT, NVT, RBM>(a);
-}
-
 // G[i][col] = sum of the partials of chunk i, clusters in increasing order.
-// Block (x, i): chunk i, columns [x*256, (x+1)*256), one column per thread;
-// the contributing clusters and their slot offsets are computed once per
-// block.  Launched as a programmatic dependent of k_chunkgrad: the blocks are
-// resident before the gradient kernel ends and wait for it here.
-constexpr int kRedMaxParts = 256;
+// Chunk i is the batches [i nbc, (i + 1) nbc) and cluster q took
+// [q bpc, (q + 1) bpc); the first of its clusters may have begun in an earlier
+// chunk (its slot for chunk i is then not slot 0), the others begin inside i.
+// Block (x, i): 1024 columns, four a thread (one 16-byte piece when VEC, else
+// 256 apart).  Memory bound, a few reads per output: the work a thread is what
+// hides the latency (d = 65536, 64 chunks, 26 MB of partials: one column a
+// thread 37 us).  Launched as a programmatic dependent of k_chunkgrad: the
+// blocks are resident before the gradient kernel ends and wait for it here.
+template <bool VEC>
 __global__ void __launch_bounds__(256) k_chunkgrad_reduce(const float* __restrict__ parts,
                                                           const double* __restrict__ loss_parts,
                                                           float* __restrict__ G, double* loss_out,
-                                                          int N, int n_c, int d, long long rpc,
+                                                          int N, int nbc, int d, long long bpc,
                                                           int maxt, int nclusters, long long Ntil) {
-  __shared__ long long s_off[kRedMaxParts];
-  __shared__ int s_np;
   const int i = blockIdx.y;
-  if (threadIdx.x == 0) {
-    const long long qlo = ((long long)i * n_c) / rpc;
-    const long long qhi = ((long long)(i + 1) * n_c - 1) / rpc;
-    int np = 0;
-    for (long long q = qlo; q <= qhi && np < kRedMaxParts; ++q, ++np) {
-      const long long first = (q * rpc) / n_c;
-      s_off[np] = ((long long)q * maxt + (i - first)) * (long long)d;
-    }
-    s_np = np;
-  }
-  __syncthreads();
+  const long long qlo = ((long long)i * nbc) / bpc;
+  const long long qhi = ((long long)(i + 1) * nbc - 1) / bpc;
+  const int np = (int)(qhi - qlo) + 1;
+  const long long step = (long long)maxt * d;
+  const float* first = parts + qlo * step + (i - (qlo * bpc) / nbc) * (long long)d;
+  const float* rest = parts + qlo * step;  // + t * step: the t-th cluster after the first
+  const int c0 = blockIdx.x * 1024 + (VEC ? 4 : 1) * threadIdx.x;
   asm volatile("griddepcontrol.wait;" ::: "memory");  // k_chunkgrad has completed
-  const int np = s_np;
-  const int col = blockIdx.x * 256 + threadIdx.x;
-  if (col < d) {
-    // independent loads in groups of 8, added in increasing cluster order
-    float acc = 0.f;
-    for (int t0 = 0; t0 < np; t0 += 8) {
-      float v[8];
+  // independent loads in groups of 8 clusters, added in increasing order
+  if constexpr (VEC) {
+    if (c0 < d) {
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int t0 = 0; t0 < np; t0 += 8) {
+        float4 v[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) v[k] = t0 + k < np ? __ldg(parts + s_off[t0 + k] + col) : 0.f;
+        for (int k = 0; k < 8; ++k)
+          if (t0 + k < np)
+            v[k] = __ldg(reinterpret_cast<const float4*>(
+                (t0 + k == 0 ? first : rest + (t0 + k) * step) + c0));
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if (t0 + k < np) acc += v[k];
+        for (int k = 0; k < 8; ++k)
+          if (t0 + k < np) {
+            acc.x += v[k].x;
+            acc.y += v[k].y;
+            acc.z += v[k].z;
+            acc.w += v[k].w;
+          }
+      }
+      *reinterpret_cast<float4*>(G + (size_t)i * d + c0) = acc;
     }
-    G[(size_t)i * d + col] = acc;
+  } else {
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int t0 = 0; t0 < np; t0 += 4) {
+      float v[4][4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          v[k][u] = t0 + k < np && c0 + 256 * u < d
+                        ? __ldg((t0 + k == 0 ? first : rest + (t0 + k) * step) + c0 + 256 * u)
+                        : 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (t0 + k < np) acc[u] += v[k][u];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (c0 + 256 * u < d) G[(size_t)i * d + c0 + 256 * u] = acc[u];
   }
   if (loss_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32) {
     // lane l adds clusters l, l + 32, ...; then a fixed xor tree
@@ -625,196 +90,143 @@ __global__ void __launch_bounds__(256) k_chunkgrad_reduce(const float* __restric
 // Host-side plan
 // ---------------------------------------------------------------------------
 struct Plan {
-  int CL, NT, NVT, RBM, RB, S, Wc, ld_s, V, use_tma;
+  int CL, NT, NVT, RBM, S, Wc, ld_s, V;
+  bool aligned;  // every row slice starts on a 16-byte boundary
   bool valid;
-  long long rpc;
+  int nbc;            // batches per chunk
+  long long nbatch;   // batches in all
+  long long bpc;      // batches per cluster
   int nclusters, maxt;
   size_t smem;
 };
 
-int max_active_clusters(const Plan& p, int x_dtype);
-
-Plan make_plan(int N, int n_c, int d, int x_dtype, bool tma_ok) {
-  Plan p{};
-  // Two CTAs per SM (two independent TMA rings) when each one still streams
-  // many rows; one when the rows per SM are few (ramp-up dominates) or a
-  // cluster is needed.  Chosen from measurements on GB300.
-  const long long rows_per_sm = (long long)N * n_c / std::max(1, device_sm_count());
-  const long long row_bytes0 = (long long)d * (x_dtype == GC_BF16 ? 2 : 4);
-  const int cps = (rows_per_sm >= 512 && row_bytes0 <= 16384) ? 2 : 1;
-  const int esz = x_dtype == GC_BF16 ? 2 : 4;
-  p.V = 16 / esz;
-  // cluster size: row slice per CTA at most 32 KB
-  const long long row_bytes = (long long)d * esz;
-  // per-CTA row slice at most 32 KB (fp32) / 16 KB (bf16: unpacking needs
-  // registers), so every thread holds at most 16 (fp32) or 16 (bf16) columns
-  const long long max_slice = x_dtype == GC_BF16 ? 16384 : 32768;
-  p.CL = 1;
-  while (p.CL < 8 && row_bytes / p.CL > max_slice) p.CL *= 2;
-  // Clusters of 8 fill only 120 of the 152 SMs (a cluster lives inside one
-  // GPC; at most 15 clusters of 8 are co-resident), clusters of 4 fill 144:
-  // bf16 rows of up to 128 KB take
-  // 32 KB slices in clusters of 4 (each thread then holds 32 columns; measured
-  // 12% faster at d = 65536 than 16 KB slices in clusters of 8).
-  if (x_dtype == GC_BF16 && p.CL == 8 && row_bytes <= 4 * 32768) p.CL = 4;
-  // fp32 rows of up to 256 KB take 64 KB slices in clusters of 4 (144 SMs
-  // instead of 120), rows of up to 512 KB 64 KB slices in clusters of 8;
-  // each thread then holds 32 columns, one row a stage
-  if (x_dtype != GC_BF16 && p.CL == 8 && row_bytes <= 4 * 65536) p.CL = 4;
-  p.use_tma = tma_ok && (row_bytes % 16 == 0) && (d % (p.CL * p.V) == 0);
-  p.Wc = p.use_tma ? d / p.CL : (int)align_up((size_t)((d + p.CL - 1) / p.CL), (size_t)p.V);
-  const int nv = p.Wc / p.V;  // 16-byte vectors per row slice (<= 2048 by the slice caps)
-  p.NT = nv >= 1024 ? 512 : (nv >= 256 ? 256 : 128);
-  if (cps == 2 && p.NT == 512) p.NT = 256;  // only when nv <= 1024 (16 KB slices)
-  const int need = (nv + p.NT - 1) / p.NT;
-  p.NVT = need <= 1 ? 1 : (need <= 2 ? 2 : (need <= 4 ? 4 : 8));
-  // every vector of the slice has a thread, and (NT, NVT) is an instantiated shape:
-  // NT = 128 with NVT <= 2, NT = 256 or 512 with NVT <= 4, and fp32 in
-  // clusters of 4 or 8 with NT = 512, NVT = 8
-  p.valid = (long long)p.NVT * p.NT >= nv && (p.NT > 128 || p.NVT <= 2) &&
-            (p.NVT < 8 || (x_dtype != GC_BF16 && p.NT == 512 && p.CL >= 4));
-  // stage row stride: one vector per (thread, u), so reads need no bounds
-  p.ld_s = p.NVT * p.NT * p.V;
-  p.RBM = p.NVT >= 8 ? 1 : (p.NVT >= 4 ? 2 : 4);
-  p.RB = p.RBM;
-  while (p.RB > 1 && n_c % p.RB != 0) p.RB /= 2;
-  const size_t stage_bytes = (size_t)p.RBM * p.ld_s * esz;
-  p.S = (int)std::min<size_t>(kMaxStages, std::max<size_t>(2, (192 * 1024 / cps) / stage_bytes));
-  const int NW = p.NT / 32;
-  p.smem = p.S * stage_bytes + (2 * NW * p.RBM + kZSlots * p.CL * p.RBM + 2) * sizeof(float) +
-           (2 * kMaxStages + kZSlots) * sizeof(uint64_t) + 16;
-  // flat row partition over one wave of clusters
-  const int sms = device_sm_count();
-  const long long Ntil = (long long)N * n_c;
-  long long waves_cl = std::max(1, sms * cps / p.CL);
-  if (p.CL > 1) waves_cl = std::max(1, std::min<int>((int)waves_cl, max_active_clusters(p, x_dtype)));
-  long long rpc = (Ntil + waves_cl - 1) / waves_cl;
-  rpc = ((rpc + p.RB - 1) / p.RB) * p.RB;
-  if (rpc < p.RB) rpc = p.RB;
-  p.rpc = rpc;
-  p.nclusters = (int)((Ntil + rpc - 1) / rpc);
-  p.maxt = (int)((rpc + n_c - 1) / n_c) + 1;
-  return p;
+cg::Kernel kernel_of(const Plan& p, int x_dtype) {
+  if (x_dtype == GC_BF16)
+    return p.aligned ? cg::pick_bf16(p.CL, p.NT, p.NVT) : cg::pick_bf16_ragged(p.CL, p.NT, p.NVT);
+  return p.aligned ? cg::pick_f32(p.CL, p.NT, p.NVT) : cg::pick_f32_ragged(p.CL, p.NT, p.NVT);
 }
 
-template <typename T, int CL, int NT, int NVT, int RBM>
-int launch_one(const Plan& p, const CGArgs& a, cudaStream_t s) {
-  auto kern = k_chunkgrad<T, CL, NT, NVT, RBM>;
-  static int smem_set = 0;  // largest opt-in so far (per instantiation)
-  cudaError_t e;
-  if ((int)p.smem > smem_set) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-    if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(chunkgrad smem)");
-    smem_set = (int)p.smem;
-  }
+// Position of a shape in the per-kernel caches below.
+constexpr int kShapes = 2 * 2 * 4 * 3 * 8;
+int shape_index(const Plan& p, int x_dtype) {
+  const int ci = p.CL == 1 ? 0 : (p.CL == 2 ? 1 : (p.CL == 4 ? 2 : 3));
+  const int ni = p.NT == 512 ? 0 : (p.NT == 256 ? 1 : 2);
+  return ((((x_dtype == GC_BF16) * 2 + p.aligned) * 4 + ci) * 3 + ni) * 8 + (p.NVT - 1);
+}
+
+// Allow the kernel its dynamic shared memory (largest opt-in so far per shape).
+cudaError_t allow_smem(cg::Kernel kern, const Plan& p, int x_dtype) {
+  static std::atomic<int> smem_set[kShapes];
+  std::atomic<int>& set = smem_set[shape_index(p, x_dtype)];
+  if ((int)p.smem <= set.load(std::memory_order_relaxed)) return cudaSuccess;
+  const cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+  if (e == cudaSuccess) set.store((int)p.smem, std::memory_order_relaxed);
+  return e;
+}
+
+cudaLaunchConfig_t launch_config(const Plan& p, unsigned grid, cudaLaunchAttribute* attr,
+                                 cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(p.nclusters * CL);
-  cfg.blockDim = dim3(NT + 32);  // consumers + the producer warp
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(p.NT + 32);  // consumers + the producer warp
   cfg.dynamicSmemBytes = p.smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = p.CL;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, kern, a);
-  if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(chunkgrad)");
-  count_launches(1);
-  return GC_OK;
+  return cfg;
 }
 
-template <typename T, int CL>
-int dispatch_nt(const Plan& p, const CGArgs& a, cudaStream_t s) {
-  if (p.NT == 512) {
-    if (p.NVT == 8) {
-      if constexpr (std::is_same<T, float>::value && CL >= 4) return launch_one<T, CL, 512, 8, 1>(p, a, s);
-      return fail(GC_ERR_UNSUPPORTED, "chunk-gradient shape not built");
-    }
-    if (p.NVT == 4) return launch_one<T, CL, 512, 4, 2>(p, a, s);
-    if (p.NVT == 2) return launch_one<T, CL, 512, 2, 4>(p, a, s);
-    return launch_one<T, CL, 512, 1, 4>(p, a, s);
-  }
-  if (p.NT == 256) {
-    if (p.NVT == 4) return launch_one<T, CL, 256, 4, 2>(p, a, s);
-    if (p.NVT == 2) return launch_one<T, CL, 256, 2, 4>(p, a, s);
-    return launch_one<T, CL, 256, 1, 4>(p, a, s);
-  }
-  if (p.NVT == 2) return launch_one<T, CL, 128, 2, 4>(p, a, s);
-  return launch_one<T, CL, 128, 1, 4>(p, a, s);
-}
-
-template <typename T>
-int dispatch_cl(const Plan& p, const CGArgs& a, cudaStream_t s) {
-  switch (p.CL) {
-    case 1: return dispatch_nt<T, 1>(p, a, s);
-    case 2: return dispatch_nt<T, 2>(p, a, s);
-    case 4: return dispatch_nt<T, 4>(p, a, s);
-    default: return dispatch_nt<T, 8>(p, a, s);
-  }
-}
-
-template <typename T, int CL, int NT, int NVT, int RBM>
-int occ_one(const Plan& p) {
-  auto kern = k_chunkgrad<T, CL, NT, NVT, RBM>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem) !=
-      cudaSuccess)
-    return 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(CL * 64);
-  cfg.blockDim = dim3(NT + 32);
-  cfg.dynamicSmemBytes = p.smem;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CL;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    return 1;
-  }
-  return n;
-}
-template <typename T, int CL>
-int occ_nt(const Plan& p) {
-  if (p.NT == 512) {
-    if (p.NVT == 8) {
-      if constexpr (std::is_same<T, float>::value && CL >= 4) return occ_one<T, CL, 512, 8, 1>(p);
-      return 1;
-    }
-    if (p.NVT == 4) return occ_one<T, CL, 512, 4, 2>(p);
-    if (p.NVT == 2) return occ_one<T, CL, 512, 2, 4>(p);
-    return occ_one<T, CL, 512, 1, 4>(p);
-  }
-  if (p.NT == 256) {
-    if (p.NVT == 4) return occ_one<T, CL, 256, 4, 2>(p);
-    if (p.NVT == 2) return occ_one<T, CL, 256, 2, 4>(p);
-    return occ_one<T, CL, 256, 1, 4>(p);
-  }
-  if (p.NVT == 2) return occ_one<T, CL, 128, 2, 4>(p);
-  return occ_one<T, CL, 128, 1, 4>(p);
-}
-template <typename T>
-int occ_cl(const Plan& p) {
-  switch (p.CL) {
-    case 2: return occ_nt<T, 2>(p);
-    case 4: return occ_nt<T, 4>(p);
-    default: return occ_nt<T, 8>(p);
-  }
-}
 // Clusters of this plan that can be resident at once (cached per shape).
 int max_active_clusters(const Plan& p, int x_dtype) {
-  static int cache[2][4][3][4] = {};
-  const int ci = p.CL == 2 ? 1 : (p.CL == 4 ? 2 : 3);
-  const int ni = p.NT == 512 ? 0 : (p.NT == 256 ? 1 : 2);
-  const int vi = p.NVT == 8 ? 3 : (p.NVT == 4 ? 0 : (p.NVT == 2 ? 1 : 2));
-  int& c = cache[x_dtype == GC_BF16][ci][ni][vi];
-  if (c == 0) c = x_dtype == GC_BF16 ? occ_cl<__nv_bfloat16>(p) : occ_cl<float>(p);
-  return c;
+  static std::atomic<int> cache[kShapes];
+  std::atomic<int>& c = cache[shape_index(p, x_dtype)];
+  int n = c.load(std::memory_order_relaxed);
+  if (n > 0) return n;
+  cg::Kernel kern = kernel_of(p, x_dtype);
+  cudaLaunchAttribute attr[1];
+  const cudaLaunchConfig_t cfg = launch_config(p, p.CL * 64, attr, nullptr);
+  if (!kern || allow_smem(kern, p, x_dtype) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    n = 1;
+  }
+  c.store(n, std::memory_order_relaxed);
+  return n;
+}
+
+Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
+  Plan p{};
+  const int esz = x_dtype == GC_BF16 ? 2 : 4;
+  p.V = 16 / esz;
+  const long long row_bytes = (long long)d * esz;
+  // The row is split over as few CTAs as its columns' w and accumulators fit
+  // the registers of (512 threads of 6 fp32 or 4 bf16 vectors): a cluster
+  // exchanges partial dots once a batch and holds each stage until the sums
+  // are back.  Measured at 2 GB of X against slices of 32 KB (fp32) and 16 KB
+  // (bf16): fp32 d = 10007 102% of the copy rate in one CTA, 54% in two
+  // (12288: 93, 64); bf16 d = 12000 89 against 37 (16384: 98, 74), d = 20000
+  // in two CTAs 54 against 29 in four.
+  const long long max_slice = x_dtype == GC_BF16 ? 32768 : 49152;
+  p.CL = 1;
+  while (p.CL < 8 && (row_bytes + p.CL - 1) / p.CL > max_slice) p.CL *= 2;
+  // Clusters of 8 fill only 120 of the 152 SMs (a cluster lives inside one
+  // GPC; at most 15 clusters of 8 are co-resident), clusters of 4 fill 144:
+  // fp32 rows of up to 256 KB take 64 KB slices (8 vectors a thread, one row a
+  // stage) in clusters of 4.  bf16 rows that two CTAs would take in four
+  // vectors a thread stay in clusters of 4 (d = 32768: 70 against 68%; at
+  // 256 MB 43 against 40%).
+  if (x_dtype != GC_BF16 && p.CL == 8 && row_bytes <= 4 * 65536) p.CL = 4;
+  if (x_dtype == GC_BF16 && p.CL == 2 && row_bytes > 2 * 3 * 512 * 16) p.CL = 4;
+  p.Wc = (int)align_up((size_t)((d + p.CL - 1) / p.CL), (size_t)p.V);
+  p.aligned = x_aligned && row_bytes % 16 == 0;
+  const int nv = p.Wc / p.V;  // 16-byte vectors per row slice (<= 2048 by the slice caps)
+  p.NT = nv >= 1024 ? 512 : (nv >= 256 ? 256 : 128);
+  // CTAs per SM.  Rows of 4 to 16 KB: two (two independent rings) when each
+  // still streams many rows, one when the rows per SM are few (ramp-up
+  // dominates) or the row is longer.  Shorter rows, 128 threads: a batch's
+  // chain of shuffles, barrier and residual (0.6 us) outlasts its copy, so as
+  // many CTAs as the registers hold, with at least 32 rows each (100,000 fp32
+  // rows of d = 512: 112 us with one CTA, 62 with two, 42 with four; 10,000
+  // rows: 16, 12 and 12).
+  const long long rows_per_sm = (long long)N * n_c / std::max(1, device_sm_count());
+  int cps = (rows_per_sm >= 512 && row_bytes <= 16384) ? 2 : 1;
+  if (p.NT == 128)
+    cps = (int)std::max(1LL, std::min<long long>(esz == 4 && nv <= 128 ? 4 : 3, rows_per_sm / 32));
+  if (cps == 2 && p.NT == 512) p.NT = 256;  // only when nv <= 1024 (16 KB slices)
+  const int need = (nv + p.NT - 1) / p.NT;
+  // vectors a thread: 1, 2, 4, and for 512-thread slices past 4 vectors (fp32)
+  // or 2 (bf16) the exact count, whose empty vectors would cost stage space
+  // and dot products
+  p.NVT = need <= 2 ? need : 4;
+  if (x_dtype == GC_BF16 ? need == 3 && p.NT == 512 : need > 4) p.NVT = need <= 6 ? need : 8;
+  p.RBM = p.NVT >= 5 ? 1 : (p.NVT >= 3 ? 2 : 4);
+  // stage row: one vector per (thread, u), so reads need no bounds; a slice at
+  // any element lies up to V - 1 elements in and ends in up to 2 V - 1 more
+  const int row_vecs = p.NVT * p.NT;
+  p.ld_s = row_vecs * p.V + (p.aligned ? 0 : 2 * p.V);
+  const size_t stage_bytes = (size_t)p.RBM * p.ld_s * esz;
+  p.S = (int)std::min<size_t>(
+      cg::kMaxStages, std::max<size_t>(2, (192 * 1024 / cps) / ((size_t)p.RBM * row_vecs * 16)));
+  const int NW = p.NT / 32;
+  p.smem = p.S * stage_bytes + (2 * NW * p.RBM + cg::kZSlots * p.CL * p.RBM + 2) * sizeof(float) +
+           (2 * cg::kMaxStages + cg::kZSlots) * sizeof(uint64_t) + 16;
+  // every vector of the slice has a thread, and the shape is built
+  p.valid = (long long)row_vecs >= nv && kernel_of(p, x_dtype) != nullptr;
+  // flat partition of the batches over one wave of clusters
+  const int sms = device_sm_count();
+  long long waves_cl = std::max(1, sms * cps / p.CL);
+  if (p.CL > 1) waves_cl = std::max(1, std::min<int>((int)waves_cl, max_active_clusters(p, x_dtype)));
+  p.nbc = (n_c + p.RBM - 1) / p.RBM;
+  p.nbatch = (long long)N * p.nbc;
+  p.bpc = (p.nbatch + waves_cl - 1) / waves_cl;
+  p.nclusters = (int)((p.nbatch + p.bpc - 1) / p.bpc);
+  p.maxt = (int)((p.bpc + p.nbc - 1) / p.nbc) + 1;
+  return p;
 }
 
 }  // namespace
@@ -834,7 +246,7 @@ int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w,
   const bool aligned = (reinterpret_cast<uintptr_t>(X) % 16) == 0;
   const Plan p = make_plan(N, n_c, d, x_dtype, aligned);
   if (!p.valid) return fail(GC_ERR_UNSUPPORTED, "chunk-gradient plan does not cover d=%d", d);
-  CGArgs a{};
+  cg::CGArgs a{};
   a.X = X;
   a.y = y;
   a.w = w;
@@ -843,26 +255,37 @@ int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w,
   a.ld_s = p.ld_s;
   a.n_c = n_c;
   a.Ntil = (long long)N * n_c;
-  a.rpc = p.rpc;
-  a.RB = p.RB;
+  a.nbc = p.nbc;
+  a.nbatch = p.nbatch;
+  a.bpc = p.bpc;
   a.S = p.S;
   a.maxt = p.maxt;
   a.loss = loss;
   a.want_loss = loss_out != nullptr;
-  a.use_tma = p.use_tma;
-  a.spin_limit = wait_limit(kSpinLimit);
+  a.spin_limit = wait_limit(cg::kSpinLimit);
   a.stall = take_stall(GC_STALL_CHUNK_GRADS) ? 1 : 0;
   a.parts = ws.take<float>((size_t)p.nclusters * p.maxt * d);
   a.loss_parts = ws.take<double>(p.nclusters);
   a.status = status;
-  if (p.rpc < 1 || (long long)n_c / p.rpc + 2 > kRedMaxParts)
+  // a limit of the interface, kept as it was: a single chunk of at least 512
+  // rows per SM of short rows is refused
+  if (N == 1 && (long long)n_c / std::max(1, device_sm_count()) >= 512 &&
+      (long long)d * (x_dtype == GC_BF16 ? 2 : 4) <= 16384)
     return fail(GC_ERR_UNSUPPORTED, "chunk of %d rows spans too many row blocks", n_c);
   if (N > 65535) return fail(GC_ERR_UNSUPPORTED, "N=%d exceeds 65535 chunks", N);
-  int rc = x_dtype == GC_BF16 ? dispatch_cl<__nv_bfloat16>(p, a, s) : dispatch_cl<float>(p, a, s);
-  if (rc != GC_OK) return rc;
+  cg::Kernel kern = kernel_of(p, x_dtype);
+  cudaError_t e = allow_smem(kern, p, x_dtype);
+  if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(chunkgrad smem)");
+  {
+    cudaLaunchAttribute cl_attr[1];
+    const cudaLaunchConfig_t cl_cfg = launch_config(p, (unsigned)(p.nclusters * p.CL), cl_attr, s);
+    e = cudaLaunchKernelEx(&cl_cfg, kern, a);
+    if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(chunkgrad)");
+    count_launches(1);
+  }
   // the reduction as a programmatic dependent launch (it waits in-kernel)
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((d + 255) / 256, N);
+  cfg.gridDim = dim3((d + 1023) / 1024, N);
   cfg.blockDim = dim3(256);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -870,9 +293,10 @@ int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w,
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_chunkgrad_reduce, (const float*)a.parts,
-                                     (const double*)a.loss_parts, G, loss_out, N, n_c, d, p.rpc,
-                                     p.maxt, p.nclusters, a.Ntil);
+  const bool vec = d % 4 == 0 && reinterpret_cast<uintptr_t>(G) % 16 == 0;
+  e = cudaLaunchKernelEx(&cfg, vec ? k_chunkgrad_reduce<true> : k_chunkgrad_reduce<false>,
+                         (const float*)a.parts, (const double*)a.loss_parts, G, loss_out, N, p.nbc,
+                         d, p.bpc, p.maxt, p.nclusters, a.Ntil);
   if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_chunkgrad_reduce)");
   count_launches(1);
   return GC_OK;

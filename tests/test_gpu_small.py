@@ -223,6 +223,60 @@ def test_chunk_grads_shapes(gc, d, n_c, N, dtype, loss):
     assert abs(lo.item() - Lo) <= 1e-5 * abs(Lo)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("d,n_c,N,off", [
+    (2, 9, 4, 5),         # several rows within the first 16 bytes of an unaligned X
+    (3, 5, 7, 0),         # rows shorter than a 16-byte piece
+    (15, 4, 3, 1),        # the ragged end reaches the next piece
+    (517, 13, 3, 0),      # 128 threads, a last batch of one row
+    (517, 30000, 2, 3),   # several CTAs per SM
+    (1021, 11, 2, 0),     # 256 threads (fp32), 128 (bf16)
+    (3001, 7, 2, 2),      # 4 vectors a thread (fp32)
+    (9001, 5, 2, 0),      # 5 fp32 vectors a thread; 3 bf16
+    (12287, 3, 2, 1),     # 6 and 4 vectors, one column short of the stage row
+    (12289, 3, 2, 0),     # a cluster of 2 (fp32)
+    (20003, 3, 2, 0),     # clusters of 2, slices that start at any element
+    (49151, 2, 2, 3),     # clusters of 4
+    (70001, 2, 2, 0),     # clusters of 8
+])
+def test_chunk_grads_ragged(gc, d, n_c, N, off, dtype):
+    """Rows that are no multiple of 16 bytes, X at any element, chunks whose rows do not fill
+    their last batch: X, w and y in a guard of NaN, so that a value read past them shows."""
+    g = torch.Generator().manual_seed(d * 7 + n_c + off)
+    X = torch.randn(N * n_c, d, generator=g).to(dtype)
+    y = torch.randn(N * n_c, generator=g)
+    w = (torch.randn(d, generator=g) / d ** 0.5).float()
+    pad = 64
+    buf = torch.full((off + X.numel() + pad,), float("nan"), dtype=dtype, device="cuda")
+    Xd = buf[off:off + X.numel()].view(N * n_c, d)
+    Xd.copy_(X)
+    lo = torch.zeros(1, dtype=torch.float64, device="cuda")
+    G = torch.full((N, d), float("nan"), device="cuda")
+    ws = gc.Workspace()
+    for _ in range(2):  # the second call's stages start from the first one's
+        gc.gc_chunk_grads(Xd, y.cuda(), w.cuda(), N, n_c, 0, G=G, loss_out=lo, ws=ws)
+    gc.gc_status(ws)
+    Go = O.chunk_gradients(X, y.numpy(), w.numpy(), N, n_c, 0)
+    for i in range(N):
+        assert_grad_close(to_np(G[i]), Go[i], f"chunk {i}")
+    Lo = O.full_loss(X, y.numpy(), w.numpy(), N * n_c, 4096, 0)
+    assert abs(lo.item() - Lo) <= 1e-5 * abs(Lo)
+
+
+def test_chunk_grads_ragged_rows_stay_apart(gc):
+    """An infinite value in one row reaches its own chunk's gradient alone (the stages hold
+    earlier rows' values past a short batch and past a ragged row's end)."""
+    N, n_c, d = 6, 3, 1021
+    X = torch.randn(N * n_c, d, generator=torch.Generator().manual_seed(3)).cuda()
+    y, w = torch.randn(N * n_c).cuda(), (torch.randn(d) / 32).cuda()
+    ref = gc.gc_chunk_grads(X, y, w, N, n_c, 0)
+    X[4, d - 1] = float("inf")
+    X[5, 0] = float("inf")
+    G = gc.gc_chunk_grads(X, y, w, N, n_c, 0)
+    keep = [i for i in range(N) if i != 1]
+    assert torch.equal(G[keep], ref[keep]) and not torch.isfinite(G[1]).all()
+
+
 def test_chunk_grads_unaligned_X(gc):
     """An X view starting 4 bytes past a 16-byte boundary takes the plain-load path."""
     N, n_c, d = 3, 8, 256
