@@ -118,6 +118,13 @@ int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w,
 // ---- encode / decode / update (k_encode.cu) -----------------------------
 int launch_encode(const double* E, const int32_t* order, const int32_t* psi, int N, int m,
                   int delta, int ell, int npat, const float* G, int d, float* T, cudaStream_t s);
+// the workers whose orders are not cyclic (k_encode_any.cu); J = workers per
+// group of the cyclic kernel
+constexpr size_t kEncodeAnySmem = 220 * 1024;
+bool encode_any_applies(int N, int m, int delta, int ell, int npat, int L);
+int launch_encode_any(const double* E, const int32_t* order, const int32_t* psi, int N, int m,
+                      int delta, int ell, int npat, const float* G, int d, int J, float* T,
+                      cudaStream_t s);
 int launch_decode_tx(const double* R, int ell, int m, const float* T, int npat, int d, float* ghat,
                      cudaStream_t s);
 int launch_sgd(float* w, const float* ghat, int d, float lr, int64_t Ntil, cudaStream_t s);

@@ -35,8 +35,9 @@ namespace gc {
 // with cp.async.wait_group, so no thread reads another's data and no barrier
 // or spin-wait is needed.
 // A transmission is summed over slots p ascending, blocks k ascending within
-// a slot -- the same order in the direct form, which a block whose workers'
-// orders are not cyclic (an explicit order) uses instead.
+// a slot -- the same order in the direct form, for a block whose workers'
+// orders are not cyclic (an explicit order): small calls sum it here from the
+// cache, larger ones leave it to k_encode_any.
 constexpr int kEncThreads = 128;
 constexpr int kEncSmemFloats = 12288;  // staged coefficients (48 KB)
 constexpr int kEncStages = 8;          // ring of chunk-stripe steps per thread
@@ -136,7 +137,8 @@ template <int DR, int V, int KB>
 __global__ void __launch_bounds__(kEncThreads, DR == 32 ? 3 : 4)
     k_encode(const double* __restrict__ E, const int32_t* __restrict__ order,
              const int32_t* __restrict__ psi, int N, int m, int delta, int ell, int npat,
-             const float* __restrict__ G, int d, int L, int J, int vec, float* __restrict__ T) {
+             const float* __restrict__ G, int d, int L, int J, int vec, int any_next,
+             float* __restrict__ T) {
   extern __shared__ __align__(16) float s_dyn[];
   __shared__ int s_np[256];               // processed counts of the group's workers (J <= 256)
   const int b = blockIdx.x;               // pattern fastest: blocks on one stripe share G in L2
@@ -158,7 +160,10 @@ __global__ void __launch_bounds__(kEncThreads, DR == 32 ? 3 : 4)
   }
   cyc = __syncthreads_and(cyc);
   const double* Eb = E + ((size_t)b * m + j0) * de;
+  // k_encode_any (when launched) may start once every block has got here or ended
+  if (any_next && threadIdx.x == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (!cyc) {
+    if (any_next) return;
     // direct form: s_e[jj][p][k]
     for (int t = threadIdx.x; t < nj * de; t += kEncThreads) s_e[t] = (float)Eb[t];
     __syncthreads();
@@ -339,7 +344,8 @@ __global__ void __launch_bounds__(kEncThreads, DR == 32 ? 3 : 4)
 template <int DR, int V, int KB>
 static int launch_enc_t(dim3 grid, size_t smem, const double* E, const int32_t* order,
                         const int32_t* psi, int N, int m, int delta, int ell, int npat,
-                        const float* G, int d, int L, int J, int vec, float* T, cudaStream_t s) {
+                        const float* G, int d, int L, int J, int vec, int any_next, float* T,
+                        cudaStream_t s) {
   static bool attr = false;
   if (!attr) {
     cudaError_t e = cudaFuncSetAttribute(k_encode<DR, V, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -347,7 +353,8 @@ static int launch_enc_t(dim3 grid, size_t smem, const double* E, const int32_t* 
     if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_encode)");
     attr = true;
   }
-  k_encode<DR, V, KB><<<grid, kEncThreads, smem, s>>>(E, order, psi, N, m, delta, ell, npat, G, d, L, J, vec, T);
+  k_encode<DR, V, KB><<<grid, kEncThreads, smem, s>>>(E, order, psi, N, m, delta, ell, npat, G, d, L, J, vec,
+                                                     any_next, T);
   return GC_OK;
 }
 
@@ -374,13 +381,14 @@ int launch_encode(const double* E, const int32_t* order, const int32_t* psi, int
   if (npat > 2147483647 || stripes > 65535 || ngroups > 65535)
     return fail(GC_ERR_UNSUPPORTED, "encode grid too large");
   const size_t smem = enc_smem_bytes(DR, V, ell, delta, J);
+  const int any_next = encode_any_applies(N, m, delta, ell, npat, L) ? 1 : 0;
   const dim3 grid((unsigned)npat, (unsigned)stripes, (unsigned)ngroups);
   int rc;
   // two blocks of a chunk per step when ell is even
 #define GC_ENC(R, VV)                                                                               \
   rc = ell % 2 == 0                                                                                 \
-           ? launch_enc_t<R, VV, 2>(grid, smem, E, order, psi, N, m, delta, ell, npat, G, d, L, J, vec, T, s) \
-           : launch_enc_t<R, VV, 1>(grid, smem, E, order, psi, N, m, delta, ell, npat, G, d, L, J, vec, T, s)
+           ? launch_enc_t<R, VV, 2>(grid, smem, E, order, psi, N, m, delta, ell, npat, G, d, L, J, vec, any_next, T, s) \
+           : launch_enc_t<R, VV, 1>(grid, smem, E, order, psi, N, m, delta, ell, npat, G, d, L, J, vec, any_next, T, s)
   switch (DR) {
     case 4: GC_ENC(4, 4); break;
     case 8: GC_ENC(8, 4); break;
@@ -390,16 +398,18 @@ int launch_encode(const double* E, const int32_t* order, const int32_t* psi, int
 #undef GC_ENC
   if (rc) return rc;
   count_launches(1);
-  return cuda_check(cudaGetLastError(), "k_encode");
+  rc = cuda_check(cudaGetLastError(), "k_encode");
+  if (rc || !any_next) return rc;
+  return launch_encode_any(E, order, psi, N, m, delta, ell, npat, G, d, J, T, s);
 }
 
-// ghat[b][k*L + c] = sum_j R[k][j] * T[b][j][c].  One thread per (b, c); R is
-// staged in dynamic shared memory as fp32 (ELL * m words, m <= kDecodeSmemM)
-// or read as fp64.  The transmissions are loaded eight workers at a time, so
-// that eight independent loads are in flight per thread (the kernel is
-// latency-bound at the sizes of one live realization).
+// ghat[b][k*L + c] = sum_j R[k][j] * T[b][j][c], j ascending.  A thread takes V
+// columns; R is staged in dynamic shared memory as fp32 (ELL * m words, m <=
+// kDecodeSmemM) or read as fp64.  The kernel streams T; eight workers' loads
+// are in flight per thread, 16 bytes each where the rows allow it (m = 256,
+// ell = 2, L = 2^19: 123 us with 4-byte loads, 84 us = 6.4 TB/s with 16).
 constexpr int kDecodeSmemM = 1024;
-template <int ELL, bool STAGED>
+template <int ELL, bool STAGED, int V>
 __global__ void k_decode_tx(const double* __restrict__ R, int m, const float* __restrict__ T,
                             int npat, int d, int L, float* __restrict__ ghat) {
   extern __shared__ float s_r[];
@@ -408,63 +418,92 @@ __global__ void k_decode_tx(const double* __restrict__ R, int m, const float* __
     __syncthreads();
   }
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)npat * L) return;
-  const int c = (int)(idx % L);
-  const int b = (int)(idx / L);
-  float acc[ELL];
+  const int LV = L / V;
+  if (idx >= (long long)npat * LV) return;
+  const int c = (int)(idx % LV) * V;
+  const int b = (int)(idx / LV);
+  float acc[ELL][V];
 #pragma unroll
-  for (int k = 0; k < ELL; ++k) acc[k] = 0.f;
+  for (int k = 0; k < ELL; ++k)
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[k][v] = 0.f;
   const float* Tb = T + (size_t)b * m * L + c;
   for (int j0 = 0; j0 < m; j0 += 8) {
-    float t[8];
+    float t[8][V];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) t[u] = j0 + u < m ? __ldg(Tb + (size_t)(j0 + u) * L) : 0.f;
+    for (int u = 0; u < 8; ++u) {
+      const float* p = Tb + (size_t)(j0 + u) * L;
+      if constexpr (V == 4) {
+        const float4 q = j0 + u < m ? __ldcs(reinterpret_cast<const float4*>(p))
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+        t[u][0] = q.x; t[u][1] = q.y; t[u][2] = q.z; t[u][3] = q.w;
+      } else {
+        t[u][0] = j0 + u < m ? __ldg(p) : 0.f;
+      }
+    }
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       if (j0 + u < m) {
 #pragma unroll
         for (int k = 0; k < ELL; ++k) {
           const float r = STAGED ? s_r[k * m + j0 + u] : (float)__ldg(R + (size_t)k * m + j0 + u);
-          acc[k] = fmaf(r, t[u], acc[k]);
+#pragma unroll
+          for (int v = 0; v < V; ++v) acc[k][v] = fmaf(r, t[u][v], acc[k][v]);
         }
       }
     }
   }
 #pragma unroll
   for (int k = 0; k < ELL; ++k) {
-    const int col = k * L + c;
-    if (col < d) ghat[(size_t)b * d + col] = acc[k];
+    const long long col = (long long)k * L + c;
+    float* o = ghat + (size_t)b * d + col;
+    if (V == 4 && col + 3 < d) {
+      *reinterpret_cast<float4*>(o) = make_float4(acc[k][0], acc[k][1 % V], acc[k][2 % V], acc[k][3 % V]);
+    } else {
+#pragma unroll
+      for (int v = 0; v < V; ++v)
+        if (col + v < d) o[v] = acc[k][v];
+    }
   }
+}
+
+template <int ELL>
+static void run_decode_tx(const double* R, int m, const float* T, int npat, int d, int L,
+                          float* ghat, cudaStream_t s) {
+  const bool staged = m <= kDecodeSmemM;
+  const size_t sm = staged ? (size_t)ELL * m * sizeof(float) : 0;
+  // four columns a thread (16-byte loads) when the rows are 16-byte pieces and
+  // that still leaves 256 threads an SM; below, one column a thread hides the
+  // latency better
+  const bool vec = staged && L % 4 == 0 && d % 4 == 0 &&
+                   (reinterpret_cast<uintptr_t>(T) | reinterpret_cast<uintptr_t>(ghat)) % 16 == 0 &&
+                   (long long)npat * L >= 1024LL * device_sm_count();
+  const int threads = 128;
+  const long long tot = (long long)npat * (vec ? L / 4 : L);
+  const unsigned blocks = (unsigned)((tot + threads - 1) / threads);
+  if (vec)
+    k_decode_tx<ELL, true, 4><<<blocks, threads, sm, s>>>(R, m, T, npat, d, L, ghat);
+  else if (staged)
+    k_decode_tx<ELL, true, 1><<<blocks, threads, sm, s>>>(R, m, T, npat, d, L, ghat);
+  else
+    k_decode_tx<ELL, false, 1><<<blocks, threads, 0, s>>>(R, m, T, npat, d, L, ghat);
 }
 
 int launch_decode_tx(const double* R, int ell, int m, const float* T, int npat, int d, float* ghat,
                      cudaStream_t s) {
   const int L = (d + ell - 1) / ell;
-  const long long tot = (long long)npat * L;
-  if (tot == 0) return GC_OK;
-  const int threads = 128;
-  const unsigned blocks = (unsigned)((tot + threads - 1) / threads);
-  const bool staged = m <= kDecodeSmemM;
-  const size_t sm = staged ? (size_t)ell * m * sizeof(float) : 0;
-#define GC_DTX(E)                                                                              \
-  case E:                                                                                      \
-    if (staged)                                                                                \
-      k_decode_tx<E, true><<<blocks, threads, sm, s>>>(R, m, T, npat, d, L, ghat);             \
-    else                                                                                       \
-      k_decode_tx<E, false><<<blocks, threads, 0, s>>>(R, m, T, npat, d, L, ghat);             \
-    break;
+  if ((long long)npat * L == 0) return GC_OK;
   switch (ell) {
-    GC_DTX(1)
-    GC_DTX(2)
-    GC_DTX(3)
-    GC_DTX(4)
-    GC_DTX(5)
-    GC_DTX(6)
-    GC_DTX(7)
-    GC_DTX(8)
+    case 1: run_decode_tx<1>(R, m, T, npat, d, L, ghat, s); break;
+    case 2: run_decode_tx<2>(R, m, T, npat, d, L, ghat, s); break;
+    case 3: run_decode_tx<3>(R, m, T, npat, d, L, ghat, s); break;
+    case 4: run_decode_tx<4>(R, m, T, npat, d, L, ghat, s); break;
+    case 5: run_decode_tx<5>(R, m, T, npat, d, L, ghat, s); break;
+    case 6: run_decode_tx<6>(R, m, T, npat, d, L, ghat, s); break;
+    case 7: run_decode_tx<7>(R, m, T, npat, d, L, ghat, s); break;
+    case 8: run_decode_tx<8>(R, m, T, npat, d, L, ghat, s); break;
     default: return fail(GC_ERR_UNSUPPORTED, "ell=%d exceeds GC_MAX_ELL", ell);
   }
-#undef GC_DTX
   count_launches(1);
   return cuda_check(cudaGetLastError(), "k_decode_tx");
 }

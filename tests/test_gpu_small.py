@@ -386,6 +386,80 @@ def test_encode_long_rows(gc, explicit, npat):
             assert float(T[b].abs().max()) == 0.0
 
 
+@pytest.mark.parametrize("N,m,delta,ell,npat,L,pad,kind", [
+    (37, 37, 5, 3, 1, 121000, 0, "random"),   # a last group of one worker, one pattern
+    (37, 37, 5, 3, 2, 61001, 2, "random"),    # two patterns, ragged rows, padded last block
+    (37, 37, 5, 3, 5, 33000, 0, "mixed"),     # four patterns and one; workers of cyclic groups
+    (64, 16, 4, 4, 3, 90003, 1, "padded"),    # three patterns of four, empty slots
+    (330, 330, 6, 2, 4, 4400, 0, "random"),   # N*ell = 660: no values held ahead
+    (330, 330, 6, 2, 4, 4399, 1, "random"),
+    (256, 256, 10, 4, 6, 1500, 0, "random"),  # two patterns at a time fit
+    (400, 400, 16, 3, 2, 2001, 0, "random"),  # one pattern at a time fits
+    (20, 20, 3, 1, 4, 300000, 0, "mixed"),
+])
+def test_encode_any_order(gc, N, m, delta, ell, npat, L, pad, kind):
+    """Eq. (2) for orders that are not cyclic, at sizes that take k_encode_any, against the sum in
+    64 bits; the first columns of every block, as a call of their own (which sums from the
+    cache), give the same bits.  Without cyclic groups an infinite value reaches only the transmissions that use it."""
+    d = ell * L - pad
+    rng = np.random.default_rng(m + L + npat)
+    order = -np.ones((m, delta), np.int32)
+    for j in range(m):
+        row = rng.choice(N, size=delta, replace=False)
+        if kind == "mixed" and j != 1:
+            row = (j + np.arange(delta)) % N
+        if kind == "padded":
+            row = row[:rng.integers(0, delta + 1)]
+        order[j, :len(row)] = row
+    psi = rng.integers(0, delta + 1, size=(npat, m)).astype(np.int32)
+    od, pd = torch.from_numpy(order).cuda(), torch.from_numpy(psi).cuda()
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    G = torch.randn(N, d, generator=gen, device="cuda")
+    E = torch.randn(npat, m, delta, ell, generator=gen, device="cuda", dtype=torch.float64)
+    E[0, 0] = torch.tensor([1e-42, -3e38, 1 + 2.0 ** -24, 1 + 3 * 2.0 ** -24], dtype=torch.float64,
+                           device="cuda").repeat(delta * ell)[:delta * ell].view(delta, ell)
+    done = torch.arange(delta, device="cuda") < pd[:, :, None]
+    assert npat * m * L * delta * ell >= 1 << 26  # k_encode_any's range
+    T = torch.full((npat, m, L), float("nan"), device="cuda")
+    gc.gc_encode_with_coeffs(E, ell, od, N, m, delta, pd, G, T=T)
+    B = torch.nn.functional.pad(G, (0, pad)).view(N, ell, L)
+    E[0, 0] = 0  # its values (huge, tiny, half-way to the next fp32) are compared as bits below
+    E32 = (E * done[..., None] * (od >= 0)[None, :, :, None]).float().double()
+    ref = torch.zeros(npat, m, L, device="cuda", dtype=torch.float64)
+    for p in range(delta):
+        for k in range(ell):
+            ref += E32[:, :, p, k, None] * B[od[:, p].clamp(min=0).long(), k].double()
+    ref[0, 0] = T[0, 0].double()
+    # delta * ell fused multiply-adds: at most delta * ell roundings of partial sums of that size
+    bound = delta * ell * 2.0 ** -24 * (E32.abs().sum((2, 3)).amax() * B.abs().max()).item()
+    assert (T.double() - ref)[torch.isfinite(ref)].abs().max().item() <= bound
+    E[0, 0] = torch.tensor([1e-42, -3e38, 1 + 2.0 ** -24, 1 + 3 * 2.0 ** -24], dtype=torch.float64,
+                           device="cuda").repeat(delta * ell)[:delta * ell].view(delta, ell)
+    cols = 40
+    Ts = gc.gc_encode_with_coeffs(E, ell, od, N, m, delta, pd, B[:, :, :cols].reshape(N, -1).contiguous())
+    same = T[:, :, :cols]
+    assert torch.equal(Ts.nan_to_num(), same.nan_to_num()) and torch.equal(Ts.isnan(), same.isnan())
+    i, c = int(order[1][0]), L // 2
+    if i >= 0 and kind != "mixed":  # the sweep of a cyclic group multiplies by zeros
+        G[i, c] = float("inf")
+        T2 = gc.gc_encode_with_coeffs(E, ell, od, N, m, delta, pd, G)
+        uses = ((od[None] == i) & done).any(2)  # npat x m
+        assert torch.equal(torch.isfinite(T2[:, 1:, c]), ~uses[:, 1:])
+        T2[:, :, c] = T[:, :, c]
+        assert torch.equal(T2.nan_to_num(), T.nan_to_num())
+
+
+@pytest.mark.parametrize("L,ell,npat,m", [(155648, 2, 1, 40), (155652, 3, 1, 7), (77824, 4, 2, 9),
+                                          (155649, 2, 1, 40), (155644, 1, 1, 16)])
+def test_decode_tx_wide(gc, L, ell, npat, m):
+    """Four columns a thread (from 1024 columns an SM on) and one give the oracle's decode."""
+    rng = np.random.default_rng(L)
+    R, T = rng.standard_normal((ell, m)), rng.standard_normal((npat, m, L)).astype(np.float32)
+    g = gc.gc_decode_tx(torch.from_numpy(R).cuda(), ell, m, torch.from_numpy(T).cuda(), ell * L)
+    for b in range(npat):
+        assert_grad_close(to_np(g[b]), O.decode(R, T[b].astype(np.float64), ell * L), f"pattern {b}")
+
+
 @pytest.mark.parametrize("delta,d,ell", [(5, 2600, 2), (9, 2599, 2), (16, 2600, 2), (16, 2599, 2),
                                          (17, 2600, 2), (32, 2600, 2), (16, 2600, 1), (16, 2600, 3),
                                          (16, 2604, 4), (16, 2601, 4)])
