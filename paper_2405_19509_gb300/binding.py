@@ -464,7 +464,7 @@ GC_DECODE_RESIDUAL = 2
 
 
 def gc_set_decode_policy(policy: int) -> None:
-    """Path of the batched decode per 128-row tile: GC_DECODE_AUTO (default),
+    """Path of the batched decode per pattern: GC_DECODE_AUTO (default),
     GC_DECODE_DENSE (tensor-core GEMM) or GC_DECODE_RESIDUAL (sum of the
     chunk gradients plus the non-identity blocks).  Process-wide."""
     _check(lib.gc_set_decode_policy(int(policy)))

@@ -134,35 +134,46 @@ int launch_live_step(const double* E, const double* R, int ell, const int32_t* o
 
 // ---- batched decode in residual form (k_decode_resid.cu) -----------------
 // Per pattern the ordered list of decode blocks that differ from I_ell (chunk
-// index and D = Pi - I); per 128-row tile of the decode the path that
-// produces its rows (tflag = 1: the tensor-core GEMM; 0: the residual kernel)
-// and, for a residual tile, the ordered list of its rows that need
-// corrections, each with a slot of squared-error partials.
+// index and D = Pi - I).
 constexpr int kResidThreads = 256;
 constexpr int kResidW = kResidThreads * 4;  // columns of one block per CTA (4 KB rows)
-constexpr int kResidRcap = 32;              // corrected rows a residual tile may hold
 struct ResidLists {
-  int32_t* nnz;        // [npat] non-identity blocks (may exceed ksp)
-  int32_t* idx;        // [npat][ksp] their chunks, ascending
-  float* D;            // [npat][ksp][ell][ell] Pi - I
-  int32_t* tflag;      // [ntiles]
-  int32_t* dlist;      // [ntiles] the GEMM's tiles, ascending
-  int32_t* ndense;     // one word: entries of dlist
-  int32_t* rslot;      // [npat*ell] slot of a corrected row of a residual tile, else -1
-  int32_t* rowlist;    // [ntiles][kResidRcap] corrected rows of each tile, ascending
-  int32_t* tcount;     // [ntiles] entries of rowlist
-  float* msp;          // [ntiles*kResidRcap][parts] squared-error partials, or null
-  int ksp;             // list capacity per pattern
-  int parts;           // partials per corrected row (column ranges x warps)
+  int32_t* nnz;   // [npat] non-identity blocks (may exceed ksp)
+  int32_t* idx;   // [npat][ksp] their chunks, ascending
+  float* D;       // [npat][ksp][ell][ell] Pi - I
+  int32_t* stat;  // patterns with more than ksp of them; blocks past the budget in
+                  // the others; patterns gathered for the GEMM
+  int32_t* dpat;  // [npat] the gathered patterns
+  float* msp;     // [npat][parts] squared-error partials, or null
+  int ksp;        // list capacity per pattern
+  int parts;      // partials per pattern (column ranges)
+};
+// Which patterns the tensor-core GEMM decodes: those with more non-identity
+// blocks than threshold() (none when any() is false).  GC_DECODE_AUTO: a
+// pattern is worth the GEMM from `budget` blocks on, but the GEMM's operand
+// split reads and writes all of G, so it runs only when some pattern's list
+// overflows or the others' blocks past the budget add up to more than that.
+struct GemmChoice {
+  int policy, budget, ksp, split_cost;
+  __device__ __forceinline__ bool any(const ResidLists& rl) const {
+    if (policy == GC_DECODE_DENSE) return true;
+    return rl.stat[0] > 0 || (policy == GC_DECODE_AUTO && rl.stat[1] > split_cost);
+  }
+  __device__ __forceinline__ int threshold(const ResidLists& rl) const {
+    if (policy == GC_DECODE_DENSE) return -1;
+    return policy == GC_DECODE_AUTO && any(rl) && budget < ksp ? budget : ksp;
+  }
 };
 int resid_ksp(int ell);
 size_t resid_ws_bytes(int N, int ell, int npat, int d);
 ResidLists carve_resid(Carve& c, int N, int ell, int npat, int d, bool want_mse);
+// counters: three words of the workspace header, zero between calls
 int launch_plan_scan(const __nv_bfloat16* Cs, int Kp, int N, int ell, int npat, int budget,
-                     int policy, const ResidLists& rl, unsigned int* done_counter, cudaStream_t s);
+                     const ResidLists& rl, unsigned int* counters, cudaStream_t s);
 int launch_gsum(const float* G, int N, int d, float* gsum, cudaStream_t s);
-int launch_decode_resid(const float* G, const float* gsum, const ResidLists& rl, int ell, int npat,
-                        int d, float* Ghat, cudaStream_t s);
+int launch_decode_resid(const float* G, const float* gsum, const ResidLists& rl,
+                        const GemmChoice& gemm, int ell, int npat, int d, float* Ghat,
+                        cudaStream_t s);
 // Process-wide path policy of the batched decode (gc_set_decode_policy).
 int decode_policy();
 

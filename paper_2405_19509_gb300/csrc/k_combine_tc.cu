@@ -24,6 +24,11 @@
 //               to Ghat and/or reduce the squared error to sum_i g_{D_i}
 //               per row; the accumulator is handed back as soon as it is
 //               read, so the epilogue of tile t overlaps the MMAs of t + 1.
+// The rows of the GEMM are those of the patterns that the plan scan leaves to
+// it, gathered by the operand split (k_split_gt) into a compact A; a row's
+// place among them does not change its value.  Ghat is written from a staged
+// 32 x 32 box, four 128-byte row pieces a warp store (32 one-row pieces where
+// rows are not 16-byte multiples).
 // Tiles are visited n-tile-major so that concurrently running CTAs share the
 // same B tile through L2.  When one 64-wide block holds all of K the output
 // write bounds the kernel and the B tile is what the copies would mostly
@@ -61,35 +66,32 @@ constexpr int A_STAGE = 2 * A_PLANE;  // 32 KB
 constexpr int kBresStages = 2;        // A ring stages of the BRES shape
 constexpr int B_TILE = 2 * B_PLANE;   // 64 KB
 // NKBR > 0: B resident (NKBR k-blocks of the current n-tile), A streamed.
-// OUT: output staging boxes for TMA stores of Ghat (none in MSE-only shapes).
+// OUT: output staging boxes for the stores of Ghat (none in MSE-only shapes).
 template <int STAGES, int EPI, int NKBR, bool OUT>
 struct Shape {
   static constexpr bool BRES = NKBR > 0;
   static constexpr int THREADS = 64 + 32 * EPI;
-  static constexpr int OUT_BYTES = OUT ? EPI * 2 * OUT_BUF : 0;  // 2 staging boxes per epilogue warp
+  static constexpr int OUT_BYTES = OUT ? EPI * OUT_BUF : 0;  // a staging box per epilogue warp
+  static constexpr int ROW_BYTES = OUT ? EPI * 256 : 0;       // 32 row offsets per epilogue warp
   static constexpr int RING = BRES ? STAGES * A_STAGE + NKBR * B_TILE : STAGES * STAGE_BYTES;
-  static constexpr size_t SMEM = (size_t)RING + OUT_BYTES + 1024 + 256;
+  static constexpr size_t SMEM = (size_t)RING + OUT_BYTES + ROW_BYTES + 1024 + 256;
   static_assert(SMEM <= 232448, "shared memory per CTA");
 };
 
 struct Params {
-  int M, K, Kp, L, ell, d;
-  int num_m_tiles, num_n_tiles, nkb;
-  long long num_tiles;
+  int K, Kp, L, ell, d;
+  int num_n_tiles, nkb;
   int vec_ok;           // d % 4 == 0 && L % 4 == 0: 16-byte row segments
-  int tma_store;        // Ghat written by TMA tensor stores (needs d == ell * L, L % 4 == 0)
-  int evict_first;      // Ghat stores marked evict-first in L2
   float* Ghat;          // npat x d or null
   const float* gsum;    // d, or null when no MSE is wanted
   float* msep;          // M x parts_per_row partial squared errors, or null
   int parts_per_row;    // num_n_tiles * (epilogue warps per TMEM lane quarter)
   long long spin_limit; // clock cycles a wait may take before the kernel gives up
   int stall;            // failure-path test: the TMA producer issues nothing
-  // The m-tiles this kernel computes (the others come from the residual
-  // decode): dlist[0 .. *ndense) in ascending order, written by the plan scan
-  // before the launch; null = every m-tile.
-  const int32_t* dlist;
-  const int32_t* ndense;
+  // row r of the GEMM is row r % ell of pattern dpat[r / ell], r < *npat_gemm * ell
+  // (both written before the launch)
+  const int32_t* dpat;
+  const int32_t* npat_gemm;
   uint32_t* status;
 };
 
@@ -107,7 +109,7 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
 template <int STAGES, int EPI, int NKBR, bool OUT>
 __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     k_combine_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                 const __grid_constant__ CUtensorMap tmC, Params p) {
+                 Params p) {
   using Sh = Shape<STAGES, EPI, NKBR, OUT>;
   constexpr bool BRES = Sh::BRES;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -115,7 +117,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
                                              ~static_cast<uintptr_t>(1023));
   uint8_t* bres = smem + STAGES * A_STAGE;                       // BRES: resident B k-blocks
   float* outbuf = reinterpret_cast<float*>(smem + Sh::RING);     // 1024-aligned
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + Sh::RING + Sh::OUT_BYTES);
+  long long* rowbuf = reinterpret_cast<long long*>(smem + Sh::RING + Sh::OUT_BYTES);
+  uint64_t* full = reinterpret_cast<uint64_t*>(smem + Sh::RING + Sh::OUT_BYTES + Sh::ROW_BYTES);
   uint64_t* empty = full + STAGES;
   uint64_t* tfull = empty + STAGES;   // [2]
   uint64_t* tempty = tfull + 2;       // [2]
@@ -154,9 +157,10 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
   // launched as a programmatic dependent of the operand split: the prologue
   // above overlaps its tail, the operands are read only after this point
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  // the tile space: nd listed m-tiles x the n-tiles, n-tile-major;
+  // the tile space: nd m-tiles x the n-tiles, n-tile-major;
   // this CTA's tiles are t = t_first, t_first + t_step, ... < t_last
-  const int nd = p.ndense ? *reinterpret_cast<volatile const int*>(p.ndense) : p.num_m_tiles;
+  const int rows = *reinterpret_cast<volatile const int*>(p.npat_gemm) * p.ell;
+  const int nd = (rows + BM - 1) / BM;
   const long long ntiles = (long long)nd * p.num_n_tiles;
   long long t_first, t_last, t_step;
   if (BRES) {
@@ -168,10 +172,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     t_last = ntiles;
     t_step = gridDim.x;
   }
-  auto tile_mt = [&](long long t) -> int {
-    const int mi = (int)(t % nd);
-    return p.dlist ? __ldg(p.dlist + mi) : mi;
-  };
+  auto tile_mt = [&](long long t) -> int { return (int)(t % nd); };
 
   if (warp == 0) {
     // ------------------------------------------------------------- producer
@@ -326,8 +327,9 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     const int e = warp - 2;        // epilogue warp index
     constexpr int SPAN = BN / (EPI / 4);  // columns per epilogue warp
     const int cbeg = (e / 4) * SPAN;
-    float* wbuf = outbuf + e * 2 * (OUT_BUF / 4);
-    uint32_t tile_it = 0, chunk_it = 0;
+    float* wbuf = outbuf + e * (OUT_BUF / 4);
+    long long* wrow = rowbuf + e * 32;  // element offset of each of the warp's rows in Ghat, -1: none
+    uint32_t tile_it = 0;
     for (long long t = t_first; t < t_last; t += t_step, ++tile_it) {
       const int ab = tile_it & 1;
       const int nt = (int)(t / nd), mt = tile_mt(t);
@@ -336,11 +338,17 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       if (!__all_sync(0xffffffffu, ready)) break;
       fence_after();
       const int row = mt * BM + quarter * 32 + lane;
-      const bool rv = row < p.M;
-      const int b = rv ? row / p.ell : 0;
-      const int k = rv ? row - b * p.ell : 0;
+      const bool rv = row < rows;
+      const int bi = rv ? row / p.ell : 0;
+      const int k = rv ? row - bi * p.ell : 0;
+      const int b = rv ? __ldg(p.dpat + bi) : 0;
       const int n0 = nt * BN;
-      float* out = p.Ghat ? p.Ghat + (size_t)b * p.d + (size_t)k * p.L : nullptr;
+      if (OUT) {
+        __syncwarp();
+        wrow[lane] = rv ? (long long)b * p.d + (long long)k * p.L : -1;
+      }
+      // columns of the row that exist: L, less in a padded last block
+      const int rlim = rv ? min(p.L, p.d - k * p.L) : 0;
       const float* gs = p.gsum ? p.gsum + (size_t)k * p.L : nullptr;
       float sq4[4] = {0.f, 0.f, 0.f, 0.f};  // four independent FMA chains
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * BN);
@@ -366,59 +374,58 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
         __syncwarp();
         tmem_ld32(taddr + cc, v);  // warp-collective: every lane, every chunk
         const int c0 = n0 + cc;
-        if (OUT && p.tma_store && c0 < p.L) {
-          // stage the 32 x 32 box (row = lane) with the 128-byte swizzle, then one TMA store
-          float* buf = wbuf + (chunk_it & 1) * (OUT_BUF / 4);
-          if (lane == 0) bulk_wait_read1();  // the store that used this buffer has read it
-          __syncwarp();
-          char* rowp = reinterpret_cast<char*>(buf) + lane * 128;
+        if (OUT && p.Ghat && c0 < p.L) {
+          // stage the 32 x 32 box (row = lane; 16-byte pieces swizzled), then
+          // store it row by row
+          __syncwarp();  // the previous box has been read
+          char* box = reinterpret_cast<char*>(wbuf);
 #pragma unroll
           for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<float4*>(rowp + ((j ^ (lane & 7)) << 4)) =
+            *reinterpret_cast<float4*>(box + lane * 128 + ((j ^ (lane & 7)) << 4)) =
                 make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           __syncwarp();
-          if (lane == 0) {
-            if (p.evict_first)
-              tma_store_2d_hint(&tmC, buf, c0, mt * BM + quarter * 32, policy_evict_first());
-            else
-              tma_store_2d(&tmC, buf, c0, mt * BM + quarter * 32);
-            bulk_commit();
-          }
-          ++chunk_it;
-        }
-        const int lim = (rv && c0 < p.L) ? min(32, min(p.L - c0, p.d - k * p.L - c0)) : 0;
-        if (lim <= 0) {
-        } else if (lim == 32 && p.vec_ok) {
-          if (out && !p.tma_store) {
-            float4* o4 = reinterpret_cast<float4*>(out + c0);
+          if (p.vec_ok) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-              o4[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-          }
-          if (gs) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const float4 g = gcur[j];
-              float df = v[4 * j] - g.x;
-              sq4[0] = fmaf(df, df, sq4[0]);
-              df = v[4 * j + 1] - g.y;
-              sq4[1] = fmaf(df, df, sq4[1]);
-              df = v[4 * j + 2] - g.z;
-              sq4[2] = fmaf(df, df, sq4[2]);
-              df = v[4 * j + 3] - g.w;
-              sq4[3] = fmaf(df, df, sq4[3]);
+            for (int it = 0; it < 8; ++it) {
+              const int rr = it * 4 + (lane >> 3), j = lane & 7;
+              const long long ro = wrow[rr];
+              const int lim_r = __shfl_sync(0xffffffffu, rlim, rr);
+              const float4 q = *reinterpret_cast<const float4*>(box + rr * 128 + ((j ^ (rr & 7)) << 4));
+              if (ro >= 0 && c0 + 4 * j < lim_r)
+                __stcs(reinterpret_cast<float4*>(p.Ghat + ro + c0 + 4 * j), q);
             }
+          } else {
+#pragma unroll 8
+            for (int rr = 0; rr < 32; ++rr) {
+              const long long ro = wrow[rr];
+              const int lim_r = __shfl_sync(0xffffffffu, rlim, rr);
+              const float q = *reinterpret_cast<const float*>(
+                  box + rr * 128 + (((lane >> 2) ^ (rr & 7)) << 4) + (lane & 3) * 4);
+              if (ro >= 0 && c0 + lane < lim_r) __stcs(p.Ghat + ro + c0 + lane, q);
+            }
+          }
+        }
+        const int lim = min(32, rlim - c0);
+        if (!gs || lim <= 0) {
+        } else if (lim == 32 && p.vec_ok) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float4 g = gcur[j];
+            float df = v[4 * j] - g.x;
+            sq4[0] = fmaf(df, df, sq4[0]);
+            df = v[4 * j + 1] - g.y;
+            sq4[1] = fmaf(df, df, sq4[1]);
+            df = v[4 * j + 2] - g.z;
+            sq4[2] = fmaf(df, df, sq4[2]);
+            df = v[4 * j + 3] - g.w;
+            sq4[3] = fmaf(df, df, sq4[3]);
           }
         } else {
 #pragma unroll
           for (int j = 0; j < 32; ++j) {
             if (j < lim) {
-              if (out && !p.tma_store) out[c0 + j] = v[j];
-              if (gs) {
-                const float df = v[j] - __ldg(gs + c0 + j);
-                sq4[j & 3] = fmaf(df, df, sq4[j & 3]);
-              }
+              const float df = v[j] - __ldg(gs + c0 + j);
+              sq4[j & 3] = fmaf(df, df, sq4[j & 3]);
             }
           }
         }
@@ -427,9 +434,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[ab]);
       if (p.msep && rv)
-        p.msep[(size_t)row * p.parts_per_row + nt * (EPI / 4) + e / 4] = (sq4[0] + sq4[1]) + (sq4[2] + sq4[3]);
+        p.msep[((size_t)b * p.ell + k) * p.parts_per_row + nt * (EPI / 4) + e / 4] = (sq4[0] + sq4[1]) + (sq4[2] + sq4[3]);
     }
-    if (lane == 0) bulk_wait_all();  // every store of this warp has completed
   }
   fence_before();
   __syncthreads();
@@ -458,149 +464,158 @@ __global__ void k_split_c(const float* __restrict__ C, int M, int K, int Kp,
   out[tot + idx] = lo;
 }
 
-// G (N x d fp32) -> planes [2][L][Kp] bf16 of Gv^T: element (c, i*ell + k') =
-// g_{D_i}[k'*L + c] (zero past d and for padding columns).  Block (x, y)
-// transposes the tile of 32 K-rows (kk = 32 y ..) by COLS columns
-// (c = COLS x ..) through shared memory: 16-byte loads along c, 16-byte
-// stores along kk (COLS = 128 for long rows, 32 when L is short and more
-// blocks are wanted).  Blocks stride over the (column tile, K tile) pairs;
-// nothing is done when *ndense is zero: no row tile of the batch is on the
-// GEMM.
+// The GEMM's operands, when some pattern takes it (nothing is done otherwise).
+// B: G (N x d fp32) -> planes [2][L][Kp] bf16 of Gv^T: element (c, i*ell + k') =
+// g_{D_i}[k'*L + c] (zero past d and for padding columns).  A block transposes
+// the tile of 64 K-rows by COLS columns through shared memory: 16-byte loads
+// along c, and 128 consecutive bytes of a plane row per eight lanes on the way
+// out (COLS = 64 for long rows, 32 when L is short and more blocks are
+// wanted).  Blocks stride over the (column tile, K tile) pairs.
+// A: the plan rows of those patterns, copied to consecutive rows (one warp a
+// pattern; places are handed out as they come, which changes no value).
 template <int COLS>
 __global__ void __launch_bounds__(256) k_split_gt(const float* __restrict__ G, int N, int d,
                                                   int ell, int L, int Kp,
                                                   __nv_bfloat16* __restrict__ out,
-                                                  const int32_t* __restrict__ ndense) {
-  constexpr int kSplitCols = COLS;
+                                                  const __nv_bfloat16* __restrict__ Cs, int npat,
+                                                  __nv_bfloat16* __restrict__ Ca, ResidLists rl,
+                                                  GemmChoice gemm) {
   constexpr int TPR = COLS / 4;            // threads per row of the load phase
   constexpr int RPP = 256 / TPR;           // rows per pass
   // the combine kernel may be scheduled now; it waits for this grid to finish
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (ndense && __ldg(ndense) == 0) return;
-  __shared__ float tile[32][kSplitCols + 1];
-  const int ncx = (L + kSplitCols - 1) / kSplitCols;
-  const long long npair = (long long)ncx * (Kp / 32);
-  for (long long pr = blockIdx.x; pr < npair; pr += gridDim.x) {
-  __syncthreads();  // the previous pair's tile has been read
-  const int c0 = (int)(pr % ncx) * kSplitCols, k0 = (int)(pr / ncx) * 32;
-  const int t = threadIdx.x;
+  if (!gemm.any(rl)) return;
+  const int t = threadIdx.x, lane = t & 31;
+  {
+    const int thr = gemm.threshold(rl);
+    const size_t plane = (size_t)npat * ell * Kp;
+    const int per_plane = ell * Kp / 8;  // 16-byte pieces of a pattern's rows in a plane
+    for (int b = (blockIdx.x * 256 + t) >> 5; b < npat; b += gridDim.x * 8) {
+      if (__ldg(rl.nnz + b) <= thr) continue;
+      int slot = 0;
+      if (lane == 0) {
+        slot = atomicAdd(rl.stat + 2, 1);
+        rl.dpat[slot] = b;
+      }
+      slot = __shfl_sync(0xffffffffu, slot, 0);
+      for (int h = 0; h < 2; ++h) {
+        const uint4* src = reinterpret_cast<const uint4*>(Cs + h * plane + (size_t)b * ell * Kp);
+        uint4* dst = reinterpret_cast<uint4*>(Ca + h * plane + (size_t)slot * ell * Kp);
+        for (int q = lane; q < per_plane; q += 32) dst[q] = __ldg(src + q);
+      }
+    }
+  }
+  __shared__ float tile[64][COLS + 1];
+  const int ncx = (L + COLS - 1) / COLS;
+  const long long npair = (long long)ncx * (Kp / 64);
   const int K = N * ell;
   const bool vec = (L % 4 == 0) && (d % 4 == 0) && (reinterpret_cast<uintptr_t>(G) % 16 == 0);
-  // load: thread t takes columns 4 (t % TPR) .. +3 of rows t / TPR + RPP r
+  const size_t plane = (size_t)L * Kp;
+  for (long long pr = blockIdx.x; pr < npair; pr += gridDim.x) {
+    __syncthreads();  // the previous pair's tile has been read
+    const int c0 = (int)(pr % ncx) * COLS, k0 = (int)(pr / ncx) * 64;
+    // load: thread t takes columns 4 (t % TPR) .. +3 of rows t / TPR + RPP r
 #pragma unroll
-  for (int r = 0; r < 32 / RPP; ++r) {
-    const int kr = t / TPR + RPP * r, kk = k0 + kr;
-    const int cc = 4 * (t % TPR), c = c0 + cc;
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
-    if (kk < K) {
-      const int i = kk / ell, kp = kk - i * ell;
-      const float* src = G + (size_t)i * d + (size_t)kp * L + c;
-      if (vec && c + 3 < L && kp * L + c + 3 < d) {
-        const float4 q = __ldg(reinterpret_cast<const float4*>(src));
-        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-      } else {
+    for (int r = 0; r < 64 / RPP; ++r) {
+      const int kr = t / TPR + RPP * r, kk = k0 + kr;
+      const int cc = 4 * (t % TPR), c = c0 + cc;
+      float v[4] = {0.f, 0.f, 0.f, 0.f};
+      if (kk < K) {
+        const int i = kk / ell, kp = kk - i * ell;
+        const float* src = G + (size_t)i * d + (size_t)kp * L + c;
+        if (vec && c + 3 < L && kp * L + c + 3 < d) {
+          const float4 q = __ldg(reinterpret_cast<const float4*>(src));
+          v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (c + e < L && kp * L + c + e < d) v[e] = __ldg(src + e);
+          for (int e = 0; e < 4; ++e)
+            if (c + e < L && kp * L + c + e < d) v[e] = __ldg(src + e);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) tile[kr][cc + e] = v[e];
+    }
+    __syncthreads();
+    // store: thread t takes K-rows 8 (t % 8) .. +7 of columns t / 8 + 32 u
+#pragma unroll
+    for (int u = 0; u < COLS / 32; ++u) {
+      const int cc = t / 8 + 32 * u, kr = 8 * (t % 8), c = c0 + cc;
+      if (c < L) {
+        uint32_t hw[4], lw[4];
+#pragma unroll
+        for (int e = 0; e < 8; e += 2) {
+          const float a = tile[kr + e][cc], b = tile[kr + e + 1][cc];
+          const __nv_bfloat16 ha = __float2bfloat16_rn(a), hb = __float2bfloat16_rn(b);
+          const __nv_bfloat16 la = __float2bfloat16_rn(a - __bfloat162float(ha));
+          const __nv_bfloat16 lb = __float2bfloat16_rn(b - __bfloat162float(hb));
+          hw[e / 2] = (uint32_t)__bfloat16_as_ushort(ha) | ((uint32_t)__bfloat16_as_ushort(hb) << 16);
+          lw[e / 2] = (uint32_t)__bfloat16_as_ushort(la) | ((uint32_t)__bfloat16_as_ushort(lb) << 16);
+        }
+        const size_t o = (size_t)c * Kp + k0 + kr;  // Kp is a multiple of 64
+        *reinterpret_cast<uint4*>(out + o) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+        *reinterpret_cast<uint4*>(out + plane + o) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
       }
     }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) tile[kr][cc + e] = v[e];
-  }
-  __syncthreads();
-  // store: thread t takes column t % COLS and K-rows 16 (t / COLS) .. +15
-  if (t < 2 * kSplitCols) {
-    const int cc = t % kSplitCols, h = t / kSplitCols, c = c0 + cc;
-    if (c < L) {
-      uint32_t hw[8], lw[8];
-#pragma unroll
-      for (int e = 0; e < 16; e += 2) {
-        const float a = tile[16 * h + e][cc], b = tile[16 * h + e + 1][cc];
-        const __nv_bfloat16 ha = __float2bfloat16_rn(a), hb = __float2bfloat16_rn(b);
-        const __nv_bfloat16 la = __float2bfloat16_rn(a - __bfloat162float(ha));
-        const __nv_bfloat16 lb = __float2bfloat16_rn(b - __bfloat162float(hb));
-        hw[e / 2] = (uint32_t)__bfloat16_as_ushort(ha) | ((uint32_t)__bfloat16_as_ushort(hb) << 16);
-        lw[e / 2] = (uint32_t)__bfloat16_as_ushort(la) | ((uint32_t)__bfloat16_as_ushort(lb) << 16);
-      }
-      const int kk = k0 + 16 * h;
-      if (kk < Kp) {  // Kp is a multiple of 64, so the 16 entries are all inside
-        const size_t plane = (size_t)L * Kp;
-        uint4* dh = reinterpret_cast<uint4*>(out + (size_t)c * Kp + kk);
-        uint4* dl = reinterpret_cast<uint4*>(out + plane + (size_t)c * Kp + kk);
-        dh[0] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-        dh[1] = make_uint4(hw[4], hw[5], hw[6], hw[7]);
-        dl[0] = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-        dl[1] = make_uint4(lw[4], lw[5], lw[6], lw[7]);
-      }
-    }
-  }
   }
 }
 
-// grad_mse[b] = (sum over the rows b*ell .. b*ell+ell-1 of their partial
-// squared errors) / d: one warp per pattern; a row of a GEMM tile sums the
-// combine's partials, a row of a residual tile the residual kernel's (none
-// for a pattern whose blocks are all I_ell: its error is exactly zero).
-// Lanes stride over a row's partials, then a fixed xor tree; rows are added
-// in order (fp32 partial sums, the result scaled in fp64).  Launched as a
-// programmatic dependent of the combine kernel.
-__global__ void k_mse_reduce_tiles(const float* __restrict__ msep, int parts,
-                                   const float* __restrict__ msp, int parts_r,
-                                   const int32_t* __restrict__ tflag, const int32_t* __restrict__ rslot,
-                                   int npat, int ell, double inv_d, double* __restrict__ grad_mse) {
+// grad_mse[b] = (partial squared errors of pattern b) / d, one warp per pattern:
+// a pattern on the GEMM sums its rows' partials row by row, any other the
+// residual kernel's (none when its blocks are all I_ell: its error is exactly
+// zero).  Lanes stride over the partials, then a fixed xor tree (fp32 partial
+// sums, the result scaled in fp64).  Launched as a programmatic dependent of
+// the combine kernel.
+__device__ __forceinline__ float warp_partials(const float* __restrict__ r, int n, int lane) {
+  float s = 0.f;
+  if (n % 4 == 0 && (reinterpret_cast<uintptr_t>(r) & 15) == 0) {
+    // 16-byte loads, four in flight a lane (up to a few thousand partials)
+    const float4* r4 = reinterpret_cast<const float4*>(r);
+    const int n4 = n / 4;
+    float4 a[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    int t = lane;
+    for (; t + 96 < n4; t += 128) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 x = __ldg(r4 + t + 32 * u);
+        a[u].x += x.x;
+        a[u].y += x.y;
+        a[u].z += x.z;
+        a[u].w += x.w;
+      }
+    }
+    for (; t < n4; t += 32) {
+      const float4 x = __ldg(r4 + t);
+      a[0].x += x.x;
+      a[0].y += x.y;
+      a[0].z += x.z;
+      a[0].w += x.w;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s += (a[u].x + a[u].y) + (a[u].z + a[u].w);
+  } else {
+    for (int t = lane; t < n; t += 32) s += __ldg(r + t);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+__global__ void k_mse_reduce(const float* __restrict__ msep, int parts, ResidLists rl,
+                             GemmChoice gemm, int npat, int ell, double inv_d,
+                             double* __restrict__ grad_mse) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const long long b = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (b >= npat) return;
+  const int nz = __ldg(rl.nnz + b);
   float tot = 0.f;
-  for (int k = 0; k < ell; ++k) {
-    const long long row = b * ell + k;
-    const float* r = nullptr;
-    int n = 0;
-    if (__ldg(tflag + (row >> 7))) {
-      r = msep + (size_t)row * parts;
-      n = parts;
-    } else {
-      const int slot = __ldg(rslot + row);
-      if (slot >= 0) {
-        r = msp + (size_t)slot * parts_r;
-        n = parts_r;
-      }
-    }
-    float s = 0.f;
-    if (n % 4 == 0 && (reinterpret_cast<uintptr_t>(r) & 15) == 0) {
-      // 16-byte loads, four in flight a lane (a row has up to a few thousand partials)
-      const float4* r4 = reinterpret_cast<const float4*>(r);
-      const int n4 = n / 4;
-      float4 a[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-      int t = lane;
-      for (; t + 96 < n4; t += 128) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const float4 x = __ldg(r4 + t + 32 * u);
-          a[u].x += x.x;
-          a[u].y += x.y;
-          a[u].z += x.z;
-          a[u].w += x.w;
-        }
-      }
-      for (; t < n4; t += 32) {
-        const float4 x = __ldg(r4 + t);
-        a[0].x += x.x;
-        a[0].y += x.y;
-        a[0].z += x.z;
-        a[0].w += x.w;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) s += (a[u].x + a[u].y) + (a[u].z + a[u].w);
-    } else {
-      for (int t = lane; t < n; t += 32) s += __ldg(r + t);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    tot += s;
+  if (nz > gemm.threshold(rl)) {
+    for (int k = 0; k < ell; ++k)
+      tot += warp_partials(msep + ((size_t)b * ell + k) * parts, parts, lane);
+  } else if (nz > 0) {
+    tot = warp_partials(rl.msp + (size_t)b * rl.parts, rl.parts, lane);
   }
   if (lane == 0) grad_mse[b] = (double)tot * inv_d;
 }
@@ -616,22 +631,6 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
       fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
   }
   return fn;
-}
-
-// 2-D fp32 map over Ghat viewed as (npat*ell) rows of L (requires d == ell*L),
-// box 32 x 32, 128-byte swizzle (matches the epilogue's staging layout).
-int make_out_map(CUtensorMap* map, float* base, long long rows, int L) {
-  auto fn = encode_fn();
-  if (!fn) return fail(GC_ERR_CUDA, "cuTensorMapEncodeTiled entry point unavailable");
-  cuuint64_t dims[2] = {(cuuint64_t)L, (cuuint64_t)rows};
-  cuuint64_t strides[1] = {(cuuint64_t)L * 4};
-  cuuint32_t box[2] = {32, 32};
-  cuuint32_t estr[2] = {1, 1};
-  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return fail(GC_ERR_CUDA, "cuTensorMapEncodeTiled(out) failed (%d)", (int)r);
-  return GC_OK;
 }
 
 // 3-D map over [2][rows][Kp] bf16 planes, box {64, box_rows, 2}, 128-byte swizzle.
@@ -652,8 +651,8 @@ int make_map(CUtensorMap* map, const void* base, int rows, int Kp, int box_rows)
 }  // namespace tc
 
 template <int STAGES, int EPI, int NKBR, bool OUT>
-int launch_tc(int grid, const CUtensorMap& mA, const CUtensorMap& mB, const CUtensorMap& mC,
-              const tc::Params& p, cudaStream_t s) {
+int launch_tc(int grid, const CUtensorMap& mA, const CUtensorMap& mB, const tc::Params& p,
+              cudaStream_t s) {
   using Sh = tc::Shape<STAGES, EPI, NKBR, OUT>;
   static bool attr_set = false;
   if (!attr_set) {
@@ -672,7 +671,7 @@ int launch_tc(int grid, const CUtensorMap& mA, const CUtensorMap& mB, const CUte
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, tc::k_combine_tc<STAGES, EPI, NKBR, OUT>, mA, mB, mC, p);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, tc::k_combine_tc<STAGES, EPI, NKBR, OUT>, mA, mB, p);
   if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_combine_tc)");
   count_launches(1);
   return cuda_check(cudaGetLastError(), "k_combine_tc");
@@ -684,6 +683,7 @@ size_t apply_ws_bytes(int N, int ell, int npat, int d) {
   const int Kp = combine_kp(N, ell);
   const int nnt = (L + tc::BN - 1) / tc::BN;
   return std::max(align_up((size_t)2 * L * Kp * 2, 256) + align_up((size_t)d * sizeof(float), 256) +
+                      plan_bytes(N, ell, npat) +
                       align_up((size_t)M * nnt * 2 * sizeof(float), 256) +
                       resid_ws_bytes(N, ell, npat, d),
                   mse_gram_ws_bytes(N, ell, d));
@@ -699,10 +699,10 @@ int launch_split_c(const float* C, int N, int ell, int npat, __nv_bfloat16* Cs, 
   return cuda_check(cudaGetLastError(), "k_split_c");
 }
 
-// The decode of a batch: the plan scan picks the path of every 128-row tile
-// (k_decode_resid.cu); residual tiles are written by the residual kernel, the
-// others by the tensor-core GEMM (whose operand split runs only when some
-// tile needs it), then the per-pattern errors are reduced.
+// The decode of a batch: the plan scan picks the path of every pattern
+// (k_decode_resid.cu); the residual kernel writes those with few non-identity
+// blocks, the tensor-core GEMM the others (its operands are prepared only when
+// there are any), then the per-pattern errors are reduced.
 int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int npat, int d,
                  float* Ghat, double* grad_mse, Carve& ws, uint32_t* status, cudaStream_t s) {
   using namespace tc;
@@ -719,71 +719,60 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
   const int nmt = (int)((M + BM - 1) / BM), nnt = (L + BN - 1) / BN;
   __nv_bfloat16* Gs = ws.take<__nv_bfloat16>((size_t)2 * L * Kp);
   float* gsum = ws.take<float>((size_t)d);
+  __nv_bfloat16* Ca = ws.take<__nv_bfloat16>((size_t)2 * M * Kp);
   float* msep_mem = ws.take<float>((size_t)M * nnt * 2);
   float* msep = grad_mse ? msep_mem : nullptr;
   const ResidLists rl = carve_resid(ws, N, ell, npat, d, grad_mse != nullptr);
-  // a residual tile may spend up to Kp / 64 corrections per pattern: about
-  // what the three MMAs per 64-wide K block cost against reading the ell
-  // blocks of one chunk gradient
-  const int budget = std::max(1, Kp / 64);
-  // header word 4: completion counter of the plan scan (zeroed with the header)
-  unsigned int* counter = reinterpret_cast<unsigned int*>(status) + 4;
-  int rc = launch_plan_scan(Cs, Kp, N, ell, npat, budget, policy, rl, counter, s);
+  // A non-identity block costs the residual path one read of a chunk gradient
+  // (4 d bytes, mostly from L2); a pattern costs the GEMM 6 Kp d flops.  At the
+  // rates of the two (about 10 TB/s, 1.6 PFLOP/s) they meet at Kp / 107 blocks;
+  // the split of G is worth about 2 N blocks.
+  GemmChoice gemm{policy, std::max(1, Kp / 64), rl.ksp, 2 * N};
+  // header words 4..6: counters of the plan scan (zeroed with the header)
+  unsigned int* counters = reinterpret_cast<unsigned int*>(status) + 4;
+  int rc = launch_plan_scan(Cs, Kp, N, ell, npat, gemm.budget, rl, counters, s);
   if (rc) return rc;
   // s = sum_i g_{D_i}: the residual rows start from it, the GEMM's MSE uses it
   rc = launch_gsum(G, N, d, gsum, s);
   if (rc) return rc;
   if (policy != GC_DECODE_DENSE) {
-    rc = launch_decode_resid(G, gsum, rl, ell, npat, d, Ghat, s);
+    rc = launch_decode_resid(G, gsum, rl, gemm, ell, npat, d, Ghat, s);
     if (rc) return rc;
   }
   {
     // a grid of a few blocks per SM striding over the tiles: it costs little
-    // to launch when no row tile is on the GEMM
-    const int cols = L >= 16384 ? 128 : 32;
-    const long long pairs = (long long)((L + cols - 1) / cols) * (Kp / 32);
-    const unsigned blocks = (unsigned)std::min<long long>(pairs, 8LL * device_sm_count());
-    if (cols == 128)
-      k_split_gt<128><<<blocks, 256, 0, s>>>(G, N, d, ell, L, Kp, Gs, rl.ndense);
+    // to launch when no pattern is on the GEMM
+    const int cols = L >= 16384 ? 64 : 32;
+    const long long pairs = (long long)((L + cols - 1) / cols) * (Kp / 64);
+    const unsigned blocks = (unsigned)std::min<long long>(std::max<long long>(pairs, (npat + 7) / 8),
+                                                          8LL * device_sm_count());
+    if (cols == 64)
+      k_split_gt<64><<<blocks, 256, 0, s>>>(G, N, d, ell, L, Kp, Gs, Cs, npat, Ca, rl, gemm);
     else
-      k_split_gt<32><<<blocks, 256, 0, s>>>(G, N, d, ell, L, Kp, Gs, rl.ndense);
+      k_split_gt<32><<<blocks, 256, 0, s>>>(G, N, d, ell, L, Kp, Gs, Cs, npat, Ca, rl, gemm);
     count_launches(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(e, "k_split_gt");
   }
-  CUtensorMap mA, mB, mC;
-  rc = make_map(&mA, Cs, (int)M, Kp, BM);
+  CUtensorMap mA, mB;
+  rc = make_map(&mA, Ca, (int)M, Kp, BM);
   if (rc) return rc;
   rc = make_map(&mB, Gs, L, Kp, BN);
   if (rc) return rc;
-  const bool tma_store = Ghat && (long long)ell * L == d && L % 4 == 0 &&
-                         reinterpret_cast<uintptr_t>(Ghat) % 16 == 0;
-  memset(&mC, 0, sizeof(mC));
-  if (tma_store) {
-    rc = make_out_map(&mC, Ghat, M, L);
-    if (rc) return rc;
-  }
   Params p{};
-  p.M = (int)M;
   p.K = K;
   p.Kp = Kp;
   p.L = L;
   p.ell = ell;
   p.d = d;
-  p.num_m_tiles = nmt;
   p.num_n_tiles = nnt;
   p.nkb = (Kp + BK - 1) / BK;
-  p.num_tiles = (long long)nmt * nnt;
-  p.vec_ok = (d % 4 == 0) && (L % 4 == 0);
-  p.tma_store = tma_store ? 1 : 0;
-  // Ghat is written once and not read back by this kernel: its lines go
-  // first when L2 needs room (measured ~1% per logistic step)
-  p.evict_first = 1;
+  p.vec_ok = (d % 4 == 0) && (L % 4 == 0) && reinterpret_cast<uintptr_t>(Ghat) % 16 == 0;
   p.Ghat = Ghat;
   p.gsum = grad_mse ? gsum : nullptr;
   p.msep = msep;
-  p.dlist = rl.dlist;
-  p.ndense = rl.ndense;
+  p.dpat = rl.dpat;
+  p.npat_gemm = rl.stat + 2;
   p.status = status;
   p.spin_limit = wait_limit(kSpin);
   p.stall = take_stall(GC_STALL_COMBINE) ? 1 : 0;
@@ -795,10 +784,10 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
   const bool two_res = p.nkb == 2 && !Ghat;
   p.parts_per_row = nnt * ((one_block || two_res) ? 2 : 1);
   const int sms = device_sm_count();
-  const int grid = (int)std::min<long long>(p.num_tiles, sms);
-  rc = one_block ? launch_tc<kBresStages, 8, 1, true>(grid, mA, mB, mC, p, s)
-       : two_res ? launch_tc<3, 8, 2, false>(grid, mA, mB, mC, p, s)
-                 : launch_tc<2, 4, 0, true>(grid, mA, mB, mC, p, s);
+  const int grid = (int)std::min<long long>((long long)nmt * nnt, sms);
+  rc = one_block ? launch_tc<kBresStages, 8, 1, true>(grid, mA, mB, p, s)
+       : two_res ? launch_tc<3, 8, 2, false>(grid, mA, mB, p, s)
+                 : launch_tc<2, 4, 0, true>(grid, mA, mB, p, s);
   if (rc) return rc;
   if (grad_mse) {
     cudaLaunchConfig_t cfg{};
@@ -810,10 +799,9 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_mse_reduce_tiles, (const float*)msep, p.parts_per_row,
-                                       (const float*)rl.msp, rl.parts, (const int32_t*)rl.tflag,
-                                       (const int32_t*)rl.rslot, npat, ell, 1.0 / (double)d, grad_mse);
-    if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_mse_reduce_tiles)");
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_mse_reduce, (const float*)msep, p.parts_per_row, rl,
+                                       gemm, npat, ell, 1.0 / (double)d, grad_mse);
+    if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_mse_reduce)");
     count_launches(1);
   }
   return GC_OK;

@@ -234,6 +234,47 @@ def test_ragged_shapes_both_paths(gc, d, ell, npat):
             assert_mse_close(float(res["grad_mse"][b]), r.grad_mse, floor, f"policy {pol} b={b}")
 
 
+@pytest.mark.parametrize("ell,d,npat,every", [
+    (4, 4096, 300, 7),    # 43 gathered patterns: a second, partial row tile
+    (3, 1000, 200, 5),    # patterns of three rows across the GEMM's tiles, padded last block
+    (2, 1601, 129, 64),   # two or three gathered patterns, rows that are no 16-byte pieces
+    (1, 2048, 40, 1),     # every pattern gathered
+])
+def test_heavy_patterns_are_gathered(gc, ell, d, npat, every):
+    """N = m = 40, delta = 8: one pattern in `every` has more non-identity blocks than its list
+    holds and takes the GEMM, wherever it stands; the others stay on the residual path under
+    the automatic and the residual policy (an exact one is the plain sum, with zero error)."""
+    N = m = 40
+    delta = 8
+    order = O.cyclic_order(N, m, delta)
+    rng = np.random.default_rng(ell * 1000 + npat)
+    R = rng.standard_normal((ell, m))
+    psi = np.full((npat, m), delta, dtype=np.int32)
+    psi[3::11, 5] = 0  # ell copies are left of every chunk
+    heavy = np.arange(every - 1, npat, every)
+    psi[heavy] = 0
+    psi[heavy, rng.integers(0, m, size=heavy.size)] = 4  # 36 of the 40 chunks have no copy
+    G32 = rng.standard_normal((N, d)).astype(np.float32)
+    Gref = G32.astype(np.float64)
+    gsum = Gref.sum(axis=0)
+    floor = 1e-8 * float(gsum @ gsum) / d
+    Rd, od, pd = dev_tensors(R, order, psi)
+    Gd = torch.from_numpy(G32).cuda()
+    nnz = (_copies(order, psi, N) < ell).sum(axis=1)
+    assert (nnz[heavy] > 32).all()
+    exact = np.flatnonzero(nnz == 0)
+    full = gc.gc_decode_batch(Rd, ell, od, N, m, delta, torch.full((1, m), delta, dtype=torch.int32, device="cuda"), Gd)["Ghat"]
+    for pol in (gc.GC_DECODE_AUTO, gc.GC_DECODE_RESIDUAL):
+        for _ in range(2):  # the counters are back at zero for the second call
+            res = _decode(gc, pol, Rd, ell, od, N, m, delta, pd, Gd)
+        Gh, ms = to_np(res["Ghat"]), to_np(res["grad_mse"])
+        assert np.all(ms[exact] == 0.0) and all(np.array_equal(Gh[b], to_np(full[0])) for b in exact)
+        for b in set(heavy) | set(range(0, npat, 13)):
+            r = O.run_pattern(R, order, psi[b], N, Gref, want_transmit=False)
+            assert_grad_close(Gh[b], r.ghat, f"policy {pol} b={b}")
+            assert_mse_close(float(ms[b]), r.grad_mse, floor, f"policy {pol} b={b}")
+
+
 def test_combine_non_projector_matrix(gc):
     """gc_decode_combine with a decode matrix whose blocks, in one pattern in
     four, are near but not exactly I (every block of such a pattern differs
