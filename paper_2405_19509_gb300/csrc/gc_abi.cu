@@ -297,10 +297,9 @@ int gc_find_encoding_coeff(const double* R, int ell, const int32_t* order, int N
   cudaStream_t s = as_stream(stream);
   Carve c(ws);
   SolveWs sw = carve_solve(c, N, m, delta, ell, npat);
-  launch_holders(order, N, m, delta, sw.h, status_of(ws), s);
   SolveOut out{E, C, delta_out, support, coef_err, est};
-  return launch_solve_impl(R, ell, psi, sw.h, N, m, delta, npat, out, sw.table, sw.bits,
-                           status_of(ws), s);
+  return launch_coeffs(R, ell, order, psi, sw.h, N, m, delta, npat, out, sw.table, sw.bits,
+                       status_of(ws), s);
 }
 
 // ---------------------------------------------------------------- encode
@@ -328,10 +327,9 @@ int gc_encode(const double* R, int ell, const int32_t* order, int N, int m, int 
   Carve c(ws);
   SolveWs sw = carve_solve(c, N, m, delta, ell, npat);
   double* E = c.take<double>((size_t)npat * m * delta * ell);
-  launch_holders(order, N, m, delta, sw.h, status_of(ws), s);
   SolveOut out{E, nullptr, nullptr, nullptr, nullptr, nullptr};
-  rc = launch_solve_impl(R, ell, psi, sw.h, N, m, delta, npat, out, sw.table, sw.bits,
-                         status_of(ws), s);
+  rc = launch_coeffs(R, ell, order, psi, sw.h, N, m, delta, npat, out, sw.table, sw.bits,
+                     status_of(ws), s);
   if (rc) return rc;
   return launch_encode(E, order, psi, N, m, delta, ell, npat, G, d, T, s);
 }

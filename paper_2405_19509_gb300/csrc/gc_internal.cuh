@@ -109,6 +109,12 @@ int launch_solve_impl(const double* R, int ell, const int32_t* psi, Holders h, i
                       int delta, int npat, SolveOut out, void* table_mem, int bits,
                       uint32_t* status, cudaStream_t s, bool build_table = true);
 
+// Algorithm 1 from the order: the holder table and the solve, or for the
+// coefficients of few problems alone one kernel that does both.
+int launch_coeffs(const double* R, int ell, const int32_t* order, const int32_t* psi, Holders h,
+                  int N, int m, int delta, int npat, SolveOut out, void* table_mem, int bits,
+                  uint32_t* status, cudaStream_t s);
+
 // ---- chunk gradients (k_chunkgrad.cu) -----------------------------------
 size_t chunkgrad_ws_bytes(int N, int n_c, int d, int x_dtype);
 int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w, int N, int n_c,

@@ -133,7 +133,6 @@ extern "C" int gc_find_encoding_coeff_noalloc(const double* R, int ell, const in
   Holders h = carve_holders(c, N);
   void* table = bits >= 0 ? c.take<char>(solve_table_bytes(N, ell, bits)) : nullptr;
   uint32_t* status = static_cast<uint32_t*>(ws);
-  launch_holders(order, N, m, delta, h, status, s);
   SolveOut out{E, C, delta_out, support, coef_err, est};
-  return launch_solve_impl(R, ell, psi, h, N, m, delta, npat, out, table, bits, status, s);
+  return launch_coeffs(R, ell, order, psi, h, N, m, delta, npat, out, table, bits, status, s);
 }

@@ -44,53 +44,49 @@ Holders carve_holders(Carve& c, int N) {
   return h;
 }
 
-// One CTA per chunk: scan order[] in (worker, slot) order and compact the
-// matches, which keeps holders sorted by worker then slot.
-__global__ void k_holders(const int32_t* __restrict__ order, int N, int m, int delta, Holders h,
-                          uint32_t* status) {
-  const int i = blockIdx.x;
-  __shared__ int s_warp[32];
-  __shared__ int s_base;
-  if (threadIdx.x == 0) s_base = 0;
-  __syncthreads();
+// One warp per chunk: scan order[] in (worker, slot) order, 128 entries a step,
+// and compact the matches, which keeps holders sorted by worker then slot.
+// Latency bound (no barriers, eight loads in flight): 256 chunks, delta 16 in
+// 3 us, against 14 with a block per chunk and three barriers per 256 entries.
+__global__ void __launch_bounds__(128) k_holders(const int32_t* __restrict__ order, int N, int m,
+                                                 int delta, Holders h, uint32_t* status) {
+  const int i = blockIdx.x * 4 + (threadIdx.x >> 5);
+  if (i >= N) return;
   const int total = m * delta;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-  for (int t0 = 0; t0 < total; t0 += blockDim.x) {
-    const int t = t0 + threadIdx.x;
-    int v = -1;
-    if (t < total) {
-      v = order[t];
-      if ((v < -1 || v >= N) && i == 0) atomicOr(status, ST_BAD_ORDER);
+  const int lane = threadIdx.x & 31;
+  int base = 0;
+  bool bad = false;
+#pragma unroll 2
+  for (int t0 = 0; t0 < total; t0 += 128) {
+    int v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = t0 + 32 * u + lane;
+      v[u] = t < total ? __ldg(order + t) : -1;
     }
-    const bool hit = (t < total) && v == i;
-    const unsigned bal = __ballot_sync(0xffffffffu, hit);
-    if (lane == 0) s_warp[warp] = __popc(bal);
-    __syncthreads();
-    int off = s_base;
-    for (int w = 0; w < warp; ++w) off += s_warp[w];
-    off += __popc(bal & ((1u << lane) - 1u));
-    if (hit) {
-      if (off < GC_MAX_REPL) {
-        h.w[(size_t)i * GC_MAX_REPL + off] = (int16_t)(t / delta);
-        h.p[(size_t)i * GC_MAX_REPL + off] = (int8_t)(t % delta);
-      } else {
-        atomicOr(status, ST_BAD_ORDER);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int t = t0 + 32 * u + lane;
+      bad |= v[u] < -1 || v[u] >= N;
+      const bool hit = v[u] == i;
+      const unsigned bal = __ballot_sync(0xffffffffu, hit);
+      if (hit) {
+        const int off = base + __popc(bal & ((1u << lane) - 1u));
+        if (off < GC_MAX_REPL) {
+          h.w[(size_t)i * GC_MAX_REPL + off] = (int16_t)(t / delta);
+          h.p[(size_t)i * GC_MAX_REPL + off] = (int8_t)(t % delta);
+        }
       }
+      base += __popc(bal);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int s = 0;
-      for (int w = 0; w < nwarp; ++w) s += s_warp[w];
-      s_base += s;
-    }
-    __syncthreads();
   }
-  if (threadIdx.x == 0) h.cnt[i] = s_base < GC_MAX_REPL ? s_base : GC_MAX_REPL;
+  if ((i == 0 && bad) || base > GC_MAX_REPL) atomicOr(status, ST_BAD_ORDER);
+  if (lane == 0) h.cnt[i] = base < GC_MAX_REPL ? base : GC_MAX_REPL;
 }
 
 void launch_holders(const int32_t* order, int N, int m, int delta, Holders h, uint32_t* status,
                     cudaStream_t s) {
-  k_holders<<<N, 256, 0, s>>>(order, N, m, delta, h, status);
+  k_holders<<<(N + 3) / 4, 128, 0, s>>>(order, N, m, delta, h, status);
   count_launches(1);
 }
 
@@ -99,7 +95,13 @@ void launch_holders(const int32_t* order, int N, int m, int delta, Holders h, ui
 // emit(h, k, v) receives X^+ row of holder h (0 for holders not in S_i).
 // Returns Delta; Pi (ell x ell) and err = ||I - Pi||_F^2 by reference.
 // ---------------------------------------------------------------------------
-template <int ELL, typename Emit>
+template <bool SHARED>
+__device__ __forceinline__ double r_load(const double* p) {
+  if constexpr (SHARED) return *p;
+  return __ldg(p);
+}
+// SHARED: R lies in shared memory.
+template <int ELL, bool SHARED = false, typename Emit>
 __device__ __forceinline__ int solve_block(const double* __restrict__ R, int m, int cnt,
                                            const int16_t* __restrict__ hw, uint32_t mask,
                                            double (&Pi)[ELL][ELL], double& err, uint32_t* status,
@@ -122,7 +124,7 @@ __device__ __forceinline__ int solve_block(const double* __restrict__ R, int m, 
       const int j = hw[h];
       double x[ELL];
 #pragma unroll
-      for (int a = 0; a < ELL; ++a) x[a] = __ldg(R + (size_t)a * m + j);
+      for (int a = 0; a < ELL; ++a) x[a] = r_load<SHARED>(R + (size_t)a * m + j);
 #pragma unroll
       for (int a = 0; a < ELL; ++a)
 #pragma unroll
@@ -193,7 +195,7 @@ __device__ __forceinline__ int solve_block(const double* __restrict__ R, int m, 
       const int j = hw[h];
       double x[ELL];
 #pragma unroll
-      for (int a = 0; a < ELL; ++a) x[a] = __ldg(R + (size_t)a * m + j);
+      for (int a = 0; a < ELL; ++a) x[a] = r_load<SHARED>(R + (size_t)a * m + j);
 #pragma unroll
       for (int k = 0; k < ELL; ++k) {
         double bk = 0.0;
@@ -218,7 +220,7 @@ __device__ __forceinline__ int solve_block(const double* __restrict__ R, int m, 
       const int j = hw[h];
       double x[ELL];
 #pragma unroll
-      for (int a = 0; a < ELL; ++a) x[a] = __ldg(R + (size_t)a * m + j);
+      for (int a = 0; a < ELL; ++a) x[a] = r_load<SHARED>(R + (size_t)a * m + j);
 #pragma unroll
       for (int k = 0; k < ELL; ++k) {
         double bk = 0.0;
@@ -249,7 +251,7 @@ __device__ __forceinline__ int solve_block(const double* __restrict__ R, int m, 
       for (int r = 0; r < MQ; ++r) Rr[r][qq] = 0.0;
 #pragma unroll
       for (int a = 0; a < ELL; ++a) {
-        Xc[qq][a] = (qq < D) ? __ldg(R + (size_t)a * m + jq[qq]) : 0.0;
+        Xc[qq][a] = (qq < D) ? r_load<SHARED>(R + (size_t)a * m + jq[qq]) : 0.0;
         Q[qq][a] = 0.0;
         Xp[qq][a] = 0.0;
       }
@@ -842,6 +844,152 @@ static void run_solve(const double* R, const int32_t* psi, Holders h, int N, int
   else
     k_patterns<ELL, false><<<grid, kPatThreads, 0, s>>>(R, psi, h, N, m, delta, npat, ppb, tb, out,
                                                        status);
+}
+
+// Coefficients alone (no decode matrix, no errors) of few (pattern, chunk)
+// problems, the encode of one or a few realizations: block (x, b) does chunks
+// 8 x .. 8 x + 7 of pattern b, one a lane of its first warp, after its warps
+// have built those chunks' holder rows from the order and staged R, all in
+// shared memory.  One launch instead of the holder table's, the zeroing of E
+// and the solve.  Latency bound by a problem's chain of fp64 operations (65
+// cycles each), so the problems are spread over many SMs: 256 chunks, delta
+// 16, ell 2, one pattern: 21 us, against 14 + 44 with one block a pattern; 20
+// chunks, delta 4: 8 us against 13 and the memset.  (32 chunks a block: 24 us;
+// four holders at once for more independent operations: no difference.)
+constexpr int kFewThreads = 256, kFewWarps = kFewThreads / 32;
+constexpr int kFewChunks = 8;      // chunks a block
+constexpr int kFewR = 4096;        // doubles of R staged (32 KB)
+constexpr int kFewBlocks = 8 * 152;  // at most: eight blocks an SM
+template <int ELL>
+__global__ void __launch_bounds__(kFewThreads) k_coeff_few(const double* __restrict__ R,
+                                                           const int32_t* __restrict__ order,
+                                                           const int32_t* __restrict__ psi, int N,
+                                                           int m, int delta, double* __restrict__ E,
+                                                           uint32_t* status) {
+  __shared__ double s_r[kFewR];
+  __shared__ int s_cnt[kFewWarps][32];
+  __shared__ __align__(16) int16_t s_w[kFewChunks][GC_MAX_REPL];
+  __shared__ int8_t s_p[kFewChunks][GC_MAX_REPL];
+  const int i0 = blockIdx.x * kFewChunks;
+  const long long b = blockIdx.y;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int total = m * delta;
+  double* Eb = E + (size_t)b * total * ELL;
+  for (int t = threadIdx.x; t < ELL * m; t += kFewThreads) s_r[t] = R[t];
+  s_cnt[warp][lane] = 0;
+  __syncwarp();
+  // warp w scans entries [t_lo, t_hi) in order: first the matches per chunk
+  // are counted, then, with the counts of the warps before it, placed
+  const int per = ((total + kFewWarps - 1) / kFewWarps + 31) / 32 * 32;
+  const int t_lo = min(total, warp * per), t_hi = min(total, t_lo + per);
+  bool bad = false;
+  // the first steps' entries are held from the counting to the placing
+  constexpr int kHeld = 16;
+  int held[kHeld];
+#pragma unroll
+  for (int u = 0; u < kHeld; ++u) {
+    const int t = t_lo + 32 * u + lane;
+    held[u] = t < t_hi ? __ldg(order + t) : -1;
+  }
+  auto step = [&](int t, int v, bool place) {
+    const bool valid = v >= 0 && v < N;
+    bad |= v < -1 || v >= N;
+    const int c = valid && v >= i0 && v < i0 + kFewChunks ? v - i0 : -1;
+    const unsigned any = __ballot_sync(0xffffffffu, c >= 0);
+    int pos = 0;
+    if (any) {  // warp-uniform
+      const unsigned same = __match_any_sync(0xffffffffu, c);
+      if (c >= 0) pos = s_cnt[warp][c] + __popc(same & ((1u << lane) - 1u));
+      __syncwarp();
+      if (c >= 0 && (same >> lane) == 1u) s_cnt[warp][c] = pos + 1;  // the last of its matches
+      __syncwarp();
+    }
+    if (!place) return;
+    // the coefficients no chunk's solve writes: empty slots (by one block),
+    // copies past GC_MAX_REPL
+    bool zero = t < t_hi && !valid && blockIdx.x == 0;
+    if (c >= 0) {
+      if (pos < GC_MAX_REPL) {
+        s_w[c][pos] = (int16_t)(t / delta);
+        s_p[c][pos] = (int8_t)(t % delta);
+      } else {
+        zero = true;
+        atomicOr(status, ST_BAD_ORDER);
+      }
+    }
+    if (zero) {
+#pragma unroll
+      for (int k = 0; k < ELL; ++k) Eb[(size_t)t * ELL + k] = 0.0;
+    }
+  };
+  auto scan = [&](bool place) {
+#pragma unroll
+    for (int u = 0; u < kHeld; ++u)
+      if (t_lo + 32 * u < t_hi) step(t_lo + 32 * u + lane, held[u], place);
+    for (int t0 = t_lo + 32 * kHeld; t0 < t_hi; t0 += 32)
+      step(t0 + lane, t0 + lane < t_hi ? __ldg(order + t0 + lane) : -1, place);
+  };
+  scan(false);
+  __syncthreads();
+  if (warp == 0) {  // exclusive sums over the warps; lane = chunk
+    int run = 0;
+#pragma unroll
+    for (int w = 0; w < kFewWarps; ++w) {
+      const int c = s_cnt[w][lane];
+      s_cnt[w][lane] = run;
+      run += c;
+    }
+  }
+  __syncthreads();
+  scan(true);
+  if (bad && blockIdx.x == 0 && b == 0) atomicOr(status, ST_BAD_ORDER);
+  __syncthreads();
+  const int i = i0 + lane;
+  if (warp != 0 || lane >= kFewChunks || i >= N) return;
+  const int cnt = min(s_cnt[kFewWarps - 1][lane], GC_MAX_REPL);  // past the last warp's matches
+  const int32_t* ps = psi + (size_t)b * m;
+  uint32_t mask = 0;
+  for (int h = 0; h < cnt; ++h) {
+    int v = __ldg(ps + s_w[lane][h]);
+    if (v < 0 || v > delta) {
+      atomicOr(status, ST_BAD_PSI);
+      v = 0;
+    }
+    if (s_p[lane][h] < v) mask |= 1u << h;
+  }
+  double Pi[ELL][ELL], err;
+  solve_block<ELL, true>(s_r, m, cnt, s_w[lane], mask, Pi, err, status, [&](int h, int k, double v) {
+    Eb[((size_t)s_w[lane][h] * delta + s_p[lane][h]) * ELL + k] = v;
+  });
+}
+
+int launch_coeffs(const double* R, int ell, const int32_t* order, const int32_t* psi, Holders h,
+                  int N, int m, int delta, int npat, SolveOut out, void* table_mem, int bits,
+                  uint32_t* status, cudaStream_t s) {
+  const bool only_e = out.E && !out.C && !out.Cs && !out.delta_out && !out.support &&
+                      !out.coef_err && !out.est;
+  const int groups = (N + kFewChunks - 1) / kFewChunks;
+  if (only_e && bits < 0 && (long long)groups * npat <= kFewBlocks && ell * m <= kFewR) {
+    const dim3 grid((unsigned)groups, (unsigned)npat);
+#define GC_FEW(E_) \
+  case E_: k_coeff_few<E_><<<grid, kFewThreads, 0, s>>>(R, order, psi, N, m, delta, out.E, status); break;
+    switch (ell) {
+      GC_FEW(1)
+      GC_FEW(2)
+      GC_FEW(3)
+      GC_FEW(4)
+      GC_FEW(5)
+      GC_FEW(6)
+      GC_FEW(7)
+      GC_FEW(8)
+      default: return fail(GC_ERR_UNSUPPORTED, "ell=%d exceeds GC_MAX_ELL", ell);
+    }
+#undef GC_FEW
+    count_launches(1);
+    return cuda_check(cudaGetLastError(), "k_coeff_few");
+  }
+  launch_holders(order, N, m, delta, h, status, s);
+  return launch_solve_impl(R, ell, psi, h, N, m, delta, npat, out, table_mem, bits, status, s);
 }
 
 // The table region is carved by the caller right after the holders.  With

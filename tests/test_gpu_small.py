@@ -334,6 +334,54 @@ def test_singular_R_flagged(gc):
     assert ei.value.code == -7 and "rank" in str(ei.value)
 
 
+@pytest.mark.parametrize("N,m,delta,ell,npat", [(1, 1, 1, 1, 1), (9, 9, 4, 2, 2), (8, 30, 5, 3, 1),
+                                                (300, 300, 14, 2, 3), (40, 7, 12, 4, 5),
+                                                (33, 33, 6, 8, 1), (70, 260, 16, 2, 1)])
+def test_few_coefficients_match_the_batched_solve(gc, N, m, delta, ell, npat):
+    """Coefficients alone of few patterns (one kernel builds the holder rows and solves) against
+    the same call with the errors (holder table, then solve), bit for bit, for random explicit
+    orders with empty slots; a psi outside [0, delta] and a chunk with too many copies are
+    flagged as there."""
+    rng = np.random.default_rng(N * 7 + m)
+    order = -np.ones((m, delta), np.int32)
+    copies = np.zeros(N, int)
+    for j in range(m):
+        row = [i for i in rng.permutation(N) if copies[i] < 32][:rng.integers(0, delta + 1)]
+        copies[row] += 1
+        order[j, :len(row)] = row
+    R = rng.standard_normal((ell, m))
+    psi = rng.integers(0, delta + 1, size=(npat, m)).astype(np.int32)
+    assert npat < 2 ** delta or npat == 1
+
+    def both(order, psi):
+        Rd, od, pd = dev_tensors(R, order, psi)
+        ws = [gc.Workspace(), gc.Workspace()]
+        n0 = gc.gc_kernel_launches()
+        E = torch.full((npat, m, delta, ell), float("nan"), dtype=torch.float64, device="cuda")
+        gc.gc_find_encoding_coeff(Rd, ell, od, N, m, delta, pd, E=E, C=False, delta_out=False,
+                                  coef_err=False, est=False, ws=ws[0])
+        assert gc.gc_kernel_launches() == n0 + 1
+        E2 = gc.gc_find_encoding_coeff(Rd, ell, od, N, m, delta, pd, ws=ws[1])["E"]
+        said = []
+        for w in ws:
+            try:
+                w.status()
+                said.append("")
+            except gc.GCError as e:
+                said.append(str(e))
+        assert said[0] == said[1] and torch.equal(E, E2)
+        return said[0]
+    both(order, psi)
+    psi[0, m // 2] = delta + 1
+    if (order[m // 2] >= 0).any():
+        assert "psi" in both(order, psi)
+    if N == 70:  # 33 copies of chunk 0, and an entry past N
+        order[:33, 0], order[40, 1] = 0, N
+        order[:33, 1:] = -1
+        psi[0, m // 2] = 0
+        assert "order" in both(order, psi)
+
+
 def test_encode_with_coeffs_matches_encode(gc):
     """Algorithm 1 then eq. (2) in two calls gives the same transmissions as
     gc_encode, and the oracle's."""
