@@ -14,15 +14,24 @@
 // copy only when its worker has finished all of its chunks (at delta_j
 // tau_j) is the completion time of the original protocol (Sec. IV).
 //
-// GB300 design: one warp per realization.  Lanes take chunks, gather their
-// holders' completion times from the holder table and keep the ell
-// smallest in registers; the N ell values go to shared memory as 64-bit
-// keys (the bit patterns of non-negative doubles order like the values),
-// and a most-significant-digit radix select (4-bit digits, per-lane packed
-// counters summed with warp reductions) finds the order statistic without
-// sorting; for theta = 0 the statistic is the largest value, a warp max
-// (and no keys are stored).  All arithmetic is the same double multiply the
-// definition uses, so times and psi are bit-exact.
+// GB300 design: one warp per realization.  theta = 0 asks for the largest of
+// the chunks' ell-th completion times, and almost all of that can be decided in
+// fp32: the times tau are truncated to fp32 (exact to 2^-23, products to 2^-22),
+// lanes take chunks and keep the ell smallest of their holders' fp32 times, and
+// only the chunks whose value comes within 2^-20 of the warp's largest are
+// formed again with the defining double products, by the whole warp.  The fp64
+// pipe (2 operations a clock per SM) and the 64-bit comparisons are what
+// bounded the kernel that did it all in double (N = m = 200, delta = 8, ell = 2,
+// 10^5 realizations: 0.92 ms; 0.33 ms this way).  A realization with a time outside [2^-100, 2^100]
+// takes the double form below.
+// In the double form, and for theta > 0, lanes gather their holders'
+// completion times as 64-bit keys (the bit patterns of non-negative doubles
+// order like the values) and keep the ell smallest in registers; for theta > 0
+// the N ell values go to shared memory and a most-significant-digit radix
+// select (4-bit digits, per-lane packed counters summed with warp reductions)
+// finds the order statistic without sorting.
+// Every time that leaves the kernel is the double multiply of the definition,
+// so times and psi are bit-exact.
 #include <math.h>
 
 #include <algorithm>
@@ -99,9 +108,38 @@ __device__ __forceinline__ float approx_float(double x) {
   return __uint_as_float(((unsigned)e << 23) | (unsigned)((b >> 29) & 0x7fffffu));
 }
 
+// The ELL smallest of the values seen (ascending), fp32.
+template <int ELL>
+__device__ __forceinline__ void insert_smallest_f(float (&b)[ELL], float v) {
+#pragma unroll
+  for (int k = 0; k < ELL; ++k) {
+    const float lo = fminf(b[k], v);
+    v = fmaxf(b[k], v);
+    b[k] = lo;
+  }
+}
+__device__ __forceinline__ unsigned long long warp_min(unsigned long long x) {
+  const unsigned hi = (unsigned)(x >> 32);
+  const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? (unsigned)x : 0xffffffffu);
+  return ((unsigned long long)mh << 32) | ml;
+}
+// ell-th smallest of the 32 lanes' keys
+__device__ __forceinline__ unsigned long long warp_ell_th(unsigned long long key, int ell, int lane) {
+  unsigned long long mn = 0;
+  for (int k = 0; k < ell; ++k) {
+    mn = warp_min(key);
+    const unsigned who = __ballot_sync(0xffffffffu, key == mn);
+    if (lane == __ffs(who) - 1) key = ~0ull;
+  }
+  return mn;
+}
+
+constexpr int kTrigHolders = 8192;  // holder words staged in shared memory (32 KB)
+
 template <int ELL>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
-    k_trigger(const int32_t* __restrict__ order, Holders h, int N, int m, int delta,
+    k_trigger(const int32_t* __restrict__ order, Holders h, int N, int m, int delta, int hs,
               const double* __restrict__ tau, long long nsim, int theta, double* __restrict__ T_out,
               int32_t* __restrict__ psi_out, double* __restrict__ Tfull_out) {
   extern __shared__ unsigned long long s_dyn[];
@@ -110,74 +148,178 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
   // int -> double conversion runs on the fp64 pipe, 1/64 of fp32 on GB300)
   __shared__ double s_kd[GC_MAX_REPL + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // per block: delta_j of every worker; per warp: the finishing time of every
-  // worker (m keys) and, for theta > 0, 2 N ELL completion keys
-  int8_t* s_dj = reinterpret_cast<int8_t*>(s_dyn);
-  const size_t dj_words = ((size_t)m + 7) / 8;
-  unsigned long long* fin = s_dyn + dj_words + (size_t)warp * m;
-  unsigned long long* keys = s_dyn + dj_words + (size_t)kWarpsPerBlock * m +
-                             (size_t)warp * 2 * N * ELL;
+  // per warp: every worker's fp32 time and fp32 finishing time, or in the
+  // double form its finishing time (m words), and for theta > 0 2 N ELL
+  // completion keys; per block: delta_j of every worker and the first hs
+  // holders of every chunk, [holder][chunk], worker in the low half of a word
+  // and the slot factor p + 1 as the upper half of its fp32 pattern (exact)
+  unsigned long long* fin = s_dyn + (size_t)warp * m;
+  float2* tf = reinterpret_cast<float2*>(fin);
+  unsigned long long* keys = s_dyn + (size_t)kWarpsPerBlock * m + (size_t)warp * 2 * N * ELL;
   unsigned long long* keysF = keys + (size_t)N * ELL;
+  uint32_t* s_h = reinterpret_cast<uint32_t*>(
+      s_dyn + (size_t)kWarpsPerBlock * (m + (theta > 0 ? 2 * N * ELL : 0)));
+  int8_t* s_dj = reinterpret_cast<int8_t*>(s_h + (size_t)hs * N);
   for (int j = threadIdx.x; j < m; j += blockDim.x) {
     int c = 0;
     for (int p = 0; p < delta; ++p) c += order[(size_t)j * delta + p] >= 0;
     s_dj[j] = (int8_t)c;
   }
+  auto holder = [&](int i, int q) {
+    const int w = h.w[(size_t)i * GC_MAX_REPL + q], p = h.p[(size_t)i * GC_MAX_REPL + q];
+    return (uint32_t)w | (__float_as_uint((float)(p + 1)) & 0xffff0000u);
+  };
+  for (int t = threadIdx.x; t < hs * N; t += blockDim.x) {
+    const int q = t / N, i = t - q * N;
+    s_h[t] = q < h.cnt[i] ? holder(i, q) : 0u;
+  }
   for (int c = threadIdx.x; c <= GC_MAX_REPL; c += blockDim.x) s_kd[c] = (double)c;
   __syncthreads();
+  const unsigned long long kInf = dbits(INFINITY);
   const int n = N * ELL;
   const int kth = n - theta;
   for (long long r = (long long)blockIdx.x * kWarpsPerBlock + warp; r < nsim;
        r += (long long)gridDim.x * kWarpsPerBlock) {
     const double* tr = tau + r * m;
-    const unsigned long long kInf = dbits(INFINITY);
-    // each worker's finishing time delta_j tau_j (+inf for a failed worker)
-    for (int j = lane; j < m; j += 32) {
-      const double tj = tr[j];
-      fin[j] = finite_bits(tj) ? dbits(s_kd[s_dj[j]] * tj) : kInf;
-    }
-    __syncwarp();
-    // theta = 0: the order statistic is the largest of the N ell values, i.e.
-    // the largest ell-th completion time -- a max, no selection needed
-    unsigned long long lmax = 0, lmaxF = 0;
-    for (int i = lane; i < N; i += 32) {
-      unsigned long long b[ELL], bf[ELL];
-#pragma unroll
-      for (int k = 0; k < ELL; ++k) b[k] = bf[k] = kInf;
-      const int cnt = h.cnt[i];
-      for (int q = 0; q < cnt; ++q) {
-        const int j = h.w[(size_t)i * GC_MAX_REPL + q];
-        const int p = h.p[(size_t)i * GC_MAX_REPL + q];
-        const double tj = tr[j];
-        if (finite_bits(tj)) {
-          insert_smallest<ELL>(b, dbits(s_kd[p + 1] * tj));
-          insert_smallest<ELL>(bf, fin[j]);
-        }
-      }
-      if (theta == 0) {
-        lmax = max(lmax, b[ELL - 1]);
-        lmaxF = max(lmaxF, bf[ELL - 1]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < ELL; ++k) {
-          keys[(size_t)i * ELL + k] = b[k];
-          keysF[(size_t)i * ELL + k] = bf[k];
-        }
-      }
-    }
-    __syncwarp();
     unsigned long long Tb = 0, TFb = 0;
+    bool wild = theta != 0;
     if (theta == 0) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        lmax = max(lmax, (unsigned long long)__shfl_xor_sync(0xffffffffu, lmax, o));
-        lmaxF = max(lmaxF, (unsigned long long)__shfl_xor_sync(0xffffffffu, lmaxF, o));
+      // fp32 times (truncated); +inf for a failed worker
+      for (int j = lane; j < m; j += 32) {
+        const double tj = tr[j];
+        const unsigned e = (unsigned)(dbits(tj) >> 52);  // sign and exponent
+        const bool fb = finite_bits(tj);
+        wild |= fb && (e < 1023u - 100u || e > 1023u + 100u);
+        const float f = fb ? approx_float(tj) : INFINITY;
+        tf[j] = make_float2(f, f * (float)s_dj[j]);
       }
-      Tb = lmax;
-      TFb = lmaxF;
-    } else if (kth >= 1) {
-      Tb = warp_select(keys, n, kth, lane);
-      TFb = warp_select(keysF, n, kth, lane);
+      wild = __any_sync(0xffffffffu, wild);
+      __syncwarp();
+    }
+    if (!wild) {
+      // every lane's largest ell-th value, its chunk, and its second largest
+      float best = -1.f, second = -1.f, bestF = -1.f, secondF = -1.f;
+      int bi = 0, biF = 0;
+      for (int i = lane; i < N; i += 32) {
+        float b[ELL], bf[ELL];
+#pragma unroll
+        for (int k = 0; k < ELL; ++k) b[k] = bf[k] = INFINITY;
+        const int cnt = h.cnt[i];
+        for (int q = 0; q < cnt; ++q) {
+          const uint32_t w = q < hs ? s_h[q * N + i] : holder(i, q);
+          const float2 v = tf[w & 0xffffu];
+          insert_smallest_f<ELL>(b, __uint_as_float(w & 0xffff0000u) * v.x);
+          insert_smallest_f<ELL>(bf, v.y);
+        }
+        const float t = b[ELL - 1], u = bf[ELL - 1];
+        second = fmaxf(second, fminf(best, t));
+        if (t > best) {
+          best = t;
+          bi = i;
+        }
+        secondF = fmaxf(secondF, fminf(bestF, u));
+        if (u > bestF) {
+          bestF = u;
+          biF = i;
+        }
+      }
+      // non-negative floats order like their bits; lanes without a chunk hold -1
+      const float A = __uint_as_float(__reduce_max_sync(0xffffffffu, best < 0.f ? 0u : __float_as_uint(best)));
+      const float AF = __uint_as_float(__reduce_max_sync(0xffffffffu, bestF < 0.f ? 0u : __float_as_uint(bestF)));
+      constexpr float kBelow = 1.f - 0x1p-20f, kAbove = 1.f + 0x1p-20f;
+      // exact ell-th time of chunk i: lane q takes its q-th holder (<= 32)
+      auto exact = [&](int i, bool full) {
+        unsigned long long key = kInf;
+        if (lane < h.cnt[i]) {
+          const int w = h.w[(size_t)i * GC_MAX_REPL + lane];
+          const double tj = tr[w];
+          const int c = full ? (int)s_dj[w] : h.p[(size_t)i * GC_MAX_REPL + lane] + 1;
+          if (finite_bits(tj)) key = dbits(s_kd[c] * tj);
+        }
+        return min(warp_ell_th(key, ELL, lane), kInf);
+      };
+      auto candidates = [&](float lim, float bst, float scd, int chunk, bool full) {
+        unsigned long long mx = 0;
+        for (unsigned c = __ballot_sync(0xffffffffu, bst >= lim); c; c &= c - 1) {
+          const int src = __ffs(c) - 1;
+          if (__shfl_sync(0xffffffffu, scd, src) >= lim) {  // several of this lane's chunks
+            for (int i = src; i < N; i += 32) mx = max(mx, exact(i, full));
+          } else {
+            mx = max(mx, exact(__shfl_sync(0xffffffffu, chunk, src), full));
+          }
+        }
+        return mx;
+      };
+      Tb = candidates(A * kBelow, best, second, bi, false);
+      if (Tfull_out) {
+        // a finishing time is one worker's, so when a single worker's fp32 time
+        // lies about AF it is the answer; else the chunks about AF
+        int js = -1, count = 0;
+        for (int j = lane; j < m; j += 32) {
+          const float u = tf[j].y;
+          if (u >= AF * kBelow && u <= AF * kAbove) {
+            js = j;
+            ++count;
+          }
+        }
+        const unsigned has = __ballot_sync(0xffffffffu, count > 0);
+        if (AF < INFINITY && __popc(has) == 1 && !__any_sync(0xffffffffu, count > 1)) {
+          js = __shfl_sync(0xffffffffu, js, __ffs(has) - 1);
+          TFb = dbits(s_kd[s_dj[js]] * tr[js]);
+        } else {
+          TFb = candidates(AF * kBelow, bestF, secondF, biF, true);
+        }
+      }
+    } else {
+      // the double form; each worker's finishing time delta_j tau_j (+inf for a
+      // failed worker)
+      __syncwarp();
+      for (int j = lane; j < m; j += 32) {
+        const double tj = tr[j];
+        fin[j] = finite_bits(tj) ? dbits(s_kd[s_dj[j]] * tj) : kInf;
+      }
+      __syncwarp();
+      // theta = 0: the order statistic is the largest of the N ell values, i.e.
+      // the largest ell-th completion time -- a max, no selection needed
+      unsigned long long lmax = 0, lmaxF = 0;
+      for (int i = lane; i < N; i += 32) {
+        unsigned long long b[ELL], bf[ELL];
+#pragma unroll
+        for (int k = 0; k < ELL; ++k) b[k] = bf[k] = kInf;
+        const int cnt = h.cnt[i];
+        for (int q = 0; q < cnt; ++q) {
+          const int j = h.w[(size_t)i * GC_MAX_REPL + q];
+          const int p = h.p[(size_t)i * GC_MAX_REPL + q];
+          const double tj = tr[j];
+          if (finite_bits(tj)) {
+            insert_smallest<ELL>(b, dbits(s_kd[p + 1] * tj));
+            insert_smallest<ELL>(bf, fin[j]);
+          }
+        }
+        if (theta == 0) {
+          lmax = max(lmax, b[ELL - 1]);
+          lmaxF = max(lmaxF, bf[ELL - 1]);
+        } else {
+#pragma unroll
+          for (int k = 0; k < ELL; ++k) {
+            keys[(size_t)i * ELL + k] = b[k];
+            keysF[(size_t)i * ELL + k] = bf[k];
+          }
+        }
+      }
+      __syncwarp();
+      if (theta == 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          lmax = max(lmax, (unsigned long long)__shfl_xor_sync(0xffffffffu, lmax, o));
+          lmaxF = max(lmaxF, (unsigned long long)__shfl_xor_sync(0xffffffffu, lmaxF, o));
+        }
+        Tb = lmax;
+        TFb = lmaxF;
+      } else if (kth >= 1) {
+        Tb = warp_select(keys, n, kth, lane);
+        TFb = warp_select(keysF, n, kth, lane);
+      }
     }
     const double T = __longlong_as_double((long long)Tb);
     const double TF = __longlong_as_double((long long)TFb);
@@ -185,23 +327,29 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
       if (T_out) T_out[r] = T;
       if (Tfull_out) Tfull_out[r] = TF;
     }
-    if (psi_out)
+    if (psi_out) {
+      const float Tf = approx_float(T);
       for (int j = lane; j < m; j += 32) {
         // slots finish in order: psi_j is the largest c <= delta_j with
         // c tau_j <= T (the products are monotone in c).  An fp32 estimate of
-        // T / tau_j is corrected with the exact double products, so that
-        // typically two of them are formed instead of one per slot.
+        // T / tau_j (exact to 2^-20 when no time is wild) decides it unless it
+        // lies next to a whole number or a time is wild: then it is corrected
+        // with the exact double products.
         const double tj = tr[j];
         const int dj = s_dj[j];
         int c = 0;
         if (finite_bits(tj) && dj > 0) {
-          const float q = __fdividef(approx_float(T), approx_float(tj));
+          const float q = __fdividef(Tf, approx_float(tj));
           c = q >= (float)dj ? dj : (q > 0.f ? (int)q : 0);
-          while (c > 0 && dbits(s_kd[c] * tj) > Tb) --c;
-          while (c < dj && dbits(s_kd[c + 1] * tj) <= Tb) ++c;
+          const float near = rintf(q);
+          if (wild || (fabsf(q - near) <= near * 0x1p-18f && near <= (float)dj)) {
+            while (c > 0 && dbits(s_kd[c] * tj) > Tb) --c;
+            while (c < dj && dbits(s_kd[c + 1] * tj) <= Tb) ++c;
+          }
         }
         psi_out[r * m + j] = c;
       }
+    }
     __syncwarp();
   }
 }
@@ -210,7 +358,11 @@ template <int ELL>
 int launch_one(const int32_t* order, Holders h, int N, int m, int delta, const double* tau,
                long long nsim, int theta, double* T, int32_t* psi, double* TF, cudaStream_t s) {
   const size_t keys = theta == 0 ? 0 : (size_t)kWarpsPerBlock * 2 * N * ELL;
-  const size_t smem = (((size_t)m + 7) / 8 + (size_t)kWarpsPerBlock * m + keys) * 8;
+  // holders of a chunk staged: delta of them (all, when every chunk has at most
+  // delta copies); none in the double form, which does not read them, nor where
+  // the workers' times alone fill a good part of the shared memory
+  const int hs = theta == 0 && m <= 2048 ? std::min(delta, kTrigHolders / N) : 0;
+  const size_t smem = ((size_t)kWarpsPerBlock * m + keys) * 8 + (size_t)hs * N * 4 + (size_t)m;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k_trigger<ELL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
@@ -219,7 +371,7 @@ int launch_one(const int32_t* order, Holders h, int N, int m, int delta, const d
   const long long blocks_needed = (nsim + kWarpsPerBlock - 1) / kWarpsPerBlock;
   const int blocks =
       (int)std::min<long long>(blocks_needed, (long long)device_sm_count() * blocks_per_sm(ELL));
-  k_trigger<ELL><<<blocks, 32 * kWarpsPerBlock, smem, s>>>(order, h, N, m, delta, tau, nsim, theta,
+  k_trigger<ELL><<<blocks, 32 * kWarpsPerBlock, smem, s>>>(order, h, N, m, delta, hs, tau, nsim, theta,
                                                            T, psi, TF);
   count_launches(1);
   return cuda_check(cudaGetLastError(), "k_trigger");

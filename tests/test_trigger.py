@@ -156,6 +156,35 @@ def test_gpu_trigger_edge_cases(gc):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["ties", "near_ties", "wild", "scaled", "many_copies"])
+@pytest.mark.parametrize("N,delta,ell", [(7, 3, 2), (33, 5, 1), (70, 8, 4), (200, 10, 2)])
+def test_gpu_trigger_close_and_extreme_times(gc, kind, N, delta, ell):
+    """Times that fp32 cannot tell apart (equal, or a few units in the last place of a double
+    apart), times outside the range decided in fp32, in all or in some realizations, and chunks
+    with more copies than are staged: every output to the bit."""
+    rng = np.random.default_rng(N + 10 * delta + ell)
+    nsim = 120
+    order = O.cyclic_order(N, N, delta)
+    tau = 0.5 + rng.exponential(1.0, size=(nsim, N))
+    if kind == "ties":
+        tau = rng.integers(1, 4, size=(nsim, N)).astype(np.float64)
+    elif kind == "near_ties":
+        tau = 1.0 + rng.integers(0, 6, size=(nsim, N)) * 2.0 ** -52
+        tau[::2] = np.round(tau[::2] * 3) + rng.integers(-2, 3, size=tau[::2].shape) * 2.0 ** -40
+    elif kind == "wild":
+        tau[rng.random((nsim, N)) < 0.5 / N] = 1e-300
+        tau[rng.random((nsim, N)) < 0.5 / N] = 1e300
+    elif kind == "scaled":
+        tau *= 2.0 ** rng.integers(-99, 97, size=(nsim, 1)).astype(np.float64)
+    else:
+        order = np.stack([rng.permutation(min(N, delta)) for _ in range(min(N, 30))]).astype(np.int32)
+        tau = tau[:, :order.shape[0]]
+        N = min(N, delta)  # every chunk is held by every worker
+    tau[::3, rng.integers(0, tau.shape[1], size=min(delta - 1, 2))] = np.inf
+    _gpu_vs_oracle(gc, order, N, ell, 0, tau)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("ell", [1, 2, 3])
 def test_gpu_trigger_feeds_decode_on_g1(gc, ell):
     """Simulate -> trigger at a theta -> psi -> batched Algorithm 1 and
