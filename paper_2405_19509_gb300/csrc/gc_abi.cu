@@ -515,6 +515,18 @@ int gc_decode_batch(const double* R, int ell, const int32_t* order, int N, int m
   SolveWs sw = carve_solve(c, N, m, delta, ell, npat);
   __nv_bfloat16* Cs = c.take<__nv_bfloat16>(plan_bytes(N, ell, npat) / sizeof(__nv_bfloat16));
   launch_holders(order, N, m, delta, sw.h, status_of(ws), s);
+  if (!Ghat && decode_policy() == GC_DECODE_AUTO && mse_gram_applies(N, ell, npat) &&
+      mse_patterns_applies(N, ell, sw.bits)) {
+    // errors alone: the memo table and the Gram matrix of the chunk blocks
+    SolveOut none{};
+    none.Kp = combine_kp(N, ell);
+    rc = launch_solve_impl(R, ell, psi, sw.h, N, m, delta, 0, none, sw.table, sw.bits,
+                           status_of(ws), s);
+    if (rc) return rc;
+    const GramMatrix gm = launch_gram(G, N, ell, d, true, c, s);
+    return launch_mse_patterns(R, ell, psi, sw.h, N, m, delta, npat, sw.table, sw.bits, gm.H,
+                               gm.H_last, d, coef_err, est, grad_mse, status_of(ws), s);
+  }
   SolveOut out{nullptr, nullptr, nullptr, nullptr, coef_err, est, Cs, combine_kp(N, ell)};
   rc = launch_solve_impl(R, ell, psi, sw.h, N, m, delta, npat, out, sw.table, sw.bits,
                          status_of(ws), s);

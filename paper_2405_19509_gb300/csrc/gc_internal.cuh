@@ -195,8 +195,20 @@ size_t apply_ws_bytes(int N, int ell, int npat, int d);
 // ---- gradient MSE through the Gram matrix of the chunk blocks (k_mse_gram.cu)
 bool mse_gram_applies(int N, int ell, int npat);
 size_t mse_gram_ws_bytes(int N, int ell, int d);
+struct GramMatrix {
+  const float* H;       // (N*ell)^2
+  const float* H_last;  // the same over the columns of a padded last block, or null
+};
+GramMatrix launch_gram(const float* G, int N, int ell, int d, bool after_table, Carve& ws,
+                       cudaStream_t s);
 int launch_mse_gram(const __nv_bfloat16* Cs, int Kp, const float* G, int N, int ell, int npat,
                     int d, double* grad_mse, Carve& ws, cudaStream_t s);
+// ... and straight from the counts and the memo table (k_mse_patterns.cu)
+bool mse_patterns_applies(int N, int ell, int bits);
+int launch_mse_patterns(const double* R, int ell, const int32_t* psi, Holders h, int N, int m,
+                        int delta, int npat, void* table_mem, int bits, const float* H,
+                        const float* H_last, int d, double* coef_err, double* est,
+                        double* grad_mse, uint32_t* status, cudaStream_t s);
 int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int npat, int d,
                  float* Ghat, double* grad_mse, Carve& ws, uint32_t* status, cudaStream_t s);
 // fp32 C (npat x ell x N*ell) -> planes

@@ -76,7 +76,12 @@ __device__ __forceinline__ void gram_load8(const float* __restrict__ G, int N, i
 __global__ void __launch_bounds__(256) k_gram_partial(const float* __restrict__ G, int N, int ell,
                                                       int d, int L, int slice, int nsa, int l_last,
                                                       int vec, float* __restrict__ partial) {
-  // staged column-major, sa[c][r], so that a thread reads 4 rows as one 16-byte load
+  // launched as a programmatic dependent of Algorithm 1's table, which it does
+  // not read (see the end)
+  // staged column-major so that a thread reads 4 rows as one 16-byte load: row r
+  // of column c lies at sa[c][r ^ 8 (c / 8)], which spreads the staging stores of
+  // a warp (8 rows x 4 column groups) over all banks (4-way conflicts without:
+  // 34 us for N*ell = 128, L = 32768; 31 with)
   __shared__ __align__(16) float sa[kGramCols][kGramTile];
   __shared__ __align__(16) float sb[kGramCols][kGramTile];
   const int K = N * ell, nt = (K + kGramTile - 1) / kGramTile;
@@ -101,8 +106,8 @@ __global__ void __launch_bounds__(256) k_gram_partial(const float* __restrict__ 
   for (int c0 = c_lo; c0 < c_hi; c0 += kGramCols) {
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      sa[8 * sq + e][sr] = xa[e];
-      sb[8 * sq + e][sr] = xb[e];
+      sa[8 * sq + e][sr ^ (8 * sq)] = xa[e];
+      sb[8 * sq + e][sr ^ (8 * sq)] = xb[e];
     }
     __syncthreads();
     if (c0 + kGramCols < c_hi) {  // the next step's columns, in flight during this one
@@ -111,8 +116,9 @@ __global__ void __launch_bounds__(256) k_gram_partial(const float* __restrict__ 
     }
 #pragma unroll 8
     for (int cc = 0; cc < kGramCols; ++cc) {
-      const float4 a4 = *reinterpret_cast<const float4*>(&sa[cc][4 * ty]);
-      const float4 b4 = *reinterpret_cast<const float4*>(&sb[cc][4 * tx]);
+      const int sw = 8 * (cc / 8);
+      const float4 a4 = *reinterpret_cast<const float4*>(&sa[cc][(4 * ty) ^ sw]);
+      const float4 b4 = *reinterpret_cast<const float4*>(&sb[cc][(4 * tx) ^ sw]);
       const float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -126,6 +132,8 @@ __global__ void __launch_bounds__(256) k_gram_partial(const float* __restrict__ 
   for (int u = 0; u < 4; ++u)
     *reinterpret_cast<float4*>(out + (4 * ty + u) * kGramTile + 4 * tx) =
         make_float4(acc[u][0], acc[u][1], acc[u][2], acc[u][3]);
+  // what is ordered after this kernel must find its predecessor complete, too
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // H_last[a][b] = H_last[b][a] = sum over the slices z < nsa of the partials,
@@ -364,8 +372,10 @@ size_t mse_gram_ws_bytes(int N, int ell, int d) {
          2 * align_up((size_t)K * K * sizeof(float), 256);
 }
 
-int launch_mse_gram(const __nv_bfloat16* Cs, int Kp, const float* G, int N, int ell, int npat,
-                    int d, double* grad_mse, Carve& ws, cudaStream_t s) {
+// H (and H_last when the last block is padded) of the chunk blocks, in ws.
+// after_table: the stream's last kernel is k_table, beside which this may start.
+GramMatrix launch_gram(const float* G, int N, int ell, int d, bool after_table, Carve& ws,
+                       cudaStream_t s) {
   const int K = N * ell;
   const int L = (d + ell - 1) / ell;
   const int l_last = d - (ell - 1) * L;  // real columns of the last block, 0 < l_last <= L
@@ -377,13 +387,29 @@ int launch_mse_gram(const __nv_bfloat16* Cs, int Kp, const float* G, int N, int 
   float* partial = ws.take<float>((size_t)ntri * nsplit * kGramTile * kGramTile);
   float* H = ws.take<float>((size_t)K * K);
   float* H_last = ws.take<float>((size_t)K * K);
-  if (npat == 0) return GC_OK;
   const bool vec = d % 4 == 0 && L % 4 == 0 && reinterpret_cast<uintptr_t>(G) % 16 == 0;
-  k_gram_partial<<<dim3((unsigned)ntri, (unsigned)nsplit), 256, 0, s>>>(
-      G, N, ell, d, L, slice, nsa, l_last, vec ? 1 : 0, partial);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)ntri, (unsigned)nsplit);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = after_table ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, k_gram_partial, G, N, ell, d, L, slice, nsa, l_last, vec ? 1 : 0, partial);
   k_gram_reduce<<<dim3((unsigned)ntri, (kGramTile * kGramTile) / 32), 256, 0, s>>>(
       partial, K, nsa, nsplit, H, H_last);
-  const float* hl = l_last < L ? H_last : nullptr;
+  count_launches(2);
+  return {H, l_last < L ? H_last : nullptr};
+}
+
+int launch_mse_gram(const __nv_bfloat16* Cs, int Kp, const float* G, int N, int ell, int npat,
+                    int d, double* grad_mse, Carve& ws, cudaStream_t s) {
+  const int K = N * ell;
+  if (npat == 0) return GC_OK;
+  const GramMatrix gm = launch_gram(G, N, ell, d, false, ws, s);
+  const float *H = gm.H, *hl = gm.H_last;
   const bool hs = K <= kHSmemMaxK;
   // H from shared memory and no padded last block: blocks of 32 warps (96 KB,
   // 64 registers a thread); otherwise blocks of 16 warps (up to 128 registers)
@@ -407,7 +433,7 @@ int launch_mse_gram(const __nv_bfloat16* Cs, int Kp, const float* G, int N, int 
   }
 #undef GC_MSEG
   if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_mse_gram)");
-  count_launches(3);
+  count_launches(1);
   return cuda_check(cudaGetLastError(), "k_mse_gram");
 }
 

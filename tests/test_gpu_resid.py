@@ -367,6 +367,52 @@ def test_large_ell_both_paths(gc, ell):
             assert_mse_close(float(res["grad_mse"][b]), r.grad_mse, floor, f"{k} l={ell} mse b={b}")
 
 
+@pytest.mark.parametrize("N,m,delta,ell,d,npat", [
+    (8, 8, 3, 1, 40, 17),        # one chunk a lane, a last batch of one pattern
+    (33, 33, 5, 2, 1003, 155),   # two chunks a lane, padded last block
+    (64, 64, 7, 3, 300, 700),    # rows' sums of 32 patterns and a remainder in every warp
+    (100, 100, 6, 2, 512, 1001), # four chunks a lane, H read through the cache
+    (64, 64, 4, 4, 256, 5000),
+    (20, 60, 4, 2, 128, 99),     # explicit order: chunks with more copies than the table has bits
+])
+def test_errors_from_counts(gc, N, m, delta, ell, d, npat):
+    """gc_mse (errors straight from the counts and the memo table) against the errors through
+    the decode plan: the coefficient error and the estimate to the bit, the gradient MSE to
+    rounding (the plan holds the blocks to 2^-17), and sampled patterns against the oracle."""
+    rng = np.random.default_rng(N * 10 + ell)
+    order = O.cyclic_order(N, N, delta) if m == N else np.stack(
+        [rng.choice(N, size=delta, replace=False) for _ in range(m)]).astype(np.int32)
+    R = rng.standard_normal((ell, m))
+    psi = rng.binomial(delta, rng.uniform(0.1, 0.9, size=(npat, 1)), size=(npat, m)).astype(np.int32)
+    psi[0], psi[1 % npat] = delta, 0
+    G32 = rng.standard_normal((N, d)).astype(np.float32)
+    Gref = G32.astype(np.float64)
+    gsum = Gref.sum(axis=0)
+    floor = 1e-8 * float(gsum @ gsum) / d
+    Rd, od, pd = dev_tensors(R, order, psi)
+    Gd = torch.from_numpy(G32).cuda()
+    ws = gc.Workspace()
+    got = gc.gc_mse(Rd, ell, od, N, m, delta, pd, Gd, ws=ws)
+    gc.gc_status(ws)
+    plan = gc.gc_decode_plan(Rd, ell, od, N, m, delta, pd)
+    via = gc.gc_decode_apply(plan["plan"], ell, N, npat, Gd, Ghat=False)["grad_mse"]
+    assert torch.equal(got["coef_err"], plan["coef_err"]) and torch.equal(got["est"], plan["est"])
+    assert (got["grad_mse"] - via).abs().max().item() <= 2e-4 * via.max().item()
+    for b in sorted({0, 1 % npat, npat - 1, *range(0, npat, max(1, npat // 12))}):
+        r = O.run_pattern(R, order, psi[b], N, Gref, want_transmit=False)
+        assert_mse_close(got["grad_mse"][b].item(), r.grad_mse, floor, f"b={b}")
+        assert abs(got["coef_err"][b].item() - r.coef_err) <= 1e-9 * max(1.0, r.coef_err)
+        assert got["est"][b].item() == r.est
+    assert got["grad_mse"][0].item() == 0.0 if (_copies(order, psi[:1], N) >= ell).all() else True
+    only = gc.gc_mse(Rd, ell, od, N, m, delta, pd, Gd, coef_err=False, est=False)
+    assert torch.equal(only["grad_mse"], got["grad_mse"])
+    if m == N:
+        psi[-1, 3] = -1
+        gc.gc_mse(Rd, ell, od, N, m, delta, torch.from_numpy(psi).cuda(), Gd, ws=ws)
+        with pytest.raises(gc.GCError, match="psi"):
+            gc.gc_status(ws)
+
+
 @pytest.mark.parametrize("N,delta,ell,d", [(10, 4, 3, 1001), (20, 8, 8, 997), (40, 6, 5, 1500)])
 def test_errors_only_gram_path(gc, N, delta, ell, d):
     """Errors only under the automatic policy (npat * ell >= 2 N ell): each
