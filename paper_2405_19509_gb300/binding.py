@@ -8,6 +8,7 @@ functions; gc_status() synchronises and reports device-detected data errors.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 
 import numpy as np
@@ -103,8 +104,26 @@ def block_length(d: int, ell: int) -> int:
     return -(-d // ell)
 
 
+# The raw handle of torch's current stream (building a Stream object for it costs 2 us a call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device())
+
+
+@functools.lru_cache(maxsize=1024)
+def _bytes(query, *sizes) -> int:
+    """A workspace size, a function of the sizes alone, asked of the library once."""
+    return int(getattr(lib, query)(*sizes))
+
+
+@functools.lru_cache(maxsize=1024)
+def _chunk_grads_bytes(N, n_c, d, x_dtype, device) -> int:
+    """... and of the number of SMs of the device."""
+    return int(lib.gc_chunk_grads_workspace(N, n_c, d, x_dtype))
 
 
 def _dev(t, dtype, name, shape=None):
@@ -113,11 +132,11 @@ def _dev(t, dtype, name, shape=None):
         return None
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype:
+    if t.dtype is not dtype:
         raise TypeError(f"{name} must be {dtype}, got {t.dtype}")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
     return t.data_ptr()
 
@@ -199,7 +218,7 @@ def gc_trigger_times(order, N: int, m: int, delta: int, tau, ell: int, theta: in
     T = out(T, (nsim,), torch.float64)
     psi = out(psi, (nsim, m), torch.int32)
     T_full = out(T_full, (nsim,), torch.float64)
-    ws, (wp, wn) = _ws(ws, lib.gc_trigger_workspace(N), dev)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_trigger_workspace", N), dev)
     _check(lib.gc_trigger_times(
         _dev(order, torch.int32, "order", (m, delta)), N, m, delta,
         _dev(tau, torch.float64, "tau", (nsim, m)), nsim, ell, theta,
@@ -217,7 +236,7 @@ def gc_chunk_grads_batched(X, y, W, N: int, n_c: int, loss: int, G=None,
         raise TypeError("X must be bfloat16")
     if G is None:
         G = torch.empty(n_w, N, d, dtype=torch.float32, device=X.device)
-    ws, (wp, wn) = _ws(ws, lib.gc_chunk_grads_batched_workspace(N, n_c, d, n_w), X.device)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_chunk_grads_batched_workspace", N, n_c, d, n_w), X.device)
     _check(lib.gc_chunk_grads_batched(
         _dev(X, torch.bfloat16, "X", (N * n_c, d)), _dev(y, torch.float32, "y", (N * n_c,)),
         _dev(W, torch.float32, "W", (n_w, d)), N, n_c, d, n_w, loss,
@@ -241,7 +260,7 @@ def gc_chunk_grads(X, y, w, N: int, n_c: int, loss: int, G=None, loss_out=None,
         raise ValueError("X must have N * n_c rows")
     if G is None:
         G = torch.empty(N, d, dtype=torch.float32, device=X.device)
-    ws, (wp, wn) = _ws(ws, gc_chunk_grads_workspace(N, n_c, d, x_dtype), X.device)
+    ws, (wp, wn) = _ws(ws, _chunk_grads_bytes(N, n_c, d, x_dtype, torch.cuda.current_device()), X.device)
     _check(lib.gc_chunk_grads(_dev(X, X.dtype, "X"), x_dtype, _dev(y, torch.float32, "y", (N * n_c,)),
                               _dev(w, torch.float32, "w", (d,)), N, n_c, d, loss,
                               _dev(G, torch.float32, "G", (N, d)),
@@ -274,7 +293,7 @@ def gc_find_encoding_coeff(R, ell, order, N, m, delta, psi, E=True, C=True, delt
         "coef_err": out(coef_err, (npat,), torch.float64),
         "est": out(est, (npat,), torch.float64),
     }
-    ws, (wp, wn) = _ws(ws, gc_coeff_workspace(N, m, delta, ell, npat), dev)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_coeff_workspace", N, m, delta, ell, npat), dev)
     _check(lib.gc_find_encoding_coeff(
         _dev(R, torch.float64, "R", (ell, m)), ell, _dev(order, torch.int32, "order", (m, delta)),
         N, m, delta, _dev(psi, torch.int32, "psi", (npat, m)), npat,
@@ -297,7 +316,7 @@ def gc_encode(R, ell, order, N, m, delta, psi, G, T=None, ws: Workspace | None =
     L = block_length(d, ell)
     if T is None:
         T = torch.empty(npat, m, L, dtype=torch.float32, device=G.device)
-    ws, (wp, wn) = _ws(ws, gc_encode_workspace(N, m, delta, ell, npat, d), G.device)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_encode_workspace", N, m, delta, ell, npat, d), G.device)
     _check(lib.gc_encode(_dev(R, torch.float64, "R", (ell, m)), ell,
                          _dev(order, torch.int32, "order", (m, delta)), N, m, delta,
                          _dev(psi, torch.int32, "psi", (npat, m)), npat,
@@ -357,7 +376,7 @@ def gc_decode_batch(R, ell, order, N, m, delta, psi, G, Ghat=True, coef_err=True
         "est": out(est, (npat,), torch.float64),
         "grad_mse": out(grad_mse, (npat,), torch.float64),
     }
-    ws, (wp, wn) = _ws(ws, gc_decode_batch_workspace(N, m, delta, ell, npat, d), dev)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_decode_batch_workspace", N, m, delta, ell, npat, d), dev)
     _check(lib.gc_decode_batch(
         _dev(R, torch.float64, "R", (ell, m)), ell, _dev(order, torch.int32, "order", (m, delta)),
         N, m, delta, _dev(psi, torch.int32, "psi", (npat, m)), npat,
@@ -373,14 +392,14 @@ def gc_decode_plan(R, ell, order, N, m, delta, psi, plan=None, coef_err=True, es
     for gc_decode_apply.  Returns dict with plan, coef_err, est."""
     npat = psi.shape[0]
     dev = psi.device
-    nb = lib.gc_decode_plan_bytes(N, ell, npat)
+    nb = _bytes("gc_decode_plan_bytes", N, ell, npat)
     if plan is None:
         plan = torch.empty(max(int(nb), 256), dtype=torch.uint8, device=dev)
     ce = coef_err if isinstance(coef_err, torch.Tensor) else (
         torch.empty(npat, dtype=torch.float64, device=dev) if coef_err else None)
     es = est if isinstance(est, torch.Tensor) else (
         torch.empty(npat, dtype=torch.float64, device=dev) if est else None)
-    ws, (wp, wn) = _ws(ws, lib.gc_decode_plan_workspace(N, m, delta, ell, npat), dev)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_decode_plan_workspace", N, m, delta, ell, npat), dev)
     _check(lib.gc_decode_plan(_dev(R, torch.float64, "R", (ell, m)), ell,
                               _dev(order, torch.int32, "order", (m, delta)), N, m, delta,
                               _dev(psi, torch.int32, "psi", (npat, m)), npat,
@@ -410,14 +429,14 @@ def gc_decode_plan_prepared(prep, R, ell, N, m, delta, psi, plan=None, coef_err=
     plan, coef_err, est."""
     npat = psi.shape[0]
     dev = psi.device
-    nb = lib.gc_decode_plan_bytes(N, ell, npat)
+    nb = _bytes("gc_decode_plan_bytes", N, ell, npat)
     if plan is None:
         plan = torch.empty(max(int(nb), 256), dtype=torch.uint8, device=dev)
     ce = coef_err if isinstance(coef_err, torch.Tensor) else (
         torch.empty(npat, dtype=torch.float64, device=dev) if coef_err else None)
     es = est if isinstance(est, torch.Tensor) else (
         torch.empty(npat, dtype=torch.float64, device=dev) if est else None)
-    ws, (wp, wn) = _ws(ws, lib.gc_decode_plan_prepared_workspace(), dev)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_decode_plan_prepared_workspace"), dev)
     _check(lib.gc_decode_plan_prepared(_dev(prep, torch.uint8, "prep"),
                                        _dev(R, torch.float64, "R", (ell, m)), ell, N, m, delta,
                                        _dev(psi, torch.int32, "psi", (npat, m)), npat,
@@ -435,7 +454,7 @@ def gc_decode_apply(plan, ell, N, npat, G, Ghat=True, grad_mse=True, ws: Workspa
         Ghat = torch.empty(npat, d, dtype=torch.float32, device=dev) if Ghat else None
     if not isinstance(grad_mse, torch.Tensor):
         grad_mse = torch.empty(npat, dtype=torch.float64, device=dev) if grad_mse else None
-    ws, (wp, wn) = _ws(ws, lib.gc_decode_apply_workspace(N, ell, npat, d), dev)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_decode_apply_workspace", N, ell, npat, d), dev)
     _check(lib.gc_decode_apply(_dev(plan, torch.uint8, "plan"), ell, N, npat,
                                _dev(G, torch.float32, "G", (N, d)), d,
                                _dev(Ghat, torch.float32, "Ghat", (npat, d)),
@@ -488,7 +507,7 @@ def gc_decode_combine(C, ell, N, G, Ghat=True, grad_mse=True, ws: Workspace | No
         Ghat = torch.empty(npat, d, dtype=torch.float32, device=dev) if Ghat else None
     if not isinstance(grad_mse, torch.Tensor):
         grad_mse = torch.empty(npat, dtype=torch.float64, device=dev) if grad_mse else None
-    ws, (wp, wn) = _ws(ws, gc_decode_combine_workspace(N, ell, npat, d), dev)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_decode_combine_workspace", N, ell, npat, d), dev)
     _check(lib.gc_decode_combine(_dev(C, torch.float32, "C", (npat, ell, N * ell)), ell, N, npat,
                                  _dev(G, torch.float32, "G", (N, d)), d,
                                  _dev(Ghat, torch.float32, "Ghat", (npat, d)),
@@ -517,7 +536,7 @@ def gc_mse(R, ell, order, N, m, delta, psi, G, coef_err=True, est=True, grad_mse
         "est": out(est, (npat,), torch.float64),
         "grad_mse": out(grad_mse, (npat,), torch.float64),
     }
-    ws, (wp, wn) = _ws(ws, gc_mse_workspace(N, m, delta, ell, npat, d), dev)
+    ws, (wp, wn) = _ws(ws, _bytes("gc_mse_workspace", N, m, delta, ell, npat, d), dev)
     _check(lib.gc_mse(
         _dev(R, torch.float64, "R", (ell, m)), ell, _dev(order, torch.int32, "order", (m, delta)),
         N, m, delta, _dev(psi, torch.int32, "psi", (npat, m)), npat,
@@ -542,13 +561,17 @@ def gc_live_step(E, R, ell, order, N, m, delta, psi, G, w, lr: float, Ntil: int,
     processed counts; T (m x L) and ghat (d) are written when given."""
     d = G.shape[1]
     L = block_length(d, ell)
-    _check(lib.gc_live_step(_dev(E.reshape(m, delta, ell), torch.float64, "E", (m, delta, ell)),
+
+    def as_shape(t, shape):
+        return t if t is None or t.shape == shape else t.reshape(shape)
+    E, psi = as_shape(E, (m, delta, ell)), as_shape(psi, (m,))
+    T, ghat = as_shape(T, (m, L)), as_shape(ghat, (d,))
+    _check(lib.gc_live_step(_dev(E, torch.float64, "E", (m, delta, ell)),
                             _dev(R, torch.float64, "R", (ell, m)), ell,
                             _dev(order, torch.int32, "order", (m, delta)), N, m, delta,
-                            _dev(psi.reshape(m), torch.int32, "psi", (m,)),
+                            _dev(psi, torch.int32, "psi", (m,)),
                             _dev(G, torch.float32, "G", (N, d)), d, float(lr), int(Ntil),
                             _dev(w, torch.float32, "w", (d,)),
-                            None if T is None else _dev(T.reshape(m, L), torch.float32, "T", (m, L)),
-                            None if ghat is None else _dev(ghat.reshape(d), torch.float32, "ghat", (d,)),
-                            _stream()))
+                            _dev(T, torch.float32, "T", (m, L)),
+                            _dev(ghat, torch.float32, "ghat", (d,)), _stream()))
     return w

@@ -47,10 +47,13 @@ static std::atomic<int> g_policy{GC_DECODE_AUTO};
 int decode_policy() { return g_policy.load(std::memory_order_relaxed); }
 
 int device_sm_count() {
+  static std::atomic<int> cache[64];  // a constant of the device
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 152;
+  if (dev >= 0 && dev < 64 && (n = cache[dev].load(std::memory_order_relaxed)) > 0) return n;
   if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
     return 152;
+  if (dev >= 0 && dev < 64) cache[dev].store(n, std::memory_order_relaxed);
   return n;
 }
 

@@ -482,9 +482,14 @@ __global__ void __launch_bounds__(256) k_split_gt(const float* __restrict__ G, i
                                                   GemmChoice gemm) {
   constexpr int TPR = COLS / 4;            // threads per row of the load phase
   constexpr int RPP = 256 / TPR;           // rows per pass
-  // the combine kernel may be scheduled now; it waits for this grid to finish
+  // the combine kernel may be scheduled now; it waits for this grid to finish,
+  // and this grid, itself a programmatic dependent of the residual kernel (which
+  // it reads nothing from), does not end before that one
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (!gemm.any(rl)) return;
+  if (!gemm.any(rl)) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   const int t = threadIdx.x, lane = t & 31;
   {
     const int thr = gemm.threshold(rl);
@@ -557,6 +562,7 @@ __global__ void __launch_bounds__(256) k_split_gt(const float* __restrict__ G, i
       }
     }
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // grad_mse[b] = (partial squared errors of pattern b) / d, one warp per pattern:
@@ -746,13 +752,20 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
     const long long pairs = (long long)((L + cols - 1) / cols) * (Kp / 64);
     const unsigned blocks = (unsigned)std::min<long long>(std::max<long long>(pairs, (npat + 7) / 8),
                                                           8LL * device_sm_count());
-    if (cols == 64)
-      k_split_gt<64><<<blocks, 256, 0, s>>>(G, N, d, ell, L, Kp, Gs, Cs, npat, Ca, rl, gemm);
-    else
-      k_split_gt<32><<<blocks, 256, 0, s>>>(G, N, d, ell, L, Kp, Gs, Cs, npat, Ca, rl, gemm);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    // not behind k_gsum alone, which lets its dependents start before the scan has ended
+    cfg.numAttrs = policy != GC_DECODE_DENSE ? 1 : 0;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, cols == 64 ? k_split_gt<64> : k_split_gt<32>, G, N, d,
+                                       ell, L, Kp, Gs, Cs, npat, Ca, rl, gemm);
+    if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_split_gt)");
     count_launches(1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_check(e, "k_split_gt");
   }
   CUtensorMap mA, mB;
   rc = make_map(&mA, Ca, (int)M, Kp, BM);

@@ -254,6 +254,8 @@ __global__ void __launch_bounds__(kResidThreads, ELL <= 2 ? 4 : (ELL <= 4 ? 3 : 
   // a programmatic dependent of the sum of the chunk gradients: s and the
   // scan's lists are complete once this wait returns
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  // the operand split may start beside this grid's last blocks
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int thr = gemm.threshold(rl);
   const int pps = (ppt + gridDim.z - 1) / gridDim.z;  // patterns per slice of a tile (<= 128)
   const int b_lo = blockIdx.x * ppt + blockIdx.z * pps;

@@ -28,6 +28,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "k_solve.cuh"
 
@@ -493,12 +494,16 @@ static void run_solve(const double* R, const int32_t* psi, Holders h, int N, int
   if (!out.E && cpl > 0) {
     // as many 128-thread blocks as are resident at once (all warps stride
     // over the patterns, so a second partial wave would only add a tail)
-    auto go = [&](auto kern) {
-      int per_sm = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, 0) != cudaSuccess ||
-          per_sm < 1) {
-        cudaGetLastError();
-        per_sm = 1;
+    auto go = [&](auto kern, int which) {
+      static std::atomic<int> resident[6];  // a constant of each kernel
+      int per_sm = resident[which].load(std::memory_order_relaxed);
+      if (per_sm == 0) {
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, 0) != cudaSuccess ||
+            per_sm < 1) {
+          cudaGetLastError();
+          per_sm = 1;
+        }
+        resident[which].store(per_sm, std::memory_order_relaxed);
       }
       const int warps = 4;  // per 128-thread block
       const int blocks =
@@ -507,12 +512,12 @@ static void run_solve(const double* R, const int32_t* psi, Holders h, int N, int
       count_launches(1);
     };
     if (cpl == 1) {
-      use_table ? go(k_patterns_warp<ELL, true, 1>) : go(k_patterns_warp<ELL, false, 1>);
+      use_table ? go(k_patterns_warp<ELL, true, 1>, 0) : go(k_patterns_warp<ELL, false, 1>, 1);
     } else if constexpr (ELL <= 4) {
       if (cpl == 2)
-        use_table ? go(k_patterns_warp<ELL, true, 2>) : go(k_patterns_warp<ELL, false, 2>);
+        use_table ? go(k_patterns_warp<ELL, true, 2>, 2) : go(k_patterns_warp<ELL, false, 2>, 3);
       else
-        use_table ? go(k_patterns_warp<ELL, true, 4>) : go(k_patterns_warp<ELL, false, 4>);
+        use_table ? go(k_patterns_warp<ELL, true, 4>, 4) : go(k_patterns_warp<ELL, false, 4>, 5);
     }
     return;
   }
