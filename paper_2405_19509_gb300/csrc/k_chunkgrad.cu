@@ -129,7 +129,7 @@ cudaLaunchConfig_t launch_config(const Plan& p, unsigned grid, cudaLaunchAttribu
                                  cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(p.NT + 32);  // consumers + the producer warp
+  cfg.blockDim = dim3(p.NT + 64);  // consumers, the producer and the reducer warp
   cfg.dynamicSmemBytes = p.smem;
   cfg.stream = s;
   attr->id = cudaLaunchAttributeClusterDimension;
@@ -165,12 +165,10 @@ Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
   p.V = 16 / esz;
   const long long row_bytes = (long long)d * esz;
   // The row is split over as few CTAs as its columns' w and accumulators fit
-  // the registers of (512 threads of 6 fp32 or 4 bf16 vectors): a cluster
-  // exchanges partial dots once a batch and holds each stage until the sums
-  // are back.  Measured at 2 GB of X against slices of 32 KB (fp32) and 16 KB
-  // (bf16): fp32 d = 10007 102% of the copy rate in one CTA, 54% in two
-  // (12288: 93, 64); bf16 d = 12000 89 against 37 (16384: 98, 74), d = 20000
-  // in two CTAs 54 against 29 in four.
+  // the registers of (512 threads of 6 fp32 or 4 bf16 vectors), so that the rows
+  // of a batch and the partial gradients are as long as they can be (2 GB of X,
+  // with the exchange of the time in the consumers' way: fp32 d = 10007 102% of
+  // the copy rate in one CTA, 54% in two; bf16 d = 16384 98 and 74).
   const long long max_slice = x_dtype == GC_BF16 ? 32768 : 49152;
   p.CL = 1;
   while (p.CL < 8 && (row_bytes + p.CL - 1) / p.CL > max_slice) p.CL *= 2;
@@ -178,8 +176,8 @@ Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
   // GPC; at most 15 clusters of 8 are co-resident), clusters of 4 fill 144:
   // fp32 rows of up to 256 KB take 64 KB slices (8 vectors a thread, one row a
   // stage) in clusters of 4.  bf16 rows that two CTAs would take in four
-  // vectors a thread stay in clusters of 4 (d = 32768: 70 against 68%; at
-  // 256 MB 43 against 40%).
+  // vectors a thread stay in clusters of 4 (d = 32768: 70 against 68%, at
+  // 256 MB 43 against 40%, before x was kept in tensor memory).
   if (x_dtype != GC_BF16 && p.CL == 8 && row_bytes <= 4 * 65536) p.CL = 4;
   if (x_dtype == GC_BF16 && p.CL == 2 && row_bytes > 2 * 3 * 512 * 16) p.CL = 4;
   p.Wc = (int)align_up((size_t)((d + p.CL - 1) / p.CL), (size_t)p.V);
@@ -188,11 +186,11 @@ Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
   p.NT = nv >= 1024 ? 512 : (nv >= 256 ? 256 : 128);
   // CTAs per SM.  Rows of 4 to 16 KB: two (two independent rings) when each
   // still streams many rows, one when the rows per SM are few (ramp-up
-  // dominates) or the row is longer.  Shorter rows, 128 threads: a batch's
-  // chain of shuffles, barrier and residual (0.6 us) outlasts its copy, so as
-  // many CTAs as the registers hold, with at least 32 rows each (100,000 fp32
-  // rows of d = 512: 112 us with one CTA, 62 with two, 42 with four; 10,000
-  // rows: 16, 12 and 12).
+  // dominates) or the row is longer.  Shorter rows, 128 threads: the chain of a
+  // batch from its dot products to its residuals outlasts its copy, so up to
+  // four CTAs (tensor memory holds four), with at least 32 rows each (measured
+  // when a batch was four rows and met at a barrier, 100,000 fp32 rows of
+  // d = 512: 112 us with one CTA, 62 with two, 42 with four).
   const long long rows_per_sm = (long long)N * n_c / std::max(1, device_sm_count());
   int cps = (rows_per_sm >= 512 && row_bytes <= 16384) ? 2 : 1;
   if (p.NT == 128)
@@ -204,7 +202,7 @@ Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
   // and dot products
   p.NVT = need <= 2 ? need : 4;
   if (x_dtype == GC_BF16 ? need == 3 && p.NT == 512 : need > 4) p.NVT = need <= 6 ? need : 8;
-  p.RBM = p.NVT >= 5 ? 1 : (p.NVT >= 3 ? 2 : 4);
+  p.RBM = p.NVT >= 5 ? 1 : (p.NVT >= 3 ? 2 : (p.NVT == 2 ? 4 : 8));
   // stage row: one vector per (thread, u), so reads need no bounds; a slice at
   // any element lies up to V - 1 elements in and ends in up to 2 V - 1 more
   const int row_vecs = p.NVT * p.NT;
@@ -213,8 +211,9 @@ Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
   p.S = (int)std::min<size_t>(
       cg::kMaxStages, std::max<size_t>(2, (192 * 1024 / cps) / ((size_t)p.RBM * row_vecs * 16)));
   const int NW = p.NT / 32;
-  p.smem = p.S * stage_bytes + (2 * NW * p.RBM + cg::kZSlots * p.CL * p.RBM + 2) * sizeof(float) +
-           (2 * cg::kMaxStages + cg::kZSlots) * sizeof(uint64_t) + 16;
+  p.smem = p.S * stage_bytes +
+           (cg::kSlots * NW * p.RBM + cg::kZSlots * p.CL * p.RBM + cg::kSlots * p.RBM) * sizeof(float) +
+           (2 * cg::kMaxStages + 2 * cg::kSlots + cg::kZSlots) * sizeof(uint64_t) + 16;
   // every vector of the slice has a thread, and the shape is built
   p.valid = (long long)row_vecs >= nv && kernel_of(p, x_dtype) != nullptr;
   // flat partition of the batches over one wave of clusters

@@ -5,17 +5,27 @@
 //
 // GB300 design: the path is HBM bound (2 flops per element read), so X is read
 // exactly once.  A cluster of CL CTAs owns a contiguous range of rows (a flat
-// partition of all N~ rows, so every SM gets the same amount of X); CTA rank q
+// partition of all batches, so every SM gets the same amount of X); CTA rank q
 // of the cluster owns the column slice [q*Wc, (q+1)*Wc).  Rows arrive through
 // a ring of S shared-memory stages filled by TMA bulk copies
 // (cp.async.bulk, one per row slice, completion on an mbarrier).  For each
-// stage of RB rows:
-//   pass 1: every thread forms partial dot products of its columns with w;
-//           they are reduced across the CTA (warp shuffles + shared memory)
-//           and, when CL > 1, across the cluster through distributed shared
-//           memory (st.shared::cluster + barrier.cluster);
-//   then:   residual r = f(z) - y01 per row (and the loss term);
-//   pass 2: acc[col] += r * x[row, col] from the same shared-memory stage.
+// batch of RB rows:
+//   pass 1: every thread forms partial dot products of its columns with w and
+//           leaves x in tensor memory; its warp's sums go to the reducer warp;
+//   the reducer warp adds the warps' sums, exchanges them across the cluster
+//           when CL > 1 (st.async into distributed shared memory), and
+//           publishes the residuals r = f(z) - y01 (and adds the loss terms);
+//   pass 2: acc[col] += r * x[row, col], x from tensor memory, two batches
+//           behind pass 1.
+// What the two separate: a stage is free as soon as its dot products are formed,
+// so nearly the whole ring is in flight (tensor memory holds the three batches
+// between the passes, 256 KB an SM that the kernel has no other use for), and
+// no warp waits at a block barrier or for the exchange.  bf16 d = 65536, 8.6 GB:
+// 1.74 ms (73% of the copy rate) with both passes from the stage, a named
+// barrier per batch and the exchange by the consumers; 1.74 with x in tensor
+// memory alone; 1.29 with the reducer warp, which then spent its time in the
+// release fence of the remote arrive; 1.22 with st.async (104%).  fp32 d =
+// 16384 .. 65536, 2 GB: 61-77% before, 86-98% now.
 // acc lives in registers; when the row range crosses into a new chunk the
 // cluster writes its partial chunk gradient to a scratch slot, and a small
 // second kernel adds the (at most a few) partials of every chunk in a fixed
@@ -69,8 +79,30 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(addr), "r"(rank));
   return out;
 }
-__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+// R floats into a peer's shared memory, counted as 4 R bytes on the peer's
+// mbarrier: no fence between the data and the signal (an arrive.release.cluster
+// after plain remote stores held the sending warp for over a microsecond).
+template <int R>
+__device__ __forceinline__ void st_async(uint32_t addr, const float (&z)[R], uint32_t bar) {
+  static_assert(R == 1 || R == 2 || R == 4, "rows per batch must be 1, 2 or 4");
+  if constexpr (R == 1)
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(
+                     addr),
+                 "r"(__float_as_uint(z[0])), "r"(bar)
+                 : "memory");
+  else if constexpr (R == 2)
+    asm volatile(
+        "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(
+            addr),
+        "r"(__float_as_uint(z[0])), "r"(__float_as_uint(z[1])), "r"(bar)
+        : "memory");
+  else
+    asm volatile(
+        "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, "
+        "[%5];" ::"r"(addr),
+        "r"(__float_as_uint(z[0])), "r"(__float_as_uint(z[1])), "r"(__float_as_uint(z[2])),
+        "r"(__float_as_uint(z[R - 1])), "r"(bar)
+        : "memory");
 }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
@@ -124,6 +156,7 @@ struct Elems {
   __device__ static __forceinline__ void unpack(const Raw& r, float (&o)[V]) {
     Vec<T>::unpack(r, o);
   }
+  __device__ static __forceinline__ uint4 words(const Raw& r) { return r; }
 };
 template <typename T, int NT>
 struct Elems<T, false, NT> {
@@ -146,14 +179,64 @@ struct Elems<T, false, NT> {
 #pragma unroll
     for (int e = 0; e < V; ++e) o[e] = r.f[e];
   }
+  // the 16 bytes they came from
+  __device__ static __forceinline__ uint4 words(const Raw& r) {
+    auto bits = [&](int e) { return __float_as_uint(r.f[e]); };
+    if constexpr (sizeof(T) == 4) {
+      return make_uint4(bits(0), bits(1), bits(2), bits(3));
+    } else {
+      auto two = [&](int e) { return (bits(e) >> 16) | bits(e + 1); };
+      return make_uint4(two(0), two(2), two(4), two(6));
+    }
+  }
 };
 
 constexpr int kMaxStages = 4;
-// DSMEM exchange slots: a peer can run at most ~1.5 batches ahead of this CTA
-// (it needs this CTA's sums of batch n + 1 before writing batch n + 4), so
-// four slots keep a slot from being rewritten before it is read.
-constexpr int kZSlots = 4;
+// Pass 1 of batch n + kAhead runs before pass 2 of batch n, which leaves the
+// reducer (and a cluster's exchange) two batches' time.
+constexpr int kAhead = 2;
+// Slots of the warps' partial dots and of the residuals, by batch.  A consumer
+// warp that writes its partials of batch m has taken the residuals of batch
+// m - kAhead - 1, so the reducer has read the partials up to m - kAhead; the
+// reducer publishes the residuals of batch n after every warp's partials of
+// batch n or later, which follow pass 2 of batch n - kAhead - 1.
+constexpr int kSlots = kAhead + 2;
+// DSMEM exchange slots.  A peer's reducer sends batch n after it has all sums of
+// batch n - 2, so this CTA has sent n - 2, having read the sums up to n - 4.
+constexpr int kZSlots = 8;
+// Tensor memory as the place of x between the two passes: a batch is at most 32
+// words a thread, one word a lane in 32 columns of its warp's lane quarter;
+// batches n .. n + kAhead are held.
+constexpr int kParkBatches = 4;
+constexpr int kParkCols = 32 * kParkBatches;  // columns a warp
+static_assert(kParkBatches > kAhead && kSlots > kAhead + 1, "slots");
+
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint4& v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "r"(v.x),
+               "r"(v.y), "r"(v.z), "r"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() {
+  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint4 tmem_ld4(uint32_t taddr) {
+  uint4 v;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(taddr)
+               : "memory");
+  return v;
+}
+// The values of loads issued before this are complete after it.
+template <int N>
+__device__ __forceinline__ void tmem_wait_ld(uint4 (&v)[N]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int k = 0; k < N; ++k)  // no use of the values moves above the wait
+    asm volatile("" : "+r"(v[k].x), "+r"(v[k].y), "+r"(v[k].z), "+r"(v[k].w)::"memory");
+}
 constexpr long long kSpinLimit = 1LL << 31;  // clock cycles (~1 s) per wait
+constexpr long long kLandCycles = 1LL << 17;  // ~70 us, far above a remote store's latency
 
 struct CGArgs {
   const void* X;
@@ -178,13 +261,6 @@ struct CGArgs {
   uint32_t* status;
 };
 
-// Arrive on the mbarrier at the same offset in cluster peer `rank`, releasing
-// this thread's prior shared::cluster stores to it.
-__device__ __forceinline__ void mbar_arrive_remote(uint64_t* bar, uint32_t rank) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(
-                   mapa(smem_u32(bar), rank))
-               : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -212,8 +288,11 @@ __device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, vol
   }
   return true;
 }
-__device__ __forceinline__ void consumer_sync(int nthreads) {
-  asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
+// A warp's bounded wait: every lane waits, then the warp goes on together.
+__device__ __forceinline__ void warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                          uint32_t* status, long long limit, bool cl = false) {
+  bounded_wait(bar, parity, abort_flag, status, limit, cl);
+  __syncwarp();
 }
 
 // Warp sums of R row partials with a halving butterfly: log2(R) exchange
@@ -221,8 +300,8 @@ __device__ __forceinline__ void consumer_sync(int nthreads) {
 // shuffles instead of 5 R.  Lane l ends with the warp sum of row l >> (5 - log2 R).
 template <int R>
 __device__ __forceinline__ float warp_sum_rows(const float (&p)[R], int lane) {
-  constexpr int LR = R >= 4 ? 2 : (R >= 2 ? 1 : 0);
-  static_assert((1 << LR) == R, "rows per batch must be 1, 2 or 4");
+  constexpr int LR = R >= 8 ? 3 : (R >= 4 ? 2 : (R >= 2 ? 1 : 0));
+  static_assert((1 << LR) == R, "rows per batch must be 1, 2, 4 or 8");
   float v[R];
 #pragma unroll
   for (int j = 0; j < R; ++j) v[j] = p[j];
@@ -263,7 +342,8 @@ struct Ring {
   }
 };
 
-// NT consumer threads (warps 0 .. NW-1) plus one producer warp (warp NW).
+// NT consumer threads (warps 0 .. NW-1), a producer warp (warp NW) and a reducer
+// warp (warp NW + 1).
 template <typename T, bool ALIGNED, int CL, int NT, int NVT, int RBM>
 __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
   constexpr int V = Vec<T>::V;
@@ -272,13 +352,17 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
   extern __shared__ __align__(128) unsigned char smem[];
   T* stages = reinterpret_cast<T*>(smem);
   const size_t stage_elems = (size_t)RBM * a.ld_s;
-  float* red = reinterpret_cast<float*>(smem + a.S * stage_elems * sizeof(T));  // [2][NW][RBM]
-  float* zcl = red + 2 * NW * RBM;                                               // [kZSlots][CL][RBM]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(zcl + kZSlots * CL * RBM + 2);    // 8-byte aligned
+  float* red = reinterpret_cast<float*>(smem + a.S * stage_elems * sizeof(T));  // [kSlots][NW][RBM]
+  float* zcl = red + kSlots * NW * RBM;                                         // [kZSlots][CL][RBM]
+  float* resid = zcl + kZSlots * CL * RBM;                                      // [kSlots][RBM]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(resid + kSlots * RBM);           // 16-byte aligned
   uint64_t* full = bars;                    // [kMaxStages] data landed
-  uint64_t* empty = bars + kMaxStages;      // [kMaxStages] consumers done with the stage
-  uint64_t* zfull = bars + 2 * kMaxStages;  // [kZSlots] every peer's partial dots arrived
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + 2 * kMaxStages + kZSlots);
+  uint64_t* empty = full + kMaxStages;      // [kMaxStages] consumers done with the stage
+  uint64_t* part = empty + kMaxStages;      // [kSlots] every warp's partial dots written
+  uint64_t* ready = part + kSlots;          // [kSlots] residuals written
+  uint64_t* zfull = ready + kSlots;         // [kZSlots] every peer's partial dots arrived
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(zfull + kZSlots);
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(zfull + kZSlots) + 1;
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = CL > 1 ? (int)cluster_rank() : 0;
@@ -305,7 +389,11 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], NW);
     }
-    for (int z = 0; z < kZSlots; ++z) mbar_init(&zfull[z], CL);
+    for (int z = 0; z < kSlots; ++z) {
+      mbar_init(&part[z], NW);
+      mbar_init(&ready[z], 1);
+    }
+    for (int z = 0; z < kZSlots; ++z) mbar_init(&zfull[z], 1);
     fence_mbar_init();
   }
   {
@@ -323,7 +411,18 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
     }
     if (!ALIGNED) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  constexpr uint32_t kTmemCols = NW / 4 * kParkCols;  // 1, 2 or 4 warps a lane quarter: 128, 256, 512
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tmem_holder)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tcw::fence_before();
   __syncthreads();
+  tcw::fence_after();
+  const uint32_t tmem_base = *tmem_holder;
   if (CL > 1) cluster_sync_all();  // every peer has started and initialised its barriers
 
   if (warp == NW) {
@@ -335,47 +434,66 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
     int issued = 0;
     long long row = r0;
     int bi = bi0;
-    for (int n = 0; n < (a.stall ? 0 : nb); ++n) {
-      const int s = n % a.S;
-      const uint32_t ph = (uint32_t)((n / a.S) & 1);
-      const int nr = bi == a.nbc - 1 ? last_rows : RBM;  // rows of this batch
-      T* st = stages + s * stage_elems;
-      if constexpr (ALIGNED) {
-        const bool ok = bounded_wait(&empty[s], ph ^ 1, abort_flag, a.status, a.spin_limit);
-        if (!__all_sync(0xffffffffu, ok && !*abort_flag)) break;
+    const int nbs = a.stall ? 0 : nb;
+    auto rows_at = [&](int k) { return k == a.nbc - 1 ? last_rows : RBM; };  // rows of batch k of a chunk
+    // the stage of batch n is free
+    auto stage_free = [&](int n) {
+      const bool ok = bounded_wait(&empty[n % a.S], (uint32_t)((n / a.S) & 1) ^ 1, abort_flag, a.status,
+                                   a.spin_limit);
+      return (bool)__all_sync(0xffffffffu, ok && !*abort_flag);
+    };
+    if constexpr (ALIGNED) {
+      for (int n = 0; n < nbs; ++n) {
+        const int s = n % a.S, nr = rows_at(bi);
+        if (!stage_free(n)) break;
         if (lane == 0) {
+          T* st = stages + s * stage_elems;
           const uint32_t row_bytes = (uint32_t)(width * sizeof(T));
           mbar_expect_tx(&full[s], row_bytes * nr);
           for (int r = 0; r < nr; ++r)
             bulk_g2s(st + (size_t)r * a.ld_s, X + (row + r) * a.d + c0, row_bytes, &full[s]);
         }
-      } else {
-        // Row r's slice starts o elements past a 16-byte boundary.  Its whole
-        // 16-byte pieces up to element pt of the stage row arrive by one bulk
-        // copy; the 2 V elements from pt on -- the last columns, then zeros
-        // over what an earlier row with a larger o may have left there -- are
-        // stored by the lanes (read from X before the wait, which hides them).
-        const uint32_t e0 = (uint32_t)row * (uint32_t)a.d + (uint32_t)c0 + xo;
-        const uint32_t dv = (uint32_t)a.d;
-        constexpr int NTL = (RBM * 2 * V + 31) / 32;
-        T tv[NTL];
-        T* tp[NTL];
+        issued = n + 1;
+        row += nr;
+        if (++bi == a.nbc) bi = 0;
+      }
+    } else {
+      // Row r's slice starts o elements past a 16-byte boundary.  Its whole
+      // 16-byte pieces up to element pt of the stage row arrive by one bulk copy;
+      // the 2 V elements from pt on -- the last columns, then zeros over what an
+      // earlier row with a larger o may have left there -- are stored by the
+      // lanes, read from X one batch ahead.
+      constexpr int NTL = (RBM * 2 * V + 31) / 32;
+      struct Tail {
+        T v[NTL];
+        int pos[NTL];  // in the stage, -1: none
+      };
+      const uint32_t dv = (uint32_t)a.d;
+      auto load_tail = [&](long long row, int nr, Tail& t) {
+        const uint32_t e0 = (uint32_t)row * dv + (uint32_t)c0 + xo;
 #pragma unroll
         for (int k = 0; k < NTL; ++k) {
-          const int t = k * 32 + lane, r = t / (2 * V);
+          const int i = k * 32 + lane, r = i / (2 * V);
           const uint32_t o = (e0 + (uint32_t)r * dv) & (V - 1);
-          const int pos = (int)((o + (uint32_t)width) & ~(uint32_t)(V - 1)) + t % (2 * V);
+          const int pos = (int)((o + (uint32_t)width) & ~(uint32_t)(V - 1)) + i % (2 * V);
           const int c = pos - (int)o;
-          tp[k] = r < nr ? st + (size_t)r * a.ld_s + pos : nullptr;
-          tv[k] = T(0.f);
-          if (r < nr && c >= 0 && c < width) tv[k] = X[(row + r) * a.d + c0 + c];
+          t.pos[k] = r < nr ? r * a.ld_s + pos : -1;
+          t.v[k] = T(0.f);
+          if (r < nr && c >= 0 && c < width) t.v[k] = X[(row + r) * a.d + c0 + c];
         }
-        const bool ok = bounded_wait(&empty[s], ph ^ 1, abort_flag, a.status, a.spin_limit);
-        if (!__all_sync(0xffffffffu, ok && !*abort_flag)) break;
+      };
+      // issue batch n, whose tail is `cur`; load the next one's
+      auto issue = [&](int n, const Tail& cur, Tail& next) {
+        const int s = n % a.S, nr = rows_at(bi);
+        const int nbi = bi + 1 == a.nbc ? 0 : bi + 1;
+        if (n + 1 < nbs) load_tail(row + nr, rows_at(nbi), next);
+        if (!stage_free(n)) return false;
+        T* st = stages + s * stage_elems;
 #pragma unroll
         for (int k = 0; k < NTL; ++k)
-          if (tp[k]) *tp[k] = tv[k];
-        const uint32_t o = (e0 + (uint32_t)lane * dv) & (V - 1);
+          if (cur.pos[k] >= 0) st[cur.pos[k]] = cur.v[k];
+        const uint32_t o =
+            ((uint32_t)row * dv + (uint32_t)c0 + xo + (uint32_t)lane * dv) & (V - 1);
         const T* src = X + (row + lane) * a.d + c0 - o;  // 16-byte aligned
         T* dst = st + (size_t)lane * a.ld_s;
         uint32_t pt = lane < nr ? (o + (uint32_t)width) & ~(uint32_t)(V - 1) : 0u;
@@ -394,16 +512,140 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
         if (lane == 0) mbar_expect_tx(&full[s], total);
         __syncwarp();
         if (bytes > 0) bulk_g2s(dst, src, bytes, &full[s]);
+        issued = n + 1;
+        row += nr;
+        bi = nbi;
+        return true;
+      };
+      Tail t0, t1;
+      if (nbs > 0) load_tail(row, rows_at(bi), t0);
+      for (int n = 0; n < nbs; n += 2) {
+        if (!issue(n, t0, t1)) break;
+        if (n + 1 < nbs && !issue(n + 1, t1, t0)) break;
       }
-      issued = n + 1;
-      row += nr;
-      if (++bi == a.nbc) bi = 0;
     }
     // drain: the CTA must not exit with copies in flight
     if (lane == 0) {
       volatile int no_abort = 0;
       for (int n = max(0, issued - a.S); n < issued; ++n)
         bounded_wait(&full[n % a.S], (uint32_t)((n / a.S) & 1), &no_abort, a.status, kSpinLimit);
+    }
+  } else if (warp == NW + 1) {
+    // ------------------------------------------------------------ reducer warp
+    // Per batch: the CTA's sums of the warps' partial dots, with clusters their
+    // exchange, the residuals and the loss; none of it in the consumers' way.
+    double loss_acc = 0.0;
+    // y of the next batches for lane r < their rows
+    const float* yp = a.y + r0 + lane;
+    int ybi = bi0, yleft = nb;
+    auto load_y = [&]() {
+      const int nr = ybi == a.nbc - 1 ? last_rows : RBM;
+      const float v = (lane < nr && yleft > 0) ? __ldg(yp) : 0.f;
+      yp += nr;
+      --yleft;
+      if (++ybi == a.nbc) ybi = 0;
+      return v;
+    };
+    float y0 = load_y(), y1 = load_y();
+    int bi = bi0;
+    // CTA sums of batch n, in every lane: the NW x RBM partials are spread over
+    // the lanes (entry j*32 + lane is warp idx % NW of row idx / NW), summed over
+    // aligned groups of NW lanes, then row r is read from the first of its group.
+    auto cta_sums = [&](int n, float (&z)[RBM]) {
+      warp_wait(&part[n % kSlots], (uint32_t)((n / kSlots) & 1), abort_flag, a.status, a.spin_limit);
+      const float* redn = red + (n % kSlots) * NW * RBM;
+      constexpr int E = NW * RBM, NCH = (E + 31) / 32;
+      float cs[NCH];
+#pragma unroll
+      for (int j = 0; j < NCH; ++j) {
+        const int idx = j * 32 + lane;
+        float t = idx < E ? redn[(idx % NW) * RBM + idx / NW] : 0.f;
+#pragma unroll
+        for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        cs[j] = t;
+      }
+#pragma unroll
+      for (int r = 0; r < RBM; ++r) z[r] = __shfl_sync(0xffffffffu, cs[(r * NW) / 32], (r * NW) % 32);
+    };
+    // Lane p writes the CTA's sums into peer p's slot; the slot's barrier waits for
+    // all peers' bytes.  After a failed wait the CTA sends no more: a peer then
+    // never receives more bytes in one phase than it expects.
+    auto send = [&](int n, const float (&z)[RBM]) {
+      uint64_t* bar = &zfull[n % kZSlots];
+      float* mine = zcl + (n % kZSlots) * CL * RBM + rank * RBM;
+      if (lane == 0) mbar_expect_tx(bar, CL * RBM * (uint32_t)sizeof(float));
+      if constexpr (CL > 1)
+        if (lane < CL && !*abort_flag)
+          st_async<RBM>(mapa(smem_u32(mine), (uint32_t)lane), z, mapa(smem_u32(bar), (uint32_t)lane));
+    };
+    // Cluster sums of batch n once every peer's have arrived: lane p * RBM + r
+    // reads peer p's sum of row r, a xor tree adds the peers.
+    auto cluster_sums = [&](int n, float (&z)[RBM]) {
+      warp_wait(&zfull[n % kZSlots], (uint32_t)((n / kZSlots) & 1), abort_flag, a.status,
+                a.spin_limit, true);
+      const float* zc = zcl + (n % kZSlots) * CL * RBM;
+      float t = lane < CL * RBM ? zc[lane] : 0.f;
+#pragma unroll
+      for (int o = RBM; o < CL * RBM; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+#pragma unroll
+      for (int r = 0; r < RBM; ++r) z[r] = __shfl_sync(0xffffffffu, t, r);
+    };
+    // Residuals of batch n from its row sums (lane r takes row r), and the loss.
+    auto publish = [&](int n, const float (&z)[RBM]) {
+      const int nr = bi == a.nbc - 1 ? last_rows : RBM;
+      if (++bi == a.nbc) bi = 0;
+      const float yv = y0;
+      y0 = y1;
+      y1 = load_y();
+      float zr = z[0];
+#pragma unroll
+      for (int r = 1; r < RBM; ++r) zr = lane == r ? z[r] : zr;
+      const float mine =
+          a.loss == GC_LSQ ? zr - yv : 1.f / (1.f + __expf(-zr)) - 0.5f * (yv + 1.f);
+      if (lane < RBM) resid[(n % kSlots) * RBM + lane] = mine;
+      __syncwarp();
+      if (lane == 0) tcw::mbar_arrive(&ready[n % kSlots]);
+      // ---- the loss: lane r adds its rows in fp64
+      if (a.want_loss && rank == 0) {
+        float lr = 0.f;
+        if (lane < nr) {
+          if (a.loss == GC_LSQ) {
+            const float e = zr - yv;
+            lr = 0.5f * e * e;
+          } else {
+            // log(1 + e^t) = max(t, 0) + log(1 + e^-|t|); the fast intrinsics
+            // are accurate to ~1e-6 absolute per row here (1 + e^-|t| lies in
+            // [1, 2]), far below the loss's 1e-5 relative tolerance
+            const float t = -yv * zr;
+            lr = fmaxf(t, 0.f) + __logf(1.f + __expf(-fabsf(t)));
+          }
+        }
+        loss_acc += (double)lr;
+      }
+    };
+    for (int n = 0; n < nb; ++n) {
+      float z[RBM];
+      cta_sums(n, z);
+      if constexpr (CL == 1) {
+        publish(n, z);
+      } else {
+        send(n, z);
+        // the sums of the batch before have had this one's time to arrive
+        if (n > 0) {
+          cluster_sums(n - 1, z);
+          publish(n - 1, z);
+        }
+      }
+    }
+    if (CL > 1 && nb > 0) {
+      float z[RBM];
+      cluster_sums(nb - 1, z);
+      publish(nb - 1, z);
+    }
+    if (a.want_loss && rank == 0) {
+#pragma unroll
+      for (int o = RBM / 2; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
+      if (lane == 0) a.loss_parts[q] = loss_acc;
     }
   } else {
     // ------------------------------------------------------------ consumer warps
@@ -429,7 +671,6 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
 #pragma unroll
       for (int e = 0; e < V2; ++e) acc[u][e] = make_float2(0.f, 0.f);
     long long cur = -1;     // chunk whose gradient acc holds
-    double loss_acc = 0.0;
     auto flush = [&](long long chunk) {
       float* dst = a.parts + ((size_t)q * a.maxt + (size_t)(chunk - first_chunk)) * a.d;
 #pragma unroll
@@ -445,7 +686,7 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
     // Stage access.  Every stage row is NVT * NT vectors long and the parts
     // the producer never writes are zero, so the reads need no masks.
     auto wait_stage = [&](const Ring& g) {
-      bounded_wait(&full[g.s], g.ph, abort_flag, a.status, a.spin_limit);
+      warp_wait(&full[g.s], g.ph, abort_flag, a.status, a.spin_limit);
     };
     auto from_stage = [&](const Ring& g) {
       const T* st = stages + (size_t)g.s * stage_elems + (ALIGNED ? tid * V : tid);
@@ -459,23 +700,22 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
         };
       }
     };
-    // x of a batch copied to registers once (kept from the dot products to pass 2)
-    auto load_x = [&](const Ring& g, typename EL::Raw (&xr)[RBM][NVT]) {
-      auto src = from_stage(g);
-#pragma unroll
-      for (int r = 0; r < RBM; ++r)
-#pragma unroll
-        for (int u = 0; u < NVT; ++u) xr[r][u] = src(r, u);
-    };
     // hand a stage back to the producer (every lane of the warp is done reading it)
     auto release = [&](const Ring& g) {
       __syncwarp();
       if (lane == 0) tcw::mbar_arrive(&empty[g.s]);
     };
-    // Dot products of batch n, reduced over the CTA (warp butterfly, then
-    // lane-parallel over (warp, row) pairs) and, with clusters, sent to every
-    // peer.  Returns the CTA sums in every lane.
-    auto dots = [&](int n, auto&& xget, float (&z)[RBM]) {
+    const uint32_t park0 =
+        tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * kParkCols);
+    auto park_slot = [&](int n) { return park0 + (uint32_t)(n % kParkBatches) * 32u; };
+    // Pass 1 of the batch at g: its dot products, reduced over the warp and left
+    // for the reducer.  x waits for pass 2 in tensor memory, so that the stage
+    // goes back to the producer at once (held until pass 2, one of a cluster's
+    // three stages was left to be in flight).
+    auto pass1 = [&](int n, const Ring& g) {
+      const uint32_t at = park_slot(n);
+      wait_stage(g);  // ends converged, as the warp-collective tensor-memory instructions need
+      auto xget = from_stage(g);
       // two packed partial sums a row (vectors u even / odd), so that the
       // FMA chain of a row is a quarter as long
       float pd[RBM];
@@ -485,73 +725,27 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
 #pragma unroll
         for (int u = 0; u < NVT; ++u) {
           float x[V];
-          EL::unpack(xget(r, u), x);
+          const typename EL::Raw raw = xget(r, u);
+          tmem_st4(at + (uint32_t)((r * NVT + u) * 4), EL::words(raw));
+          EL::unpack(raw, x);
 #pragma unroll
           for (int e = 0; e < V2; ++e)
             p2[u & 1] = __ffma2_rn(make_float2(x[2 * e], x[2 * e + 1]), wv[u][e], p2[u & 1]);
         }
         pd[r] = (p2[0].x + p2[0].y) + (p2[1].x + p2[1].y);
       }
-      constexpr int kRowShift = 5 - (RBM >= 4 ? 2 : (RBM >= 2 ? 1 : 0));
+      release(g);
+      __syncwarp();
+      tmem_wait_st();
+      constexpr int kRowShift = 5 - (RBM >= 8 ? 3 : (RBM >= 4 ? 2 : (RBM >= 2 ? 1 : 0)));
       const float ws_ = warp_sum_rows<RBM>(pd, lane);
-      float* redn = red + (n & 1) * NW * RBM;
-      if ((lane & ((1 << kRowShift) - 1)) == 0) redn[warp * RBM + (lane >> kRowShift)] = ws_;
-      consumer_sync(NT);
-      // CTA sums: the NW x RBM partials are spread over the lanes (entry
-      // j*32 + lane is warp (idx % NW) of row idx / NW), summed over aligned
-      // groups of NW lanes, then row r is read from the first lane of its group.
-      constexpr int E = NW * RBM, NCH = (E + 31) / 32;
-      float cs[NCH];
-#pragma unroll
-      for (int j = 0; j < NCH; ++j) {
-        const int idx = j * 32 + lane;
-        float t = idx < E ? redn[(idx % NW) * RBM + idx / NW] : 0.f;
-#pragma unroll
-        for (int o = NW / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        cs[j] = t;
-      }
-#pragma unroll
-      for (int r = 0; r < RBM; ++r) z[r] = __shfl_sync(0xffffffffu, cs[(r * NW) / 32], (r * NW) % 32);
-      if (CL > 1 && tid < CL && !*abort_flag) {
-        // thread p writes the CTA sums into peer p's slot and arrives there
-        // (release).  After a failed wait the CTA sends no more: a peer then
-        // never receives more arrivals in one phase than it expects.
-        float* zc = zcl + (n % kZSlots) * CL * RBM;
-        const uint32_t peer = (uint32_t)tid;
-#pragma unroll
-        for (int r = 0; r < RBM; ++r)
-          st_cluster_f32(mapa(smem_u32(zc + rank * RBM + r), peer), z[r]);
-        mbar_arrive_remote(&zfull[n % kZSlots], peer);
-      }
+      if ((lane & ((1 << kRowShift) - 1)) == 0)
+        red[((n % kSlots) * NW + warp) * RBM + (lane >> kRowShift)] = ws_;
+      __syncwarp();
+      if (lane == 0) tcw::mbar_arrive(&part[n % kSlots]);
     };
-    // Cluster sums of batch n once every peer's CTA sums have arrived: lane
-    // p * RBM + r reads peer p's sum of row r, a xor tree adds the peers.
-    auto cluster_sums = [&](int n, float (&z)[RBM]) {
-      bounded_wait(&zfull[n % kZSlots], (uint32_t)((n / kZSlots) & 1), abort_flag, a.status,
-                   a.spin_limit, true);
-      const float* zc = zcl + (n % kZSlots) * CL * RBM;
-      float t = lane < CL * RBM ? zc[lane] : 0.f;
-#pragma unroll
-      for (int o = RBM; o < CL * RBM; o <<= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-#pragma unroll
-      for (int r = 0; r < RBM; ++r) z[r] = __shfl_sync(0xffffffffu, t, r);
-    };
-
-    // y of a batch for lane r < its rows, loaded two batches ahead (off the
-    // critical path between the dot products and the residuals)
-    const float* yp = a.y + r0 + lane;  // row of the batch y is loaded for next
-    int ybi = bi0, yleft = nb;
-    auto load_y = [&]() {
-      const int nr = ybi == a.nbc - 1 ? last_rows : RBM;
-      const float v = (lane < nr && yleft > 0) ? __ldg(yp) : 0.f;
-      yp += nr;
-      --yleft;
-      if (++ybi == a.nbc) ybi = 0;
-      return v;
-    };
-    float y0 = load_y(), y1 = load_y();
-    // Residuals, loss and pass 2 (acc += r * x) of the batch at g from its row sums z.
-    auto finish = [&](const Ring& g, const float (&z)[RBM], auto&& xget) {
+    // Pass 2 (acc += r * x) of the batch at g.
+    auto pass2 = [&](int n, const Ring& g) {
       if (cur < 0 || g.bi == 0) {  // a new chunk (a batch never straddles chunks)
         if (cur >= 0) flush(cur);
 #pragma unroll
@@ -561,45 +755,22 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
         cur = cur < 0 ? first_chunk : cur + 1;
       }
       const int nr = g.bi == a.nbc - 1 ? last_rows : RBM;
-      const float yv = y0;
-      y0 = y1;
-      y1 = load_y();
-      // ---- residuals: lane r < RBM takes row r, then a broadcast
-      float zr = z[0];
-#pragma unroll
-      for (int r = 1; r < RBM; ++r) zr = lane == r ? z[r] : zr;
-      const float mine =
-          a.loss == GC_LSQ ? zr - yv : 1.f / (1.f + __expf(-zr)) - 0.5f * (yv + 1.f);
+      const uint32_t at = park_slot(n);
+      warp_wait(&ready[n % kSlots], (uint32_t)((n / kSlots) & 1), abort_flag, a.status, a.spin_limit);
       float res[RBM];
 #pragma unroll
-      for (int r = 0; r < RBM; ++r) res[r] = __shfl_sync(0xffffffffu, mine, r);
-      // ---- the loss: lane r < RB of warp 0 takes row r (fp32), one fp64 add per batch
-      if (a.want_loss && rank == 0 && warp == 0) {
-        float lr = 0.f;
-        if (lane < nr) {
-          if (a.loss == GC_LSQ) {
-            const float e = zr - yv;
-            lr = 0.5f * e * e;
-          } else {
-            // log(1 + e^t) = max(t, 0) + log(1 + e^-|t|); the fast intrinsics
-            // are accurate to ~1e-6 absolute per row here (1 + e^-|t| lies in
-            // [1, 2]), far below the loss's 1e-5 relative tolerance, and keep
-            // warp 0 from lagging behind the others at every batch
-            const float t = -yv * zr;
-            lr = fmaxf(t, 0.f) + __logf(1.f + __expf(-fabsf(t)));
-          }
-        }
-#pragma unroll
-        for (int o = 2; o > 0; o >>= 1) lr += __shfl_xor_sync(0xffffffffu, lr, o);
-        if (lane == 0) loss_acc += (double)lr;
-      }
-      // ---- pass 2 (rows past nr hold an earlier batch's values: skipped)
+      for (int r = 0; r < RBM; ++r) res[r] = resid[(n % kSlots) * RBM + r];
+      // rows past nr hold an earlier batch's values: skipped
       auto add_row = [&](int r) {
+        uint4 xr[NVT];
+#pragma unroll
+        for (int u = 0; u < NVT; ++u) xr[u] = tmem_ld4(at + (uint32_t)((r * NVT + u) * 4));
+        tmem_wait_ld(xr);
         const float2 rr = make_float2(res[r], res[r]);
 #pragma unroll
         for (int u = 0; u < NVT; ++u) {
           float x[V];
-          EL::unpack(xget(r, u), x);
+          Vec<T>::unpack(xr[u], x);
 #pragma unroll
           for (int e = 0; e < V2; ++e)
             acc[u][e] = __ffma2_rn(rr, make_float2(x[2 * e], x[2 * e + 1]), acc[u][e]);
@@ -615,64 +786,42 @@ __device__ __forceinline__ void chunkgrad_body(const CGArgs& a) {
       }
     };
 
-    // x in registers when they fit beside acc and w (fp32 rows; not bf16,
-    // whose unpacked vectors would spill)
-    constexpr bool kXRegs = NVT * RBM * V <= 32;
     Ring g{0, 0u, bi0, (uint32_t)r0 * (uint32_t)a.d + (uint32_t)c0 + xo};
-    if (CL == 1 && kXRegs) {
-      // One pass over the stage: x stays in registers from the dot products to
-      // pass 2, so the stage goes back to the producer as soon as it is read.
-      for (int n = 0; n < nb; ++n, g.next<ALIGNED>(a, RBM)) {
-        typename EL::Raw xr[RBM][NVT];
-        float z[RBM];
-        wait_stage(g);
-        load_x(g, xr);
-        release(g);
-        auto xget = [&](int r, int u) { return xr[r][u]; };
-        dots(n, xget, z);
-        finish(g, z, xget);
-      }
-    } else if (CL == 1) {
-      for (int n = 0; n < nb; ++n, g.next<ALIGNED>(a, RBM)) {
-        float z[RBM];
-        wait_stage(g);
-        dots(n, from_stage(g), z);
-        finish(g, z, from_stage(g));
-        release(g);
-      }
-    } else {
-      // Clusters: batch n + 1's dot products and send run before the wait for
-      // batch n's cluster sums (software pipelining); pass 2 re-reads the
-      // stage, which is handed back afterwards.
-      float znext[RBM];
-      Ring g1 = g;
-      if (nb > 0) {
-        wait_stage(g1);
-        dots(0, from_stage(g1), znext);
+    Ring g1 = g;
+    for (int n = 0; n < min(kAhead, nb); ++n, g1.next<ALIGNED>(a, RBM)) pass1(n, g1);
+    for (int n = 0; n < nb; ++n, g.next<ALIGNED>(a, RBM)) {
+      if (n + kAhead < nb) {
+        pass1(n + kAhead, g1);
         g1.next<ALIGNED>(a, RBM);
       }
-      for (int n = 0; n < nb; ++n, g.next<ALIGNED>(a, RBM), g1.next<ALIGNED>(a, RBM)) {
-        if (n + 1 < nb) {
-          wait_stage(g1);
-          dots(n + 1, from_stage(g1), znext);
-        }
-        float z[RBM];
-        cluster_sums(n, z);
-        finish(g, z, from_stage(g));
-        release(g);
-      }
+      pass2(n, g);
     }
     // the reduction kernel may be scheduled now (it waits for this grid to
     // finish); not earlier, so that work on other streams keeps the SMs' room
     if (tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (cur >= 0) flush(cur);
-    if (tid == 0 && rank == 0) a.loss_parts[q] = loss_acc;
   }
-  if (CL > 1) cluster_sync_all();  // no CTA leaves while a peer may still address it
+  tcw::fence_before();
+  if (CL > 1)
+    cluster_sync_all();  // no CTA leaves while a peer may still address it
+  else
+    __syncthreads();
+  tcw::fence_after();
+  if (CL > 1 && *abort_flag) {
+    // after a failed wait sums that peers sent before the barrier may still be
+    // on their way into this CTA's shared memory: let them land
+    for (const long long t0 = clock64(); clock64() - t0 < kLandCycles;) {
+    }
+  }
+  __syncwarp();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                 "r"(kTmemCols)
+                 : "memory");
 }
 
 template <typename T, bool ALIGNED, int CL, int NT, int NVT, int RBM>
-__global__ void __launch_bounds__(NT + 32, 1) k_chunkgrad(CGArgs a) {
+__global__ void __launch_bounds__(NT + 64, 1) k_chunkgrad(CGArgs a) {
   chunkgrad_body<T, ALIGNED, CL, NT, NVT, RBM>(a);
 }
 
@@ -687,9 +836,9 @@ Kernel pick_shape(int NT, int NVT) {
     if (NT == 512 && NVT == 2) return k_chunkgrad<T, ALIGNED, 1, 512, 2, 4>;
     if (NT == 256 && NVT == 4) return k_chunkgrad<T, ALIGNED, 1, 256, 4, 2>;
     if (NT == 256 && NVT == 2) return k_chunkgrad<T, ALIGNED, 1, 256, 2, 4>;
-    if (NT == 256 && NVT == 1) return k_chunkgrad<T, ALIGNED, 1, 256, 1, 4>;
+    if (NT == 256 && NVT == 1) return k_chunkgrad<T, ALIGNED, 1, 256, 1, 8>;
     if (NT == 128 && NVT == 2) return k_chunkgrad<T, ALIGNED, 1, 128, 2, 4>;
-    if (NT == 128 && NVT == 1) return k_chunkgrad<T, ALIGNED, 1, 128, 1, 4>;
+    if (NT == 128 && NVT == 1) return k_chunkgrad<T, ALIGNED, 1, 128, 1, 8>;
   }
   if constexpr (kF32 ? CL <= 4 : CL != 2)
     if (NT == 512 && NVT == 4) return k_chunkgrad<T, ALIGNED, CL, 512, 4, 2>;
