@@ -512,13 +512,16 @@ __global__ void __launch_bounds__(256) k_split_gt(const float* __restrict__ G, i
   }
   __shared__ float tile[64][COLS + 1];
   const int ncx = (L + COLS - 1) / COLS;
-  const long long npair = (long long)ncx * (Kp / 64);
+  const int nkt = Kp / 64;
+  const long long npair = (long long)ncx * nkt;
   const int K = N * ell;
   const bool vec = (L % 4 == 0) && (d % 4 == 0) && (reinterpret_cast<uintptr_t>(G) % 16 == 0);
   const size_t plane = (size_t)L * Kp;
   for (long long pr = blockIdx.x; pr < npair; pr += gridDim.x) {
     __syncthreads();  // the previous pair's tile has been read
-    const int c0 = (int)(pr % ncx) * COLS, k0 = (int)(pr / ncx) * 64;
+    // K tiles fastest: the blocks running at a time write whole plane rows
+    // (2 Kp bytes), not 128 bytes of each of many
+    const int c0 = (int)(pr / nkt) * COLS, k0 = (int)(pr % nkt) * 64;
     // load: thread t takes columns 4 (t % TPR) .. +3 of rows t / TPR + RPP r
 #pragma unroll
     for (int r = 0; r < 64 / RPP; ++r) {

@@ -405,9 +405,10 @@ int launch_encode(const double* E, const int32_t* order, const int32_t* psi, int
 
 // ghat[b][k*L + c] = sum_j R[k][j] * T[b][j][c], j ascending.  A thread takes V
 // columns; R is staged in dynamic shared memory as fp32 (ELL * m words, m <=
-// kDecodeSmemM) or read as fp64.  The kernel streams T; eight workers' loads
-// are in flight per thread, 16 bytes each where the rows allow it (m = 256,
-// ell = 2, L = 2^19: 123 us with 4-byte loads, 84 us = 6.4 TB/s with 16).
+// kDecodeSmemM) or read as fp64.  The kernel streams T; eight 16-byte loads of
+// workers' rows are in flight per thread where the rows allow it, else sixteen
+// 4-byte ones (m = 256, ell = 2, L = 2^19, 16-byte loads: 77 us = 7.0 TB/s, 123 us
+// with eight of 4 bytes; four patterns of m = 200, ell = 3, L = 87383: 60 and 73).
 constexpr int kDecodeSmemM = 1024;
 template <int ELL, bool STAGED, int V>
 __global__ void k_decode_tx(const double* __restrict__ R, int m, const float* __restrict__ T,
@@ -428,10 +429,11 @@ __global__ void k_decode_tx(const double* __restrict__ R, int m, const float* __
 #pragma unroll
     for (int v = 0; v < V; ++v) acc[k][v] = 0.f;
   const float* Tb = T + (size_t)b * m * L + c;
-  for (int j0 = 0; j0 < m; j0 += 8) {
-    float t[8][V];
+  constexpr int U = V == 4 ? 8 : 16;  // workers' loads in flight
+  for (int j0 = 0; j0 < m; j0 += U) {
+    float t[U][V];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < U; ++u) {
       const float* p = Tb + (size_t)(j0 + u) * L;
       if constexpr (V == 4) {
         const float4 q = j0 + u < m ? __ldcs(reinterpret_cast<const float4*>(p))
@@ -442,7 +444,7 @@ __global__ void k_decode_tx(const double* __restrict__ R, int m, const float* __
       }
     }
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < U; ++u) {
       if (j0 + u < m) {
 #pragma unroll
         for (int k = 0; k < ELL; ++k) {
