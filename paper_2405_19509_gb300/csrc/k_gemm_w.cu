@@ -24,6 +24,13 @@
 //           boxes per K block: LBO = 8 KB between the 64-element MN atoms,
 //           SBO = 1 KB between 8-row K groups); B = R^T planes of chunk i.
 //           The epilogue writes G[w][i][col] (coalesced along col per w).
+// GEMM 1 has few tiles (one per 256 rows of X) with a long K: the tiles past the
+// last whole wave of CTAs are cut into K ranges, enough of them to fill the
+// waves, whose partial Z go to scratch; k_resid_sum adds them in order and
+// forms the residuals.  The ranges are dealt K-major, so that the CTAs of a
+// moment read the same part of W.  (65,536 rows, d = 65536, n_w = 256: 256 tiles
+// on 152 SMs took two waves, 3.29 ms; 2.90 and 0.04.  4,096 rows, d = 8192,
+// n_w = 64, both GEMMs: 136 and 54 us.)
 // Tiles are visited so that concurrently running CTAs share the B operand
 // through L2 (all of W in MODE 0; R_i of one chunk in MODE 1).  Every wait
 // is bounded (GC_ERR_TIMEOUT, drain, return).
@@ -53,6 +60,10 @@ struct WParams {
   long long num_tiles;
   int num_m_tiles;   // MODE 0: ceil(N~ / 256); MODE 1: ceil(d / 256) (per chunk)
   int nkb;           // 64-wide K blocks per tile
+  // MODE 0: tiles [0, full_tiles) are one unit each, the split_tiles after them
+  // nsplit units each (unit full_tiles + kr * split_tiles + t)
+  int full_tiles, split_tiles, nsplit;
+  float* part;       // MODE 0: partial Z of the split units, [t * nsplit + kr][n_w][256]
   int stages;
   int stage_bytes;   // 2 * A_BYTES + 256 * n_w
   int nbuf;          // accumulator buffers (2 when 2 * n_w <= 256)
@@ -64,6 +75,18 @@ struct WParams {
   int stall;  // failure-path test: the TMA producer issues nothing
   uint32_t* status;
 };
+
+// Unit u of MODE 0: its tile and K blocks [kb0, kb1); slot of its partial
+// result, -1 for a whole tile.
+struct Unit {
+  int tile, kb0, kb1, slot;
+};
+__device__ __forceinline__ Unit unit_at(const WParams& p, long long u) {
+  if (u < p.full_tiles) return {(int)u, 0, p.nkb, -1};
+  const int v = (int)(u - p.full_tiles), kr = v / p.split_tiles, t = v - kr * p.split_tiles;
+  return {p.full_tiles + t, (int)((long long)kr * p.nkb / p.nsplit),
+          (int)((long long)(kr + 1) * p.nkb / p.nsplit), t * p.nsplit + kr};
+}
 
 template <int MODE>
 __global__ void __launch_bounds__(kThreadsW, 1)
@@ -116,15 +139,19 @@ __global__ void __launch_bounds__(kThreadsW, 1)
       bool ok = !p.stall;
       for (long long t = blockIdx.x; t < p.num_tiles && ok; t += gridDim.x) {
         int a_x, a_y;  // MODE 0: (k, row0); MODE 1: (col0, row0)
+        int kb0 = 0, kb1 = p.nkb;
         if (MODE == 0) {
+          const Unit un = unit_at(p, t);
           a_x = 0;
-          a_y = (int)(t * TM);
+          a_y = un.tile * TM;
+          kb0 = un.kb0;
+          kb1 = un.kb1;
         } else {
           const int i = (int)(t / p.num_m_tiles), mt = (int)(t % p.num_m_tiles);
           a_x = mt * TM;
           a_y = i * p.n_c;
         }
-        for (int kb = 0; kb < p.nkb; ++kb, ++it) {
+        for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const int s = it % S;
           const uint32_t ph = (it / S) & 1;
           if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, p.status, p.spin_limit)) {
@@ -165,7 +192,13 @@ __global__ void __launch_bounds__(kThreadsW, 1)
         // half h accumulates at column ab * 2 n_w + h n_w (nbuf 2) or h * 256 (nbuf 1)
         const uint32_t d0 = tmem_base + (uint32_t)(p.nbuf == 2 ? ab * 2 * n_w : 0);
         const uint32_t d1 = d0 + (uint32_t)(p.nbuf == 2 ? n_w : 256);
-        for (int kb = 0; kb < p.nkb; ++kb, ++it) {
+        int kb0 = 0, kb1 = p.nkb;
+        if (MODE == 0) {
+          const Unit un = unit_at(p, t);
+          kb0 = un.kb0;
+          kb1 = un.kb1;
+        }
+        for (int kb = kb0; kb < kb1; ++kb, ++it) {
           const int s = it % S;
           if (!mbar_wait(&full[s], (it / S) & 1, abort_flag, p.status, p.spin_limit)) {
             ok = false;
@@ -183,7 +216,7 @@ __global__ void __launch_bounds__(kThreadsW, 1)
                                           : sdesc(a1 + ks * 2048, A_BYTES / 2, 1024);
             const uint64_t bh = sdesc(b0 + ks * 32, 16, 1024);
             const uint64_t bl = sdesc(b0 + b_plane + ks * 32, 16, 1024);
-            const uint32_t acc = (kb > 0 || ks > 0) ? 1u : 0u;
+            const uint32_t acc = (kb > kb0 || ks > 0) ? 1u : 0u;
             mma_bf16(d0, x0, bh, idesc, acc);
             mma_bf16(d0, x0, bl, idesc, 1u);
             mma_bf16(d1, x1, bh, idesc, acc);
@@ -213,7 +246,23 @@ __global__ void __launch_bounds__(kThreadsW, 1)
       const uint32_t col_base = (uint32_t)(p.nbuf == 2 ? ab * 2 * n_w + half * n_w : half * 256);
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + col_base;
       if (MODE == 0) {
-        const long long row = t * TM + half * BM + quarter * 32 + lane;
+        const Unit un = unit_at(p, t);
+        const long long row = (long long)un.tile * TM + half * BM + quarter * 32 + lane;
+        if (un.slot >= 0) {
+          // part of K: the raw sums, consecutive rows for each w
+          float* out = p.part + (size_t)un.slot * n_w * TM + half * BM + quarter * 32 + lane;
+          for (int c = 0; c < n_w / 32; ++c) {
+            float v[32];
+            __syncwarp();
+            tmem_ld32(taddr + (uint32_t)(c * 32), v);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) out[(size_t)(c * 32 + j) * TM] = v[j];
+          }
+          fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&tempty[ab]);
+          continue;
+        }
         const bool rv = row < p.Ntil;
         const float yv = rv ? __ldg(p.y + row) : 0.f;
         const float y01 = p.loss == GC_LSQ ? yv : 0.5f * (yv + 1.f);
@@ -263,14 +312,95 @@ __global__ void __launch_bounds__(kThreadsW, 1)
   }
 }
 
-// W (n_w x d fp32) -> planes [2][n_w][d] bf16: hi = bf16(w), lo = bf16(w - hi).
-__global__ void k_split_w(const float* __restrict__ W, long long n, __nv_bfloat16* __restrict__ out) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
-  const float v = W[idx];
-  const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-  out[idx] = hi;
-  out[n + idx] = __float2bfloat16_rn(v - __bfloat162float(hi));
+// R^T planes of the rows whose tiles were split along K: the partial Z in range
+// order, then the residual.  One thread per (w, four rows).
+__global__ void __launch_bounds__(256) k_resid_sum(const float* __restrict__ part, int nsplit, int n_w,
+                                                   int first_tile, int split_tiles, long long Ntil,
+                                                   const float* __restrict__ y, int loss,
+                                                   __nv_bfloat16* __restrict__ Rt) {
+  const long long idx = (long long)blockIdx.x * 256 + threadIdx.x;
+  const int q = (int)(idx % (TM / 4));
+  const long long wt = idx / (TM / 4);
+  const int w = (int)(wt % n_w), t = (int)(wt / n_w);
+  const long long row = (long long)(first_tile + t) * TM + 4 * q;
+  if (t >= split_tiles || row >= Ntil) return;  // N~ is a multiple of 128
+  const float* src = part + ((size_t)t * nsplit * n_w + w) * TM + 4 * q;
+  float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int k = 0; k < nsplit; ++k) {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(src + (size_t)k * n_w * TM));
+    z.x += v.x;
+    z.y += v.y;
+    z.z += v.z;
+    z.w += v.w;
+  }
+  const float zz[4] = {z.x, z.y, z.z, z.w};
+  __nv_bfloat16 hi[4], lo[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const float yv = __ldg(y + row + e);
+    const float y01 = loss == GC_LSQ ? yv : 0.5f * (yv + 1.f);
+    const float r = (loss == GC_LSQ ? zz[e] : 1.f / (1.f + __expf(-zz[e]))) - y01;
+    hi[e] = __float2bfloat16_rn(r);
+    lo[e] = __float2bfloat16_rn(r - __bfloat162float(hi[e]));
+  }
+  auto two = [](__nv_bfloat16 a, __nv_bfloat16 b) {
+    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+  };
+  *reinterpret_cast<uint2*>(Rt + (size_t)w * Ntil + row) = make_uint2(two(hi[0], hi[1]), two(hi[2], hi[3]));
+  *reinterpret_cast<uint2*>(Rt + ((size_t)n_w + w) * Ntil + row) =
+      make_uint2(two(lo[0], lo[1]), two(lo[2], lo[3]));
+}
+
+// How GEMM 1's `tiles` tiles of nkb K blocks are dealt to `sms` CTAs: the tiles
+// past the last whole wave in nsplit K ranges.  The count with the least time by
+// the measured rates: 1.34 us a K block of a 256 x 256 tile, 8 us an epilogue
+// (it is not overlapped), the partials' bytes at 6 TB/s.
+struct Split {
+  int full_tiles, split_tiles, nsplit;
+};
+Split split_of(int tiles, int nkb, int n_w, int sms) {
+  const int full = tiles / sms * sms, rem = tiles - full;
+  if (rem == 0) return {tiles, 0, 1};
+  const double kb_us = 1.34 * n_w / 256, epi_us = 8.0 * n_w / 256;
+  Split best{tiles, 0, 1};
+  double t_best = nkb * kb_us + epi_us;
+  for (int s = 2; s <= 64 && nkb / s >= 8 && (long long)rem * s <= 5LL * sms; ++s) {
+    const int rounds = (rem * s + sms - 1) / sms;
+    const double t = rounds * ((double)nkb / s * kb_us + epi_us) +
+                     5.0 + 2.0 * rem * s * n_w * TM * 4 / 6e6;
+    if (t < t_best) {
+      t_best = t;
+      best = {full, rem, s};
+    }
+  }
+  return best;
+}
+
+// W (n_w x d fp32) -> planes [2][n_w][d] bf16: hi = bf16(w), lo = bf16(w - hi);
+// four elements a thread (n is a multiple of 4, W of 16 bytes when vec).
+__global__ void __launch_bounds__(256) k_split_w(const float* __restrict__ W, long long n, int vec,
+                                                 __nv_bfloat16* __restrict__ out) {
+  const long long i = 4 * ((long long)blockIdx.x * 256 + threadIdx.x);
+  if (i >= n) return;
+  float v[4];
+  if (vec) {
+    const float4 q = __ldg(reinterpret_cast<const float4*>(W + i));
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) v[e] = __ldg(W + i + e);
+  }
+  uint32_t h[2], l[2];
+#pragma unroll
+  for (int e = 0; e < 4; e += 2) {
+    const __nv_bfloat16 ha = __float2bfloat16_rn(v[e]), hb = __float2bfloat16_rn(v[e + 1]);
+    const __nv_bfloat16 la = __float2bfloat16_rn(v[e] - __bfloat162float(ha));
+    const __nv_bfloat16 lb = __float2bfloat16_rn(v[e + 1] - __bfloat162float(hb));
+    h[e / 2] = (uint32_t)__bfloat16_as_ushort(ha) | ((uint32_t)__bfloat16_as_ushort(hb) << 16);
+    l[e / 2] = (uint32_t)__bfloat16_as_ushort(la) | ((uint32_t)__bfloat16_as_ushort(lb) << 16);
+  }
+  *reinterpret_cast<uint2*>(out + i) = make_uint2(h[0], h[1]);
+  *reinterpret_cast<uint2*>(out + n + i) = make_uint2(l[0], l[1]);
 }
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn_w() {
@@ -336,7 +466,9 @@ int launch_w(const CUtensorMap& mA, const CUtensorMap& mB, const WParams& p, cud
 
 size_t gemmw_ws_bytes(int N, int n_c, int d, int n_w) {
   const size_t Ntil = (size_t)N * n_c;
-  return align_up((size_t)2 * n_w * d * 2, 256) + align_up((size_t)2 * n_w * Ntil * 2, 256);
+  const Split sp = split_of((int)((Ntil + TM - 1) / TM), std::max(1, d / BK), n_w, device_sm_count());
+  return align_up((size_t)2 * n_w * d * 2, 256) + align_up((size_t)2 * n_w * Ntil * 2, 256) +
+         align_up((size_t)sp.split_tiles * sp.nsplit * n_w * TM * sizeof(float), 256);
 }
 
 int launch_chunkgrad_batched(const void* X, const float* y, const float* W, int N, int n_c, int d,
@@ -347,7 +479,8 @@ int launch_chunkgrad_batched(const void* X, const float* y, const float* W, int 
   __nv_bfloat16* Rt = ws.take<__nv_bfloat16>((size_t)2 * n_w * Ntil);
   {
     const long long n = (long long)n_w * d;
-    k_split_w<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(W, n, Wp);
+    const int vec = reinterpret_cast<uintptr_t>(W) % 16 == 0;
+    k_split_w<<<(unsigned)((n / 4 + 255) / 256), 256, 0, s>>>(W, n, vec, Wp);
     count_launches(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_check(e, "k_split_w");
@@ -375,10 +508,23 @@ int launch_chunkgrad_batched(const void* X, const float* y, const float* W, int 
   rc = map_planes(&mB, Wp, n_w, d);
   if (rc) return rc;
   p.num_m_tiles = (int)((Ntil + TM - 1) / TM);
-  p.num_tiles = p.num_m_tiles;
   p.nkb = d / BK;
+  const Split sp = split_of(p.num_m_tiles, p.nkb, n_w, device_sm_count());
+  p.full_tiles = sp.full_tiles;
+  p.split_tiles = sp.split_tiles;
+  p.nsplit = sp.nsplit;
+  p.part = ws.take<float>((size_t)sp.split_tiles * sp.nsplit * n_w * TM);
+  p.num_tiles = sp.full_tiles + (long long)sp.split_tiles * sp.nsplit;
   rc = launch_w<0>(mA, mB, p, s);
   if (rc) return rc;
+  if (sp.split_tiles > 0) {
+    const long long threads = (long long)sp.split_tiles * n_w * (TM / 4);
+    k_resid_sum<<<(unsigned)((threads + 255) / 256), 256, 0, s>>>(
+        p.part, sp.nsplit, n_w, sp.full_tiles, sp.split_tiles, Ntil, y, loss, Rt);
+    count_launches(1);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_check(e, "k_resid_sum");
+  }
   // GEMM 2: G_i = X_i^T R_i
   rc = map_2d(&mA, X, Ntil, d, 64);
   if (rc) return rc;

@@ -51,6 +51,31 @@ def test_batched_chunk_grads_match_oracle(gc, N, n_c, d, n_w, loss):
             assert_grad_close(Gn[w, i], ref[i], f"w {w} chunk {i}")
 
 
+@pytest.mark.parametrize("N,n_c,d,n_w,loss", [
+    (3, 128, 4096, 64, 1),       # two tiles in K ranges, the last one half full
+    (2, 64, 1024, 32, 0),        # one tile, the fewest K blocks that are split
+    (2, 19968, 1024, 32, 1),     # a whole wave of tiles and four split ones
+    (6, 192, 1152, 256, 0),      # K blocks that the ranges do not divide
+])
+def test_batched_split_tiles(gc, N, n_c, d, n_w, loss):
+    """GEMM 1's tiles past the last whole wave are cut into K ranges: against the same sums in
+    64 bits.  z is a sum of d products of 2^-17 operands, G one of n_c: 1e-4 of the largest."""
+    X, y, W = _case(N, n_c, d, n_w, loss, 5 + d)
+    Xd, yd, Wd = X.cuda(), y.cuda(), W.cuda()
+    ws = gc.Workspace()
+    G = torch.full((n_w, N, d), float("nan"), device="cuda")
+    for _ in range(2):
+        gc.gc_chunk_grads_batched(Xd, yd, Wd, N, n_c, loss, G=G, ws=ws)
+    gc.gc_status(ws)
+    for i in range(N):
+        x, yy = Xd[i * n_c:(i + 1) * n_c].double(), yd[i * n_c:(i + 1) * n_c, None].double()
+        z = x @ Wd.double().T
+        r = torch.sigmoid(z) - 0.5 * (yy + 1) if loss else z - yy
+        ref = r.T @ x
+        err = (G[:, i].double() - ref).abs().amax(1) / ref.abs().amax(1)
+        assert err.max().item() <= 1e-4
+
+
 def test_batched_matches_single_w_path(gc):
     """Column w of the batched result equals gc_chunk_grads at w (bf16 X)."""
     N, n_c, d, n_w = 8, 256, 1024, 64
