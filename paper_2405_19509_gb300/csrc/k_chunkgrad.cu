@@ -23,7 +23,7 @@ __global__ void __launch_bounds__(256) k_chunkgrad_reduce(const float* __restric
                                                           const double* __restrict__ loss_parts,
                                                           float* __restrict__ G, double* loss_out,
                                                           int N, int nbc, int d, long long bpc,
-                                                          int maxt, int nclusters, long long Ntil) {
+                                                          int maxt, int nloss, long long Ntil) {
   const int i = blockIdx.y;
   const long long qlo = ((long long)i * nbc) / bpc;
   const long long qhi = ((long long)(i + 1) * nbc - 1) / bpc;
@@ -77,9 +77,9 @@ __global__ void __launch_bounds__(256) k_chunkgrad_reduce(const float* __restric
       if (c0 + 256 * u < d) G[(size_t)i * d + c0 + 256 * u] = acc[u];
   }
   if (loss_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32) {
-    // lane l adds clusters l, l + 32, ...; then a fixed xor tree
+    // lane l adds parts l, l + 32, ...; then a fixed xor tree
     double t = 0.0;
-    for (int q = threadIdx.x; q < nclusters; q += 32) t += loss_parts[q];
+    for (int q = threadIdx.x; q < nloss; q += 32) t += loss_parts[q];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     if (threadIdx.x == 0) *loss_out = t / (double)Ntil;
@@ -98,6 +98,8 @@ struct Plan {
   long long bpc;      // batches per cluster
   int nclusters, maxt;
   size_t smem;
+  bool by_warp;       // short rows: the clusters are single warps
+  int blocks;         // of the short-row kernel
 };
 
 cg::Kernel kernel_of(const Plan& p, int x_dtype) {
@@ -228,14 +230,49 @@ Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
   return p;
 }
 
+// Short rows: a block per share of the batches, two blocks an SM when every
+// warp of them has one.
+Plan make_short_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
+  Plan p{};
+  const int esz = x_dtype == GC_BF16 ? 2 : 4;
+  p.V = 16 / esz;
+  const int nv = (d + p.V - 1) / p.V;
+  if (nv > cg::short_vecs(x_dtype == GC_BF16)) return p;
+  p.CL = 1;
+  p.NVT = (nv + 31) / 32;
+  p.NT = cg::kShortThreads;
+  p.RBM = cg::short_rows(p.NVT, x_dtype == GC_BF16);
+  p.aligned = x_aligned && (long long)d * esz % 16 == 0;
+  p.valid = true;
+  p.nbc = (n_c + p.RBM - 1) / p.RBM;
+  p.nbatch = (long long)N * p.nbc;
+  const int warps = p.NT / 32;
+  // Chunks of few batches go to single warps, as a block's would meet after each of
+  // them with most having nothing to add (256 chunks of 4 rows: 5.4 us, by blocks 14);
+  // chunks that give every warp a batch do not, unless a warp's range is whole chunks:
+  // their partials would be as many bytes as the rows (256 chunks of 16 rows of 768
+  // bf16: by warps 13 us, by blocks 7.9).
+  p.by_warp = p.nbc < warps || N >= 2 * warps * device_sm_count();
+  const long long blocks =
+      std::max(1LL, std::min((p.nbatch + warps - 1) / warps, 2LL * device_sm_count()));
+  const long long ranges = p.by_warp ? blocks * warps : blocks;
+  p.bpc = (p.nbatch + ranges - 1) / ranges;
+  p.nclusters = (int)((p.nbatch + p.bpc - 1) / p.bpc);
+  p.blocks = p.by_warp ? (p.nclusters + warps - 1) / warps : p.nclusters;
+  p.maxt = (int)((p.bpc + p.nbc - 1) / p.nbc) + 1;
+  return p;
+}
+
 }  // namespace
 
 size_t chunkgrad_ws_bytes(int N, int n_c, int d, int x_dtype) {
   const Plan p = make_plan(N, n_c, d, x_dtype, true);
   const Plan p2 = make_plan(N, n_c, d, x_dtype, false);
-  const size_t parts = std::max((size_t)p.nclusters * p.maxt, (size_t)p2.nclusters * p2.maxt) *
+  const Plan p3 = make_short_plan(N, n_c, d, x_dtype, true);  // alignment does not change its sizes
+  const size_t parts = std::max({(size_t)p.nclusters * p.maxt, (size_t)p2.nclusters * p2.maxt,
+                                 (size_t)p3.nclusters * p3.maxt}) *
                        (size_t)d * sizeof(float);
-  const size_t lp = (size_t)std::max(p.nclusters, p2.nclusters) * sizeof(double);
+  const size_t lp = (size_t)std::max({p.nclusters, p2.nclusters, p3.nclusters}) * sizeof(double);
   return align_up(parts, 256) + align_up(lp, 256);
 }
 
@@ -243,7 +280,10 @@ int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w,
                      int d, int loss, float* G, double* loss_out, Carve& ws, uint32_t* status,
                      cudaStream_t s) {
   const bool aligned = (reinterpret_cast<uintptr_t>(X) % 16) == 0;
-  const Plan p = make_plan(N, n_c, d, x_dtype, aligned);
+  const bool stall = take_stall(GC_STALL_CHUNK_GRADS);
+  // an armed stall withholds the ring kernel's copies: that kernel then
+  const Plan ps = stall ? Plan{} : make_short_plan(N, n_c, d, x_dtype, aligned);
+  const Plan p = ps.valid ? ps : make_plan(N, n_c, d, x_dtype, aligned);
   if (!p.valid) return fail(GC_ERR_UNSUPPORTED, "chunk-gradient plan does not cover d=%d", d);
   cg::CGArgs a{};
   a.X = X;
@@ -259,10 +299,11 @@ int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w,
   a.bpc = p.bpc;
   a.S = p.S;
   a.maxt = p.maxt;
+  a.by_warp = p.by_warp;
   a.loss = loss;
   a.want_loss = loss_out != nullptr;
   a.spin_limit = wait_limit(cg::kSpinLimit);
-  a.stall = take_stall(GC_STALL_CHUNK_GRADS) ? 1 : 0;
+  a.stall = stall ? 1 : 0;
   a.parts = ws.take<float>((size_t)p.nclusters * p.maxt * d);
   a.loss_parts = ws.take<double>(p.nclusters);
   a.status = status;
@@ -272,10 +313,16 @@ int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w,
       (long long)d * (x_dtype == GC_BF16 ? 2 : 4) <= 16384)
     return fail(GC_ERR_UNSUPPORTED, "chunk of %d rows spans too many row blocks", n_c);
   if (N > 65535) return fail(GC_ERR_UNSUPPORTED, "N=%d exceeds 65535 chunks", N);
-  cg::Kernel kern = kernel_of(p, x_dtype);
-  cudaError_t e = allow_smem(kern, p, x_dtype);
-  if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(chunkgrad smem)");
-  {
+  cudaError_t e = cudaSuccess;
+  if (ps.valid) {
+    cg::pick_short(x_dtype == GC_BF16, p.aligned, p.NVT)<<<p.blocks, p.NT, 0, s>>>(a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return cuda_check(e, "k_chunkgrad_short");
+    count_launches(1);
+  } else {
+    cg::Kernel kern = kernel_of(p, x_dtype);
+    e = allow_smem(kern, p, x_dtype);
+    if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(chunkgrad smem)");
     cudaLaunchAttribute cl_attr[1];
     const cudaLaunchConfig_t cl_cfg = launch_config(p, (unsigned)(p.nclusters * p.CL), cl_attr, s);
     e = cudaLaunchKernelEx(&cl_cfg, kern, a);
@@ -295,7 +342,7 @@ int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w,
   const bool vec = d % 4 == 0 && reinterpret_cast<uintptr_t>(G) % 16 == 0;
   e = cudaLaunchKernelEx(&cfg, vec ? k_chunkgrad_reduce<true> : k_chunkgrad_reduce<false>,
                          (const float*)a.parts, (const double*)a.loss_parts, G, loss_out, N, p.nbc,
-                         d, p.bpc, p.maxt, p.nclusters, a.Ntil);
+                         d, p.bpc, p.maxt, ps.valid ? p.blocks : p.nclusters, a.Ntil);
   if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_chunkgrad_reduce)");
   count_launches(1);
   return GC_OK;

@@ -252,6 +252,7 @@ struct CGArgs {
   long long bpc;  // batches per cluster
   int S;          // stages
   int maxt;       // chunk slots per cluster in `parts`
+  int by_warp;    // short rows: a range of batches is a warp's, not a block's
   int loss;
   int want_loss;
   long long spin_limit;  // clock cycles a wait may take before the kernel gives up
@@ -300,8 +301,8 @@ __device__ __forceinline__ void warp_wait(uint64_t* bar, uint32_t parity, volati
 // shuffles instead of 5 R.  Lane l ends with the warp sum of row l >> (5 - log2 R).
 template <int R>
 __device__ __forceinline__ float warp_sum_rows(const float (&p)[R], int lane) {
-  constexpr int LR = R >= 8 ? 3 : (R >= 4 ? 2 : (R >= 2 ? 1 : 0));
-  static_assert((1 << LR) == R, "rows per batch must be 1, 2, 4 or 8");
+  constexpr int LR = R >= 16 ? 4 : R >= 8 ? 3 : (R >= 4 ? 2 : (R >= 2 ? 1 : 0));
+  static_assert((1 << LR) == R, "rows per batch must be a power of two up to 16");
   float v[R];
 #pragma unroll
   for (int j = 0; j < R; ++j) v[j] = p[j];
@@ -871,6 +872,15 @@ Kernel pick_f32(int CL, int NT, int NVT);
 Kernel pick_f32_ragged(int CL, int NT, int NVT);
 Kernel pick_bf16(int CL, int NT, int NVT);
 Kernel pick_bf16_ragged(int CL, int NT, int NVT);
+// rows of at most 32 K vectors, a warp a row (k_chunkgrad_short.cu); four vectors of
+// bf16 a lane do not fit the registers (d = 1000: 81% of the copy rate against the
+// ring kernel's 75% at 2 GB, but 256 chunks of 16 rows 15 us against 9)
+constexpr int short_vecs(bool bf16) { return bf16 ? 96 : 128; }
+constexpr int kShortThreads = 256;
+// rows a batch: 16 vectors a lane (half of that for bf16, whose unpacked values
+// would not fit the registers)
+constexpr int short_rows(int K, bool bf16) { return (K == 1 ? 16 : (K == 2 ? 8 : 4)) >> (bf16 ? 1 : 0); }
+Kernel pick_short(bool bf16, bool aligned, int K);
 
 }  // namespace cg
 }  // namespace gc

@@ -277,6 +277,28 @@ def test_chunk_grads_ragged_rows_stay_apart(gc):
     assert torch.equal(G[keep], ref[keep]) and not torch.isfinite(G[1]).all()
 
 
+@pytest.mark.parametrize("d,n_c,N,off,dtype", [
+    (1, 33, 5, 0, torch.float32),
+    (127, 129, 3, 1, torch.float32),      # one vector a lane, the last not full
+    (128, 16, 40, 0, torch.float32),      # every lane's vector full
+    (129, 70, 4, 0, torch.float32),       # two vectors a lane
+    (260, 41, 3, 0, torch.float32),       # three
+    (512, 9, 50, 0, torch.float32),       # four, full
+    (511, 1000, 9, 2, torch.float32),     # ranges that end within a chunk
+    (1, 40, 5, 1, torch.bfloat16),        # every second row starts in the middle of a word
+    (255, 65, 3, 1, torch.bfloat16),
+    (256, 30, 4, 1, torch.bfloat16),      # one word more than the lanes hold
+    (257, 1, 70, 0, torch.bfloat16),
+    (700, 21, 5, 2, torch.bfloat16),
+    (767, 600, 9, 3, torch.bfloat16),     # odd rows that fill every word but half of one
+    (768, 10, 30, 0, torch.bfloat16),
+])
+def test_chunk_grads_short_rows(gc, d, n_c, N, off, dtype):
+    """Rows that a warp takes whole: every count of vectors a lane, aligned and from any
+    element, first and last rows of X at a guard of NaN."""
+    test_chunk_grads_ragged(gc, d, n_c, N, off, dtype)
+
+
 def test_chunk_grads_unaligned_X(gc):
     """An X view starting 4 bytes past a 16-byte boundary takes the plain-load path."""
     N, n_c, d = 3, 8, 256
