@@ -48,7 +48,10 @@ constexpr int kWarpsPerBlock = 4;
 // the tau loads of many realizations in flight.
 constexpr int blocks_per_sm(int ell) { return ell <= 3 ? 12 : 8; }
 
-// k-th smallest (1-based, 1 <= k <= n) of n keys in shared memory, by warp.
+// k-th smallest (1-based, 1 <= k <= n) of n keys in shared memory, by warp.  Once
+// a single key is left under the prefix it is the answer (of a few hundred
+// distinct times after about six of the sixteen digits; N = m = 200, delta = 8,
+// ell = 2, theta = 10, 10^5 realizations: 1.92 ms with all sixteen, 1.55 so).
 __device__ unsigned long long warp_select(const unsigned long long* keys, int n, int k, int lane) {
   unsigned long long prefix = 0, mask = 0;
   for (int shift = 60; shift >= 0; shift -= 4) {
@@ -61,12 +64,13 @@ __device__ unsigned long long warp_select(const unsigned long long* keys, int n,
         else hi += 1ull << (8 * (dg - 8));
       }
     }
-    int cum = 0, digit = 15;
+    int cum = 0, digit = 15, left = 0;
     for (int dg = 0; dg < 16; ++dg) {
       const unsigned c = (unsigned)(((dg < 8 ? lo : hi) >> (8 * (dg & 7))) & 255u);
       const int tot = (int)__reduce_add_sync(0xffffffffu, c);
       if (cum + tot >= k) {
         digit = dg;
+        left = tot;
         break;
       }
       cum += tot;
@@ -74,6 +78,14 @@ __device__ unsigned long long warp_select(const unsigned long long* keys, int n,
     k -= cum;
     prefix |= (unsigned long long)digit << shift;
     mask |= 15ull << shift;
+    if (left == 1) {
+      unsigned long long found = 0;
+      for (int t = lane; t < n; t += 32)
+        if ((keys[t] & mask) == prefix) found = keys[t];
+      const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(found >> 32));
+      const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)found);  // 0 in the other lanes
+      return ((unsigned long long)hi << 32) | lo;
+    }
   }
   return prefix;
 }
@@ -106,6 +118,12 @@ __device__ __forceinline__ float approx_float(double x) {
   if (e <= 0) return 0.f;
   if (e >= 255) return 3.0e38f;
   return __uint_as_float(((unsigned)e << 23) | (unsigned)((b >> 29) & 0x7fffffu));
+}
+
+// outside [2^-100, 2^100], or negative (from the sign and the exponent)
+__device__ __forceinline__ bool far_out(double x) {
+  const unsigned e = (unsigned)(dbits(x) >> 52);
+  return e < 1023u - 100u || e > 1023u + 100u;
 }
 
 // The ELL smallest of the values seen (ascending), fp32.
@@ -182,21 +200,20 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
        r += (long long)gridDim.x * kWarpsPerBlock) {
     const double* tr = tau + r * m;
     unsigned long long Tb = 0, TFb = 0;
-    bool wild = theta != 0;
+    bool wild = false;  // a time outside the range in which fp32 decides
     if (theta == 0) {
       // fp32 times (truncated); +inf for a failed worker
       for (int j = lane; j < m; j += 32) {
         const double tj = tr[j];
-        const unsigned e = (unsigned)(dbits(tj) >> 52);  // sign and exponent
         const bool fb = finite_bits(tj);
-        wild |= fb && (e < 1023u - 100u || e > 1023u + 100u);
+        wild |= fb && far_out(tj);
         const float f = fb ? approx_float(tj) : INFINITY;
         tf[j] = make_float2(f, f * (float)s_dj[j]);
       }
       wild = __any_sync(0xffffffffu, wild);
       __syncwarp();
     }
-    if (!wild) {
+    if (theta == 0 && !wild) {
       // every lane's largest ell-th value, its chunk, and its second largest
       float best = -1.f, second = -1.f, bestF = -1.f, secondF = -1.f;
       int bi = 0, biF = 0;
@@ -276,8 +293,11 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
       __syncwarp();
       for (int j = lane; j < m; j += 32) {
         const double tj = tr[j];
-        fin[j] = finite_bits(tj) ? dbits(s_kd[s_dj[j]] * tj) : kInf;
+        const bool fb = finite_bits(tj);
+        wild |= fb && far_out(tj);
+        fin[j] = fb ? dbits(s_kd[s_dj[j]] * tj) : kInf;
       }
+      wild = __any_sync(0xffffffffu, wild);  // for psi below
       __syncwarp();
       // theta = 0: the order statistic is the largest of the N ell values, i.e.
       // the largest ell-th completion time -- a max, no selection needed

@@ -182,6 +182,7 @@ def test_gpu_trigger_close_and_extreme_times(gc, kind, N, delta, ell):
         N = min(N, delta)  # every chunk is held by every worker
     tau[::3, rng.integers(0, tau.shape[1], size=min(delta - 1, 2))] = np.inf
     _gpu_vs_oracle(gc, order, N, ell, 0, tau)
+    _gpu_vs_oracle(gc, order, N, ell, 1 + N * ell // 5, tau)  # psi is decided in fp32 as well
 
 
 @pytest.mark.gpu
