@@ -994,7 +994,7 @@ def logistic_arm(args, rank, world, local_rank):
         m * 4 + m * delta * ell * 8,                                          # psi read; E written
         N * d * 4 + m * L * 4 * 2 + d * 4 * 3,                                # G read; T; ghat; w
     ]
-    srcs = [["k_chunkgrad.cu"], ["k_solve.cu"], ["k_decode_resid.cu"], ["k_solve.cu"],
+    srcs = [["k_chunkgrad.cu", "k_chunkgrad.cuh"], ["k_solve.cu"], ["k_decode_resid.cu"], ["k_solve.cu"],
             ["k_encode.cu"]]
     # the dominant kernel: the longer of the two HBM-bound calls on the
     # critical path (chunk gradients in g1, decode-combine in g2)
