@@ -100,14 +100,15 @@ __global__ void __launch_bounds__(kAnyThreads, 1)
     const long long lo = nitem * blockIdx.x / gridDim.x, hi = nitem * (blockIdx.x + 1) / gridDim.x;
     const bool ahead = rows * kAnyCols <= kAnyPre * kAnyThreads;
     // value u of the tile at column c0 for this thread (VEC four columns): row
-    // r0 + u * rstep, column cl of the tile.  A row ends at L, the last block's at l_last.
-    const int l_last = d - (ELL - 1) * L;
+    // r0 + u * rstep, column cl of the tile.  Block k ends at L or where the row does,
+    // which for d < (ELL - 1) L is before the last block (d = 5, ELL = 4: L = 2, blocks
+    // of 2, 2, 1 and no columns).
     const int r0 = threadIdx.x / (VEC ? kAnyCols / 4 : kAnyCols);
     constexpr int kRstep = kAnyThreads / (VEC ? kAnyCols / 4 : kAnyCols);
     const int cl = VEC ? 4 * (threadIdx.x % (kAnyCols / 4)) : lane;
     auto fetch = [&](int c0, int u, float (&v)[VEC ? 4 : 1]) {
       const int r = r0 + u * kRstep, i = r / ELL, k = r - i * ELL;
-      const bool in = r < rows && c0 + cl < (k == ELL - 1 ? l_last : L);
+      const bool in = r < rows && c0 + cl < min(L, d - k * L);
       const float* src = G + (size_t)i * d + (k * L + c0 + cl);
       if constexpr (VEC) {
         const float4 q = in ? __ldg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);

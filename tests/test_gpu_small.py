@@ -519,6 +519,31 @@ def test_encode_any_order(gc, N, m, delta, ell, npat, L, pad, kind):
         assert torch.equal(T2.nan_to_num(), T.nan_to_num())
 
 
+@pytest.mark.parametrize("ell,d", [(4, 1), (4, 2), (4, 5), (3, 1), (3, 5)])
+def test_encode_any_order_short_rows(gc, ell, d):
+    """k_encode_any on rows so short that blocks before the last one are padded too, or empty,
+    G in a guard of NaN: against the sum in 64 bits (delta * ell fused multiply-adds)."""
+    N = m = 200
+    delta, L = 8, -(-d // ell)
+    npat = -(-(1 << 26) // (m * L * delta * ell))  # k_encode_any's range
+    rng = np.random.default_rng(10 * ell + d)
+    order = np.stack([rng.choice(N, size=delta, replace=False) for _ in range(m)]).astype(np.int32)
+    od = torch.from_numpy(order).cuda()
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    psi = torch.randint(0, delta + 1, (npat, m), generator=gen, device="cuda", dtype=torch.int32)
+    buf = torch.full((16 + N * d + 16,), float("nan"), device="cuda")
+    G = buf[16:16 + N * d].view(N, d)
+    G.copy_(torch.randn(N, d, generator=gen, device="cuda"))
+    E = torch.randn(npat, m, delta, ell, generator=gen, device="cuda", dtype=torch.float64)
+    T = gc.gc_encode_with_coeffs(E, ell, od, N, m, delta, psi, G)
+    B = torch.nn.functional.pad(G, (0, ell * L - d)).view(N, ell, L).double()
+    E.mul_((torch.arange(delta, device="cuda") < psi[:, :, None])[..., None])
+    ref = sum(torch.einsum("bmk,mkc->bmc", E[:, :, p].float().double(), B[od[:, p].long()])
+              for p in range(delta))
+    bound = delta * ell * 2.0 ** -24 * (E.abs().sum((2, 3)).amax() * B.abs().max()).item()
+    assert (T.double() - ref).abs().max().item() <= bound
+
+
 @pytest.mark.parametrize("L,ell,npat,m", [(155648, 2, 1, 40), (155652, 3, 1, 7), (77824, 4, 2, 9),
                                           (155649, 2, 1, 40), (155644, 1, 1, 16)])
 def test_decode_tx_wide(gc, L, ell, npat, m):
