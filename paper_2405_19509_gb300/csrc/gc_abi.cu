@@ -518,7 +518,7 @@ int gc_decode_batch(const double* R, int ell, const int32_t* order, int N, int m
   SolveWs sw = carve_solve(c, N, m, delta, ell, npat);
   __nv_bfloat16* Cs = c.take<__nv_bfloat16>(plan_bytes(N, ell, npat) / sizeof(__nv_bfloat16));
   launch_holders(order, N, m, delta, sw.h, status_of(ws), s);
-  if (!Ghat && decode_policy() == GC_DECODE_AUTO && mse_gram_applies(N, ell, npat) &&
+  if (!Ghat && decode_policy() == GC_DECODE_AUTO && mse_gram_applies(N, ell, npat, d) &&
       mse_patterns_applies(N, ell, sw.bits)) {
     // errors alone: the memo table and the Gram matrix of the chunk blocks
     SolveOut none{};

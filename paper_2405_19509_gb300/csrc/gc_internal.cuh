@@ -193,7 +193,7 @@ inline size_t plan_bytes(int N, int ell, int npat) {
 // scratch of the GEMM side given the planes (G planes, sum of G, MSE partials)
 size_t apply_ws_bytes(int N, int ell, int npat, int d);
 // ---- gradient MSE through the Gram matrix of the chunk blocks (k_mse_gram.cu)
-bool mse_gram_applies(int N, int ell, int npat);
+bool mse_gram_applies(int N, int ell, int npat, int d);
 size_t mse_gram_ws_bytes(int N, int ell, int d);
 struct GramMatrix {
   const float* H;       // (N*ell)^2

@@ -723,7 +723,7 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
   const int policy = decode_policy();
   // errors only, and enough patterns to amortise one Gram matrix of the
   // chunk blocks: each pattern's MSE is a quadratic form in it
-  if (!Ghat && grad_mse && policy == GC_DECODE_AUTO && mse_gram_applies(N, ell, npat))
+  if (!Ghat && grad_mse && policy == GC_DECODE_AUTO && mse_gram_applies(N, ell, npat, d))
     return launch_mse_gram(Cs, Kp, G, N, ell, npat, d, grad_mse, ws, s);
   const int nmt = (int)((M + BM - 1) / BM), nnt = (L + BN - 1) / BN;
   __nv_bfloat16* Gs = ws.take<__nv_bfloat16>((size_t)2 * L * Kp);

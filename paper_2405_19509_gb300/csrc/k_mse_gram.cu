@@ -357,9 +357,14 @@ int gram_splits(int L) {
 
 }  // namespace
 
-bool mse_gram_applies(int N, int ell, int npat) {
+// Taken when the patterns amortise H, and no block but the last is padded: one
+// padded range and one H_last is all that the sums know.  (Rows shorter than
+// (ell - 1) ceil(d / ell) columns, d = 5 with ell = 4 among them, are not worth a
+// Gram matrix: at most ell (ell - 1) columns.)
+bool mse_gram_applies(int N, int ell, int npat, int d) {
   const int K = N * ell;
-  return K <= kGramMaxK && (long long)npat * ell >= 2LL * K;
+  const long long L = ((long long)d + ell - 1) / ell;
+  return K <= kGramMaxK && (long long)npat * ell >= 2LL * K && d >= (ell - 1) * L;
 }
 
 size_t mse_gram_ws_bytes(int N, int ell, int d) {
@@ -378,7 +383,7 @@ GramMatrix launch_gram(const float* G, int N, int ell, int d, bool after_table, 
                        cudaStream_t s) {
   const int K = N * ell;
   const int L = (d + ell - 1) / ell;
-  const int l_last = d - (ell - 1) * L;  // real columns of the last block, 0 < l_last <= L
+  const int l_last = d - (ell - 1) * L;  // real columns of the last block, 0 <= l_last <= L
   const int nt = (K + kGramTile - 1) / kGramTile;
   const int ntri = nt * (nt + 1) / 2;
   const int nsa = gram_splits(l_last);                  // slices of [0, l_last)

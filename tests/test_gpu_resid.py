@@ -444,3 +444,32 @@ def test_errors_only_gram_path(gc, N, delta, ell, d):
         r = O.run_pattern(R, order, psi[b], N, Gref, want_transmit=False)
         assert_mse_close(float(mg[b]), r.grad_mse, floor, f"gram b={b}")
         assert_mse_close(float(mg[b]), float(mf[b]), floor, f"gram vs decode b={b}")
+
+
+@pytest.mark.parametrize("N,delta,ell,d", [(10, 4, 4, 5), (10, 4, 4, 6), (7, 3, 3, 1), (12, 8, 8, 20),
+                                           (9, 4, 4, 1)])
+def test_errors_only_short_rows(gc, N, delta, ell, d):
+    """Errors only of rows so short that blocks before the last one are padded (d = 5, ell = 4:
+    blocks of 2, 2, 1 and no columns) or the last one is empty (d = 6), with G in a guard of NaN:
+    the two error calls against the oracle."""
+    m, npat = N, 2 * N + 7
+    rng = np.random.default_rng(7 * N + d)
+    order = O.cyclic_order(N, m, delta)
+    R = rng.standard_normal((ell, m))
+    psi = rng.integers(0, delta + 1, size=(npat, m)).astype(np.int32)
+    psi[0], psi[1] = delta, 0
+    G = rng.standard_normal((N, d)).astype(np.float32)
+    Gref = G.astype(np.float64)
+    gsum = Gref.sum(axis=0)
+    floor = 1e-8 * float(gsum @ gsum) / d
+    Rd, od, pd = dev_tensors(R, order, psi)
+    buf = torch.full((64 + N * d + 64,), float("nan"), device="cuda")
+    Gd = buf[64:64 + N * d].view(N, d)
+    Gd.copy_(torch.from_numpy(G))
+    ms = gc.gc_mse(Rd, ell, od, N, m, delta, pd, Gd)["grad_mse"]
+    plan = gc.gc_decode_plan(Rd, ell, od, N, m, delta, pd)["plan"]
+    ma = gc.gc_decode_apply(plan, ell, N, npat, Gd, Ghat=False)["grad_mse"]
+    for b in range(npat):
+        r = O.run_pattern(R, order, psi[b], N, Gref, want_transmit=False)
+        assert_mse_close(ms[b].item(), r.grad_mse, floor, f"gc_mse b={b}")
+        assert_mse_close(ma[b].item(), r.grad_mse, floor, f"gc_decode_apply b={b}")
