@@ -725,6 +725,9 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
   // chunk blocks: each pattern's MSE is a quadratic form in it
   if (!Ghat && grad_mse && policy == GC_DECODE_AUTO && mse_gram_applies(N, ell, npat, d))
     return launch_mse_gram(Cs, Kp, G, N, ell, npat, d, grad_mse, ws, s);
+  // the scan and the gathering read the plan's rows in 8- and 16-byte pieces
+  if (reinterpret_cast<uintptr_t>(Cs) % 16 != 0)
+    return fail(GC_ERR_WORKSPACE, "plan must be 16-byte aligned");
   const int nmt = (int)((M + BM - 1) / BM), nnt = (L + BN - 1) / BN;
   __nv_bfloat16* Gs = ws.take<__nv_bfloat16>((size_t)2 * L * Kp);
   float* gsum = ws.take<float>((size_t)d);

@@ -121,6 +121,11 @@ def test_device_entry_validation_before_launch():
                              ctypes.c_void_p(4096), need - 1, None) == -6
     assert L.gc_decode_batch(fake, 2, fake, 6, 6, 3, fake, 4, fake, 64, fake, None, None, None,
                              ctypes.c_void_p(4096 + 8), need, None) == -6
+    # a plan on no 16-byte boundary: its rows are read in 16-byte pieces
+    aw = L.gc_decode_apply_workspace(6, 2, 4, 64)
+    assert L.gc_decode_apply(ctypes.c_void_p(4096 + 8), 2, 6, 4, fake, 64, fake, None, fake, aw,
+                             None) == -6
+    assert "plan" in gc.gc_last_error()
     # neither output requested
     assert L.gc_decode_batch(fake, 2, fake, 6, 6, 3, fake, 4, fake, 64, None, None, None, None,
                              ctypes.c_void_p(4096), need, None) == -1
