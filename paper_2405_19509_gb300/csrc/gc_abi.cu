@@ -140,6 +140,9 @@ int gc_chunk_grads_batched(const void* X, const float* y, const float* W, int N,
   if (reinterpret_cast<uintptr_t>(X) % 16 != 0) return fail(GC_ERR_ARG, "X must be 16-byte aligned");
   if (!ws || ws_bytes < gc_chunk_grads_batched_workspace(N, n_c, d, n_w))
     return fail(GC_ERR_WORKSPACE, "workspace too small");
+  // the operand planes and partial sums are written and read in 8- and 16-byte pieces
+  if (reinterpret_cast<uintptr_t>(ws) % 16 != 0)
+    return fail(GC_ERR_WORKSPACE, "workspace must be 16-byte aligned");
   Carve c(ws);
   return launch_chunkgrad_batched(X, y, W, N, n_c, d, n_w, loss, G, c, status_of(ws),
                                   as_stream(stream));

@@ -164,7 +164,12 @@ def test_batched_chunk_grads_validation():
     assert L.gc_chunk_grads_batched(nul, nul, nul, 2, 128, 200, 32, 0, nul, nul, 0, nul) == -3
     assert L.gc_chunk_grads_batched(nul, nul, nul, 2, 100, 256, 32, 0, nul, nul, 0, nul) == -3
     assert L.gc_chunk_grads_batched(nul, nul, nul, 2, 128, 256, 32, 0, nul, nul, 0, nul) == -1
-    assert L.gc_chunk_grads_batched_workspace(2, 128, 256, 32) > 256
+    need = L.gc_chunk_grads_batched_workspace(2, 128, 256, 32)
+    assert need > 256
+    # a workspace on no 16-byte boundary: its planes are written in 8-byte pieces
+    q = ctypes.c_void_p(4096)
+    assert L.gc_chunk_grads_batched(q, q, q, 2, 128, 256, 32, 0, q, ctypes.c_void_p(4096 + 4), need,
+                                    nul) == -6
 
 
 def test_binding_without_library_raises(tmp_path):
