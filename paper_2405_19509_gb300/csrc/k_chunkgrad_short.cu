@@ -179,7 +179,10 @@ __global__ void __launch_bounds__(32 * kShortWarps, 2) k_chunkgrad_short(CGArgs 
         pd[r] = p2.x + p2.y;
       }
       const float z = warp_sum_rows<RB>(pd, lane);
-      const float mine = a.loss == GC_LSQ ? z - yv : 1.f / (1.f + __expf(-z)) - 0.5f * (yv + 1.f);
+      // a row past the chunk's end is zeros, whose dot with an infinite w is NaN: its
+      // residual is zero whatever the dot
+      const float mine = my >= nr ? 0.f
+                         : a.loss == GC_LSQ ? z - yv : 1.f / (1.f + __expf(-z)) - 0.5f * (yv + 1.f);
       if (a.want_loss && my < nr && (lane & ((1 << kShift) - 1)) == 0) {
         if (a.loss == GC_LSQ) {
           const float e = z - yv;

@@ -299,6 +299,32 @@ def test_chunk_grads_short_rows(gc, d, n_c, N, off, dtype):
     test_chunk_grads_ragged(gc, d, n_c, N, off, dtype)
 
 
+@pytest.mark.parametrize("d,n_c,dtype", [(64, 20, torch.float32), (301, 12, torch.float32),
+                                         (500, 12, torch.float32), (255, 9, torch.bfloat16),
+                                         (504, 28, torch.bfloat16), (1021, 6, torch.float32)])
+def test_chunk_grads_infinite_w(gc, d, n_c, dtype):
+    """An infinite parameter under the logistic loss saturates every row (residuals of 0 or 1, so
+    the gradients are finite); the zeros that stand for rows past a chunk's last one add nothing.
+    An infinite feature reaches its own chunk alone."""
+    N = 5
+    gen = torch.Generator(device="cuda").manual_seed(d)
+    X = torch.randn(N * n_c, d, generator=gen, device="cuda").to(dtype)
+    X[X == 0] = 1
+    y = torch.where(torch.rand(N * n_c, generator=gen, device="cuda") < 0.5, 1.0, -1.0)
+    w = torch.randn(d, generator=gen, device="cuda")
+    w[d // 2] = float("inf")
+    G = gc.gc_chunk_grads(X, y, w, N, n_c, 1)
+    r = (X[:, d // 2].float() > 0).double() - 0.5 * (y + 1).double()
+    ref = (r[:, None] * X.double()).view(N, n_c, d).sum(1)
+    assert_grad_close(to_np(G), to_np(ref))
+    w[d // 2] = 0.5
+    G = gc.gc_chunk_grads(X, y, w, N, n_c, 0)
+    X[n_c + 1, d - 1] = float("inf")
+    G1 = gc.gc_chunk_grads(X, y, w, N, n_c, 0)
+    keep = [0, 2, 3, 4]
+    assert torch.equal(G1[keep], G[keep]) and not torch.isfinite(G1[1]).all()
+
+
 def test_chunk_grads_unaligned_X(gc):
     """An X view starting 4 bytes past a 16-byte boundary takes the plain-load path."""
     N, n_c, d = 3, 8, 256
