@@ -159,50 +159,69 @@ __global__ void __launch_bounds__(1024, 1) k_mse_patterns(
     if (n > 0) {
       __syncwarp();
       const int nz = n * ELL;
-      for (int t0 = 0; t0 < nz; t0 += 32) {
-        // lane's own entry e' = t0 + lane (past the end: zero values)
-        const bool in = t0 + lane < nz;
-        const uint32_t* own = list + (size_t)(in ? t0 + lane : 0) * EW;
-        const uint32_t a2 = own[ELL] >> 16;
-        float u[ELL];
+      // the rows' forms, over the lanes; SKIP leaves the entries that are zero in a row out of it
+      auto forms = [&](auto skip) {
+        constexpr bool SKIP = decltype(skip)::value;
 #pragma unroll
-        for (int k = 0; k < ELL; ++k) u[k] = 0.f;
-#pragma unroll 4
-        for (int e = 0; e < nz; ++e) {
-          uint32_t w[EW];
-          if constexpr (EW == 2) {
-            const uint2 x = *reinterpret_cast<const uint2*>(list + (size_t)e * EW);
-            w[0] = x.x;
-            w[1] = x.y;
-          } else {
+        for (int k = 0; k < ELL; ++k) q[k] = 0.f;
+        for (int t0 = 0; t0 < nz; t0 += 32) {
+          // lane's own entry e' = t0 + lane (past the end: zero values)
+          const bool in = t0 + lane < nz;
+          const uint32_t* own = list + (size_t)(in ? t0 + lane : 0) * EW;
+          const uint32_t a2 = own[ELL] >> 16;
+          float u[ELL];
 #pragma unroll
-            for (int k = 0; k < EW; k += 4) {
-              if (k <= ELL) {
-                const uint4 x = *reinterpret_cast<const uint4*>(list + (size_t)e * EW + k);
-                w[k] = x.x;
-                w[k + 1] = x.y;
-                w[k + 2] = x.z;
-                w[k + 3] = x.w;
+          for (int k = 0; k < ELL; ++k) u[k] = 0.f;
+#pragma unroll (SKIP ? 1 : 4)
+          for (int e = 0; e < nz; ++e) {
+            uint32_t w[EW];
+            if constexpr (EW == 2) {
+              const uint2 x = *reinterpret_cast<const uint2*>(list + (size_t)e * EW);
+              w[0] = x.x;
+              w[1] = x.y;
+            } else {
+#pragma unroll
+              for (int k = 0; k < EW; k += 4) {
+                if (k <= ELL) {
+                  const uint4 x = *reinterpret_cast<const uint4*>(list + (size_t)e * EW + k);
+                  w[k] = x.x;
+                  w[k + 1] = x.y;
+                  w[k + 2] = x.z;
+                  w[k + 3] = x.w;
+                }
               }
             }
+            const uint32_t at = (w[ELL] & 0xffffu) + a2;
+            const float hv = HS ? s_h[at] : __ldg(H + at);
+#pragma unroll
+            for (int k = 0; k < ELL; ++k) {
+              const float v = __uint_as_float(w[k]);
+              const float f = fmaf(v, PAD && k == ELL - 1 ? __ldg(H_last + at) : hv, u[k]);
+              u[k] = SKIP && v == 0.f ? u[k] : f;
+            }
           }
-          const uint32_t at = (w[ELL] & 0xffffu) + a2;
-          const float hv = HS ? s_h[at] : __ldg(H + at);
+          if (in) {
 #pragma unroll
-          for (int k = 0; k < ELL; ++k)
-            u[k] = fmaf(__uint_as_float(w[k]), PAD && k == ELL - 1 ? __ldg(H_last + at) : hv, u[k]);
+            for (int k = 0; k < ELL; ++k) {
+              const float v = __uint_as_float(own[k]);
+              q[k] = SKIP && v == 0.f ? q[k] : fmaf(v, u[k], q[k]);
+            }
+          }
         }
-        if (in) {
+        // each row over the lanes
 #pragma unroll
-          for (int k = 0; k < ELL; ++k) q[k] = fmaf(__uint_as_float(own[k]), u[k], q[k]);
+        for (int k = 0; k < ELL; ++k) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) q[k] += __shfl_xor_sync(0xffffffffu, q[k], o);
         }
-      }
-      // each row over the lanes
+      };
+      forms(std::false_type{});
+      // the list is that of all rows; an entry that is zero in one of them must not
+      // meet an infinite value of H there
+      bool finite = true;
 #pragma unroll
-      for (int k = 0; k < ELL; ++k) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) q[k] += __shfl_xor_sync(0xffffffffu, q[k], o);
-      }
+      for (int k = 0; k < ELL; ++k) finite &= fabsf(q[k]) <= 3.4028235e38f;
+      if (ELL > 1 && !finite) forms(std::true_type{});  // warp-uniform
       def = (int)__reduce_add_sync(0xffffffffu, (unsigned)def);
       __syncwarp();  // the list is rewritten by the next pattern
     }

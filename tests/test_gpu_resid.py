@@ -473,3 +473,37 @@ def test_errors_only_short_rows(gc, N, delta, ell, d):
         r = O.run_pattern(R, order, psi[b], N, Gref, want_transmit=False)
         assert_mse_close(ms[b].item(), r.grad_mse, floor, f"gc_mse b={b}")
         assert_mse_close(ma[b].item(), r.grad_mse, floor, f"gc_decode_apply b={b}")
+
+
+@pytest.mark.parametrize("N,delta,ell,L,pad", [(16, 4, 2, 40, 0), (40, 5, 3, 33, 2), (80, 6, 3, 20, 1)])
+def test_errors_from_counts_infinite_feature(gc, N, delta, ell, L, pad):
+    """An infinite value in one block of one chunk makes infinite (or NaN, where infinities of
+    both signs meet) the errors whose decode has a non-zero departure on that block, and no
+    other: with coefficients on the axes, so that incomplete chunks have exactly decoded blocks."""
+    m, npat, d = N, 400, ell * L - pad
+    rng = np.random.default_rng(N + ell)
+    order = O.cyclic_order(N, m, delta)
+    R = np.zeros((ell, m))
+    R[rng.integers(0, ell, size=m), np.arange(m)] = 1.0
+    R[:, ::4] = rng.standard_normal(R[:, ::4].shape)
+    i = N // 2
+    R[:, i] = np.eye(ell)[1]  # worker i starts with chunk i: its copy alone gives block 1
+    psi = rng.binomial(delta, rng.uniform(0.05, 0.6, size=(npat, 1)), size=(npat, m)).astype(np.int32)
+    psi[0], psi[1] = delta, 0
+    psi[0, 1::4] = 0
+    G = rng.standard_normal((N, d)).astype(np.float32)
+    G[:, L + 3] = 1 + np.abs(G[:, L + 3])
+    Gf = G.copy()
+    G[i, L + 3] = np.inf
+    Rd, od, pd = dev_tensors(R, order, psi)
+    both = [gc.gc_mse(Rd, ell, od, N, m, delta, pd, torch.from_numpy(g).cuda())["grad_mse"]
+            for g in (G, Gf)]
+    got, fin = to_np(both[0]), to_np(both[1])
+    D = _copies(order, psi, N)[:, i]
+    C = to_np(gc.gc_find_encoding_coeff(Rd, ell, od, N, m, delta, pd, E=False, coef_err=False,
+                                        est=False)["C"]).reshape(npat, ell, N, ell)
+    hit = np.array([np.any(C[b, :, i, 1] != np.eye(ell)[:, 1]) for b in range(npat)])
+    assert got[1] == np.inf                              # no chunk finished: the whole sum is missing
+    assert np.array_equal(np.isfinite(got), ~hit)
+    assert (~hit & (D < ell)).any() and hit.any()        # incomplete chunks that decode the block
+    assert np.array_equal(got[~hit], fin[~hit])
