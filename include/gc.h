@@ -195,7 +195,8 @@ int gc_chunk_ordering(const uint8_t* A_h, int N, int m, int delta, int32_t* orde
  *        matrix of w_w, the layout the decode entry points take).
  *   Limits: 32 <= n_w <= 256, n_w % 32 == 0; d % 128 == 0; n_c % 64 == 0;
  *   N * n_c % 128 == 0.  No loss output.
- * Workspace: gc_chunk_grads_batched_workspace(N, n_c, d, n_w) bytes.
+ * Workspace: gc_chunk_grads_batched_workspace(N, n_c, d, n_w) bytes, 16-byte aligned;
+ * the size depends on the current device's number of SMs, so ask with that device current.
  */
 size_t gc_chunk_grads_batched_workspace(int N, int n_c, int d, int n_w);
 int gc_chunk_grads_batched(const void* X, const float* y, const float* W, int N, int n_c, int d,
@@ -240,7 +241,8 @@ int gc_trigger_times(const int32_t* order, int N, int m, int delta, const double
  *          (GC_LSQ, y01 = y) or the logistic sigmoid (GC_LOGISTIC,
  *          y01 = (y + 1) / 2).  Un-normalised sums, as in Sec. I.
  * loss_out NULL or one device double: L = (1/N~) sum_i l(x_i, y_i, w).
- * Requires d >= 1, n_c >= 1, N >= 1.  One pass over X.
+ * Requires d >= 1, n_c >= 1, N >= 1.  One pass over X.  The workspace size depends on the
+ * current device's number of SMs.
  */
 size_t gc_chunk_grads_workspace(int N, int n_c, int d, int x_dtype);
 int gc_chunk_grads(const void* X, int x_dtype, const float* y, const float* w, int N, int n_c,

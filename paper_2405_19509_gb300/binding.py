@@ -121,9 +121,9 @@ def _bytes(query, *sizes) -> int:
 
 
 @functools.lru_cache(maxsize=1024)
-def _chunk_grads_bytes(N, n_c, d, x_dtype, device) -> int:
-    """... and of the number of SMs of the device."""
-    return int(lib.gc_chunk_grads_workspace(N, n_c, d, x_dtype))
+def _device_bytes(device, query, *sizes) -> int:
+    """... of the sizes and of the number of SMs of the current device."""
+    return int(getattr(lib, query)(*sizes))
 
 
 def _dev(t, dtype, name, shape=None):
@@ -236,7 +236,8 @@ def gc_chunk_grads_batched(X, y, W, N: int, n_c: int, loss: int, G=None,
         raise TypeError("X must be bfloat16")
     if G is None:
         G = torch.empty(n_w, N, d, dtype=torch.float32, device=X.device)
-    ws, (wp, wn) = _ws(ws, _bytes("gc_chunk_grads_batched_workspace", N, n_c, d, n_w), X.device)
+    ws, (wp, wn) = _ws(ws, _device_bytes(torch.cuda.current_device(), "gc_chunk_grads_batched_workspace",
+                                        N, n_c, d, n_w), X.device)
     _check(lib.gc_chunk_grads_batched(
         _dev(X, torch.bfloat16, "X", (N * n_c, d)), _dev(y, torch.float32, "y", (N * n_c,)),
         _dev(W, torch.float32, "W", (n_w, d)), N, n_c, d, n_w, loss,
@@ -260,7 +261,8 @@ def gc_chunk_grads(X, y, w, N: int, n_c: int, loss: int, G=None, loss_out=None,
         raise ValueError("X must have N * n_c rows")
     if G is None:
         G = torch.empty(N, d, dtype=torch.float32, device=X.device)
-    ws, (wp, wn) = _ws(ws, _chunk_grads_bytes(N, n_c, d, x_dtype, torch.cuda.current_device()), X.device)
+    ws, (wp, wn) = _ws(ws, _device_bytes(torch.cuda.current_device(), "gc_chunk_grads_workspace",
+                                        N, n_c, d, x_dtype), X.device)
     _check(lib.gc_chunk_grads(_dev(X, X.dtype, "X"), x_dtype, _dev(y, torch.float32, "y", (N * n_c,)),
                               _dev(w, torch.float32, "w", (d,)), N, n_c, d, loss,
                               _dev(G, torch.float32, "G", (N, d)),

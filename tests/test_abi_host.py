@@ -172,6 +172,36 @@ def test_batched_chunk_grads_validation():
                                     nul) == -6
 
 
+@pytest.mark.parametrize("call", ["gc_chunk_grads", "gc_chunk_grads_batched"])
+def test_workspace_size_is_asked_per_device(monkeypatch, call):
+    """The chunk-gradient workspaces depend on the device's SM count: with another device current
+    the library is asked again."""
+    gc = _lib()
+    import torch
+    from paper_2405_19509_gb300 import binding
+    sms, asked = {0: 152, 1: 132}, []
+    device = [0]
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: device[0])
+    monkeypatch.setattr(binding.lib, call + "_workspace", lambda *a: 1000 * sms[device[0]])
+
+    class Stop(Exception):
+        pass
+
+    class Ws:
+        def get(self, nbytes):
+            asked.append(nbytes)
+            raise Stop
+    X = torch.zeros(2 * 64, 128, dtype=torch.bfloat16)
+    y, w = torch.zeros(128), torch.zeros(128) if call == "gc_chunk_grads" else torch.zeros(32, 128)
+    try:
+        for device[0] in (0, 1, 0):
+            with pytest.raises(Stop):
+                getattr(gc, call)(X, y, w, 2, 64, 0, G=torch.zeros(1), ws=Ws())
+    finally:
+        binding._device_bytes.cache_clear()  # of these made-up sizes
+    assert asked == [152000, 132000, 152000]
+
+
 def test_binding_without_library_raises(tmp_path):
     """The package has no CPU fallback: a copy of its Python files without
     libgc.so beside them refuses to import, naming the missing library."""
