@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "gc.h"
 
 namespace gc {
@@ -58,6 +60,24 @@ struct Carve {
 };
 
 int device_sm_count();
+
+// A kernel's opt-in to `bytes` of dynamic shared memory, always the same number: once per
+// device, whose attribute it is.  Threads may meet here; at worst both set it.
+struct SmemOptIn {
+  std::atomic<uint64_t> devices{0};  // bit = device ordinal
+  template <typename Kern>
+  cudaError_t operator()(Kern kern, size_t bytes) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
+    if (devices.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) devices.fetch_or(bit, std::memory_order_release);
+    return e;
+  }
+};
+constexpr size_t kSmemMax = 227 * 1024;  // a block's, static and dynamic
 
 // Launch accounting for gc_kernel_launches().
 void count_launches(int n);

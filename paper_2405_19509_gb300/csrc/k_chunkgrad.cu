@@ -116,15 +116,10 @@ int shape_index(const Plan& p, int x_dtype) {
   return ((((x_dtype == GC_BF16) * 2 + p.aligned) * 4 + ci) * 3 + ni) * 8 + (p.NVT - 1);
 }
 
-// Allow the kernel its dynamic shared memory (largest opt-in so far per shape).
+// Allow the kernel its dynamic shared memory (all there is: a shape's depends on the ring).
 cudaError_t allow_smem(cg::Kernel kern, const Plan& p, int x_dtype) {
-  static std::atomic<int> smem_set[kShapes];
-  std::atomic<int>& set = smem_set[shape_index(p, x_dtype)];
-  if ((int)p.smem <= set.load(std::memory_order_relaxed)) return cudaSuccess;
-  const cudaError_t e =
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-  if (e == cudaSuccess) set.store((int)p.smem, std::memory_order_relaxed);
-  return e;
+  static SmemOptIn allow[kShapes];
+  return allow[shape_index(p, x_dtype)](kern, kSmemMax);
 }
 
 cudaLaunchConfig_t launch_config(const Plan& p, unsigned grid, cudaLaunchAttribute* attr,

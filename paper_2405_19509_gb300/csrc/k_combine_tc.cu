@@ -663,13 +663,9 @@ template <int STAGES, int EPI, int NKBR, bool OUT>
 int launch_tc(int grid, const CUtensorMap& mA, const CUtensorMap& mB, const tc::Params& p,
               cudaStream_t s) {
   using Sh = tc::Shape<STAGES, EPI, NKBR, OUT>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(tc::k_combine_tc<STAGES, EPI, NKBR, OUT>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Sh::SMEM);
-    if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_combine_tc)");
-    attr_set = true;
-  }
+  static SmemOptIn allow;
+  cudaError_t e = allow(tc::k_combine_tc<STAGES, EPI, NKBR, OUT>, Sh::SMEM);
+  if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_combine_tc)");
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(Sh::THREADS);
@@ -680,7 +676,7 @@ int launch_tc(int grid, const CUtensorMap& mA, const CUtensorMap& mB, const tc::
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, tc::k_combine_tc<STAGES, EPI, NKBR, OUT>, mA, mB, p);
+  e = cudaLaunchKernelEx(&cfg, tc::k_combine_tc<STAGES, EPI, NKBR, OUT>, mA, mB, p);
   if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_combine_tc)");
   count_launches(1);
   return cuda_check(cudaGetLastError(), "k_combine_tc");

@@ -346,13 +346,10 @@ static int launch_enc_t(dim3 grid, size_t smem, const double* E, const int32_t* 
                         const int32_t* psi, int N, int m, int delta, int ell, int npat,
                         const float* G, int d, int L, int J, int vec, int any_next, float* T,
                         cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_encode<DR, V, KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)((kEncSmemFloats + kEncStages * kEncThreads * V) * sizeof(float)));
-    if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_encode)");
-    attr = true;
-  }
+  static SmemOptIn allow;
+  const cudaError_t e =
+      allow(k_encode<DR, V, KB>, (kEncSmemFloats + kEncStages * kEncThreads * V) * sizeof(float));
+  if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_encode)");
   k_encode<DR, V, KB><<<grid, kEncThreads, smem, s>>>(E, order, psi, N, m, delta, ell, npat, G, d, L, J, vec,
                                                      any_next, T);
   return GC_OK;
@@ -618,14 +615,9 @@ static cudaError_t launch_live_t(unsigned blocks, size_t smem, const double* E, 
                                  const int32_t* order, const int32_t* psi, int N, int m, int delta,
                                  const float* G, int d, int L, float scale, float* w, float* T,
                                  float* ghat, cudaStream_t s) {
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(k_live_step<ELL, SG>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)kLiveSmemMax);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn allow;
+  const cudaError_t e = allow(k_live_step<ELL, SG>, kLiveSmemMax);
+  if (e != cudaSuccess) return e;
   k_live_step<ELL, SG><<<blocks, kLiveThreads, smem, s>>>(E, R, order, psi, N, m, delta, G, d, L,
                                                           scale, w, T, ghat);
   return cudaSuccess;

@@ -296,13 +296,9 @@ int launch_any_t(size_t smem, const double* E, const int32_t* order, const int32
                  int m, int delta, int npat, const float* G, int d, int L, int J, float* T,
                  cudaStream_t s) {
   auto kern = k_encode_any<PB, ELL, VEC>;
-  static bool attr_set = false;
-  if (!attr_set) {
-    const cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kEncodeAnySmem);
-    if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_encode_any)");
-    attr_set = true;
-  }
+  static SmemOptIn allow;
+  cudaError_t e = allow(kern, kEncodeAnySmem);
+  if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_encode_any)");
   const long long items = (long long)((L + kAnyCols - 1) / kAnyCols) * ((npat + PB - 1) / PB);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)std::min<long long>(items, device_sm_count()));
@@ -314,8 +310,7 @@ int launch_any_t(size_t smem, const double* E, const int32_t* order, const int32
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e =
-      cudaLaunchKernelEx(&cfg, kern, E, order, psi, N, m, delta, npat, G, d, L, J, T);
+  e = cudaLaunchKernelEx(&cfg, kern, E, order, psi, N, m, delta, npat, G, d, L, J, T);
   if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_encode_any)");
   count_launches(1);
   return GC_OK;

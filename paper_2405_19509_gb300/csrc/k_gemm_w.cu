@@ -449,13 +449,9 @@ int map_planes(CUtensorMap* map, const void* base, int rows, long long cols) {
 template <int MODE>
 int launch_w(const CUtensorMap& mA, const CUtensorMap& mB, const WParams& p, cudaStream_t s) {
   const size_t smem = (size_t)p.stages * p.stage_bytes + 1024 + 256;
-  static size_t smem_set = 0;
-  if (smem > smem_set) {
-    cudaError_t e = cudaFuncSetAttribute(k_gemm_w<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_gemm_w)");
-    smem_set = smem;
-  }
+  static SmemOptIn allow;
+  const cudaError_t e = allow(k_gemm_w<MODE>, kSmemMax);
+  if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_gemm_w)");
   const int grid = (int)std::min<long long>(p.num_tiles, device_sm_count());
   k_gemm_w<MODE><<<grid, kThreadsW, smem, s>>>(mA, mB, p);
   count_launches(1);

@@ -335,14 +335,11 @@ cudaError_t launch_mse_gram_t(int blocks, size_t smem, const __nv_bfloat16* Cs, 
                               int ell, int npat, const float* H, const float* H_last, double inv_d,
                               double* grad_mse, cudaStream_t s) {
   if (HS) {
-    static bool attr = false;
-    if (!attr) {
-      const cudaError_t e = cudaFuncSetAttribute(
-          k_mse_gram<HS, KW, W, PAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-          (int)(((size_t)kHSmemMaxK * kHSmemMaxK + W * 2 * kHSmemMaxK) * sizeof(float)));
-      if (e != cudaSuccess) return e;
-      attr = true;
-    }
+    static SmemOptIn allow;
+    const cudaError_t e =
+        allow(k_mse_gram<HS, KW, W, PAD>,
+              ((size_t)kHSmemMaxK * kHSmemMaxK + W * 2 * kHSmemMaxK) * sizeof(float));
+    if (e != cudaSuccess) return e;
   }
   k_mse_gram<HS, KW, W, PAD><<<blocks, W * 32, smem, s>>>(Cs, Kp, N, ell, npat, H, H_last,
                                                            inv_d, grad_mse);

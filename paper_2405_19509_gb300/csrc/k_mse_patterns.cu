@@ -267,12 +267,9 @@ cudaError_t launch_t(const Shape& sh, int blocks, const double* R, const int32_t
                      const float* H_last, double inv_d, double* coef_err, double* est,
                      double* grad_mse, uint32_t* status, cudaStream_t s) {
   auto kern = k_mse_patterns<ELL, CPL, HS, PAD>;
-  static bool attr = false;
-  if (!attr) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
-    if (e != cudaSuccess) return e;
-    attr = true;
-  }
+  static SmemOptIn allow;
+  const cudaError_t e = allow(kern, 220 * 1024);
+  if (e != cudaSuccess) return e;
   kern<<<blocks, sh.warps * 32, sh.smem, s>>>(R, psi, h, N, m, delta, npat, tb, H, H_last, inv_d,
                                               coef_err, est, grad_mse, status);
   return cudaSuccess;

@@ -202,6 +202,43 @@ def test_workspace_size_is_asked_per_device(monkeypatch, call):
     assert asked == [152000, 132000, 152000]
 
 
+def test_shared_memory_opt_in_per_device(tmp_path):
+    """The opt-in to large shared memory is an attribute of the device: every device gets its own,
+    once (against a stand-in for the two runtime calls)."""
+    import shutil
+    import subprocess
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    if not (shutil.which("g++") and os.path.exists(os.path.join(cuda, "cuda_runtime.h"))):
+        pytest.skip("no g++ or no CUDA headers")
+    src = tmp_path / "t.cpp"
+    src.write_text("""
+#include <cstdio>
+#include "gc_internal.cuh"
+static int dev = 0, calls = 0;
+extern "C" cudaError_t CUDARTAPI cudaGetDevice(int* d) { *d = dev; return cudaSuccess; }
+extern "C" cudaError_t CUDARTAPI cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) {
+  ++calls;
+  return cudaSuccess;
+}
+int main() {
+  static gc::SmemOptIn allow;
+  const void* kernel = nullptr;
+  for (int d : {0, 0, 1, 1, 0, 70, 70}) {
+    dev = d;
+    if (allow(kernel, 4096) != cudaSuccess) return 1;
+    printf("%d ", calls);
+  }
+}
+""")
+    exe = tmp_path / "t"
+    subprocess.run(["g++", "-std=c++17", "-w", "-I", cuda, "-I", os.path.join(ROOT, "include"), "-I",
+                    os.path.join(ROOT, "paper_2405_19509_gb300", "csrc"), str(src), "-o", str(exe)],
+                   check=True, timeout=300)
+    out = subprocess.run([str(exe)], check=True, capture_output=True, text=True, timeout=60).stdout
+    assert out.split() == ["1", "1", "2", "2", "2", "3", "4"]  # 70: past the ones remembered
+
+
 def test_binding_without_library_raises(tmp_path):
     """The package has no CPU fallback: a copy of its Python files without
     libgc.so beside them refuses to import, naming the missing library."""
