@@ -19,11 +19,12 @@
 // fp32: the times tau are truncated to fp32 (exact to 2^-23, products to 2^-22),
 // lanes take chunks and keep the ell smallest of their holders' fp32 times, and
 // only the chunks whose value comes within 2^-20 of the warp's largest are
-// formed again with the defining double products, by the whole warp.  The fp64
-// pipe (2 operations a clock per SM) and the 64-bit comparisons are what
+// formed again with the defining double products, by the whole warp; when more
+// than a few do (workers of one speed), the products themselves are compared.
+// The fp64 pipe (2 operations a clock per SM) and the 64-bit comparisons are what
 // bounded the kernel that did it all in double (N = m = 200, delta = 8, ell = 2,
-// 10^5 realizations: 0.92 ms; 0.33 ms this way).  A realization with a time outside [2^-100, 2^100]
-// takes the double form below.
+// 10^5 realizations: 0.92 ms; 0.34 this way, 0.42 with all chunks tied).  A
+// realization with a time outside [2^-100, 2^100] takes the double form below.
 // In the double form, and for theta > 0, lanes gather their holders'
 // completion times as 64-bit keys (the bit patterns of non-negative doubles
 // order like the values) and keep the ell smallest in registers; for theta > 0
@@ -48,13 +49,27 @@ constexpr int kWarpsPerBlock = 4;
 // the tau loads of many realizations in flight.
 constexpr int blocks_per_sm(int ell) { return ell <= 3 ? 12 : 8; }
 
-// k-th smallest (1-based, 1 <= k <= n) of n keys in shared memory, by warp.  Once
-// a single key is left under the prefix it is the answer (of a few hundred
-// distinct times after about six of the sixteen digits; N = m = 200, delta = 8,
-// ell = 2, theta = 10, 10^5 realizations: 1.92 ms with all sixteen, 1.55 so).
+// k-th smallest (1-based, 1 <= k <= n) of n keys in shared memory, by warp: a radix
+// select over the 4-bit digits in which the keys that are left differ, until they are all
+// the same (N = m = 200, delta = 8, ell = 2, theta = 10, 10^5 realizations: 1.31 ms; 1.92 with
+// all sixteen digits).
 __device__ unsigned long long warp_select(const unsigned long long* keys, int n, int k, int lane) {
   unsigned long long prefix = 0, mask = 0;
-  for (int shift = 60; shift >= 0; shift -= 4) {
+  for (;;) {
+    unsigned long long all = ~0ull, any = 0;
+    for (int t = lane; t < n; t += 32) {
+      const unsigned long long key = keys[t];
+      if ((key & mask) == prefix) {
+        all &= key;
+        any |= key;
+      }
+    }
+    all = ((unsigned long long)__reduce_and_sync(0xffffffffu, (unsigned)(all >> 32)) << 32) |
+          __reduce_and_sync(0xffffffffu, (unsigned)all);
+    any = ((unsigned long long)__reduce_or_sync(0xffffffffu, (unsigned)(any >> 32)) << 32) |
+          __reduce_or_sync(0xffffffffu, (unsigned)any);
+    if (all == any) return all;
+    const int shift = (63 - __clzll((long long)(all ^ any))) & ~3;  // the digits above are common
     unsigned long long lo = 0, hi = 0;  // 8-bit counters for digits 0..7 and 8..15
     for (int t = lane; t < n; t += 32) {
       const unsigned long long key = keys[t];
@@ -64,30 +79,20 @@ __device__ unsigned long long warp_select(const unsigned long long* keys, int n,
         else hi += 1ull << (8 * (dg - 8));
       }
     }
-    int cum = 0, digit = 15, left = 0;
+    int cum = 0, digit = 15;
     for (int dg = 0; dg < 16; ++dg) {
       const unsigned c = (unsigned)(((dg < 8 ? lo : hi) >> (8 * (dg & 7))) & 255u);
       const int tot = (int)__reduce_add_sync(0xffffffffu, c);
       if (cum + tot >= k) {
         digit = dg;
-        left = tot;
         break;
       }
       cum += tot;
     }
     k -= cum;
-    prefix |= (unsigned long long)digit << shift;
-    mask |= 15ull << shift;
-    if (left == 1) {
-      unsigned long long found = 0;
-      for (int t = lane; t < n; t += 32)
-        if ((keys[t] & mask) == prefix) found = keys[t];
-      const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(found >> 32));
-      const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)found);  // 0 in the other lanes
-      return ((unsigned long long)hi << 32) | lo;
-    }
+    mask = ~0ull << shift;
+    prefix = (all & (mask << 4)) | ((unsigned long long)digit << shift);
   }
-  return prefix;
 }
 
 // Keep the ELL smallest keys seen so far (ascending).  Keys are the bit
@@ -153,9 +158,13 @@ __device__ __forceinline__ unsigned long long warp_ell_th(unsigned long long key
   return mn;
 }
 
+constexpr float kBelow = 1.f - 0x1p-20f, kAbove = 1.f + 0x1p-20f;
+// Chunks about the largest time that a warp forms one by one; more of them are ties.
+constexpr int kTrigExact = 4;
 constexpr int kTrigHolders = 8192;  // holder words staged in shared memory (32 KB)
 
-template <int ELL>
+// ZERO: theta = 0 (two kernels, each with the registers it needs).
+template <int ELL, bool ZERO>
 __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
     k_trigger(const int32_t* __restrict__ order, Holders h, int N, int m, int delta, int hs,
               const double* __restrict__ tau, long long nsim, int theta, double* __restrict__ T_out,
@@ -176,7 +185,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
   unsigned long long* keys = s_dyn + (size_t)kWarpsPerBlock * m + (size_t)warp * 2 * N * ELL;
   unsigned long long* keysF = keys + (size_t)N * ELL;
   uint32_t* s_h = reinterpret_cast<uint32_t*>(
-      s_dyn + (size_t)kWarpsPerBlock * (m + (theta > 0 ? 2 * N * ELL : 0)));
+      s_dyn + (size_t)kWarpsPerBlock * (m + (ZERO ? 0 : 2 * N * ELL)));
   int8_t* s_dj = reinterpret_cast<int8_t*>(s_h + (size_t)hs * N);
   for (int j = threadIdx.x; j < m; j += blockDim.x) {
     int c = 0;
@@ -201,7 +210,9 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
     const double* tr = tau + r * m;
     unsigned long long Tb = 0, TFb = 0;
     bool wild = false;  // a time outside the range in which fp32 decides
-    if (theta == 0) {
+    unsigned tied = 0;  // 1: T, 2: T_full: more chunks about the largest time than are formed one by one
+    float topT = 0.f, topF = 0.f;
+    if (ZERO) {
       // fp32 times (truncated); +inf for a failed worker
       for (int j = lane; j < m; j += 32) {
         const double tj = tr[j];
@@ -213,7 +224,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
       wild = __any_sync(0xffffffffu, wild);
       __syncwarp();
     }
-    if (theta == 0 && !wild) {
+    if (ZERO && !wild) {
       // every lane's largest ell-th value, its chunk, and its second largest
       float best = -1.f, second = -1.f, bestF = -1.f, secondF = -1.f;
       int bi = 0, biF = 0;
@@ -243,7 +254,6 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
       // non-negative floats order like their bits; lanes without a chunk hold -1
       const float A = __uint_as_float(__reduce_max_sync(0xffffffffu, best < 0.f ? 0u : __float_as_uint(best)));
       const float AF = __uint_as_float(__reduce_max_sync(0xffffffffu, bestF < 0.f ? 0u : __float_as_uint(bestF)));
-      constexpr float kBelow = 1.f - 0x1p-20f, kAbove = 1.f + 0x1p-20f;
       // exact ell-th time of chunk i: lane q takes its q-th holder (<= 32)
       auto exact = [&](int i, bool full) {
         unsigned long long key = kInf;
@@ -255,19 +265,20 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
         }
         return min(warp_ell_th(key, ELL, lane), kInf);
       };
-      auto candidates = [&](float lim, float bst, float scd, int chunk, bool full) {
+      // the largest time: of the few chunks about top (one as a rule); else a tie
+      auto largest = [&](float top, float bst, float scd, int chunk, bool full) {
+        const float lim = top * kBelow;
+        const unsigned lanes = __ballot_sync(0xffffffffu, bst >= lim);
         unsigned long long mx = 0;
-        for (unsigned c = __ballot_sync(0xffffffffu, bst >= lim); c; c &= c - 1) {
-          const int src = __ffs(c) - 1;
-          if (__shfl_sync(0xffffffffu, scd, src) >= lim) {  // several of this lane's chunks
-            for (int i = src; i < N; i += 32) mx = max(mx, exact(i, full));
-          } else {
-            mx = max(mx, exact(__shfl_sync(0xffffffffu, chunk, src), full));
-          }
+        if (__popc(lanes) > kTrigExact || __any_sync(0xffffffffu, scd >= lim)) {
+          tied |= full ? 2u : 1u;
+        } else {
+          for (unsigned c = lanes; c; c &= c - 1)
+            mx = max(mx, exact(__shfl_sync(0xffffffffu, chunk, __ffs(c) - 1), full));
         }
         return mx;
       };
-      Tb = candidates(A * kBelow, best, second, bi, false);
+      Tb = largest(A, best, second, bi, false);
       if (Tfull_out) {
         // a finishing time is one worker's, so when a single worker's fp32 time
         // lies about AF it is the answer; else the chunks about AF
@@ -284,10 +295,43 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
           js = __shfl_sync(0xffffffffu, js, __ffs(has) - 1);
           TFb = dbits(s_kd[s_dj[js]] * tr[js]);
         } else {
-          TFb = candidates(AF * kBelow, bestF, secondF, biF, true);
+          TFb = largest(AF, bestF, secondF, biF, true);
         }
       }
-    } else {
+      topT = A;
+      topF = AF;
+    }
+    if (tied) {
+      // The answer is one of the double products whose fp32 value lies about topT, and a
+      // worker has at most one of them (two slots are 3% apart): when they are all the same
+      // number, however many workers and chunks are tied, that is it.  So for T_full.
+      // Otherwise the double form decides.  (Chunk by chunk, 10^5 realizations of 200
+      // workers at equal speeds took 5.3 ms; 0.42 so, 0.93 all in double.)
+      unsigned left = 0;
+#pragma unroll 1
+      for (; tied; tied &= tied - 1) {
+        const bool full = !(tied & 1u);
+        const float top = full ? topF : topT;
+        unsigned long long mn = ~0ull, mx = 0;
+        for (int j = lane; j < m; j += 32) {
+          const float f = tf[j].x, dj = (float)s_dj[j];
+          const float c = full ? dj : rintf(__fdividef(top, f)), u = c * f;
+          if (u >= top * kBelow && u <= top * kAbove && c >= 1.f && c <= dj) {
+            const unsigned long long key = dbits(s_kd[(int)c] * tr[j]);
+            mn = min(mn, key);
+            mx = max(mx, key);
+          }
+        }
+        mn = warp_min(mn);
+        const bool inf = !(top < INFINITY);  // a chunk without ell finite copies
+        if (!inf && mn != ~warp_min(~mx)) left = 1;
+        if (inf) mn = kInf;
+        if (full) TFb = mn;
+        else Tb = mn;
+      }
+      tied = left;
+    }
+    if (!ZERO || wild || tied) {
       // the double form; each worker's finishing time delta_j tau_j (+inf for a
       // failed worker)
       __syncwarp();
@@ -316,7 +360,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
             insert_smallest<ELL>(bf, fin[j]);
           }
         }
-        if (theta == 0) {
+        if (ZERO) {
           lmax = max(lmax, b[ELL - 1]);
           lmaxF = max(lmaxF, bf[ELL - 1]);
         } else {
@@ -328,7 +372,7 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
         }
       }
       __syncwarp();
-      if (theta == 0) {
+      if (ZERO) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           lmax = max(lmax, (unsigned long long)__shfl_xor_sync(0xffffffffu, lmax, o));
@@ -383,15 +427,15 @@ int launch_one(const int32_t* order, Holders h, int N, int m, int delta, const d
   // the workers' times alone fill a good part of the shared memory
   const int hs = theta == 0 && m <= 2048 ? std::min(delta, kTrigHolders / N) : 0;
   const size_t smem = ((size_t)kWarpsPerBlock * m + keys) * 8 + (size_t)hs * N * 4 + (size_t)m;
+  auto kern = theta == 0 ? k_trigger<ELL, true> : k_trigger<ELL, false>;
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_trigger<ELL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_check(e, "cudaFuncSetAttribute(k_trigger)");
   }
   const long long blocks_needed = (nsim + kWarpsPerBlock - 1) / kWarpsPerBlock;
   const int blocks =
       (int)std::min<long long>(blocks_needed, (long long)device_sm_count() * blocks_per_sm(ELL));
-  k_trigger<ELL><<<blocks, 32 * kWarpsPerBlock, smem, s>>>(order, h, N, m, delta, hs, tau, nsim, theta,
+  kern<<<blocks, 32 * kWarpsPerBlock, smem, s>>>(order, h, N, m, delta, hs, tau, nsim, theta,
                                                            T, psi, TF);
   count_launches(1);
   return cuda_check(cudaGetLastError(), "k_trigger");

@@ -186,6 +186,31 @@ def test_gpu_trigger_close_and_extreme_times(gc, kind, N, delta, ell):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("kind", ["equal", "two_speeds", "tenths", "few_near", "one_slow"])
+@pytest.mark.parametrize("N,delta,ell", [(5, 3, 1), (33, 5, 2), (70, 8, 4), (200, 10, 3)])
+def test_gpu_trigger_tied_chunks(gc, kind, N, delta, ell):
+    """Many chunks that finish together: at one and the same double (equal times, two speeds), at
+    doubles that differ in the last place (3 * 0.1 and 0.3), a few of them only, and one slow
+    worker whose last chunks tie; every output to the bit, for several theta."""
+    rng = np.random.default_rng(3 * N + ell)
+    nsim = 70
+    order = O.cyclic_order(N, N, delta)
+    tau = np.ones((nsim, N))
+    if kind == "two_speeds":
+        tau[rng.random((nsim, N)) < 0.3] = 3.0
+    elif kind == "tenths":
+        tau = rng.integers(1, 4, size=(nsim, N)) * 0.1
+    elif kind == "few_near":
+        tau = 0.5 + rng.exponential(1.0, size=(nsim, N))
+        tau[:, ::5] = 4.0 + rng.integers(0, 3, size=tau[:, ::5].shape) * 2.0 ** -50
+    elif kind == "one_slow":
+        tau[:, N // 2] = 50.0
+    tau[::4, rng.integers(0, N, size=1)] = np.inf
+    for theta in (0, 1, N * ell // 3):
+        _gpu_vs_oracle(gc, order, N, ell, theta, tau)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("ell", [1, 2, 3])
 def test_gpu_trigger_feeds_decode_on_g1(gc, ell):
     """Simulate -> trigger at a theta -> psi -> batched Algorithm 1 and
