@@ -168,8 +168,9 @@ struct ResidLists {
   int32_t* idx;   // [npat][ksp] their chunks, ascending
   float* D;       // [npat][ksp][ell][ell] Pi - I
   int32_t* stat;  // patterns with more than ksp of them; blocks past the budget in
-                  // the others; patterns gathered for the GEMM
+                  // the others; patterns gathered for the GEMM; its direct tiles
   int32_t* dpat;  // [npat] the gathered patterns
+  int32_t* dtile; // [ceil(npat / (128 / ell))] the direct tiles
   float* msp;     // [npat][parts] squared-error partials, or null
   int ksp;        // list capacity per pattern
   int parts;      // partials per pattern (column ranges)
@@ -179,8 +180,11 @@ struct ResidLists {
 // pattern is worth the GEMM from `budget` blocks on, but the GEMM's operand
 // split reads and writes all of G, so it runs only when some pattern's list
 // overflows or the others' blocks past the budget add up to more than that.
+// A row tile of the GEMM is 128 / ell consecutive patterns of the plan (a direct
+// tile) where these are all on the GEMM, or direct_share sixteenths of them are:
+// nothing is copied and whole boxes are stored.  The others are gathered.
 struct GemmChoice {
-  int policy, budget, ksp, split_cost;
+  int policy, budget, ksp, split_cost, direct_share;
   __device__ __forceinline__ bool any(const ResidLists& rl) const {
     if (policy == GC_DECODE_DENSE) return true;
     return rl.stat[0] > 0 || (policy == GC_DECODE_AUTO && rl.stat[1] > split_cost);

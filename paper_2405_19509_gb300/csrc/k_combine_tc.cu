@@ -25,10 +25,12 @@
 //               per row; the accumulator is handed back as soon as it is
 //               read, so the epilogue of tile t overlaps the MMAs of t + 1.
 // The rows of the GEMM are those of the patterns that the plan scan leaves to
-// it, gathered by the operand split (k_split_gt) into a compact A; a row's
-// place among them does not change its value.  Ghat is written from a staged
-// 32 x 32 box, four 128-byte row pieces a warp store (32 one-row pieces where
-// rows are not 16-byte multiples).
+// it: whole row tiles of the plan where nearly all patterns are (direct tiles),
+// the others gathered by the operand split (k_split_gt) into a compact A; a row's
+// place among them does not change its value.  Ghat is written from staged
+// 32 x 32 boxes: one TMA tensor store each where the warp's rows are consecutive
+// rows of Ghat, else four 128-byte row pieces a warp store (32 one-row pieces
+// where rows are not 16-byte multiples).
 // Tiles are visited n-tile-major so that concurrently running CTAs share the
 // same B tile through L2.  When one 64-wide block holds all of K the output
 // write bounds the kernel and the B tile is what the copies would mostly
@@ -43,6 +45,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "tc_ptx.cuh"
 
@@ -71,7 +74,7 @@ template <int STAGES, int EPI, int NKBR, bool OUT>
 struct Shape {
   static constexpr bool BRES = NKBR > 0;
   static constexpr int THREADS = 64 + 32 * EPI;
-  static constexpr int OUT_BYTES = OUT ? EPI * OUT_BUF : 0;  // a staging box per epilogue warp
+  static constexpr int OUT_BYTES = OUT ? EPI * 2 * OUT_BUF : 0;  // 2 staging boxes per epilogue warp
   static constexpr int ROW_BYTES = OUT ? EPI * 256 : 0;       // 32 row offsets per epilogue warp
   static constexpr int RING = BRES ? STAGES * A_STAGE + NKBR * B_TILE : STAGES * STAGE_BYTES;
   static constexpr size_t SMEM = (size_t)RING + OUT_BYTES + ROW_BYTES + 1024 + 256;
@@ -81,17 +84,20 @@ struct Shape {
 struct Params {
   int K, Kp, L, ell, d;
   int num_n_tiles, nkb;
+  int npat, ppt;        // patterns; patterns per row tile of the plan (128 / ell)
   int vec_ok;           // d % 4 == 0 && L % 4 == 0: 16-byte row segments
+  int tma_store;        // Ghat is (npat * ell) rows of L with 16-byte pieces: tensor stores
   float* Ghat;          // npat x d or null
   const float* gsum;    // d, or null when no MSE is wanted
   float* msep;          // M x parts_per_row partial squared errors, or null
   int parts_per_row;    // num_n_tiles * (epilogue warps per TMEM lane quarter)
   long long spin_limit; // clock cycles a wait may take before the kernel gives up
   int stall;            // failure-path test: the TMA producer issues nothing
-  // row r of the GEMM is row r % ell of pattern dpat[r / ell], r < *npat_gemm * ell
-  // (both written before the launch)
-  const int32_t* dpat;
-  const int32_t* npat_gemm;
+  // m-tiles t < stat[3]: rows of the plan from pattern dtile[t] * ppt on, those above
+  // the threshold; after them row r of the compact A, r < stat[2] * ell, is row r % ell
+  // of pattern dpat[r / ell] (all written before the launch)
+  ResidLists rl;
+  GemmChoice gemm;
   uint32_t* status;
 };
 
@@ -108,7 +114,8 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
 
 template <int STAGES, int EPI, int NKBR, bool OUT>
 __global__ void __launch_bounds__(64 + 32 * EPI, 1)
-    k_combine_tc(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+    k_combine_tc(const __grid_constant__ CUtensorMap tmP, const __grid_constant__ CUtensorMap tmA,
+                 const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmC,
                  Params p) {
   using Sh = Shape<STAGES, EPI, NKBR, OUT>;
   constexpr bool BRES = Sh::BRES;
@@ -157,10 +164,11 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
   // launched as a programmatic dependent of the operand split: the prologue
   // above overlaps its tail, the operands are read only after this point
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  // the tile space: nd m-tiles x the n-tiles, n-tile-major;
+  // the tile space: nd m-tiles (the direct ones first) x the n-tiles, n-tile-major;
   // this CTA's tiles are t = t_first, t_first + t_step, ... < t_last
-  const int rows = *reinterpret_cast<volatile const int*>(p.npat_gemm) * p.ell;
-  const int nd = (rows + BM - 1) / BM;
+  const int rows = *reinterpret_cast<volatile const int*>(p.rl.stat + 2) * p.ell;
+  const int ndir = *reinterpret_cast<volatile const int*>(p.rl.stat + 3);
+  const int nd = ndir + (rows + BM - 1) / BM;
   const long long ntiles = (long long)nd * p.num_n_tiles;
   long long t_first, t_last, t_step;
   if (BRES) {
@@ -173,6 +181,13 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     t_step = gridDim.x;
   }
   auto tile_mt = [&](long long t) -> int { return (int)(t % nd); };
+  // A's rows of m-tile mt at K block kb: of the plan, or of the compact copy
+  auto load_a = [&](uint8_t* st, int kb, int mt, uint64_t* bar) {
+    if (mt < ndir)
+      tma_load_3d(st, &tmP, kb * BK, __ldg(p.rl.dtile + mt) * p.ppt * p.ell, 0, bar);
+    else
+      tma_load_3d(st, &tmA, kb * BK, (mt - ndir) * BM, 0, bar);
+  };
 
   if (warp == 0) {
     // ------------------------------------------------------------- producer
@@ -200,9 +215,8 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
             ok = false;
             break;
           }
-          uint8_t* st = smem + s * A_STAGE;
           mbar_expect_tx(&full[s], A_STAGE);
-          tma_load_3d(st, &tmA, kb * BK, mt * BM, 0, &full[s]);
+          load_a(smem + s * A_STAGE, kb, mt, &full[s]);
         }
       }
       // drain: every issued copy has landed before the CTA may exit
@@ -224,7 +238,7 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
           }
           uint8_t* st = smem + s * STAGE_BYTES;
           mbar_expect_tx(&full[s], STAGE_BYTES);
-          tma_load_3d(st, &tmA, kb * BK, mt * BM, 0, &full[s]);
+          load_a(st, kb, mt, &full[s]);
           tma_load_3d(st + 2 * A_PLANE, &tmB, kb * BK, nt * BN, 0, &full[s]);
         }
       }
@@ -327,9 +341,11 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
     const int e = warp - 2;        // epilogue warp index
     constexpr int SPAN = BN / (EPI / 4);  // columns per epilogue warp
     const int cbeg = (e / 4) * SPAN;
-    float* wbuf = outbuf + e * (OUT_BUF / 4);
+    float* wbuf = outbuf + e * 2 * (OUT_BUF / 4);
     long long* wrow = rowbuf + e * 32;  // element offset of each of the warp's rows in Ghat, -1: none
-    uint32_t tile_it = 0;
+    const int thr = t_first < t_last ? p.gemm.threshold(p.rl) : 0;
+    const uint64_t evict_first = policy_evict_first();  // Ghat is not read back here
+    uint32_t tile_it = 0, chunk_it = 0;
     for (long long t = t_first; t < t_last; t += t_step, ++tile_it) {
       const int ab = tile_it & 1;
       const int nt = (int)(t / nd), mt = tile_mt(t);
@@ -337,13 +353,25 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
       const bool ready = mbar_wait(&tfull[ab], (tile_it >> 1) & 1, abort_flag, p.status, p.spin_limit);
       if (!__all_sync(0xffffffffu, ready)) break;
       fence_after();
-      const int row = mt * BM + quarter * 32 + lane;
-      const bool rv = row < rows;
-      const int bi = rv ? row / p.ell : 0;
-      const int k = rv ? row - bi * p.ell : 0;
-      const int b = rv ? __ldg(p.dpat + bi) : 0;
+      // this lane's row: row k of pattern b, if the GEMM's
+      int row = quarter * 32 + lane, b, row0 = 0;
+      bool rv;
+      if (mt < ndir) {
+        const int first = __ldg(p.rl.dtile + mt) * p.ppt, pl = row / p.ell;
+        b = first + pl;
+        rv = pl < p.ppt && b < p.npat && __ldg(p.rl.nnz + b) > thr;
+        row0 = first * p.ell + quarter * 32;
+      } else {
+        row += (mt - ndir) * BM;
+        rv = row < rows;
+        b = rv ? __ldg(p.rl.dpat + row / p.ell) : 0;
+      }
+      const int k = rv ? row % p.ell : 0;
+      // all 32 rows, consecutive ones of Ghat: stored as boxes
+      const bool boxes = OUT && p.tma_store && mt < ndir && __all_sync(0xffffffffu, rv);
       const int n0 = nt * BN;
       if (OUT) {
+        if (!boxes && lane == 0) bulk_wait_read<0>();  // the boxes are written without a look below
         __syncwarp();
         wrow[lane] = rv ? (long long)b * p.d + (long long)k * p.L : -1;
       }
@@ -360,82 +388,117 @@ __global__ void __launch_bounds__(64 + 32 * EPI, 1)
         for (int j = 0; j < 8; ++j)
           gnext[j] = __ldg(reinterpret_cast<const float4*>(gs + n0 + cbeg) + j);
       }
+      auto chunks = [&](auto whole) {
+        constexpr bool BOXES = decltype(whole)::value;
 #pragma unroll 1
-      for (int cc = cbeg; cc < cbeg + SPAN; cc += 32) {
-        float v[32];
-        float4 gcur[8];
+        for (int cc = cbeg; cc < cbeg + SPAN; cc += 32) {
+          float v[32];
+          float4 gcur[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) gcur[j] = gnext[j];
-        if (fast_gs && cc + 32 < cbeg + SPAN && n0 + cc + 64 <= p.L) {
+          for (int j = 0; j < 8; ++j) gcur[j] = gnext[j];
+          if (fast_gs && cc + 32 < cbeg + SPAN && n0 + cc + 64 <= p.L) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            gnext[j] = __ldg(reinterpret_cast<const float4*>(gs + n0 + cc + 32) + j);
-        }
-        __syncwarp();
-        tmem_ld32(taddr + cc, v);  // warp-collective: every lane, every chunk
-        const int c0 = n0 + cc;
-        if (OUT && p.Ghat && c0 < p.L) {
-          // stage the 32 x 32 box (row = lane; 16-byte pieces swizzled), then
-          // store it row by row
-          __syncwarp();  // the previous box has been read
-          char* box = reinterpret_cast<char*>(wbuf);
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<float4*>(box + lane * 128 + ((j ^ (lane & 7)) << 4)) =
-                make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            for (int j = 0; j < 8; ++j)
+              gnext[j] = __ldg(reinterpret_cast<const float4*>(gs + n0 + cc + 32) + j);
+          }
           __syncwarp();
-          if (p.vec_ok) {
+          tmem_ld32(taddr + cc, v);  // warp-collective: every lane, every chunk
+          const int c0 = n0 + cc;
+          if (OUT && p.Ghat && c0 < p.L) {
+            // stage the 32 x 32 box (row = lane; 128-byte swizzle of 16-byte pieces),
+            // then store it whole or row by row
+            float* buf = wbuf + (chunk_it++ & 1) * (OUT_BUF / 4);
+            if (BOXES && lane == 0) bulk_wait_read<1>();  // the store that used this box has read it
+            __syncwarp();  // and the warp the box before
+            char* box = reinterpret_cast<char*>(buf);
 #pragma unroll
-            for (int it = 0; it < 8; ++it) {
-              const int rr = it * 4 + (lane >> 3), j = lane & 7;
-              const long long ro = wrow[rr];
-              const int lim_r = __shfl_sync(0xffffffffu, rlim, rr);
-              const float4 q = *reinterpret_cast<const float4*>(box + rr * 128 + ((j ^ (rr & 7)) << 4));
-              if (ro >= 0 && c0 + 4 * j < lim_r)
-                __stcs(reinterpret_cast<float4*>(p.Ghat + ro + c0 + 4 * j), q);
+            for (int j = 0; j < 8; ++j)
+              *reinterpret_cast<float4*>(box + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+                  make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            if (BOXES) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (BOXES) {
+              if (lane == 0) {
+                tma_store_2d_hint(&tmC, buf, c0, row0, evict_first);
+                bulk_commit();
+              }
+            } else if (p.vec_ok) {
+              // four rows' pieces out of shared memory, then their stores (a load behind a
+              // store is not moved before it)
+#pragma unroll
+              for (int i0 = 0; i0 < 8; i0 += 4) {
+                float4 q[4];
+                long long ro[4];
+                bool in[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                  const int rr = (i0 + u) * 4 + (lane >> 3), j = lane & 7;
+                  ro[u] = wrow[rr];
+                  in[u] = c0 + 4 * j < __shfl_sync(0xffffffffu, rlim, rr);  // rlim: 0 where ro is -1
+                  q[u] = *reinterpret_cast<const float4*>(box + rr * 128 + ((j ^ (rr & 7)) << 4));
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                  if (in[u])
+                    __stcs(reinterpret_cast<float4*>(p.Ghat + ro[u] + c0 + 4 * (lane & 7)), q[u]);
+              }
+            } else {
+#pragma unroll
+              for (int r0 = 0; r0 < 32; r0 += 8) {
+                float q[8];
+                long long ro[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  const int rr = r0 + u;
+                  ro[u] = wrow[rr];
+                  q[u] = *reinterpret_cast<const float*>(box + rr * 128 + (((lane >> 2) ^ (rr & 7)) << 4) +
+                                                         (lane & 3) * 4);
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                  const int lim_r = __shfl_sync(0xffffffffu, rlim, r0 + u);
+                  if (c0 + lane < lim_r) __stcs(p.Ghat + ro[u] + c0 + lane, q[u]);
+                }
+              }
+            }
+          }
+          const int lim = min(32, rlim - c0);
+          if (!gs || lim <= 0) {
+          } else if (lim == 32 && p.vec_ok) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float4 g = gcur[j];
+              float df = v[4 * j] - g.x;
+              sq4[0] = fmaf(df, df, sq4[0]);
+              df = v[4 * j + 1] - g.y;
+              sq4[1] = fmaf(df, df, sq4[1]);
+              df = v[4 * j + 2] - g.z;
+              sq4[2] = fmaf(df, df, sq4[2]);
+              df = v[4 * j + 3] - g.w;
+              sq4[3] = fmaf(df, df, sq4[3]);
             }
           } else {
-#pragma unroll 8
-            for (int rr = 0; rr < 32; ++rr) {
-              const long long ro = wrow[rr];
-              const int lim_r = __shfl_sync(0xffffffffu, rlim, rr);
-              const float q = *reinterpret_cast<const float*>(
-                  box + rr * 128 + (((lane >> 2) ^ (rr & 7)) << 4) + (lane & 3) * 4);
-              if (ro >= 0 && c0 + lane < lim_r) __stcs(p.Ghat + ro + c0 + lane, q);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              if (j < lim) {
+                const float df = v[j] - __ldg(gs + c0 + j);
+                sq4[j & 3] = fmaf(df, df, sq4[j & 3]);
+              }
             }
           }
         }
-        const int lim = min(32, rlim - c0);
-        if (!gs || lim <= 0) {
-        } else if (lim == 32 && p.vec_ok) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float4 g = gcur[j];
-            float df = v[4 * j] - g.x;
-            sq4[0] = fmaf(df, df, sq4[0]);
-            df = v[4 * j + 1] - g.y;
-            sq4[1] = fmaf(df, df, sq4[1]);
-            df = v[4 * j + 2] - g.z;
-            sq4[2] = fmaf(df, df, sq4[2]);
-            df = v[4 * j + 3] - g.w;
-            sq4[3] = fmaf(df, df, sq4[3]);
-          }
-        } else {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (j < lim) {
-              const float df = v[j] - __ldg(gs + c0 + j);
-              sq4[j & 3] = fmaf(df, df, sq4[j & 3]);
-            }
-          }
-        }
-      }
+      };
+      if (OUT && boxes)
+        chunks(std::true_type{});
+      else
+        chunks(std::false_type{});
       fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&tempty[ab]);
       if (p.msep && rv)
         p.msep[((size_t)b * p.ell + k) * p.parts_per_row + nt * (EPI / 4) + e / 4] = (sq4[0] + sq4[1]) + (sq4[2] + sq4[3]);
     }
+    if (OUT && lane == 0) bulk_wait_all();  // every tensor store of this warp has completed
   }
   fence_before();
   __syncthreads();
@@ -471,8 +534,10 @@ __global__ void k_split_c(const float* __restrict__ C, int M, int K, int Kp,
 // along c, and 128 consecutive bytes of a plane row per eight lanes on the way
 // out (COLS = 64 for long rows, 32 when L is short and more blocks are
 // wanted).  Blocks stride over the (column tile, K tile) pairs.
-// A: the plan rows of those patterns, copied to consecutive rows (one warp a
-// pattern; places are handed out as they come, which changes no value).
+// A: if the 128 / ell patterns of a row tile of the plan are all on the GEMM, or enough
+// of them for the choice, the tile is listed; else the rows of those that are are copied
+// to consecutive rows (a block eight patterns, a warp each; places are handed out as
+// they come, which changes no value).
 template <int COLS>
 __global__ void __launch_bounds__(256) k_split_gt(const float* __restrict__ G, int N, int d,
                                                   int ell, int L, int Kp,
@@ -492,22 +557,37 @@ __global__ void __launch_bounds__(256) k_split_gt(const float* __restrict__ G, i
   }
   const int t = threadIdx.x, lane = t & 31;
   {
-    const int thr = gemm.threshold(rl);
+    __shared__ int s_base;
+    __shared__ unsigned s_heavy[4];
+    const int thr = gemm.threshold(rl), ppt = 128 / ell;
     const size_t plane = (size_t)npat * ell * Kp;
     const int per_plane = ell * Kp / 8;  // 16-byte pieces of a pattern's rows in a plane
-    for (int b = (blockIdx.x * 256 + t) >> 5; b < npat; b += gridDim.x * 8) {
-      if (__ldg(rl.nnz + b) <= thr) continue;
-      int slot = 0;
-      if (lane == 0) {
-        slot = atomicAdd(rl.stat + 2, 1);
-        rl.dpat[slot] = b;
+    const int parts = (ppt + 7) / 8;     // of a row tile, eight patterns each
+    const int nunit = (npat + ppt - 1) / ppt * parts, warp = t >> 5;
+    for (int unit = blockIdx.x; unit < nunit; unit += gridDim.x) {
+      const int seg = unit / parts, part = unit - seg * parts;
+      const int cnt = min(ppt, npat - seg * ppt);
+      const bool heavy = t < cnt && __ldg(rl.nnz + seg * ppt + t) > thr;
+      const unsigned bal = __ballot_sync(0xffffffffu, heavy);
+      if (lane == 0 && warp < 4) s_heavy[warp] = bal;
+      const int n = __syncthreads_count(heavy);
+      const bool direct = n > 0 && (n == cnt || 16 * n >= gemm.direct_share * cnt);
+      const unsigned mine = direct ? 0u : (s_heavy[part / 4] >> (8 * (part % 4))) & 0xffu;
+      if (t == 0) {
+        if (direct && part == 0) rl.dtile[atomicAdd(rl.stat + 3, 1)] = seg;
+        if (mine) s_base = atomicAdd(rl.stat + 2, __popc(mine));
       }
-      slot = __shfl_sync(0xffffffffu, slot, 0);
-      for (int h = 0; h < 2; ++h) {
-        const uint4* src = reinterpret_cast<const uint4*>(Cs + h * plane + (size_t)b * ell * Kp);
-        uint4* dst = reinterpret_cast<uint4*>(Ca + h * plane + (size_t)slot * ell * Kp);
-        for (int q = lane; q < per_plane; q += 32) dst[q] = __ldg(src + q);
+      __syncthreads();
+      if ((mine >> warp) & 1u) {
+        const int b = seg * ppt + part * 8 + warp, slot = s_base + __popc(mine & ((1u << warp) - 1u));
+        if (lane == 0) rl.dpat[slot] = b;
+        for (int h = 0; h < 2; ++h) {
+          const uint4* src = reinterpret_cast<const uint4*>(Cs + h * plane + (size_t)b * ell * Kp);
+          uint4* dst = reinterpret_cast<uint4*>(Ca + h * plane + (size_t)slot * ell * Kp);
+          for (int q = lane; q < per_plane; q += 32) dst[q] = __ldg(src + q);
+        }
       }
+      __syncthreads();  // s_base and s_heavy have been read
     }
   }
   __shared__ float tile[64][COLS + 1];
@@ -642,6 +722,22 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
+// 2-D fp32 map over Ghat viewed as (npat*ell) rows of L (requires d == ell*L),
+// box 32 x 32, 128-byte swizzle (matches the epilogue's staging layout).
+int make_out_map(CUtensorMap* map, float* base, long long rows, int L) {
+  auto fn = encode_fn();
+  if (!fn) return fail(GC_ERR_CUDA, "cuTensorMapEncodeTiled entry point unavailable");
+  cuuint64_t dims[2] = {(cuuint64_t)L, (cuuint64_t)rows};
+  cuuint64_t strides[1] = {(cuuint64_t)L * 4};
+  cuuint32_t box[2] = {32, 32};
+  cuuint32_t estr[2] = {1, 1};
+  CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) return fail(GC_ERR_CUDA, "cuTensorMapEncodeTiled(out) failed (%d)", (int)r);
+  return GC_OK;
+}
+
 // 3-D map over [2][rows][Kp] bf16 planes, box {64, box_rows, 2}, 128-byte swizzle.
 int make_map(CUtensorMap* map, const void* base, int rows, int Kp, int box_rows) {
   auto fn = encode_fn();
@@ -660,8 +756,8 @@ int make_map(CUtensorMap* map, const void* base, int rows, int Kp, int box_rows)
 }  // namespace tc
 
 template <int STAGES, int EPI, int NKBR, bool OUT>
-int launch_tc(int grid, const CUtensorMap& mA, const CUtensorMap& mB, const tc::Params& p,
-              cudaStream_t s) {
+int launch_tc(int grid, const CUtensorMap& mP, const CUtensorMap& mA, const CUtensorMap& mB,
+              const CUtensorMap& mC, const tc::Params& p, cudaStream_t s) {
   using Sh = tc::Shape<STAGES, EPI, NKBR, OUT>;
   static SmemOptIn allow;
   cudaError_t e = allow(tc::k_combine_tc<STAGES, EPI, NKBR, OUT>, Sh::SMEM);
@@ -676,7 +772,7 @@ int launch_tc(int grid, const CUtensorMap& mA, const CUtensorMap& mB, const tc::
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, tc::k_combine_tc<STAGES, EPI, NKBR, OUT>, mA, mB, p);
+  e = cudaLaunchKernelEx(&cfg, tc::k_combine_tc<STAGES, EPI, NKBR, OUT>, mP, mA, mB, mC, p);
   if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_combine_tc)");
   count_launches(1);
   return cuda_check(cudaGetLastError(), "k_combine_tc");
@@ -735,7 +831,13 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
   // (4 d bytes, mostly from L2); a pattern costs the GEMM 6 Kp d flops.  At the
   // rates of the two (about 10 TB/s, 1.6 PFLOP/s) they meet at Kp / 107 blocks;
   // the split of G is worth about 2 N blocks.
-  GemmChoice gemm{policy, std::max(1, Kp / 64), rl.ksp, 2 * N};
+  const bool tma_store = Ghat && (long long)ell * L == d && L % 4 == 0 &&
+                         reinterpret_cast<uintptr_t>(Ghat) % 16 == 0;
+  // The GEMM of one or two K blocks is bound by its output, which direct tiles store
+  // as boxes (N = 30, ell = 4, d = 2^20, 128 patterns, 97% of them on the GEMM: plan and
+  // decode 365 us, 403 all gathered); with more, only rows that it has to multiply.
+  const int direct_share = Kp <= 128 && tma_store ? 12 : 17;
+  GemmChoice gemm{policy, std::max(1, Kp / 64), rl.ksp, 2 * N, direct_share};
   // header words 4..6: counters of the plan scan (zeroed with the header)
   unsigned int* counters = reinterpret_cast<unsigned int*>(status) + 4;
   int rc = launch_plan_scan(Cs, Kp, N, ell, npat, gemm.budget, rl, counters, s);
@@ -769,12 +871,22 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
     if (e != cudaSuccess) return cuda_check(e, "cudaLaunchKernelEx(k_split_gt)");
     count_launches(1);
   }
-  CUtensorMap mA, mB;
+  CUtensorMap mP, mA, mB, mC;
+  rc = make_map(&mP, Cs, (int)M, Kp, BM);
+  if (rc) return rc;
   rc = make_map(&mA, Ca, (int)M, Kp, BM);
   if (rc) return rc;
   rc = make_map(&mB, Gs, L, Kp, BN);
   if (rc) return rc;
+  memset(&mC, 0, sizeof(mC));
+  if (tma_store) {
+    rc = make_out_map(&mC, Ghat, M, L);
+    if (rc) return rc;
+  }
   Params p{};
+  p.npat = npat;
+  p.ppt = 128 / ell;
+  p.tma_store = tma_store ? 1 : 0;
   p.K = K;
   p.Kp = Kp;
   p.L = L;
@@ -786,8 +898,8 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
   p.Ghat = Ghat;
   p.gsum = grad_mse ? gsum : nullptr;
   p.msep = msep;
-  p.dpat = rl.dpat;
-  p.npat_gemm = rl.stat + 2;
+  p.rl = rl;
+  p.gemm = gemm;
   p.status = status;
   p.spin_limit = wait_limit(kSpin);
   p.stall = take_stall(GC_STALL_COMBINE) ? 1 : 0;
@@ -800,9 +912,9 @@ int launch_apply(const __nv_bfloat16* Cs, const float* G, int N, int ell, int np
   p.parts_per_row = nnt * ((one_block || two_res) ? 2 : 1);
   const int sms = device_sm_count();
   const int grid = (int)std::min<long long>((long long)nmt * nnt, sms);
-  rc = one_block ? launch_tc<kBresStages, 8, 1, true>(grid, mA, mB, p, s)
-       : two_res ? launch_tc<3, 8, 2, false>(grid, mA, mB, p, s)
-                 : launch_tc<2, 4, 0, true>(grid, mA, mB, p, s);
+  rc = one_block ? launch_tc<kBresStages, 8, 1, true>(grid, mP, mA, mB, mC, p, s)
+       : two_res ? launch_tc<3, 8, 2, false>(grid, mP, mA, mB, mC, p, s)
+                 : launch_tc<2, 4, 0, true>(grid, mP, mA, mB, mC, p, s);
   if (rc) return rc;
   if (grad_mse) {
     cudaLaunchConfig_t cfg{};

@@ -56,6 +56,7 @@ ResidLists carve_resid(Carve& c, int N, int ell, int npat, int d, bool want_mse)
   r.D = c.take<float>((size_t)npat * r.ksp * ell * ell);
   r.stat = c.take<int32_t>(4);
   r.dpat = c.take<int32_t>(npat);
+  r.dtile = c.take<int32_t>(npat / (128 / ell) + 1);
   float* msp = c.take<float>((size_t)npat * r.parts);
   r.msp = want_mse ? msp : nullptr;
   return r;
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(kScanThreads) k_plan_scan(const __nv_bfloat16*
       __threadfence();
       rl.stat[0] = (int)atomicExch(counters + 1, 0u);
       rl.stat[1] = (int)atomicExch(counters + 2, 0u);
-      rl.stat[2] = 0;  // patterns on the GEMM, counted by their gathering
+      rl.stat[2] = rl.stat[3] = 0;  // counted by the operand split
     }
   }
 }

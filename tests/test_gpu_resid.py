@@ -275,6 +275,47 @@ def test_heavy_patterns_are_gathered(gc, ell, d, npat, every):
             assert_mse_close(float(ms[b]), r.grad_mse, floor, f"policy {pol} b={b}")
 
 
+@pytest.mark.parametrize("ell,d,npat,step", [
+    (4, 4096, 200, 9),    # row tiles of 32 patterns, three or four of them light: stored as boxes and by rows
+    (2, 2048, 130, 40),   # one K block, tiles of 64, a last one of two
+    (1, 512, 300, 100),   # tiles of 128
+    (3, 1200, 127, 50),   # tiles of 42 patterns, 126 rows
+    (4, 4092, 100, 6),    # five of 32 light; rows of 1023: no boxes, gathered
+    (5, 2000, 60, 16),    # tiles of 25
+])
+def test_mostly_heavy_row_tiles(gc, ell, d, npat, step):
+    """N = m = 20, delta = 4: nearly every pattern is on the GEMM, which then takes whole row tiles
+    of the plan; the few exact ones in between stay the plain sum, with zero error."""
+    N = m = 20
+    delta = 4 if ell <= 4 else ell
+    order = O.cyclic_order(N, m, delta)
+    rng = np.random.default_rng(ell * 100 + npat)
+    R = rng.standard_normal((ell, m))
+    psi = np.zeros((npat, m), dtype=np.int32)
+    psi[np.arange(npat), rng.integers(0, m, size=npat)] = delta
+    light = np.arange(step - 1, npat, step)
+    psi[light] = delta
+    G32 = rng.standard_normal((N, d)).astype(np.float32)
+    Gref = G32.astype(np.float64)
+    gsum = Gref.sum(axis=0)
+    floor = 1e-8 * float(gsum @ gsum) / d
+    Rd, od, pd = dev_tensors(R, order, psi)
+    Gd = torch.from_numpy(G32).cuda()
+    full = gc.gc_decode_batch(Rd, ell, od, N, m, delta, torch.full((1, m), delta, dtype=torch.int32, device="cuda"), Gd)["Ghat"]
+    buf = torch.full((npat + 2, d), float("nan"), device="cuda")
+    for _ in range(2):  # the counters are back at zero for the second call
+        ms = gc.gc_decode_batch(Rd, ell, od, N, m, delta, pd, Gd, Ghat=buf[1:-1])["grad_mse"]
+    Gh, ms = to_np(buf[1:-1]), to_np(ms)
+    assert torch.isnan(buf[0]).all() and torch.isnan(buf[-1]).all()
+    for b in range(npat):
+        if b in light:
+            assert np.array_equal(Gh[b], to_np(full[0])) and ms[b] == 0.0
+        else:
+            r = O.run_pattern(R, order, psi[b], N, Gref, want_transmit=False)
+            assert_grad_close(Gh[b], r.ghat, f"b={b}")
+            assert_mse_close(float(ms[b]), r.grad_mse, floor, f"b={b}")
+
+
 def test_combine_non_projector_matrix(gc):
     """gc_decode_combine with a decode matrix whose blocks, in one pattern in
     four, are near but not exactly I (every block of such a pattern differs
