@@ -402,12 +402,15 @@ int launch_encode(const double* E, const int32_t* order, const int32_t* psi, int
 
 // ghat[b][k*L + c] = sum_j R[k][j] * T[b][j][c], j ascending.  A thread takes V
 // columns; R is staged in dynamic shared memory as fp32 (ELL * m words, m <=
-// kDecodeSmemM) or read as fp64.  The kernel streams T; eight 16-byte loads of
-// workers' rows are in flight per thread where the rows allow it, else sixteen
-// 4-byte ones (m = 256, ell = 2, L = 2^19, 16-byte loads: 77 us = 7.0 TB/s, 123 us
-// with eight of 4 bytes; four patterns of m = 200, ell = 3, L = 87383: 60 and 73).
+// kDecodeSmemM) or read as fp64.  The kernel streams T with U loads of workers' rows
+// in flight per thread: eight of 16 bytes where the rows allow it and ell >= 2, else
+// of 4 bytes, sixteen from 64 workers on (their last, partial step is what a few
+// workers would mostly run) and eight below.  m = 256, ell = 2, L = 2^19: 76 us = 7.1
+// TB/s with 16-byte loads, 90 with either of 4 bytes.  ell = 1, m = 256, L = 2^20: 161 us
+// with sixteen, 169 with eight, 256 with 16-byte loads (m = 200, L = 20000, 8 patterns 25, 32
+// and 95).  m = 50, ell = 3, L = 101, 3,000 patterns: 16.3 us with sixteen, 12.3 with eight.
 constexpr int kDecodeSmemM = 1024;
-template <int ELL, bool STAGED, int V>
+template <int ELL, bool STAGED, int V, int U>
 __global__ void k_decode_tx(const double* __restrict__ R, int m, const float* __restrict__ T,
                             int npat, int d, int L, float* __restrict__ ghat) {
   extern __shared__ float s_r[];
@@ -426,7 +429,6 @@ __global__ void k_decode_tx(const double* __restrict__ R, int m, const float* __
 #pragma unroll
     for (int v = 0; v < V; ++v) acc[k][v] = 0.f;
   const float* Tb = T + (size_t)b * m * L + c;
-  constexpr int U = V == 4 ? 8 : 16;  // workers' loads in flight
   for (int j0 = 0; j0 < m; j0 += U) {
     float t[U][V];
 #pragma unroll
@@ -474,18 +476,21 @@ static void run_decode_tx(const double* R, int m, const float* T, int npat, int 
   // four columns a thread (16-byte loads) when the rows are 16-byte pieces and
   // that still leaves 256 threads an SM; below, one column a thread hides the
   // latency better
-  const bool vec = staged && L % 4 == 0 && d % 4 == 0 &&
+  constexpr bool kVec = ELL >= 2;
+  const bool vec = kVec && staged && L % 4 == 0 && d % 4 == 0 &&
                    (reinterpret_cast<uintptr_t>(T) | reinterpret_cast<uintptr_t>(ghat)) % 16 == 0 &&
                    (long long)npat * L >= 1024LL * device_sm_count();
   const int threads = 128;
   const long long tot = (long long)npat * (vec ? L / 4 : L);
   const unsigned blocks = (unsigned)((tot + threads - 1) / threads);
-  if (vec)
-    k_decode_tx<ELL, true, 4><<<blocks, threads, sm, s>>>(R, m, T, npat, d, L, ghat);
-  else if (staged)
-    k_decode_tx<ELL, true, 1><<<blocks, threads, sm, s>>>(R, m, T, npat, d, L, ghat);
-  else
-    k_decode_tx<ELL, false, 1><<<blocks, threads, 0, s>>>(R, m, T, npat, d, L, ghat);
+  auto run = [&](auto kern) { kern<<<blocks, threads, sm, s>>>(R, m, T, npat, d, L, ghat); };
+  if (vec) {
+    if constexpr (kVec) run(k_decode_tx<ELL, true, 4, 8>);
+  } else if (staged) {
+    m >= 64 ? run(k_decode_tx<ELL, true, 1, 16>) : run(k_decode_tx<ELL, true, 1, 8>);
+  } else {
+    run(k_decode_tx<ELL, false, 1, 16>);
+  }
 }
 
 int launch_decode_tx(const double* R, int ell, int m, const float* T, int npat, int d, float* ghat,
