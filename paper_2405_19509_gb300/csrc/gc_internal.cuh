@@ -147,7 +147,8 @@ int launch_encode(const double* E, const int32_t* order, const int32_t* psi, int
 // the workers whose orders are not cyclic (k_encode_any.cu); J = workers per
 // group of the cyclic kernel
 constexpr size_t kEncodeAnySmem = 220 * 1024;
-bool encode_any_applies(int N, int m, int delta, int ell, int npat, int L);
+bool encode_any_applies(int N, int m, int delta, int ell, int npat, int d, const float* G,
+                        const float* T);
 int launch_encode_any(const double* E, const int32_t* order, const int32_t* psi, int N, int m,
                       int delta, int ell, int npat, const float* G, int d, int J, float* T,
                       cudaStream_t s);

@@ -378,7 +378,7 @@ int launch_encode(const double* E, const int32_t* order, const int32_t* psi, int
   if (npat > 2147483647 || stripes > 65535 || ngroups > 65535)
     return fail(GC_ERR_UNSUPPORTED, "encode grid too large");
   const size_t smem = enc_smem_bytes(DR, V, ell, delta, J);
-  const int any_next = encode_any_applies(N, m, delta, ell, npat, L) ? 1 : 0;
+  const int any_next = encode_any_applies(N, m, delta, ell, npat, d, G, T) ? 1 : 0;
   const dim3 grid((unsigned)npat, (unsigned)stripes, (unsigned)ngroups);
   int rc;
   // two blocks of a chunk per step when ell is even

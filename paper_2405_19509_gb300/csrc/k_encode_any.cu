@@ -291,6 +291,12 @@ int any_patterns(int N, int m, int delta, int ell, int npat) {
   return 0;
 }
 
+// rows of G and T are 16-byte pieces
+bool any_vec(int L, int d, const float* G, const float* T) {
+  return L % 4 == 0 && d % 4 == 0 &&
+         (reinterpret_cast<uintptr_t>(G) | reinterpret_cast<uintptr_t>(T)) % 16 == 0;
+}
+
 template <int PB, int ELL, bool VEC>
 int launch_any_t(size_t smem, const double* E, const int32_t* order, const int32_t* psi, int N,
                  int m, int delta, int npat, const float* G, int d, int L, int J, float* T,
@@ -319,13 +325,27 @@ int launch_any_t(size_t smem, const double* E, const int32_t* order, const int32
 }  // namespace
 
 // Whether k_encode_any takes the groups that are not cyclic.  The order lies on
-// the device, so the launch is paid for cyclic orders as well (about 3 us with
+// the device, so the launch is paid for cyclic orders as well (about 2 us with
 // its scan of the order): only from 2^26 multiply-adds on, where the form that
-// reads the cache takes 60 us (0.9 us per 2^20).
-bool encode_any_applies(int N, int m, int delta, int ell, int npat, int L) {
-  return ell <= 4 && N < 32768 && m <= 4096 &&
-         (long long)npat * m * L * delta * ell >= (1LL << 26) &&
-         any_patterns(N, m, delta, ell, npat) > 0;
+// reads the cache takes 35-55 us.  That form takes 0.5-1 us per 2^20 multiply-adds, of
+// whole blocks of 512 columns, by the sizes and by how many slots are finished; a tile here
+// 1.2 us (rows that are no 16-byte pieces 0.9 us more a pattern) and its multiply-adds at 43
+// a nanosecond.  So few workers or few blocks on long rows stay there: ell = 1, delta = 4,
+// L = 2^20, m = 16 53 us against 256 here, m = 50 182 and 287; ell = 2, L = 2^19, m = 50 147 and 163,
+// m = 64 199 and 172; ell = 4, delta = 8, L = 2^18, m = 20 126 and 91.
+bool encode_any_applies(int N, int m, int delta, int ell, int npat, int d, const float* G,
+                        const float* T) {
+  const int L = (d + ell - 1) / ell;
+  const double fmas = (double)npat * m * L * delta * ell;
+  if (ell > 4 || N >= 32768 || m > 4096 || fmas < (double)(1 << 26)) return false;
+  const int PB = any_patterns(N, m, delta, ell, npat);
+  if (PB == 0) return false;
+  const long long items = (long long)((L + kAnyCols - 1) / kAnyCols) * ((npat + PB - 1) / PB);
+  const long long rounds = (items + device_sm_count() - 1) / device_sm_count();
+  const double item_us = 1.25 + (any_vec(L, d, G, T) ? 0.0 : 0.9 * PB) +
+                         (double)m * delta * ell * kAnyCols * PB / 43e3;
+  const double whole = (double)((L + 511) / 512 * 512) / L;
+  return (double)rounds * item_us < fmas * whole / (1 << 20) * 0.7;
 }
 
 int launch_encode_any(const double* E, const int32_t* order, const int32_t* psi, int N, int m,
@@ -334,8 +354,7 @@ int launch_encode_any(const double* E, const int32_t* order, const int32_t* psi,
   const int L = (d + ell - 1) / ell;
   const int PB = any_patterns(N, m, delta, ell, npat);
   const size_t smem = any_smem(N, m, delta, ell, PB);
-  const bool vec = L % 4 == 0 && d % 4 == 0 &&
-                   (reinterpret_cast<uintptr_t>(G) | reinterpret_cast<uintptr_t>(T)) % 16 == 0;
+  const bool vec = any_vec(L, d, G, T);
   auto go = [&](auto launch) {
     return launch(smem, E, order, psi, N, m, delta, npat, G, d, L, J, T, s);
   };

@@ -545,6 +545,25 @@ def test_encode_any_order(gc, N, m, delta, ell, npat, L, pad, kind):
         assert torch.equal(T2.nan_to_num(), T.nan_to_num())
 
 
+@pytest.mark.parametrize("m,delta,ell,npat,L,pad,kind,taken", [
+    (100, 8, 3, 1, 40000, 0, "random", True),    # one pattern
+    (100, 8, 3, 2, 20001, 2, "random", True),    # two, ragged rows, padded last block
+    (100, 6, 4, 3, 10003, 1, "padded", True),    # three patterns of four, empty slots
+    (100, 6, 1, 4, 30000, 0, "mixed", True),     # workers of cyclic groups
+    (16, 4, 1, 1, 1 << 20, 0, "random", False),  # few workers on long rows: summed from the cache
+])
+def test_encode_any_order_choice(gc, m, delta, ell, npat, L, pad, kind, taken):
+    """The same sums on both sides of the rule that gives a call to k_encode_any (a second launch)."""
+    order = np.stack([(np.arange(delta) * 3 + 2 * j) % m for j in range(m)]).astype(np.int32)
+    od = torch.from_numpy(order).cuda()
+    E = torch.zeros(npat, m, delta, ell, dtype=torch.float64, device="cuda")
+    psi = torch.full((npat, m), delta, dtype=torch.int32, device="cuda")
+    n0 = gc.gc_kernel_launches()
+    gc.gc_encode_with_coeffs(E, ell, od, m, m, delta, psi, torch.zeros(m, ell * L - pad, device="cuda"))
+    assert gc.gc_kernel_launches() - n0 == (2 if taken else 1)
+    test_encode_any_order(gc, m, m, delta, ell, npat, L, pad, kind)
+
+
 @pytest.mark.parametrize("ell,d", [(4, 1), (4, 2), (4, 5), (3, 1), (3, 5)])
 def test_encode_any_order_short_rows(gc, ell, d):
     """k_encode_any on rows so short that blocks before the last one are padded too, or empty,
@@ -561,7 +580,9 @@ def test_encode_any_order_short_rows(gc, ell, d):
     G = buf[16:16 + N * d].view(N, d)
     G.copy_(torch.randn(N, d, generator=gen, device="cuda"))
     E = torch.randn(npat, m, delta, ell, generator=gen, device="cuda", dtype=torch.float64)
+    n0 = gc.gc_kernel_launches()
     T = gc.gc_encode_with_coeffs(E, ell, od, N, m, delta, psi, G)
+    assert gc.gc_kernel_launches() - n0 == 2
     B = torch.nn.functional.pad(G, (0, ell * L - d)).view(N, ell, L).double()
     E.mul_((torch.arange(delta, device="cuda") < psi[:, :, None])[..., None])
     ref = sum(torch.einsum("bmk,mkc->bmc", E[:, :, p].float().double(), B[od[:, p].long()])
