@@ -166,16 +166,20 @@ Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
   // of a batch and the partial gradients are as long as they can be (2 GB of X,
   // with the exchange of the time in the consumers' way: fp32 d = 10007 102% of
   // the copy rate in one CTA, 54% in two; bf16 d = 16384 98 and 74).
-  const long long max_slice = x_dtype == GC_BF16 ? 32768 : 49152;
+  // With less than 160 KB of X an SM the rows are so few that this leaves SMs idle, or a
+  // partial gradient to every few rows (bf16 d = 16384: 32 rows 16.0 us, 11.9 with slices of
+  // half the size, 640 rows 24.3 and 20.2; fp32 d = 24576, 32 rows 10.3 and 9.1).
+  const bool few = (long long)N * n_c * row_bytes < (160LL << 10) * device_sm_count();
+  const long long max_slice = x_dtype == GC_BF16 ? (few ? 16384 : 32768) : (few ? 32768 : 49152);
   p.CL = 1;
   while (p.CL < 8 && (row_bytes + p.CL - 1) / p.CL > max_slice) p.CL *= 2;
   // Clusters of 8 fill only 120 of the 152 SMs (a cluster lives inside one
   // GPC; at most 15 clusters of 8 are co-resident), clusters of 4 fill 144:
   // fp32 rows of up to 256 KB take 64 KB slices (8 vectors a thread, one row a
-  // stage) in clusters of 4.  bf16 rows that two CTAs would take in four
+  // stage) in clusters of 4, bf16 rows of up to 128 KB 32 KB slices.  bf16 rows that two CTAs would take in four
   // vectors a thread stay in clusters of 4 (d = 32768: 70 against 68%, at
   // 256 MB 43 against 40%, before x was kept in tensor memory).
-  if (x_dtype != GC_BF16 && p.CL == 8 && row_bytes <= 4 * 65536) p.CL = 4;
+  if (p.CL == 8 && row_bytes <= 4 * (x_dtype == GC_BF16 ? 32768 : 65536)) p.CL = 4;
   if (x_dtype == GC_BF16 && p.CL == 2 && row_bytes > 2 * 3 * 512 * 16) p.CL = 4;
   p.Wc = (int)align_up((size_t)((d + p.CL - 1) / p.CL), (size_t)p.V);
   p.aligned = x_aligned && row_bytes % 16 == 0;

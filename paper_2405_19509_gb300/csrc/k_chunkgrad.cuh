@@ -850,7 +850,7 @@ Kernel pick_shape(int NT, int NVT) {
       if (NT == 512 && NVT == 8) return k_chunkgrad<T, ALIGNED, CL, 512, 8, 1>;
   } else {
     if (NT == 512 && NVT == 3) return k_chunkgrad<T, ALIGNED, CL, 512, 3, 2>;
-    if constexpr (CL == 4) {
+    if constexpr (CL == 2 || CL == 4) {
       if (NT == 512 && NVT == 2) return k_chunkgrad<T, ALIGNED, CL, 512, 2, 4>;
       if (NT == 256 && NVT == 4) return k_chunkgrad<T, ALIGNED, CL, 256, 4, 2>;
     }
