@@ -522,7 +522,7 @@ int gc_decode_batch(const double* R, int ell, const int32_t* order, int N, int m
   __nv_bfloat16* Cs = c.take<__nv_bfloat16>(plan_bytes(N, ell, npat) / sizeof(__nv_bfloat16));
   launch_holders(order, N, m, delta, sw.h, status_of(ws), s);
   if (!Ghat && decode_policy() == GC_DECODE_AUTO && mse_gram_applies(N, ell, npat, d) &&
-      mse_patterns_applies(N, ell, sw.bits)) {
+      mse_patterns_applies(N, ell, sw.bits, npat)) {
     // errors alone: the memo table and the Gram matrix of the chunk blocks
     SolveOut none{};
     none.Kp = combine_kp(N, ell);

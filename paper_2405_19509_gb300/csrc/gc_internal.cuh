@@ -229,7 +229,7 @@ GramMatrix launch_gram(const float* G, int N, int ell, int d, bool after_table, 
 int launch_mse_gram(const __nv_bfloat16* Cs, int Kp, const float* G, int N, int ell, int npat,
                     int d, double* grad_mse, Carve& ws, cudaStream_t s);
 // ... and straight from the counts and the memo table (k_mse_patterns.cu)
-bool mse_patterns_applies(int N, int ell, int bits);
+bool mse_patterns_applies(int N, int ell, int bits, int npat);
 int launch_mse_patterns(const double* R, int ell, const int32_t* psi, Holders h, int N, int m,
                         int delta, int npat, void* table_mem, int bits, const float* H,
                         const float* H_last, int d, double* coef_err, double* est,

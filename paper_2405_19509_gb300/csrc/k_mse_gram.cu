@@ -279,7 +279,8 @@ __global__ void __launch_bounds__(W * 32) k_mse_gram(const __nv_bfloat16* __rest
       sweep(std::integral_constant<int, KW>{});
     float q = 0.f;
 #pragma unroll
-    for (int t = 0; t < KW; ++t) q = fmaf(v2[t], uu[t], q);
+    for (int t = 0; t < KW; ++t)
+      q = v2[t] != 0.f ? fmaf(v2[t], uu[t], q) : q;  // lanes past the list may hold an infinite uu
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
     if (lane == 0) {  // fp64 work on one lane only

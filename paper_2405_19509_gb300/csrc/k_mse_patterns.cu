@@ -251,11 +251,13 @@ struct Shape {
   int warps;
   size_t smem;
 };
-// H in shared memory when it fits beside the lists of at least 16 warps
+// H in shared memory when it fits beside the lists of at least 16 warps; with ell = 3
+// past 128 rows the warps are worth more (N = 64, delta = 5, 20,000 patterns: 0.90 ms, 0.61
+// through the cache; ell = 2, N = 100 0.35 and 0.48, ell = 4, N = 40 0.35 and 0.60)
 Shape shape_of(int N, int ell) {
   const size_t K = (size_t)N * ell, list = K * entry_words(ell) * 4, limit = 220 * 1024;
   for (int w : {32, 24, 16})
-    if (K * K * 4 + w * list <= limit) return {true, w, K * K * 4 + w * list};
+    if ((ell != 3 || K <= 128) && K * K * 4 + w * list <= limit) return {true, w, K * K * 4 + w * list};
   for (int w : {32, 24, 16})
     if (w * list <= limit) return {false, w, w * list};
   return {false, 0, 0};
@@ -278,9 +280,15 @@ cudaError_t launch_t(const Shape& sh, int blocks, const double* R, const int32_t
 }  // namespace
 
 // Taken when the memo table is (its blocks are gathered), for the sizes the
-// register-resident holders cover.
-bool mse_patterns_applies(int N, int ell, int bits) {
-  return bits >= 0 && ell <= 4 && N <= 128 && shape_of(N, ell).warps > 0;
+// register-resident holders cover.  Past N*ell = 160 a warp's pattern costs more here
+// than in k_mse_gram, whose warps hold a row's entries in registers, until there are
+// several for each warp: N = 100, delta = 6, ell = 2, p = 0.5 2,000 patterns 40 us from the plan and
+// 74 here, 20,000 102 and 105; N = 64, ell = 4 2,000 206 and 306, 20,000 1517 and 1677; but
+// N = 128, ell = 2, 10^5 patterns 513 and 260.
+bool mse_patterns_applies(int N, int ell, int bits, int npat) {
+  const int K = N * ell;
+  return bits >= 0 && ell <= 4 && N <= 128 && shape_of(N, ell).warps > 0 &&
+         (K <= 160 || (npat >= 16384 && (ell < 4 || K < 256)));
 }
 
 int launch_mse_patterns(const double* R, int ell, const int32_t* psi, Holders h, int N, int m,

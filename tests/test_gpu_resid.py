@@ -411,8 +411,8 @@ def test_large_ell_both_paths(gc, ell):
 @pytest.mark.parametrize("N,m,delta,ell,d,npat", [
     (8, 8, 3, 1, 40, 17),        # one chunk a lane, a last batch of one pattern
     (33, 33, 5, 2, 1003, 155),   # two chunks a lane, padded last block
-    (64, 64, 7, 3, 300, 700),    # rows' sums of 32 patterns and a remainder in every warp
-    (100, 100, 6, 2, 512, 1001), # four chunks a lane, H read through the cache
+    (64, 64, 7, 3, 300, 700),    # N ell = 192, few patterns: from the plan
+    (100, 100, 6, 2, 512, 1001), # N ell = 200, few patterns: from the plan
     (64, 64, 4, 4, 256, 5000),
     (20, 60, 4, 2, 128, 99),     # explicit order: chunks with more copies than the table has bits
 ])
@@ -452,6 +452,52 @@ def test_errors_from_counts(gc, N, m, delta, ell, d, npat):
         gc.gc_mse(Rd, ell, od, N, m, delta, torch.from_numpy(psi).cuda(), Gd, ws=ws)
         with pytest.raises(gc.GCError, match="psi"):
             gc.gc_status(ws)
+
+
+@pytest.mark.parametrize("N,delta,ell,d,npat,direct", [
+    (50, 5, 3, 312, 700, True),      # H read through the cache, two chunks a lane
+    (50, 5, 3, 310, 700, True),      # ... and a padded last block
+    (100, 4, 1, 64, 3000, True),     # four chunks a lane, H in shared memory
+    (80, 6, 3, 200, 16383, False),   # N ell = 240: one pattern too few
+    (80, 6, 3, 200, 16384, True),    # four chunks a lane, through the cache, padded
+    (100, 6, 2, 128, 16400, True),   # four chunks a lane, H in shared memory beside 16 warps
+    (50, 5, 4, 130, 16384, True),    # ell = 4 through the cache, padded
+    (64, 5, 4, 128, 16384, False),   # N ell = 256, ell = 4
+    (128, 6, 2, 130, 16384, True),   # N ell = 256, ell = 2
+])
+def test_errors_from_counts_or_plan(gc, N, delta, ell, d, npat, direct):
+    """Every form of the error kernel that gc_mse chooses, and the rule that leaves the others to the
+    plan (a launch more): against the errors of the plan, and sampled patterns against the
+    definition (each chunk's projector from the pseudo-inverse of its finished columns)."""
+    m = N
+    rng = np.random.default_rng(N)
+    order = O.cyclic_order(N, m, delta)
+    R = rng.standard_normal((ell, m))
+    psi = rng.binomial(delta, rng.uniform(0.1, 0.9, size=(npat, 1)), size=(npat, m)).astype(np.int32)
+    psi[0], psi[1] = delta, 0
+    G32 = rng.standard_normal((N, d)).astype(np.float32)
+    Rd, od, pd = dev_tensors(R, order, psi)
+    Gd = torch.from_numpy(G32).cuda()
+    n0 = gc.gc_kernel_launches()
+    got = gc.gc_mse(Rd, ell, od, N, m, delta, pd, Gd)
+    assert gc.gc_kernel_launches() - n0 == (5 if direct else 6)
+    plan = gc.gc_decode_plan(Rd, ell, od, N, m, delta, pd)
+    via = gc.gc_decode_apply(plan["plan"], ell, N, npat, Gd, Ghat=False)["grad_mse"]
+    assert torch.equal(got["coef_err"], plan["coef_err"]) and torch.equal(got["est"], plan["est"])
+    assert (got["grad_mse"] - via).abs().max().item() <= 2e-4 * via.max().item()
+    L = -(-d // ell)
+    B = np.pad(G32.astype(np.float64), ((0, 0), (0, ell * L - d))).reshape(N, ell, L)
+    floor = 1e-8 * float(np.square(G32.sum(0, dtype=np.float64)).sum()) / d
+    for b in sorted({0, 1, npat - 1, *rng.integers(0, npat, size=12).tolist()}):
+        e, ce = np.zeros((ell, L)), 0.0
+        for i in range(N):
+            S = [(i - p) % N for p in range(delta) if psi[b, (i - p) % N] > p]
+            if len(S) < ell:
+                D = (R[:, S] @ np.linalg.pinv(R[:, S]) if S else np.zeros((ell, ell))) - np.eye(ell)
+                e += D @ B[i]
+                ce += np.square(D).sum()
+        assert_mse_close(got["grad_mse"][b].item(), np.square(e.reshape(-1)[:d]).sum() / d, floor, f"b={b}")
+        assert abs(got["coef_err"][b].item() - ce) <= 1e-9 * max(1.0, ce)
 
 
 @pytest.mark.parametrize("N,delta,ell,d", [(10, 4, 3, 1001), (20, 8, 8, 997), (40, 6, 5, 1500)])
