@@ -189,19 +189,18 @@ Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
   // still streams many rows, one when the rows per SM are few (ramp-up
   // dominates) or the row is longer.  Shorter rows, 128 threads: the chain of a
   // batch from its dot products to its residuals outlasts its copy, so up to
-  // four CTAs (tensor memory holds four), with at least 32 rows each (measured
-  // when a batch was four rows and met at a barrier, 100,000 fp32 rows of
-  // d = 512: 112 us with one CTA, 62 with two, 42 with four).
+  // three CTAs, with at least 32 rows each.  (Rows of at most 128 fp32 or 96 bf16
+  // vectors come here with an armed stall alone, see launch_chunkgrad.)
   const long long rows_per_sm = (long long)N * n_c / std::max(1, device_sm_count());
   int cps = (rows_per_sm >= 512 && row_bytes <= 16384) ? 2 : 1;
   if (p.NT == 128)
-    cps = (int)std::max(1LL, std::min<long long>(esz == 4 && nv <= 128 ? 4 : 3, rows_per_sm / 32));
+    cps = (int)std::max(1LL, std::min(3LL, rows_per_sm / 32));
   if (cps == 2 && p.NT == 512) p.NT = 256;  // only when nv <= 1024 (16 KB slices)
   const int need = (nv + p.NT - 1) / p.NT;
   // vectors a thread: 1, 2, 4, and for 512-thread slices past 4 vectors (fp32)
   // or 2 (bf16) the exact count, whose empty vectors would cost stage space
   // and dot products
-  p.NVT = need <= 2 ? need : 4;
+  p.NVT = need <= 2 ? (p.NT == 128 && esz == 4 ? 2 : need) : 4;
   if (x_dtype == GC_BF16 ? need == 3 && p.NT == 512 : need > 4) p.NVT = need <= 6 ? need : 8;
   p.RBM = p.NVT >= 5 ? 1 : (p.NVT >= 3 ? 2 : (p.NVT == 2 ? 4 : 8));
   // stage row: one vector per (thread, u), so reads need no bounds; a slice at

@@ -109,16 +109,12 @@ __device__ __forceinline__ void cluster_sync_all() {
                    : "memory");
 }
 
-// Load V elements (16 bytes) of a row slice from shared memory as floats.
+// V elements (16 bytes) of a row slice, as they lie and as floats.
 template <typename T>
 struct Vec;
 template <>
 struct Vec<float> {
   static constexpr int V = 4;
-  __device__ static __forceinline__ void load(const float* p, float (&o)[4]) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
-  }
   __device__ static __forceinline__ uint4 load_raw(const float* p) {
     return *reinterpret_cast<const uint4*>(p);
   }
@@ -130,9 +126,6 @@ struct Vec<float> {
 template <>
 struct Vec<__nv_bfloat16> {
   static constexpr int V = 8;
-  __device__ static __forceinline__ void load(const __nv_bfloat16* p, float (&o)[8]) {
-    unpack(load_raw(p), o);
-  }
   __device__ static __forceinline__ uint4 load_raw(const __nv_bfloat16* p) {
     return *reinterpret_cast<const uint4*>(p);
   }
@@ -839,7 +832,8 @@ Kernel pick_shape(int NT, int NVT) {
     if (NT == 256 && NVT == 2) return k_chunkgrad<T, ALIGNED, 1, 256, 2, 4>;
     if (NT == 256 && NVT == 1) return k_chunkgrad<T, ALIGNED, 1, 256, 1, 8>;
     if (NT == 128 && NVT == 2) return k_chunkgrad<T, ALIGNED, 1, 128, 2, 4>;
-    if (NT == 128 && NVT == 1) return k_chunkgrad<T, ALIGNED, 1, 128, 1, 8>;
+    if constexpr (!kF32)
+      if (NT == 128 && NVT == 1) return k_chunkgrad<T, ALIGNED, 1, 128, 1, 8>;
   }
   if constexpr (kF32 ? CL <= 4 : CL != 2)
     if (NT == 512 && NVT == 4) return k_chunkgrad<T, ALIGNED, CL, 512, 4, 2>;

@@ -353,8 +353,10 @@ __global__ void __launch_bounds__(256) k_resid_sum(const float* __restrict__ par
 
 // How GEMM 1's `tiles` tiles of nkb K blocks are dealt to `sms` CTAs: the tiles
 // past the last whole wave in nsplit K ranges.  The count with the least time by
-// the measured rates: 1.34 us a K block of a 256 x 256 tile, 8 us an epilogue
-// (it is not overlapped), the partials' bytes at 6 TB/s.
+// rates measured at n_w = 256 and taken as proportional to it: 1.34 us a K block of a
+// 256 x 256 tile, 8 us an epilogue, the partials' bytes at 6 TB/s.  The epilogue is
+// added to each round, as it is at n_w = 256; up to n_w = 128 the accumulators are
+// doubled and it overlaps the next tile, so there the splits are a little too few.
 struct Split {
   int full_tiles, split_tiles, nsplit;
 };

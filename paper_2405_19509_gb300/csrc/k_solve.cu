@@ -545,7 +545,6 @@ static void run_solve(const double* R, const int32_t* psi, Holders h, int N, int
 constexpr int kFewThreads = 256, kFewWarps = kFewThreads / 32;
 constexpr int kFewChunks = 8;      // chunks a block
 constexpr int kFewR = 4096;        // doubles of R staged (32 KB)
-constexpr int kFewBlocks = 8 * 152;  // at most: eight blocks an SM
 template <int ELL>
 __global__ void __launch_bounds__(kFewThreads) k_coeff_few(const double* __restrict__ R,
                                                            const int32_t* __restrict__ order,
@@ -655,7 +654,7 @@ int launch_coeffs(const double* R, int ell, const int32_t* order, const int32_t*
   const bool only_e = out.E && !out.C && !out.Cs && !out.delta_out && !out.support &&
                       !out.coef_err && !out.est;
   const int groups = (N + kFewChunks - 1) / kFewChunks;
-  if (only_e && bits < 0 && (long long)groups * npat <= kFewBlocks && ell * m <= kFewR) {
+  if (only_e && bits < 0 && (long long)groups * npat <= 8LL * device_sm_count() && ell * m <= kFewR) {
     const dim3 grid((unsigned)groups, (unsigned)npat);
 #define GC_FEW(E_) \
   case E_: k_coeff_few<E_><<<grid, kFewThreads, 0, s>>>(R, order, psi, N, m, delta, out.E, status); break;
