@@ -166,10 +166,10 @@ Plan make_plan(int N, int n_c, int d, int x_dtype, bool x_aligned) {
   // of a batch and the partial gradients are as long as they can be (2 GB of X,
   // with the exchange of the time in the consumers' way: fp32 d = 10007 102% of
   // the copy rate in one CTA, 54% in two; bf16 d = 16384 98 and 74).
-  // With less than 160 KB of X an SM the rows are so few that this leaves SMs idle, or a
-  // partial gradient to every few rows (bf16 d = 16384: 32 rows 16.0 us, 11.9 with slices of
-  // half the size, 640 rows 24.3 and 20.2; fp32 d = 24576, 32 rows 10.3 and 9.1).
-  const bool few = (long long)N * n_c * row_bytes < (160LL << 10) * device_sm_count();
+  // Fewer than five rows an SM leave SMs idle that way, or write a partial gradient for
+  // every few rows (bf16 d = 16384: 32 rows 16.0 us, 11.9 with slices of half the size, 640
+  // rows 24.3 and 20.2; d = 10007, 1024 rows 12.1 and 14.6; fp32 d = 24576, 32 rows 10.3 and 9.1).
+  const bool few = (long long)N * n_c < 5LL * device_sm_count();
   const long long max_slice = x_dtype == GC_BF16 ? (few ? 16384 : 32768) : (few ? 32768 : 49152);
   p.CL = 1;
   while (p.CL < 8 && (row_bytes + p.CL - 1) / p.CL > max_slice) p.CL *= 2;

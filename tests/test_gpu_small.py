@@ -266,11 +266,11 @@ def test_chunk_grads_ragged(gc, d, n_c, N, off, dtype):
 @pytest.mark.parametrize("d,n_c,N,dtype", [
     (16384, 4, 3, torch.bfloat16),    # two CTAs of 512 threads a row
     (12285, 5, 2, torch.bfloat16),    # two of 256, ragged
-    (12288, 400, 9, torch.bfloat16),  # as many rows as one CTA takes whole
+    (12288, 90, 9, torch.bfloat16),   # as many rows as one CTA takes whole
     (40000, 3, 2, torch.bfloat16),    # four, three vectors a thread
     (24576, 4, 2, torch.float32),     # four
     (10000, 7, 3, torch.float32),     # two
-    (10000, 90, 30, torch.float32),   # whole
+    (10000, 27, 30, torch.float32),   # whole
 ])
 def test_chunk_grads_few_long_rows(gc, d, n_c, N, dtype):
     """Few rows are cut into smaller slices than many."""
