@@ -160,7 +160,7 @@ __device__ __forceinline__ unsigned long long warp_ell_th(unsigned long long key
 
 constexpr float kBelow = 1.f - 0x1p-20f, kAbove = 1.f + 0x1p-20f;
 // Chunks about the largest time that a warp forms one by one; more of them are ties.
-constexpr int kTrigExact = 4;
+constexpr int kTrigExact = 2;
 constexpr int kTrigHolders = 8192;  // holder words staged in shared memory (32 KB)
 
 // ZERO: theta = 0 (two kernels, each with the registers it needs).
@@ -268,13 +268,15 @@ __global__ void __launch_bounds__(32 * kWarpsPerBlock, blocks_per_sm(ELL))
       // the largest time: of the few chunks about top (one as a rule); else a tie
       auto largest = [&](float top, float bst, float scd, int chunk, bool full) {
         const float lim = top * kBelow;
-        const unsigned lanes = __ballot_sync(0xffffffffu, bst >= lim);
+        unsigned lanes = __ballot_sync(0xffffffffu, bst >= lim);
         unsigned long long mx = 0;
-        if (__popc(lanes) > kTrigExact || __any_sync(0xffffffffu, scd >= lim)) {
-          tied |= full ? 2u : 1u;
-        } else {
-          for (unsigned c = lanes; c; c &= c - 1)
-            mx = max(mx, exact(__shfl_sync(0xffffffffu, chunk, __ffs(c) - 1), full));
+        for (int left = kTrigExact; lanes; lanes &= lanes - 1) {
+          const int src = __ffs(lanes) - 1;
+          if (left-- == 0 || __shfl_sync(0xffffffffu, scd, src) >= lim) {
+            tied |= full ? 2u : 1u;
+            break;
+          }
+          mx = max(mx, exact(__shfl_sync(0xffffffffu, chunk, src), full));
         }
         return mx;
       };
