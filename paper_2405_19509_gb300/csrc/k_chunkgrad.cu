@@ -309,7 +309,7 @@ int launch_chunkgrad(const void* X, int x_dtype, const float* y, const float* w,
   // rows per SM of short rows is refused
   if (N == 1 && (long long)n_c / std::max(1, device_sm_count()) >= 512 &&
       (long long)d * (x_dtype == GC_BF16 ? 2 : 4) <= 16384)
-    return fail(GC_ERR_UNSUPPORTED, "chunk of %d rows spans too many row blocks", n_c);
+    return fail(GC_ERR_UNSUPPORTED, "one chunk of %d short rows: at most 512 per SM", n_c);
   if (N > 65535) return fail(GC_ERR_UNSUPPORTED, "N=%d exceeds 65535 chunks", N);
   cudaError_t e = cudaSuccess;
   if (ps.valid) {

@@ -1,13 +1,13 @@
 """The two paths of the batched decode against the oracle and each other.
 
 Every decode block Pi_{b,i} is I_ell when Delta_i >= ell (Sec. II-A), so the
-library writes the rows of a 128-row tile either as sum_i g_{D_i} plus the
-non-identity blocks (residual path) or by the tensor-core GEMM C . G; the
-choice is made per tile on the device (gc_set_decode_policy).  These tests
-force each policy and let the automatic one mix them: tiles of exact and of
-approximate patterns side by side, patterns straddling two tiles (ell = 3),
-lists longer than the residual path holds, ragged block lengths, and a
-decode matrix that is not a projector (gc_decode_combine)."""
+library writes a pattern either as sum_i g_{D_i} plus its non-identity blocks
+(residual path) or by the tensor-core GEMM C . G; the choice is made per
+pattern on the device (gc_set_decode_policy).  These tests force each policy
+and let the automatic one mix them: exact and approximate patterns side by
+side, patterns straddling two row tiles (ell = 3), lists longer than the
+residual path holds, row tiles that are mostly the GEMM's, ragged block
+lengths, and a decode matrix that is not a projector (gc_decode_combine)."""
 import numpy as np
 import pytest
 import torch
@@ -55,9 +55,9 @@ def _copies(order, psi, N):
 
 
 def _residual_rows(nnz, ell, ksp):
-    """Rows the residual policy leaves off the GEMM: a 128-row tile stays on
-    the residual path unless a pattern overlapping it has more than `ksp`
-    non-identity blocks or more than 32 of its rows need corrections."""
+    """Rows that the residual policy leaves off the GEMM (it goes by pattern; this
+    keeps those of 128-row tiles without a pattern of more than `ksp` blocks and
+    with at most 32 corrected rows, a part of them)."""
     npat = nnz.shape[0]
     M = npat * ell
     row_pat = np.arange(M) // ell
@@ -81,8 +81,7 @@ def _tiny_G():
 @pytest.mark.parametrize("ell", [1, 2, 3])
 def test_policies_every_tiny_pattern(gc, ell):
     """All 4,096 patterns of the 6-worker workload plus 256 seeded ones under
-    each policy: decoded gradients and errors against the oracle (tiles with
-    more than 32 corrected rows stay on the GEMM under every policy)."""
+    each policy: decoded gradients and errors against the oracle."""
     cfg = get("tiny")
     N, m, delta, d = cfg.N, cfg.m, cfg.delta, cfg.d
     order = O.cyclic_order(N, m, delta)
@@ -107,8 +106,8 @@ def test_policies_every_tiny_pattern(gc, ell):
 @pytest.mark.parametrize("ell", [2, 3])
 def test_mixed_and_straddling_tiles(gc, ell):
     """Runs of 64 exact patterns (all workers finished) alternate with runs of
-    uniformly random ones, so the automatic policy sends some tiles to each
-    path; with ell = 3 patterns straddle tile boundaries."""
+    uniformly random ones, so the automatic policy may send some patterns to
+    each path; with ell = 3 patterns straddle the GEMM's row tiles."""
     cfg = get("tiny")
     N, m, delta, d = cfg.N, cfg.m, cfg.delta, cfg.d
     order = O.cyclic_order(N, m, delta)
@@ -140,9 +139,9 @@ def test_mixed_and_straddling_tiles(gc, ell):
 
 def test_list_overflow_goes_to_the_gemm(gc):
     """m = N = 64, delta = 8, l = 2 with Binomial(8, 0.3) patterns: nearly every
-    pattern needs corrections, more rows than a residual tile holds (32), so
-    even the residual policy must decode those tiles on the GEMM; sampled
-    patterns, the heaviest included, against the oracle."""
+    pattern needs corrections, those with more than the list holds (32) on the
+    GEMM even under the residual policy; sampled patterns, the heaviest
+    included, against the oracle."""
     cfg = get("mse_sweep")
     N, m, delta, ell, d = cfg.N, cfg.m, cfg.delta, 2, 2048
     order = O.cyclic_order(N, m, delta)
@@ -168,7 +167,7 @@ def test_list_overflow_goes_to_the_gemm(gc):
 
 def _sparse_stragglers(rng, npat, m, delta, every):
     """Every worker finished, except in every `every`-th pattern (offset 1),
-    whose counts are uniform in 0..delta: residual tiles with corrected rows."""
+    whose counts are uniform in 0..delta: corrected patterns among exact ones."""
     psi = np.full((npat, m), delta, dtype=np.int32)
     idx = np.arange(1, npat, every)
     psi[idx] = rng.integers(0, delta + 1, size=(idx.size, m))
@@ -178,7 +177,7 @@ def _sparse_stragglers(rng, npat, m, delta, every):
 @pytest.mark.parametrize("ell", [1, 2, 3])
 def test_sparse_stragglers_tiny(gc, ell):
     """4096 patterns of the 6-worker workload, one in five with stragglers:
-    the residual tiles now hold corrected rows (the list and slot machinery);
+    corrected patterns among exact ones on the residual path;
     every pattern against the oracle under each policy."""
     cfg = get("tiny")
     N, m, delta, d = cfg.N, cfg.m, cfg.delta, cfg.d
@@ -367,7 +366,7 @@ def test_combine_non_projector_matrix(gc):
 def test_large_ell_both_paths(gc, ell):
     """The widest communication factors of the build: N = m = 10 chunks and
     workers, delta = 8, l = 5 and 8 (at l = 8 exact recovery needs every copy;
-    lists hold 8 blocks, so longer ones send their tiles to the GEMM), d not a
+    lists hold 8 blocks, patterns with more take the GEMM), d not a
     multiple of l.  Mostly exact patterns, mild stragglers and a few uniform
     ones; every pattern against the oracle under each policy."""
     N = m = 10

@@ -340,7 +340,7 @@ def test_chunk_grads_infinite_w(gc, d, n_c, dtype):
 
 
 def test_chunk_grads_unaligned_X(gc):
-    """An X view starting 4 bytes past a 16-byte boundary takes the plain-load path."""
+    """An X view starting 4 bytes past a 16-byte boundary: short rows read word by word."""
     N, n_c, d = 3, 8, 256
     base = torch.randn(N * n_c * d + 1, generator=torch.Generator().manual_seed(9))
     X = base[1:].view(N * n_c, d)
