@@ -408,7 +408,8 @@ int launch_encode(const double* E, const int32_t* order, const int32_t* psi, int
 // workers would mostly run) and eight below.  m = 256, ell = 2, L = 2^19: 76 us = 7.1
 // TB/s with 16-byte loads, 90 with either of 4 bytes.  ell = 1, m = 256, L = 2^20: 161 us
 // with sixteen, 169 with eight, 256 with 16-byte loads (m = 200, L = 20000, 8 patterns 25, 32
-// and 95).  m = 50, ell = 3, L = 101, 3,000 patterns: 16.3 us with sixteen, 12.3 with eight.
+// and 95).  m = 50, ell = 3, L = 101, 3,000 patterns: 16.3 us with sixteen, 12.3 with eight;
+// but 5 patterns of m = 38, ell = 3, L = 11040 (with their encode) 41.9 and 44.0.
 constexpr int kDecodeSmemM = 1024;
 template <int ELL, bool STAGED, int V, int U>
 __global__ void k_decode_tx(const double* __restrict__ R, int m, const float* __restrict__ T,
@@ -487,7 +488,9 @@ static void run_decode_tx(const double* R, int m, const float* T, int npat, int 
   if (vec) {
     if constexpr (kVec) run(k_decode_tx<ELL, true, 4, 8>);
   } else if (staged) {
-    m >= 64 ? run(k_decode_tx<ELL, true, 1, 16>) : run(k_decode_tx<ELL, true, 1, 8>);
+    // ... and with more than two steps' workers where few threads are there to load
+    const bool deep = m >= 64 || (m > 32 && tot < 1024LL * device_sm_count());
+    deep ? run(k_decode_tx<ELL, true, 1, 16>) : run(k_decode_tx<ELL, true, 1, 8>);
   } else {
     run(k_decode_tx<ELL, false, 1, 16>);
   }

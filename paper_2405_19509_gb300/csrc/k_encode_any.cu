@@ -108,8 +108,9 @@ __global__ void __launch_bounds__(kAnyThreads, 1)
     const int cl = VEC ? 4 * (threadIdx.x % (kAnyCols / 4)) : lane;
     auto fetch = [&](int c0, int u, float (&v)[VEC ? 4 : 1]) {
       const int r = r0 + u * kRstep, i = r / ELL, k = r - i * ELL;
-      const bool in = r < rows && c0 + cl < min(L, d - k * L);
-      const float* src = G + (size_t)i * d + (k * L + c0 + cl);
+      const int col = k * L + c0 + cl;
+      const bool in = r < rows && c0 + cl < L && col < d;
+      const float* src = G + (size_t)i * d + col;
       if constexpr (VEC) {
         const float4 q = in ? __ldg(reinterpret_cast<const float4*>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
         v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
